@@ -1,23 +1,15 @@
-// npm_tc.cu -- tensor-core path of the NPM forward pass on sm_103a.
+// npm_tc.cu -- tensor-core path on sm_103a: the training kernel, the
+// arrangement of the weights for the MMAs, the model's tensor-core state and
+// the dispatch of the forward kernels (npm_tc_forward.cuh, npm_tc_tiny.cu).
 //
-// One persistent CTA of 128 threads walks 128-query tiles; thread t owns query
-// t of the tile, which is row t of every MMA and lane t of tensor memory.
-// Per tile:
-//   encode : thread t gathers the 8 corners of every level from the FP16
-//            grid copy, blends in FP32 (Sec. 5.1, Eq. 11), appends the
-//            product-mode SH encodings (Sec. 4.3), and writes its row of the
-//            BF16 activation tile A (shared memory, UMMA K-major layout).
-//   layers : one elected thread issues tcgen05.mma kind::f16 (BF16 x BF16 ->
-//            FP32 in TMEM), M = 128, N = layer width, K in steps of 16, and
-//            commits to an mbarrier; every thread then reads its accumulator
-//            row with tcgen05.ld, applies ReLU and writes the next A row.
-//   decode : the last accumulator row (4K FP32 raw outputs) stays in
-//            registers; the thread maps it (Table 1), samples a lobe and a
-//            direction (Sec. 5.3) and evaluates the mixture (Eq. 4) in FP32.
-// Weights (BF16, pre-arranged in the UMMA layout) arrive once per CTA by a
-// bulk asynchronous copy. Every wait on an mbarrier is bounded: on timeout
-// the kernel records NPM_ERR_TIMEOUT in the status word, releases its tensor
-// memory and returns.
+// The training kernel runs one CTA of 256 threads over 128-sample tiles, two
+// threads per sample; activations and gradients are BF16 operand tiles in
+// shared memory (UMMA K-major layout), one elected thread issues
+// tcgen05.mma kind::f16 with FP32 accumulation in tensor memory and commits
+// to an mbarrier, and the threads read their accumulator lanes with
+// tcgen05.ld. Weights arrive once per CTA by a bulk asynchronous copy. Every
+// wait on an mbarrier is bounded: on timeout the kernel records
+// NPM_ERR_TIMEOUT in the status word, releases its tensor memory and returns.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdlib.h>
@@ -39,44 +31,6 @@ namespace {
 // --------------------------------------------------------------- encode
 
 // Thread t writes row t of A (BF16, kp columns) for its query.
-// Table entry loads: FP16 copy (inference) or FP32 master (training).
-__device__ __forceinline__ float2 load_feat2(const __half* g, uint32_t idx) {
-    const uint32_t raw = __ldg(reinterpret_cast<const unsigned int*>(g) + idx);
-    return __half22float2(*reinterpret_cast<const __half2*>(&raw));
-}
-__device__ __forceinline__ float2 load_feat2(const float* g, uint32_t idx) {
-    return __ldg(reinterpret_cast<const float2*>(g) + idx);
-}
-// Features 4h .. 4h+3 of entry idx of a table with F = 4 or 8 features: the
-// raw 8-byte FP16 or 16-byte FP32 vector, widened to float4 at use.
-__device__ __forceinline__ uint2 load_raw4(const __half* g, uint32_t idx, int F, int h) {
-    return __ldg(reinterpret_cast<const uint2*>(g) + (size_t)idx * (F >> 2) + h);
-}
-__device__ __forceinline__ float4 load_raw4(const float* g, uint32_t idx, int F, int h) {
-    return __ldg(reinterpret_cast<const float4*>(g) + (size_t)idx * (F >> 2) + h);
-}
-__device__ __forceinline__ float4 widen4(uint2 raw) {
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ float4 widen4(float4 v) { return v; }
-__device__ __forceinline__ float load_feat(const __half* e, int f) { return __half2float(e[f]); }
-__device__ __forceinline__ float load_feat(const float* e, int f) { return __ldg(e + f); }
-
-// Entry index of corner c of a cell (the corner_idx8 formula for one
-// corner). The two-level gather below issues each corner's load as soon as
-// its index is formed, which schedules better there than forming all 16
-// indices first.
-__device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const Cell& cl, int c) {
-    const uint32_t i = cl.c[0] + (c & 1), j = cl.c[1] + ((c >> 1) & 1), k = cl.c[2] + ((c >> 2) & 1);
-    if ((cfg.dense_mask >> l) & 1u) {
-        const uint32_t D = (uint32_t)cfg.level_res[l];
-        return bounded_index(i + D * (j + D * k), D * D * D);
-    }
-    return (i ^ (j * 2654435761u) ^ (k * 805459861u)) & cfg.table_mask;
-}
-
 // F2: the grid has 2 features per level (compile-time), so two levels' 16
 // corner loads can be in flight before blending; other grids take the
 // generic per-level path (fewer registers).
@@ -263,470 +217,6 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
     }
     const int kend = pad_all ? kp : min(kp, (k + 7) & ~7);
     for (; k < kend; ++k) store_one(sA, tile_off(row, k, kp), 0.0f, lo);
-}
-
-// --------------------------------------------------------------- decode
-
-// KEXACT: the model has exactly KMAX lobes (no per-lobe bound checks).
-template <int KMAX, bool KEXACT>
-__device__ __forceinline__ void tc_decode(const TcCfg& tc, const float (&raw)[4 * KMAX], int64_t j,
-                                          bool valid, int64_t ld, const float* __restrict__ uin,
-                                          float ufrac, bool sample, float* __restrict__ dir_out,
-                                          float* __restrict__ pdf_out,
-                                          float* __restrict__ mix_out, bool log_pdf) {
-    const DevCfg& cfg = tc.base;
-    const int K = KEXACT ? KMAX : cfg.K;
-    Lobe lob[KMAX];
-    float cn[KMAX];
-    float mx = -INFINITY;
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i)
-        if (i < K) mx = fmaxf(mx, raw[4 * i]);
-    float ssum = 0.0f;
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i)
-        if (i < K) {
-            lob[i].lam = __expf(raw[4 * i] - mx);
-            ssum += lob[i].lam;
-        }
-    const float inv = __fdividef(1.0f, ssum);  // ssum in [1, K]
-#pragma unroll
-    for (int i = 0; i < KMAX; ++i)
-        if (i < K) {
-            lob[i].lam *= inv;
-            float th, ph;
-            decode_lobe_fast(cfg.kappa_act, raw[4 * i + 1], raw[4 * i + 2], raw[4 * i + 3], lob[i], &th, &ph);
-            cn[i] = vmf_scaled_norm_fast(lob[i].kap);
-            if (mix_out && valid) {
-                mix_out[(4 * i + 0) * ld + j] = lob[i].lam;
-                mix_out[(4 * i + 1) * ld + j] = lob[i].kap;
-                mix_out[(4 * i + 2) * ld + j] = th;
-                mix_out[(4 * i + 3) * ld + j] = ph;
-            }
-        }
-    float w[3] = {0.0f, 0.0f, 1.0f};
-    bool uni = false;
-    if (sample) {
-        float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
-        if (valid) {
-            u0 = uin[j];
-            u1 = uin[ld + j];
-            u2 = uin[2 * ld + j];
-            uni = ufrac > 0.0f && uin[3 * ld + j] < ufrac;
-        }
-        if (uni) {
-            uniform_sphere(u1, u2, w);
-        } else {
-            // Smallest lobe i with u0 < lambda_0 + ... + lambda_i (last if none).
-            int sel = K - 1;
-            float cum = 0.0f;
-            bool found = false;
-#pragma unroll
-            for (int i = 0; i < KMAX; ++i)
-                if (i < K) {
-                    cum += lob[i].lam;
-                    if (!found && u0 < cum) {
-                        sel = i;
-                        found = true;
-                    }
-                }
-            Lobe sl = lob[0];
-#pragma unroll
-            for (int i = 1; i < KMAX; ++i)
-                if (i == sel) sl = lob[i];
-            if (tc.fp32) vmf_sample(sl, u1, u2, w);  // the FP32 path's sampler
-            else vmf_sample_rp(sl, u1, u2, w);
-        }
-    } else if (valid) {
-        w[0] = uin[j];
-        w[1] = uin[ld + j];
-        w[2] = uin[2 * ld + j];
-    }
-    float pv = 0.0f;
-    if (!sample && log_pdf) {
-        // log V (Eq. 4 in log-sum-exp form), the weights' logs taken from
-        // the logits so that they stay finite where lambda_i underflows.
-        const float lnorm = mx + __logf(ssum);
-        float a[KMAX];
-        float m = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i)
-            if (i < K) {
-                const float d = lob[i].mu[0] * w[0] + lob[i].mu[1] * w[1] + lob[i].mu[2] * w[2];
-                a[i] = (raw[4 * i] - lnorm) + __logf(cn[i]) + lob[i].kap * (d - 1.0f);
-                m = fmaxf(m, a[i]);
-            }
-        float s = 0.0f;
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i)
-            if (i < K) s += __expf(a[i] - m);
-        pv = m + __logf(s);
-    } else {
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i)
-            if (i < K) pv += lob[i].lam * vmf_eval_fast(lob[i], cn[i], w[0], w[1], w[2]);
-        if (sample && ufrac > 0.0f) pv = ufrac * kInv4Pi + (1.0f - ufrac) * pv;
-    }
-    if (valid) {
-        if (sample) {
-            dir_out[j] = w[0];
-            dir_out[ld + j] = w[1];
-            dir_out[2 * ld + j] = w[2];
-        }
-        pdf_out[j] = pv;
-    }
-}
-
-// Warp-per-query form of the decode, sample and density (Table 1, Sec. 5.3,
-// Eq. 4): lane l of a warp owns lobe l mod KMAX of one query, so a warp
-// serves 32 / KMAX queries per pass and KMAX passes cover its 32 rows. The
-// raw outputs of the tile are staged in shared memory (row stride 4 KMAX + 4
-// floats keeps both the row writes and the lobe reads free of bank
-// conflicts). Softmax and density are reductions over the query's lanes;
-// the lobe choice takes the running sum of the weights in lobe order (a
-// serial scan, the same rounding as the thread-per-row form) and a ballot;
-// every lane samples its own lobe and the chosen lane's direction is
-// broadcast. Measured against tc_decode (one thread per query).
-template <int KMAX>
-__device__ __forceinline__ void tc_decode_warp(const TcCfg& tc, const float* __restrict__ sRaw, int warp, int lane,
-                                               int64_t j0, int64_t n, int64_t ld, const float* __restrict__ uin,
-                                               float ufrac, bool sample, float* __restrict__ dir_out,
-                                               float* __restrict__ pdf_out, float* __restrict__ mix_out,
-                                               bool log_pdf) {
-    constexpr int RS = 4 * KMAX + 4;
-    constexpr int QP = 32 / KMAX;  // queries per pass
-    constexpr unsigned kAll = 0xffffffffu;
-    const DevCfg& cfg = tc.base;
-    const int K = cfg.K;
-    const int i = lane & (KMAX - 1);
-    const int qsub = lane / KMAX;
-    const unsigned seg = KMAX == 32 ? kAll : (((1u << KMAX) - 1u) << (qsub * KMAX));
-    const bool act = i < K;
-#pragma unroll 1
-    for (int p = 0; p < KMAX; ++p) {
-        const int r = warp * 32 + p * QP + qsub;
-        const int64_t j = j0 + r;
-        const bool valid = j < n;
-        const float4 rv = *reinterpret_cast<const float4*>(sRaw + r * RS + 4 * i);
-        float mx = act ? rv.x : -INFINITY;
-#pragma unroll
-        for (int o = 1; o < KMAX; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kAll, mx, o));
-        const float e = act ? __expf(rv.x - mx) : 0.0f;
-        float ssum = e;
-#pragma unroll
-        for (int o = 1; o < KMAX; o <<= 1) ssum += __shfl_xor_sync(kAll, ssum, o);
-        Lobe L;
-        L.lam = e * __fdividef(1.0f, ssum);
-        float th, ph;
-        decode_lobe_fast(cfg.kappa_act, rv.y, rv.z, rv.w, L, &th, &ph);
-        const float cn = vmf_scaled_norm_fast(L.kap);
-        if (mix_out && valid && act) {
-            mix_out[(4 * i + 0) * ld + j] = L.lam;
-            mix_out[(4 * i + 1) * ld + j] = L.kap;
-            mix_out[(4 * i + 2) * ld + j] = th;
-            mix_out[(4 * i + 3) * ld + j] = ph;
-        }
-        float w[3] = {0.0f, 0.0f, 1.0f};
-        bool uni = false;
-        if (sample) {
-            float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
-            if (valid) {
-                u0 = uin[j];
-                u1 = uin[ld + j];
-                u2 = uin[2 * ld + j];
-                uni = ufrac > 0.0f && uin[3 * ld + j] < ufrac;
-            }
-            // Running sum of the weights in lobe order.
-            float cum = i == 0 ? L.lam : 0.0f;
-#pragma unroll
-            for (int k = 1; k < KMAX; ++k) {
-                const float prev = __shfl_up_sync(kAll, cum, 1);
-                if (i == k) cum = prev + L.lam;
-            }
-            const unsigned hit = __ballot_sync(kAll, act && u0 < cum) & seg;
-            const int sel = hit ? __ffs(hit) - 1 - qsub * KMAX : K - 1;
-            float d[3];
-            if (uni) uniform_sphere(u1, u2, d);
-            else vmf_sample_rp(L, u1, u2, d);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) w[a] = __shfl_sync(kAll, d[a], qsub * KMAX + sel);
-        } else if (valid) {
-            w[0] = uin[j];
-            w[1] = uin[ld + j];
-            w[2] = uin[2 * ld + j];
-        }
-        float pv;
-        if (!sample && log_pdf) {
-            const float dd = L.mu[0] * w[0] + L.mu[1] * w[1] + L.mu[2] * w[2];
-            const float a = act ? (rv.x - mx) - __logf(ssum) + __logf(cn) + L.kap * (dd - 1.0f) : -INFINITY;
-            float m = a;
-#pragma unroll
-            for (int o = 1; o < KMAX; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-            float sx = act ? __expf(a - m) : 0.0f;
-#pragma unroll
-            for (int o = 1; o < KMAX; o <<= 1) sx += __shfl_xor_sync(kAll, sx, o);
-            pv = m + __logf(sx);
-        } else {
-            pv = act ? L.lam * vmf_eval_fast(L, cn, w[0], w[1], w[2]) : 0.0f;
-#pragma unroll
-            for (int o = 1; o < KMAX; o <<= 1) pv += __shfl_xor_sync(kAll, pv, o);
-            if (sample && ufrac > 0.0f) pv = ufrac * kInv4Pi + (1.0f - ufrac) * pv;
-        }
-        if (valid && i == 0) {
-            if (sample) {
-                dir_out[j] = w[0];
-                dir_out[ld + j] = w[1];
-                dir_out[2 * ld + j] = w[2];
-            }
-            pdf_out[j] = pv;
-        }
-    }
-}
-
-// --------------------------------------------------------------- kernel
-
-// NL > 0: the network has exactly NL layers and KMAX lobes (loops over
-// layers, output chunks and lobes unrolled at compile time); NL = 0: any
-// layer count and K <= KMAX. WARPDEC: the warp-per-query decode
-// (tc_decode_warp) instead of one thread per query. G32: the grid table is
-// the FP32 master table (the FP32-accuracy mode). G: tile groups per CTA.
-// Grid table type of the forward kernel: the FP16 copy, or the FP32 master
-// table (inference weights) in the FP32-accuracy mode.
-template <bool G32>
-using GridT = typename std::conditional<G32, float, __half>::type;
-
-// A CTA of G tile groups (128 threads each) holds one copy of the weights;
-// each group has its own activation tiles, tensor-memory columns, MMA
-// barrier and named barrier, and walks its own tiles. Such a CTA runs alone
-// on its SM; single-group CTAs are compiled for as many per SM as the
-// shapes that use them fit.
-__host__ __device__ constexpr int tc_min_blocks(int kmax, bool f2, int nl, int g) {
-    return g > 1 ? 1 : (kmax == 4 && !f2) ? (nl == 3 ? 8 : 6) : (kmax == 8 ? 3 : 1);
-}
-
-template <int KMAX, bool F2, int NL, bool WARPDEC = false, bool G32 = false, int G = 1>
-__global__ void __launch_bounds__(kThreads * G, tc_min_blocks(KMAX, F2, NL, G)) k_forward_tc(const __grid_constant__ TcCfg tc,
-                                                         const GridT<G32>* __restrict__ grid_h,
-                                                         const uint8_t* __restrict__ wblob,
-                                                         const __grid_constant__ QueryBatch qb,
-                                                         int* __restrict__ status) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    const int nsplit = tc.split ? 2 : 1;               // activation tiles (hi, residual)
-    const int nw = (tc.split || tc.f16) ? 2 : 1;       // weight blobs (hi, residual)
-    const int g = G > 1 ? (int)(threadIdx.x >> 7) : 0;  // tile group
-    const int t = G > 1 ? (int)(threadIdx.x & 127) : (int)threadIdx.x;  // row of the group's tile
-    const int warp = t >> 5;                            // warp of the group (its TMEM lane quarter)
-    const uint32_t gbytes = nsplit * (tc.a0_bytes + tc.a_bytes);  // activation tiles of a group
-    uint8_t* sW = smem;
-    uint8_t* sG0 = smem + nw * tc.w_bytes;
-    uint8_t* sA = sG0 + g * gbytes + nsplit * tc.a0_bytes;  // inputs of layers >= 1
-    uint8_t* sA0 = tc.a0_bytes ? sG0 + g * gbytes : sA;    // layer-0 input (encoding)
-    const uint32_t a0_lo = tc.a0_bytes ? tc.a0_bytes : tc.a_bytes;  // its residual tile
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sG0 + G * gbytes);  // [0] weights, [1 + g] mma
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 1 + G);
-    const uint32_t bar_mma = smem_u32(&bars[1 + g]);
-    const uint32_t bar_w = smem_u32(&bars[0]);
-    // Tensor-memory columns of the CTA (a power of two: the groups' columns
-    // rounded up).
-    uint32_t cta_cols = 32;
-    while (cta_cols < (uint32_t)G * tc.tmem_cols) cta_cols <<= 1;
-
-    if (threadIdx.x < 32) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(tslot)),
-                     "r"(cta_cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i <= G; ++i) mbar_init(smem_u32(&bars[i]), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tslot + (uint32_t)g * tc.tmem_cols;
-
-    // Weights: one bulk asynchronous copy global -> shared.
-    if (threadIdx.x == 0) {
-        const uint32_t wb = (uint32_t)nw * tc.w_bytes;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_w), "r"(wb)
-                     : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                smem_u32(sW)),
-            "l"(wblob), "r"(wb), "r"(bar_w)
-            : "memory");
-    }
-    // The all-zero 8-column chunks of the encoding are written once: the
-    // layer-0 buffer holds nothing else.
-    if (tc.a0_bytes) {
-        const int kp0 = tc.layer[0].Kp;
-        for (int c = (tc.enc_width + 7) >> 3; c < (kp0 >> 3); ++c) {
-            *reinterpret_cast<uint4*>(sA0 + tile_off(t, 8 * c, kp0)) = make_uint4(0u, 0u, 0u, 0u);
-            if (tc.split)
-                *reinterpret_cast<uint4*>(sA0 + a0_lo + tile_off(t, 8 * c, kp0)) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
-    bool ok = !__syncthreads_or(threadIdx.x < 32 && !mbar_wait_bounded(bar_w, 0));
-    uint32_t phase = 0;
-    const uint32_t sA_addr = smem_u32(sA), sA0_addr = smem_u32(sA0);
-    const uint32_t sW_addr = smem_u32(sW);
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const int L = NL > 0 ? NL : tc.base.n_layers;
-    constexpr int kUnrollL = NL > 0 ? NL : 1;
-    constexpr int kUnrollC = NL > 0 ? NPM_MAX_WIDTH / 16 : 1;
-
-    int64_t ntiles = qb.total_tiles, n0 = qb.seg[0].n;
-    if (qb.n_dev) {
-        n0 = *qb.n_dev;
-        ntiles = (n0 + kTile - 1) / kTile;
-    }
-    const int64_t stride = (int64_t)gridDim.x * G;
-    for (int64_t tile = (int64_t)blockIdx.x * G + g; ok && tile < ntiles; tile += stride) {
-        int sg = 0;
-        while (sg + 1 < qb.nseg && tile >= qb.seg[sg + 1].tile0) ++sg;
-        const QuerySeg& S = qb.seg[sg];
-        const int64_t n = (sg == 0 && qb.n_dev) ? n0 : S.n;
-        const int64_t ld = S.ld;
-        const int64_t j = (tile - S.tile0) * kTile + t;
-        const bool valid = j < n;
-        // Into L2 while this tile is encoded and run through the MLP: its
-        // uniforms (or directions), which the decode reads last, and the
-        // next tile's positions. Lane l of warp 3 takes row l >> 2 (0-3:
-        // uniforms, 4-6: next positions), quarter l & 3 (128 bytes) of the
-        // 512-byte rows.
-        if (warp == 3) {
-            const int lane = t & 31, r = lane >> 2;
-            const int64_t b0 = (tile - S.tile0) * kTile + 32 * (lane & 3);
-            if (r < 4) {
-                if ((r < 3 || S.ufrac > 0.0f) && b0 < n)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(S.uin + r * ld + b0));
-            } else if (r < 7) {
-                const int64_t nt = tile + stride;
-                if (nt < ntiles) {
-                    int s2 = sg;
-                    while (s2 + 1 < qb.nseg && nt >= qb.seg[s2 + 1].tile0) ++s2;
-                    const QuerySeg& S2 = qb.seg[s2];
-                    const int64_t b2 = (nt - S2.tile0) * kTile + 32 * (lane & 3);
-                    const int64_t n2 = (s2 == 0 && qb.n_dev) ? n0 : S2.n;
-                    if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + (r - 4) * S2.ld + b2));
-                }
-            }
-        }
-        // Without a layer-0 buffer of its own the encoding also rewrites
-        // the zero chunks (the hidden layers reuse the buffer).
-        tc_encode<F2>(tc, grid_h, j, valid, ld, S.pos, S.aux, sA0, t, tc.split ? a0_lo : 0u, tc.a0_bytes == 0, 0,
-                      tc.base.n_levels, true);
-        fence_async_smem();
-        tc_fence_before();
-        tc_group_sync(g);
-        uint32_t raw[4 * KMAX / 16][16];
-#pragma unroll kUnrollL
-        for (int l = 0; l < L; ++l) {
-            const TcLayer& ly = tc.layer[l];
-            if (t == 0) {
-                tc_fence_after();
-                const uint32_t sbo = (uint32_t)(ly.Kp >> 3) * 128u;
-                const uint32_t a_addr = l == 0 ? sA0_addr : sA_addr;
-                const uint32_t a_lo = l == 0 ? a0_lo : tc.a_bytes;
-                for (int s = 0; s < (ly.Kp >> 4); ++s) {
-                    const uint64_t ad = umma_desc(a_addr + s * 256u, 128u, sbo);
-                    const uint64_t bd = umma_desc(sW_addr + ly.w_off + s * 256u, 128u, sbo);
-                    mma_bf16(tmem, ad, bd, ly.idesc, s > 0 ? 1u : 0u);
-                    if (tc.split || tc.f16) {
-                        // hi*lo (the weights' residual) and, when split,
-                        // lo*hi (the activations' residual)
-                        const uint64_t bdl = umma_desc(sW_addr + tc.w_bytes + ly.w_off + s * 256u, 128u, sbo);
-                        mma_bf16(tmem, ad, bdl, ly.idesc, 1u);
-                        if (tc.split) {
-                            const uint64_t adl = umma_desc(a_addr + a_lo + s * 256u, 128u, sbo);
-                            mma_bf16(tmem, adl, bd, ly.idesc, 1u);
-                        }
-                    }
-                }
-                mma_commit(bar_mma);
-            }
-            // Warp 0 (which holds the issuing thread) waits on the MMA's
-            // barrier; the other warps wait in the group barrier, issuing
-            // nothing, and see the accumulators after its fence.
-            const bool done = warp != 0 || mbar_wait_bounded(bar_mma, phase);
-            phase ^= 1u;
-            ok = !tc_group_sync_or(g, !done);
-            if (!ok) break;
-            tc_fence_after();
-            if (l < L - 1) {
-                const int kp_next = tc.layer[l + 1].Kp;
-#pragma unroll kUnrollC
-                for (int c0 = 0; c0 < ly.Np; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)c0, r);
-                    tmem_wait16(r);
-                    float v[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = fmaxf(__uint_as_float(r[i]), 0.0f);
-                    store16_fwd(sA, tile_off(t, c0, kp_next), tile_off(t, c0 + 8, kp_next), v,
-                                tc.split ? tc.a_bytes : 0u, tc.f16 != 0);
-                }
-                fence_async_smem();
-                tc_fence_before();
-                tc_group_sync(g);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4 * KMAX / 16; ++c)
-                    if (c * 16 < ly.Np) tmem_ld16(tmem + lane_base + (uint32_t)(c * 16), raw[c]);
-#pragma unroll
-                for (int c = 0; c < 4 * KMAX / 16; ++c)
-                    if (c * 16 < ly.Np) tmem_wait16(raw[c]);
-                tc_fence_before();
-            }
-        }
-        if (!ok) break;
-        if constexpr (WARPDEC) {
-            // Stage the raw outputs in the activation buffer (free until the
-            // next tile's encode), then decode a query per 32 / KMAX lanes.
-            constexpr int RS = 4 * KMAX + 4;
-            float* sRaw = reinterpret_cast<float*>(sA);
-#pragma unroll
-            for (int c = 0; c < 4 * KMAX / 16; ++c)
-                if (c * 16 < tc.layer[L - 1].Np)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        *reinterpret_cast<uint4*>(sRaw + t * RS + 16 * c + 4 * q) =
-                            make_uint4(raw[c][4 * q], raw[c][4 * q + 1], raw[c][4 * q + 2], raw[c][4 * q + 3]);
-            tc_group_sync(g);
-            tc_decode_warp<KMAX>(tc, sRaw, warp, t & 31, (tile - S.tile0) * kTile, n, ld, S.uin, S.ufrac,
-                                 qb.sample != 0, S.dir, S.pdf, S.mix, qb.log_pdf != 0);
-            tc_group_sync(g);
-        } else {
-            float rawf[4 * KMAX];
-#pragma unroll
-            for (int c = 0; c < 4 * KMAX / 16; ++c)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) rawf[c * 16 + i] = __uint_as_float(raw[c][i]);
-            tc_decode<KMAX, (NL > 0)>(tc, rawf, j, valid, ld, S.uin, S.ufrac, qb.sample != 0, S.dir, S.pdf, S.mix,
-                                      qb.log_pdf != 0);
-        }
-    }
-    if (!ok) {
-        if (t == 0) atomicOr(status, kStatusTimeout);
-        // Before the tensor memory is released: wait again, bounded, for this
-        // group's own asynchronous work that may still be in flight (the
-        // weights' bulk copy; the MMA batch whose wait gave up, the phase
-        // before `phase`).
-        if (warp == 0) {
-            (void)mbar_wait_bounded(bar_w, 0);
-            (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(cta_cols)
-                     : "memory");
-    }
 }
 
 // Master FP32 weights (packed [out][in] per layer) -> BF16 blob in the UMMA
@@ -1339,8 +829,6 @@ struct TcState {
     // blob in the split layout; otherwise training reads wblob.
     uint8_t* wblob_train = nullptr;
     uint8_t* wblob_inf = nullptr;  // of the moving average, when inference uses it
-    size_t smem = 0;
-    int grid = 0;
     TcCfg train_cfg;     // copy of cfg for training (split operands)
     TcTrain train;
     bool can_train = false;
@@ -1398,12 +886,13 @@ npm_status tc_create(npm_handle* h) {
     t.fp32 = c.precision == NPM_FP32_TC ? 1 : 0;
     const uint32_t nsplit = t.split ? 2u : 1u;
     const uint32_t nw = (t.split || t.f16) ? 2u : 1u;
-    uint32_t cols = 32;
-    while ((int)cols < maxnp) cols <<= 1;
-    t.tmem_cols = cols;
+    int maxkp = 16;
+    for (int l = 0; l < c.n_layers; ++l) maxkp = std::max(maxkp, t.layer[l].Kp);
+    t.d_cols = (uint32_t)((maxnp + 31) / 32 * 32);
+    t.a_cols = (uint32_t)(maxkp / 2);
+    t.g_cols = t.d_cols + nsplit * t.a_cols;
     t.enc_width = enc_width;
-    s->smem = nw * t.w_bytes + nsplit * (t.a0_bytes + t.a_bytes) + 64;
-    if (s->smem > 200 * 1024 || c.K > 16) {
+    if (nw * t.w_bytes + nsplit * (t.a0_bytes + t.a_bytes) + 64 > 200 * 1024 || c.K > 16) {
         delete s;
         return NPM_ERR_UNSUPPORTED;
     }
@@ -1530,80 +1019,6 @@ cudaError_t tc_refresh_weights(npm_handle* h, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Shared memory of a k_forward_tc CTA of G tile groups: the weight blobs,
-// each group's activation tiles, the barriers and the tensor-memory slot.
-static size_t tc_group_smem(const TcState* s, int G) {
-    const TcCfg& c = s->cfg;
-    const size_t nw = (c.split || c.f16) ? 2 : 1, nsplit = c.split ? 2 : 1;
-    return nw * c.w_bytes + (size_t)G * nsplit * (c.a0_bytes + c.a_bytes) + 8 * (1 + G) + 16;
-}
-
-// Whether a CTA of G tile groups fits one SM (shared and tensor memory).
-static bool tc_groups_fit(const TcState* s, int G) {
-    uint32_t cols = 32;
-    while (cols < (uint32_t)G * s->cfg.tmem_cols) cols <<= 1;
-    return cols <= 512u && tc_group_smem(s, G) + 1024 <= 227 * 1024;
-}
-
-// Whether a group's activation tiles hold the raw outputs of a 128-row tile
-// staged for the warp-per-query decode (row stride 4 KMAX + 4 floats).
-static bool tc_stage_fits(const TcState* s, int kmax) {
-    return (size_t)(s->cfg.split ? 2 : 1) * s->cfg.a_bytes >= (size_t)kTile * (4 * kmax + 4) * sizeof(float);
-}
-
-template <int KMAX, bool F2, int NL, bool WARPDEC = false, bool G32 = false, int G = 1>
-static cudaError_t launch_tc(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStream_t st) {
-    TcState* s = h->tc;
-    if (WARPDEC && !tc_stage_fits(s, KMAX)) return cudaErrorInvalidValue;  // the dispatch checks this
-    auto kern = k_forward_tc<KMAX, F2, NL, WARPDEC, G32, G>;
-    // CTAs per SM from registers (the instance's count, queried once) and
-    // tensor memory; then carve out just the shared memory they need so the
-    // rest stays L1 for the grid gathers.
-    static std::atomic<int> regs{-1};
-    int nregs = regs.load(std::memory_order_relaxed);
-    if (nregs < 0) {
-        cudaFuncAttributes fa;
-        cudaError_t ea = cudaFuncGetAttributes(&fa, kern);
-        if (ea != cudaSuccess) return ea;
-        nregs = fa.numRegs;
-        regs.store(nregs, std::memory_order_relaxed);
-    }
-    const int regs_cta = ((nregs + 7) / 8 * 8) * kThreads;
-    int per_sm = regs_cta > 0 ? 65536 / regs_cta : 1;
-    const int tmem_cap = (int)(512u / s->cfg.tmem_cols);
-    if (per_sm > tmem_cap) per_sm = tmem_cap;
-    if (per_sm > 16) per_sm = 16;
-    while (per_sm > 1 && (size_t)per_sm * (s->smem + 1024) > 227 * 1024) --per_sm;
-    static std::atomic<int> env_ctas{INT32_MIN + 1};
-    const int v = env_override("NPM_TC_CTAS_PER_SM", env_ctas);
-    if (v >= 1 && v < per_sm) per_sm = v;
-    if (per_sm < 1) per_sm = 1;
-    const size_t smem = G > 1 ? tc_group_smem(s, G) : s->smem;
-    if (G > 1) per_sm = 1;  // one CTA of G groups per SM
-    static std::atomic<uint64_t> attrs{~0ull};
-    cudaError_t e = set_smem_attrs(kern, smem, carveout_percent((size_t)per_sm * (smem + 1024)), attrs);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t t0 = 0;
-    for (int i = 0; i < qb.nseg; ++i) {
-        qb.seg[i].tile0 = t0;
-        t0 += (qb.seg[i].n + kTile - 1) / kTile;
-    }
-    qb.total_tiles = t0;
-    const int64_t hint = (qb.n_dev ? (max_n + kTile - 1) / kTile : t0 + G - 1) / G;
-    int64_t g = (int64_t)per_sm * sms;
-    if (g > hint) g = hint < 1 ? 1 : hint;
-    int* status = reinterpret_cast<int*>(h->scalars + 8);
-    const uint8_t* wb = h->ema ? s->wblob_inf : s->wblob;  // inference weights
-    const GridT<G32>* grid;
-    if constexpr (G32) grid = h->ema ? h->ema : h->params;  // the inference parameters
-    else grid = h->grid_h;
-    kern<<<(int)g, kThreads * G, smem, st>>>(s->cfg, grid, wb, qb, status);
-    return cudaGetLastError();
-}
-
 template <int KMAX, bool F2>
 static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,
                                    const float* dir, const float* rad, const float* spdf, const float* dlogv,
@@ -1666,66 +1081,25 @@ cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, con
 }
 
 cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStream_t st, bool pdl) {
-    const int K = h->cfg.K, L = h->cfg.n_layers;
-    const bool f2 = h->cfg.feat_per_level == 2;
+    const TcState* s = h->tc;
+    const TcCfg& c = s->cfg;
+    const uint8_t* wb = h->ema ? s->wblob_inf : s->wblob;  // inference weights
+    int* status = status_word(h);
+    const long long limit = 1ll << 32;  // the tensor-core kernels' fixed bound
     // The FP32-accuracy mode gathers from the FP32 table.
-    // Up to eight lobes it runs three tile groups per CTA sharing one copy
-    // of the weights where they fit (more tiles in flight per SM for the
-    // gathers' latency than separate CTAs, whose weight copies fill the
-    // shared memory).
-    if (h->tc->cfg.fp32) {
-        const bool grp = tc_groups_fit(h->tc, 3);
-        if (K <= 4) {
-            if (grp) return f2 ? launch_tc<4, true, 0, false, true, 3>(h, qb, max_n, st)
-                               : launch_tc<4, false, 0, false, true, 3>(h, qb, max_n, st);
-            return f2 ? launch_tc<4, true, 0, false, true>(h, qb, max_n, st)
-                      : launch_tc<4, false, 0, false, true>(h, qb, max_n, st);
-        }
-        if (K <= 8) {
-            if (grp) return f2 ? launch_tc<8, true, 0, false, true, 3>(h, qb, max_n, st)
-                               : launch_tc<8, false, 0, false, true, 3>(h, qb, max_n, st);
-            return f2 ? launch_tc<8, true, 0, false, true>(h, qb, max_n, st)
-                      : launch_tc<8, false, 0, false, true>(h, qb, max_n, st);
-        }
-        return f2 ? launch_tc<16, true, 0, false, true>(h, qb, max_n, st)
-                  : launch_tc<16, false, 0, false, true>(h, qb, max_n, st);
-    }
+    if (c.fp32) return launch_fwd_ops<kTwoFp16>(c, inf_params(h), wb, qb, max_n, status, limit, false, st);
     // The small serving networks get their own kernel (npm_tc_tiny.cu);
     // tuning override NPM_TC_TINY=0 selects the general kernel instead.
     static std::atomic<int> env_tiny{INT32_MIN + 1};
-    if (tiny_qualifies(h->tc->cfg) && env_override("NPM_TC_TINY", env_tiny) != 0) {
-        const uint8_t* wb = h->ema ? h->tc->wblob_inf : h->tc->wblob;
-        return launch_tiny(h->tc->cfg, h->tc->smem, h->grid_h, wb, qb, max_n, reinterpret_cast<int*>(h->scalars + 8), st,
-                           pdl);
-    }
-    // Tuning override NPM_TC_DECODE=1: the warp-per-query decode in the
-    // general kernel (built for the four- and eight-lobe instances; it stages
-    // the raw outputs in the activation buffers, which must hold them).
+    if (tiny_qualifies(c) && env_override("NPM_TC_TINY", env_tiny) != 0)
+        return launch_tiny(c, h->grid_h, wb, qb, max_n, status, st, pdl);
+    // Tuning override NPM_TC_DECODE=1: the warp-per-query decode (up to eight
+    // lobes).
     static std::atomic<int> env_dec{INT32_MIN + 1};
-    const TcCfg& c = h->tc->cfg;
-    const int kmax = K <= 4 ? 4 : 8;
-    const bool fits = tc_stage_fits(h->tc, kmax);
-    if (env_override("NPM_TC_DECODE", env_dec) == 1 && K <= 8 && fits) {
-        if (K <= 4) {
-            if (L == 3 && K == 4 && !f2) return launch_tc<4, false, 3, true>(h, qb, max_n, st);
-            return f2 ? launch_tc<4, true, 0, true>(h, qb, max_n, st) : launch_tc<4, false, 0, true>(h, qb, max_n, st);
-        }
-        return f2 ? launch_tc<8, true, 0, true>(h, qb, max_n, st) : launch_tc<8, false, 0, true>(h, qb, max_n, st);
-    }
-    // The small three-layer four-lobe networks get an instance with the layer
-    // and lobe loops unrolled (measured faster there; on the four-layer
-    // paper-shaped networks unrolling was slower).
-    if (K <= 4) {
-        if (L == 3 && K == 4 && !f2) return launch_tc<4, false, 3>(h, qb, max_n, st);
-        return f2 ? launch_tc<4, true, 0>(h, qb, max_n, st) : launch_tc<4, false, 0>(h, qb, max_n, st);
-    }
-    if (K <= 8) {
-        // Hash-grid networks: three tile groups sharing the weights, where
-        // they fit (more tiles in flight for the gathers).
-        if (f2 && tc_groups_fit(h->tc, 3)) return launch_tc<8, true, 0, false, false, 3>(h, qb, max_n, st);
-        return f2 ? launch_tc<8, true, 0>(h, qb, max_n, st) : launch_tc<8, false, 0>(h, qb, max_n, st);
-    }
-    return f2 ? launch_tc<16, true, 0>(h, qb, max_n, st) : launch_tc<16, false, 0>(h, qb, max_n, st);
+    const bool warp_decode = c.base.K <= 8 && env_override("NPM_TC_DECODE", env_dec) == 1;
+    if (c.f16) return launch_fwd_ops<kOneFp16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
+    if (c.split) return launch_fwd_ops<kTwoBf16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
+    return launch_fwd_ops<kOneBf16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
 }
 
 npm_status tc_query(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,

@@ -8,6 +8,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "npm_device.cuh"
 
 namespace npm {
@@ -38,7 +40,10 @@ struct TcCfg {
                        // with split, activations FP16 plus an FP16 residual too
     int fp32;          // 1: the FP32-accuracy mode (split FP16 operands, FP32
                        // grid table, the FP32 path's sampler)
-    uint32_t tmem_cols;
+    // Tensor-memory columns of a forward tile group: d_cols of accumulator,
+    // then one a_cols wide block per activation part (two 16-bit values to a
+    // column); g_cols in all.
+    uint32_t d_cols, a_cols, g_cols;
     int enc_width;     // meaningful network inputs
 };
 
@@ -67,6 +72,18 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// The same with the A operand in tensor memory: lane m holds row m, each
+// 32-bit column two consecutive K elements (eight columns per K step of 16).
+__device__ __forceinline__ void mma_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -111,6 +128,47 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
         if (clock64() - t0 > (1ll << 32)) return false;
     return true;
 }
+
+// Wait bounded by `limit` SM clock cycles (<= 0: one non-blocking test).
+__device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, long long limit) {
+    if (limit <= 0) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        return ok != 0;
+    }
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, parity))
+        if (clock64() - t0 > limit) return false;
+    return true;
+}
+
+// N consecutive 32-bit columns of this thread's TMEM lane written from
+// registers; tmem_wait_st completes the thread's earlier stores.
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[1]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(r[0]) : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[2]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(r[0]), "r"(r[1])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 16 consecutive FP32 columns of this thread's TMEM lane. The values are
 // valid only after tmem_wait16 on the same registers.
@@ -206,47 +264,6 @@ __device__ __forceinline__ void store16(uint8_t* sA, uint32_t off0, uint32_t off
     }
 }
 
-// Forward-pass form of store16. With a residual tile, hi is v truncated to
-// BF16 (its upper 16 bits: one byte permute per pair) and the residual
-// v - hi, exact in FP32 and of the same sign as v, is rounded to BF16 (one
-// packed subtraction and one conversion per pair); the product error that
-// split BF16 drops stays below 2^-15 relative. Without a residual tile, v is
-// rounded to nearest (to FP16 with saturation when f16).
-__device__ __forceinline__ void store16_fwd(uint8_t* sA, uint32_t off0, uint32_t off1, const float (&v)[16],
-                                            uint32_t lo_off, bool f16 = false) {
-    uint32_t h[8];
-    if (f16) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) h[i] = pack_f16_sat(v[2 * i], v[2 * i + 1]);
-        if (lo_off) {
-            // FP16 residuals v - hi, rounded to nearest.
-            uint32_t l[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) l[i] = f16_residual(h[i], v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4*>(sA + lo_off + off0) = make_uint4(l[0], l[1], l[2], l[3]);
-            *reinterpret_cast<uint4*>(sA + lo_off + off1) = make_uint4(l[4], l[5], l[6], l[7]);
-        }
-    } else if (lo_off) {
-        uint32_t l[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t a = __float_as_uint(v[2 * i]), b = __float_as_uint(v[2 * i + 1]);
-            h[i] = __byte_perm(a, b, 0x7632);
-            const float2 nh = make_float2(__uint_as_float((a & 0xffff0000u) ^ 0x80000000u),
-                                          __uint_as_float((b & 0xffff0000u) ^ 0x80000000u));
-            const float2 r = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), nh);
-            l[i] = pack_bf16(r.x, r.y);
-        }
-        *reinterpret_cast<uint4*>(sA + lo_off + off0) = make_uint4(l[0], l[1], l[2], l[3]);
-        *reinterpret_cast<uint4*>(sA + lo_off + off1) = make_uint4(l[4], l[5], l[6], l[7]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) h[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-    }
-    *reinterpret_cast<uint4*>(sA + off0) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(sA + off1) = make_uint4(h[4], h[5], h[6], h[7]);
-}
-
 // One or two BF16 values (and their residuals when lo_off != 0), or FP16
 // values when f16.
 __device__ __forceinline__ void store_pair(uint8_t* sA, uint32_t off, float a, float b, uint32_t lo_off,
@@ -310,16 +327,78 @@ __device__ __forceinline__ void vmf_sample_rp(const Lobe& L, float u1, float u2,
     for (int a = 0; a < 3; ++a) out[a] = lx * tt[a] + ly * bb[a] + W * L.mu[a];
 }
 
+// ------------------------------------------------------------ grid gathers
+
+// Table entry loads: FP16 copy (inference) or FP32 master (training).
+__device__ __forceinline__ float2 load_feat2(const __half* g, uint32_t idx) {
+    const uint32_t raw = __ldg(reinterpret_cast<const unsigned int*>(g) + idx);
+    return __half22float2(*reinterpret_cast<const __half2*>(&raw));
+}
+__device__ __forceinline__ float2 load_feat2(const float* g, uint32_t idx) {
+    return __ldg(reinterpret_cast<const float2*>(g) + idx);
+}
+// Features 4h .. 4h+3 of entry idx of a table with F = 4 or 8 features: the
+// raw 8-byte FP16 or 16-byte FP32 vector, widened to float4 at use.
+__device__ __forceinline__ uint2 load_raw4(const __half* g, uint32_t idx, int F, int h) {
+    return __ldg(reinterpret_cast<const uint2*>(g) + (size_t)idx * (F >> 2) + h);
+}
+__device__ __forceinline__ float4 load_raw4(const float* g, uint32_t idx, int F, int h) {
+    return __ldg(reinterpret_cast<const float4*>(g) + (size_t)idx * (F >> 2) + h);
+}
+__device__ __forceinline__ float4 widen4(uint2 raw) {
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
+    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float4 widen4(float4 v) { return v; }
+__device__ __forceinline__ float load_feat(const __half* e, int f) { return __half2float(e[f]); }
+__device__ __forceinline__ float load_feat(const float* e, int f) { return __ldg(e + f); }
+
+// Entry index of corner c of a cell (the corner_idx8 formula for one
+// corner). The two-level gather below issues each corner's load as soon as
+// its index is formed, which schedules better there than forming all 16
+// indices first.
+__device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const Cell& cl, int c) {
+    const uint32_t i = cl.c[0] + (c & 1), j = cl.c[1] + ((c >> 1) & 1), k = cl.c[2] + ((c >> 2) & 1);
+    if ((cfg.dense_mask >> l) & 1u) {
+        const uint32_t D = (uint32_t)cfg.level_res[l];
+        return bounded_index(i + D * (j + D * k), D * D * D);
+    }
+    return (i ^ (j * 2654435761u) ^ (k * 805459861u)) & cfg.table_mask;
+}
+
+// ------------------------------------------------------- forward kernels
+
+// Byte offset of the staging space behind the weights, the barriers and the
+// tensor-memory slot of a forward CTA of G tile groups.
+__host__ __device__ inline uint32_t fwd_stage_off(uint32_t wbytes, int G) {
+    return (wbytes + 8u * (1u + (uint32_t)G) + 16u + 15u) & ~15u;
+}
+
+// The general forward in one operand format (npm_tc_forward.cuh; one
+// translation unit per format): grid is the FP16 table, or the FP32 table in
+// the formats of FP32 accuracy.
+template <int OPS>
+cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
+                           int* status, long long wait_limit, bool warp_decode, cudaStream_t st);
+
+// Operand formats (parts from the highest):
+//   kOneBf16   activations and weights rounded to BF16
+//   kOneFp16   activations rounded to FP16, weights FP16 plus residual
+//   kTwoBf16   activations and weights BF16 plus residual
+//   kTwoFp16   activations and weights FP16 plus residual, FP32 grid table
+enum : int { kOneBf16 = 0, kOneFp16 = 1, kTwoBf16 = 2, kTwoFp16 = 3 };
+
 // Fused forward of the small serving networks (npm_tc_tiny.cu): radiance
 // mode, one dense level of 4 features, three layers of at most 32 outputs
 // (padded input 16), K = 4, softplus kappa, layer 0 sharing the activation
-// buffer. launch_tiny takes the general kernel's configuration, shared
-// memory size, FP16 grid and weight blob. With pdl the kernel is launched as
+// buffer. launch_tiny takes the general kernel's configuration, FP16 grid
+// and weight blob. With pdl the kernel is launched as
 // a programmatic dependent of the stream's previous kernel: its prologue
 // (tensor-memory allocation, copies of the weights and grid) overlaps that
 // kernel, which therefore must not write the weights or the grid.
 bool tiny_qualifies(const TcCfg& c);
-cudaError_t launch_tiny(const TcCfg& c, size_t smem, const __half* grid_h, const uint8_t* wblob, QueryBatch& qb,
+cudaError_t launch_tiny(const TcCfg& c, const __half* grid_h, const uint8_t* wblob, QueryBatch& qb,
                         int64_t max_n, int* status, cudaStream_t st, bool pdl = false);
 
 }  // namespace tc

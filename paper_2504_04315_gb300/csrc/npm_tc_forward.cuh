@@ -1,0 +1,772 @@
+// npm_tc_forward.cuh -- tensor-core forward pass (encode, MLP, sample and
+// density) on sm_103a with the activations in tensor memory.
+//
+// One persistent CTA per SM holds G tile groups of 128 threads that share one
+// copy of the weights in shared memory. Thread t of a group owns query t of
+// the group's 128-query tile, which is lane t of its tensor-memory columns.
+// Per tile:
+//   encode : the thread gathers the 8 corners of every level, blends them in
+//            FP32 (Sec. 5.1, Eq. 11), appends the product-mode SH encodings
+//            (Sec. 4.3), splits the values into 16-bit operand parts and
+//            stores them into its lane of the activation columns (tcgen05.st).
+//   layers : one elected thread issues tcgen05.mma kind::f16 with the
+//            activations as the A operand in tensor memory and the weights as
+//            the B operand in shared memory (M = 128, N = layer width, K in
+//            steps of 16, FP32 accumulation) and commits to an mbarrier; every
+//            thread reads its accumulator lane (tcgen05.ld), applies ReLU and
+//            stores the next layer's operand parts.
+//   decode : the last accumulator lane (4K FP32 raw outputs) in registers is
+//            mapped (Table 1), sampled (Sec. 5.3) and evaluated (Eq. 4).
+// Weights arrive once per CTA by a bulk asynchronous copy; the first tile is
+// encoded meanwhile. Every wait on an mbarrier is bounded: on timeout the
+// kernel records kStatusTimeout in the status word, drains what it has in
+// flight (bounded), releases its tensor memory and returns.
+//
+// What bounds it on hash grids is the gathers: the L1 takes one request per
+// lane and cycle, about 6 requests per level and query. Activations in tensor
+// memory leave shared memory to the weights alone, so the rest of the 256 KB
+// stays L1 and four groups (16 warps, 128 registers) fit where activation
+// tiles in shared memory left room for one to three. Measured against those
+// (GB300, one call): 64-wide product-mode network in the FP32-accuracy mode,
+// 300,007 queries, 339 -> 140 us (one group -> four); paper-shaped hash grid,
+// FP16, 2,073,600 queries, 869 -> 719 us (three -> four); eight dense levels
+// of four features, split BF16, 250,007 densities, 102 -> 72 us.
+#pragma once
+
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <atomic>
+
+#include "npm_kernels.h"
+#include "npm_tc.cuh"
+
+namespace npm {
+namespace tc {
+
+template <int OPS>
+struct OpsTraits {
+    static constexpr int parts = OPS == kOneBf16 || OPS == kOneFp16 ? 1 : 2;  // of an activation
+    static constexpr int wparts = OPS == kOneBf16 ? 1 : 2;                    // of a weight
+    static constexpr bool fp32 = OPS == kTwoFp16;  // FP32 grid table and sampler
+    using GridT = typename std::conditional<fp32, float, __half>::type;
+};
+
+// Tile groups a CTA is compiled for: four at 128 registers; two for up to
+// sixteen lobes, whose raw outputs alone take 64.
+__host__ __device__ constexpr int fwd_groups(int kmax) { return kmax > 8 ? 2 : 4; }
+
+// ----------------------------------------------------------- operands
+
+// The operand parts of a pair of values (the first in the low half).
+template <int OPS>
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[OpsTraits<OPS>::parts]) {
+    if constexpr (OPS == kOneFp16) {
+        p[0] = pack_f16_sat(a, b);
+    } else if constexpr (OPS == kOneBf16) {
+        p[0] = pack_bf16(a, b);
+    } else if constexpr (OPS == kTwoFp16) {
+        p[0] = pack_f16_sat(a, b);
+        p[1] = f16_residual(p[0], a, b);
+    } else {
+        p[0] = pack_bf16(a, b);
+        p[1] = pack_bf16(a - __uint_as_float(p[0] << 16), b - __uint_as_float(p[0] & 0xffff0000u));
+    }
+}
+
+// The same of max(a, 0), max(b, 0) (hidden layers). Split BF16 truncates the
+// high part: the residual is then never negative and ReLU comes with both
+// conversions.
+template <int OPS>
+__device__ __forceinline__ void relu_split_pair(float a, float b, uint32_t (&p)[OpsTraits<OPS>::parts]) {
+    if constexpr (OPS == kOneFp16) {
+        asm("cvt.rn.satfinite.relu.f16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
+    } else if constexpr (OPS == kOneBf16) {
+        asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
+    } else if constexpr (OPS == kTwoFp16) {
+        split_pair<OPS>(fmaxf(a, 0.0f), fmaxf(b, 0.0f), p);
+    } else {
+        asm("cvt.rz.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
+        const float ra = a - __uint_as_float(p[0] << 16), rb = b - __uint_as_float(p[0] & 0xffff0000u);
+        asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[1]) : "f"(rb), "f"(ra));
+    }
+}
+
+// N (1, 2, 4 or 8) operand pairs of this thread's row into the activation
+// columns col .. col + N of every part. All 32 lanes take part.
+template <int OPS, int N>
+__device__ __forceinline__ void put_pairs(uint32_t act, uint32_t part_cols, uint32_t col,
+                                          const uint32_t (&v)[N][OpsTraits<OPS>::parts]) {
+#pragma unroll
+    for (int p = 0; p < OpsTraits<OPS>::parts; ++p) {
+        uint32_t r[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] = v[i][p];
+        tmem_st(act + p * part_cols + col, r);
+    }
+}
+
+// ------------------------------------------------------------- encode
+
+// Two levels' corner features are gathered before either is blended, so that
+// 16 loads (F = 2) are in flight.
+template <typename GT>
+__device__ __forceinline__ void gather_level2(const DevCfg& cfg, const GT* __restrict__ grid, int l, const Cell& cl,
+                                              float2 (&v)[8]) {
+    const GT* g = grid + (size_t)cfg.level_off[l] * 2;
+#pragma unroll
+    for (int c = 0; c < 8; c += 2)
+        gather_pair2(g, cfg.level_off[l], corner_idx1(cfg, l, cl, c), corner_idx1(cfg, l, cl, c + 1), v[c], v[c + 1]);
+}
+
+__device__ __forceinline__ float2 blend_level2(const Cell& cl, const float2 (&v)[8]) {
+    float w[8];
+    corner_w8(cl, w);
+    float2 a = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        a.x = fmaf(w[c], v[c].x, a.x);
+        a.y = fmaf(w[c], v[c].y, a.y);
+    }
+    return a;
+}
+
+// Features 4h .. 4h + 3 of a level of F = 4 or 8 features.
+template <typename GT>
+__device__ __forceinline__ float4 blend_level4(const DevCfg& cfg, const GT* __restrict__ grid, int l, const Cell& cl,
+                                               int F, int h) {
+    const GT* g = grid + (size_t)cfg.level_off[l] * F;
+    uint32_t idx[8];
+    corner_idx8(cfg, l, cl, idx);
+    decltype(load_raw4(g, 0u, F, 0)) raw[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) raw[c] = load_raw4(g, idx[c], F, h);
+    float w[8];
+    corner_w8(cl, w);
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float4 v = widen4(raw[c]);
+        a.x = fmaf(w[c], v.x, a.x);
+        a.y = fmaf(w[c], v.y, a.y);
+        a.z = fmaf(w[c], v.z, a.z);
+        a.w = fmaf(w[c], v.w, a.w);
+    }
+    return a;
+}
+
+// Values of a row one after another, stored in pairs.
+template <int OPS>
+struct RowPacker {
+    uint32_t act, part_cols;
+    int k;
+    float prev;
+    __device__ __forceinline__ void put(float v) {
+        if (k & 1) {
+            uint32_t p[1][OpsTraits<OPS>::parts];
+            split_pair<OPS>(prev, v, p[0]);
+            __syncwarp();
+            put_pairs<OPS, 1>(act, part_cols, (uint32_t)(k >> 1), p);
+        }
+        prev = v;
+        ++k;
+    }
+};
+
+// The network input of query (x, y, z): this thread's row of the activation
+// columns, padded with zeros to the layer's kp values. FEAT: features per
+// level (2 or 4), or 0 for any.
+template <int FEAT, int OPS>
+__device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTraits<OPS>::GridT* __restrict__ grid,
+                                           float x, float y, float z, const float (&ax)[7], uint32_t act) {
+    const DevCfg& cfg = tc.base;
+    constexpr int P = OpsTraits<OPS>::parts;
+    const uint32_t pc = tc.a_cols;
+    __syncwarp();
+    const int L = cfg.n_levels, F = FEAT ? FEAT : cfg.feat;
+    if constexpr (FEAT == 2) {
+        int l = 0;
+        for (; l + 1 < L; l += 2) {
+            const Cell c0 = make_cell(x, y, z, cfg.level_res[l]), c1 = make_cell(x, y, z, cfg.level_res[l + 1]);
+            float2 v0[8], v1[8];
+            gather_level2(cfg, grid, l, c0, v0);
+            gather_level2(cfg, grid, l + 1, c1, v1);
+            const float2 a = blend_level2(c0, v0), b = blend_level2(c1, v1);
+            uint32_t p[2][P];
+            split_pair<OPS>(a.x, a.y, p[0]);
+            split_pair<OPS>(b.x, b.y, p[1]);
+            __syncwarp();
+            put_pairs<OPS, 2>(act, pc, (uint32_t)l, p);
+        }
+        if (l < L) {
+            const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
+            float2 v0[8];
+            gather_level2(cfg, grid, l, c0, v0);
+            const float2 a = blend_level2(c0, v0);
+            uint32_t p[1][P];
+            split_pair<OPS>(a.x, a.y, p[0]);
+            __syncwarp();
+            put_pairs<OPS, 1>(act, pc, (uint32_t)l, p);
+        }
+    } else if (FEAT == 4 || F == 4 || F == 8) {
+#pragma unroll(FEAT == 4 ? 2 : 1)
+        for (int l = 0; l < L; ++l) {
+            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            for (int h = 0; h < (F >> 2); ++h) {
+                const float4 a = blend_level4(cfg, grid, l, cl, F, h);
+                uint32_t p[2][P];
+                split_pair<OPS>(a.x, a.y, p[0]);
+                split_pair<OPS>(a.z, a.w, p[1]);
+                put_pairs<OPS, 2>(act, pc, (uint32_t)((l * F + 4 * h) >> 1), p);
+            }
+        }
+    } else {
+        RowPacker<OPS> row{act, pc, 0, 0.0f};
+        for (int l = 0; l < L; ++l) {
+            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            if (F == 2) {
+                float2 v[8];
+                gather_level2(cfg, grid, l, cl, v);
+                const float2 a = blend_level2(cl, v);
+                row.put(a.x);
+                row.put(a.y);
+            } else {  // F = 1
+                const auto* g = grid + cfg.level_off[l];
+                uint32_t idx[8];
+                float w[8];
+                corners8(cfg, l, cl, idx, w);
+                float s = 0.0f;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s = fmaf(w[c], load_feat(g + idx[c], 0), s);
+                row.put(s);
+            }
+        }
+        if (cfg.mode != NPM_PRODUCT && (row.k & 1)) row.put(0.0f);
+        if (cfg.mode == NPM_PRODUCT) {
+            float e[21];
+            sh_band4(ax[0], ax[1], ax[2], e);
+            sh_band2(ax[3], ax[4], ax[5], e + 16);
+            e[20] = ax[6];
+#pragma unroll
+            for (int i = 0; i < 21; ++i) row.put(e[i]);
+            if (row.k & 1) row.put(0.0f);
+        }
+    }
+    uint32_t col = (uint32_t)(cfg.grid_feats + 1) >> 1;
+    if (cfg.mode == NPM_PRODUCT) {
+        if (F != 1 && !(FEAT == 0 && F == 2)) {
+            // An even number of grid features: 21 values and one zero.
+            float e[22];
+            sh_band4(ax[0], ax[1], ax[2], e);
+            sh_band2(ax[3], ax[4], ax[5], e + 16);
+            e[20] = ax[6];
+            e[21] = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 22; i += 2) {
+                uint32_t p[1][P];
+                split_pair<OPS>(e[i], e[i + 1], p[0]);
+                put_pairs<OPS, 1>(act, pc, col + (uint32_t)(i >> 1), p);
+            }
+        }
+        col = (uint32_t)(cfg.grid_feats + 22) >> 1;
+    }
+    const uint32_t end = (uint32_t)tc.layer[0].Kp >> 1;
+    for (; col < end; ++col) {
+        const uint32_t p[1][P] = {};
+        put_pairs<OPS, 1>(act, pc, col, p);
+    }
+}
+
+// --------------------------------------------------------------- decode
+
+// Table 1, sampling (Sec. 5.3) and density (Eq. 4) of one query from its raw
+// outputs. Only the chosen lobe is decoded for the sample; the density then
+// decodes lobe by lobe, so that no array of decoded lobes stays live (nine
+// lobe decodes instead of eight, half the registers).
+struct QueryIo {
+    int64_t j, ld;
+    bool valid;
+    float u[4];  // uniforms when sampling, direction when evaluating
+    float ufrac;
+    float* dir;
+    float* pdf;
+    float* mix;
+};
+
+template <int KMAX, bool FP32>
+__device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&rawu)[KMAX / 4][16], const QueryIo& q,
+                                           bool sample, bool log_pdf) {
+    const int K = cfg.K;
+    auto raw = [&](int i) { return __uint_as_float(rawu[i >> 4][i & 15]); };
+    float mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+        if (i < K) mx = fmaxf(mx, raw(4 * i));
+    float lam[KMAX], ssum = 0.0f;
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+        if (i < K) {
+            lam[i] = __expf(raw(4 * i) - mx);
+            ssum += lam[i];
+        }
+    const float inv = __fdividef(1.0f, ssum);  // ssum in [1, K]
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+        if (i < K) lam[i] *= inv;
+    float w[3] = {q.u[0], q.u[1], q.u[2]};
+    if (sample) {
+        // Smallest lobe i with u0 < lambda_0 + ... + lambda_i (last if none).
+        float cum = 0.0f, rk = raw(1), rt = raw(2), rp = raw(3);
+        bool found = false;
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i)
+            if (i < K) {
+                cum += lam[i];
+                if (!found) {
+                    rk = raw(4 * i + 1);
+                    rt = raw(4 * i + 2);
+                    rp = raw(4 * i + 3);
+                }
+                found = found || q.u[0] < cum;
+            }
+        if (q.ufrac > 0.0f && q.u[3] < q.ufrac) {
+            uniform_sphere(q.u[1], q.u[2], w);
+        } else {
+            Lobe sl;
+            decode_lobe_fast(cfg.kappa_act, rk, rt, rp, sl, nullptr, nullptr);
+            if (FP32) vmf_sample(sl, q.u[1], q.u[2], w);
+            else vmf_sample_rp(sl, q.u[1], q.u[2], w);
+        }
+    }
+    float pv = 0.0f;
+    if (!sample && log_pdf) {
+        // log V (Eq. 4 in log-sum-exp form), the weights' logs taken from the
+        // logits so that they stay finite where lambda_i underflows.
+        const float lnorm = mx + __logf(ssum);
+        float m = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i)
+            if (i < K) {
+                Lobe lb;
+                decode_lobe_fast(cfg.kappa_act, raw(4 * i + 1), raw(4 * i + 2), raw(4 * i + 3), lb, nullptr, nullptr);
+                const float d = lb.mu[0] * w[0] + lb.mu[1] * w[1] + lb.mu[2] * w[2];
+                lam[i] = (raw(4 * i) - lnorm) + __logf(vmf_scaled_norm_fast(lb.kap)) + lb.kap * (d - 1.0f);
+                m = fmaxf(m, lam[i]);
+            }
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i)
+            if (i < K) s += __expf(lam[i] - m);
+        pv = m + __logf(s);
+    } else {
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i)
+            if (i < K) {
+                Lobe lb;
+                float th, ph;
+                decode_lobe_fast(cfg.kappa_act, raw(4 * i + 1), raw(4 * i + 2), raw(4 * i + 3), lb, &th, &ph);
+                if (q.mix && q.valid) {
+                    float* mo = q.mix + (int64_t)(4 * i) * q.ld + q.j;
+                    mo[0] = lam[i];
+                    mo[q.ld] = lb.kap;
+                    mo[2 * q.ld] = th;
+                    mo[3 * q.ld] = ph;
+                }
+                pv += lam[i] * vmf_eval_fast(lb, vmf_scaled_norm_fast(lb.kap), w[0], w[1], w[2]);
+            }
+        if (sample && q.ufrac > 0.0f) pv = q.ufrac * kInv4Pi + (1.0f - q.ufrac) * pv;
+    }
+    if (q.valid) {
+        if (sample) {
+            q.dir[q.j] = w[0];
+            q.dir[q.ld + q.j] = w[1];
+            q.dir[2 * q.ld + q.j] = w[2];
+        }
+        q.pdf[q.j] = pv;
+    }
+}
+
+// Warp-per-query form of the decode, sample and density (Table 1, Sec. 5.3,
+// Eq. 4): lane l of a warp owns lobe l mod KMAX of one query, so a warp
+// serves 32 / KMAX queries per pass and KMAX passes cover its 32 rows. The
+// raw outputs of the tile are staged in shared memory (row stride 4 KMAX + 4
+// floats keeps both the row writes and the lobe reads free of bank
+// conflicts). Softmax and density are reductions over the query's lanes;
+// the lobe choice takes the running sum of the weights in lobe order (a
+// serial scan, the same rounding as the thread-per-row form) and a ballot;
+// every lane samples its own lobe and the chosen lane's direction is
+// broadcast. Measured against tc_decode (one thread per query).
+template <int KMAX>
+__device__ __forceinline__ void tc_decode_warp(const TcCfg& tc, const float* __restrict__ sRaw, int warp, int lane,
+                                               int64_t j0, int64_t n, int64_t ld, const float* __restrict__ uin,
+                                               float ufrac, bool sample, float* __restrict__ dir_out,
+                                               float* __restrict__ pdf_out, float* __restrict__ mix_out,
+                                               bool log_pdf) {
+    constexpr int RS = 4 * KMAX + 4;
+    constexpr int QP = 32 / KMAX;  // queries per pass
+    constexpr unsigned kAll = 0xffffffffu;
+    const DevCfg& cfg = tc.base;
+    const int K = cfg.K;
+    const int i = lane & (KMAX - 1);
+    const int qsub = lane / KMAX;
+    const unsigned seg = KMAX == 32 ? kAll : (((1u << KMAX) - 1u) << (qsub * KMAX));
+    const bool act = i < K;
+#pragma unroll 1
+    for (int p = 0; p < KMAX; ++p) {
+        const int r = warp * 32 + p * QP + qsub;
+        const int64_t j = j0 + r;
+        const bool valid = j < n;
+        const float4 rv = *reinterpret_cast<const float4*>(sRaw + r * RS + 4 * i);
+        float mx = act ? rv.x : -INFINITY;
+#pragma unroll
+        for (int o = 1; o < KMAX; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kAll, mx, o));
+        const float e = act ? __expf(rv.x - mx) : 0.0f;
+        float ssum = e;
+#pragma unroll
+        for (int o = 1; o < KMAX; o <<= 1) ssum += __shfl_xor_sync(kAll, ssum, o);
+        Lobe L;
+        L.lam = e * __fdividef(1.0f, ssum);
+        float th, ph;
+        decode_lobe_fast(cfg.kappa_act, rv.y, rv.z, rv.w, L, &th, &ph);
+        const float cn = vmf_scaled_norm_fast(L.kap);
+        if (mix_out && valid && act) {
+            mix_out[(4 * i + 0) * ld + j] = L.lam;
+            mix_out[(4 * i + 1) * ld + j] = L.kap;
+            mix_out[(4 * i + 2) * ld + j] = th;
+            mix_out[(4 * i + 3) * ld + j] = ph;
+        }
+        float w[3] = {0.0f, 0.0f, 1.0f};
+        bool uni = false;
+        if (sample) {
+            float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
+            if (valid) {
+                u0 = uin[j];
+                u1 = uin[ld + j];
+                u2 = uin[2 * ld + j];
+                uni = ufrac > 0.0f && uin[3 * ld + j] < ufrac;
+            }
+            // Running sum of the weights in lobe order.
+            float cum = i == 0 ? L.lam : 0.0f;
+#pragma unroll
+            for (int k = 1; k < KMAX; ++k) {
+                const float prev = __shfl_up_sync(kAll, cum, 1);
+                if (i == k) cum = prev + L.lam;
+            }
+            const unsigned hit = __ballot_sync(kAll, act && u0 < cum) & seg;
+            const int sel = hit ? __ffs(hit) - 1 - qsub * KMAX : K - 1;
+            float d[3];
+            if (uni) uniform_sphere(u1, u2, d);
+            else vmf_sample_rp(L, u1, u2, d);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) w[a] = __shfl_sync(kAll, d[a], qsub * KMAX + sel);
+        } else if (valid) {
+            w[0] = uin[j];
+            w[1] = uin[ld + j];
+            w[2] = uin[2 * ld + j];
+        }
+        float pv;
+        if (!sample && log_pdf) {
+            const float dd = L.mu[0] * w[0] + L.mu[1] * w[1] + L.mu[2] * w[2];
+            const float a = act ? (rv.x - mx) - __logf(ssum) + __logf(cn) + L.kap * (dd - 1.0f) : -INFINITY;
+            float m = a;
+#pragma unroll
+            for (int o = 1; o < KMAX; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
+            float sx = act ? __expf(a - m) : 0.0f;
+#pragma unroll
+            for (int o = 1; o < KMAX; o <<= 1) sx += __shfl_xor_sync(kAll, sx, o);
+            pv = m + __logf(sx);
+        } else {
+            pv = act ? L.lam * vmf_eval_fast(L, cn, w[0], w[1], w[2]) : 0.0f;
+#pragma unroll
+            for (int o = 1; o < KMAX; o <<= 1) pv += __shfl_xor_sync(kAll, pv, o);
+            if (sample && ufrac > 0.0f) pv = ufrac * kInv4Pi + (1.0f - ufrac) * pv;
+        }
+        if (valid && i == 0) {
+            if (sample) {
+                dir_out[j] = w[0];
+                dir_out[ld + j] = w[1];
+                dir_out[2 * ld + j] = w[2];
+            }
+            pdf_out[j] = pv;
+        }
+    }
+}
+
+// --------------------------------------------------------------- kernel
+
+// The MMAs of one layer: every K step of each product of parts, the smallest
+// products first, so that the large ones meet the accumulator's rounding only
+// Kp / 16 times. Issued by one thread.
+template <int OPS>
+__device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, uint32_t acc, uint32_t act,
+                                            uint32_t sW_addr) {
+    const uint64_t b0 = umma_desc(sW_addr + ly.w_off, 128u, (uint32_t)(ly.Kp >> 3) * 128u);
+    const int nk = ly.Kp >> 4;
+    uint32_t accum = 0u;
+    auto product = [&](int ap, int wp) {
+        const uint64_t b = b0 + (uint64_t)wp * (tc.w_bytes >> 4);
+        const uint32_t a = act + (uint32_t)ap * tc.a_cols;
+        for (int s = 0; s < nk; ++s) {
+            mma_tmem_a(acc, a + 8u * (uint32_t)s, b + (uint64_t)(16 * s), ly.idesc, accum);
+            accum = 1u;
+        }
+    };
+    if constexpr (OpsTraits<OPS>::parts == 2) product(1, 0);
+    if constexpr (OpsTraits<OPS>::wparts == 2) product(0, 1);
+    product(0, 0);
+}
+
+// WARPDEC: the warp-per-query decode (tc_decode_warp) from raw outputs staged
+// in shared memory.
+template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
+__global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
+    k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ grid,
+                 const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
+                 long long wait_limit) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int G = (int)(blockDim.x >> 7);
+    const int g = (int)(threadIdx.x >> 7);   // tile group
+    const int t = (int)(threadIdx.x & 127);  // row of the group's tile
+    const int warp = t >> 5;                 // warp of the group (its tensor-memory lane quarter)
+    const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * tc.w_bytes;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + wbytes);  // [0] weights, [1 + g] MMAs
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 1 + G);
+    const uint32_t bar_w = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[1 + g]);
+    uint32_t cta_cols = 32;
+    while (cta_cols < (uint32_t)G * tc.g_cols) cta_cols <<= 1;
+
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(cta_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int i = 0; i <= G; ++i) mbar_init(smem_u32(&bars[i]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_w), "r"(wbytes) : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                smem_u32(smem)),
+            "l"(wblob), "r"(wbytes), "r"(bar_w)
+            : "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    // This group's columns: the accumulator, then the activations' parts.
+    const uint32_t acc = *tslot + (uint32_t)g * tc.g_cols, act = acc + tc.d_cols;
+    const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+    const uint32_t sW_addr = smem_u32(smem);
+    const int L = tc.base.n_layers;
+    const bool sample = qb.sample != 0;
+
+    int64_t ntiles = qb.total_tiles, n0 = qb.seg[0].n;
+    if (qb.n_dev) {
+        n0 = *qb.n_dev;
+        ntiles = (n0 + kTile - 1) / kTile;
+    }
+    bool ok = true, issued = false;
+    uint32_t phase = 0;
+    // Tiles are dealt to the CTAs first and to a CTA's groups second, so a
+    // batch of fewer tiles than groups spreads over as many SMs as it can.
+    const int64_t stride = (int64_t)gridDim.x * G;
+    for (int64_t tile = blockIdx.x + (int64_t)g * gridDim.x; tile < ntiles; tile += stride) {
+        int sg = 0;
+        while (sg + 1 < qb.nseg && tile >= qb.seg[sg + 1].tile0) ++sg;
+        const QuerySeg& S = qb.seg[sg];
+        const int64_t n = (sg == 0 && qb.n_dev) ? n0 : S.n;
+        const int64_t ld = S.ld;
+        QueryIo q;
+        q.j = (tile - S.tile0) * kTile + t;
+        q.ld = ld;
+        q.valid = q.j < n;
+        q.ufrac = S.ufrac;
+        q.dir = S.dir;
+        q.pdf = S.pdf;
+        q.mix = S.mix;
+        float x = 0.0f, y = 0.0f, z = 0.0f;
+        float ax[7] = {0.0f, 0.0f, 1.0f, 0.0f, 0.0f, 1.0f, 0.0f};
+        if (q.valid) {
+            x = S.pos[q.j];
+            y = S.pos[ld + q.j];
+            z = S.pos[2 * ld + q.j];
+            if (tc.base.mode == NPM_PRODUCT)
+#pragma unroll
+                for (int i = 0; i < 7; ++i) ax[i] = S.aux[i * ld + q.j];
+        }
+        if (warp == 3) {
+            // The group's next tile's positions into L2 (three 512-byte rows).
+            const int lane = t & 31, r = lane >> 2;
+            const int64_t nt = tile + stride;
+            if (r < 3 && nt < ntiles) {
+                int s2 = sg;
+                while (s2 + 1 < qb.nseg && nt >= qb.seg[s2 + 1].tile0) ++s2;
+                const QuerySeg& S2 = qb.seg[s2];
+                const int64_t b2 = (nt - S2.tile0) * kTile + 32 * (lane & 3);
+                const int64_t n2 = (s2 == 0 && qb.n_dev) ? n0 : S2.n;
+                if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + r * S2.ld + b2));
+            }
+        }
+        encode_row<FEAT, OPS>(tc, grid, x, y, z, ax, act + lanes);
+        // The uniforms (or the direction), loaded now so that their latency
+        // passes during the layers.
+        q.u[0] = q.u[1] = q.u[3] = 0.0f;
+        q.u[2] = sample ? 0.0f : 1.0f;
+        if (q.valid) {
+            q.u[0] = S.uin[q.j];
+            q.u[1] = S.uin[ld + q.j];
+            q.u[2] = S.uin[2 * ld + q.j];
+            if (q.ufrac > 0.0f) q.u[3] = S.uin[3 * ld + q.j];
+        }
+        __syncwarp();
+        tmem_wait_st();
+        tc_fence_before();
+        if (tc_group_sync_or(g, !ok)) {
+            ok = false;
+            break;
+        }
+        uint32_t raw[KMAX / 4][16];
+        for (int l = 0; l < L; ++l) {
+            const TcLayer& ly = tc.layer[l];
+            if (t == 0) {
+                // The weights have arrived (once per CTA).
+                if (!issued) ok = mbar_wait_limit(bar_w, 0, wait_limit);
+                if (ok) {
+                    tc_fence_after();
+                    issue_layer<OPS>(tc, ly, acc, act, sW_addr);
+                    mma_commit(bar_mma);
+                    issued = true;
+                }
+            }
+            // Every warp waits on the MMAs' barrier; a wait that gives up is
+            // made known to the group at its next barrier.
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_limit(bar_mma, phase, wait_limit));
+            phase ^= 1u;
+            tc_fence_after();
+            if (l < L - 1) {
+                if (ok) {
+#pragma unroll 2
+                    for (int c0 = 0; c0 < ly.Np; c0 += 16) {
+                        uint32_t r[16];
+                        tmem_ld16(acc + lanes + (uint32_t)c0, r);
+                        tmem_wait16(r);
+                        uint32_t p[8][OpsTraits<OPS>::parts];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            relu_split_pair<OPS>(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), p[i]);
+                        put_pairs<OPS, 8>(act + lanes, tc.a_cols, (uint32_t)(c0 >> 1), p);
+                    }
+                    tmem_wait_st();
+                }
+                tc_fence_before();
+                if (tc_group_sync_or(g, !ok)) {
+                    ok = false;
+                    break;
+                }
+            } else if (ok) {
+#pragma unroll
+                for (int c = 0; c < KMAX / 4; ++c)
+                    if (c * 16 < ly.Np) tmem_ld16(acc + lanes + (uint32_t)(c * 16), raw[c]);
+#pragma unroll
+                for (int c = 0; c < KMAX / 4; ++c)
+                    if (c * 16 < ly.Np) tmem_wait16(raw[c]);
+                tc_fence_before();
+            }
+        }
+        if constexpr (WARPDEC) {
+            // Stage the raw outputs, then decode a query per 32 / KMAX lanes.
+            constexpr int RS = 4 * KMAX + 4;
+            float* sRaw = reinterpret_cast<float*>(smem + fwd_stage_off(wbytes, G)) + g * kTile * RS;
+            if (tc_group_sync_or(g, !ok)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int c = 0; c < KMAX / 4; ++c)
+                if (c * 16 < tc.layer[L - 1].Np)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        *reinterpret_cast<uint4*>(sRaw + t * RS + 16 * c + 4 * i) =
+                            make_uint4(raw[c][4 * i], raw[c][4 * i + 1], raw[c][4 * i + 2], raw[c][4 * i + 3]);
+            tc_group_sync(g);
+            tc_decode_warp<KMAX>(tc, sRaw, warp, t & 31, (tile - S.tile0) * kTile, n, ld, S.uin, S.ufrac, sample, S.dir,
+                                 S.pdf, S.mix, qb.log_pdf != 0);
+        } else {
+            if (ok) decode_row<KMAX, OpsTraits<OPS>::fp32>(tc.base, raw, q, sample, qb.log_pdf != 0);
+        }
+    }
+    if (!ok && (t & 31) == 0) atomicOr(status, kStatusTimeout);
+    // Before the tensor and shared memory are released: whatever a wait gave
+    // up on and may still be in flight (the weights' bulk copy; this group's
+    // last MMAs, of the phase before `phase`), again with a bound.
+    if (threadIdx.x == 32) (void)mbar_wait_bounded(bar_w, 0);
+    if (t == 0 && !ok && issued) (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(cta_cols) : "memory");
+    }
+}
+
+// ------------------------------------------------------------- launcher
+
+// Tile groups of a CTA: as many as the instance is compiled for and the
+// 512 tensor-memory columns hold.
+inline int fwd_group_count(const TcCfg& c, int kmax) {
+    int G = fwd_groups(kmax);
+    for (; G > 1; --G) {
+        uint32_t cols = 32;
+        while (cols < (uint32_t)G * c.g_cols) cols <<= 1;
+        if (cols <= 512u) break;
+    }
+    return G;
+}
+
+template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
+cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
+                       int* status, long long wait_limit, cudaStream_t st) {
+    auto kern = k_forward_tc<KMAX, FEAT, OPS, WARPDEC>;
+    const int G = fwd_group_count(c, KMAX);
+    const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * c.w_bytes;
+    size_t smem = fwd_stage_off(wbytes, G);
+    if (WARPDEC) smem += (size_t)G * kTile * (4 * KMAX + 4) * sizeof(float);
+    static std::atomic<uint64_t> attrs{~0ull};
+    cudaError_t e = set_smem_attrs(kern, smem, carveout_percent(smem + 1024), attrs);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int64_t t0 = 0;
+    for (int i = 0; i < qb.nseg; ++i) {
+        qb.seg[i].tile0 = t0;
+        t0 += (qb.seg[i].n + kTile - 1) / kTile;
+    }
+    qb.total_tiles = t0;
+    int64_t blocks = qb.n_dev ? (max_n + kTile - 1) / kTile : t0;
+    if (blocks > sms) blocks = sms;
+    if (blocks < 1) blocks = 1;
+    kern<<<(int)blocks, kThreads * G, smem, st>>>(
+        c, static_cast<const typename OpsTraits<OPS>::GridT*>(grid), wblob, qb, status, wait_limit);
+    return cudaGetLastError();
+}
+
+// The instance of an operand format for this model: up to eight lobes with
+// 2, 4 or any features per level, or sixteen lobes.
+template <int OPS>
+cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
+                           int* status, long long wait_limit, bool warp_decode, cudaStream_t st) {
+    if (c.base.K > 8) return launch_fwd<16, 0, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+    if constexpr (!OpsTraits<OPS>::fp32)
+        if (warp_decode) return launch_fwd<8, 0, OPS, true>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+    if (c.base.feat == 2) return launch_fwd<8, 2, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+    if (c.base.feat == 4) return launch_fwd<8, 4, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+    return launch_fwd<8, 0, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+}
+
+}  // namespace tc
+}  // namespace npm

@@ -1,0 +1,10 @@
+// npm_tc_fwd_fp32tc.cu -- the tensor-core forward kernel (npm_tc_forward.cuh) in the
+// FP32-accuracy (split FP16) operand format.
+#include "npm_tc_forward.cuh"
+
+namespace npm {
+namespace tc {
+template cudaError_t launch_fwd_ops<kTwoFp16>(const TcCfg&, const void*, const uint8_t*, QueryBatch&, int64_t, int*,
+                                        long long, bool, cudaStream_t);
+}  // namespace tc
+}  // namespace npm

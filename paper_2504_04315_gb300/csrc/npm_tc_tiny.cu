@@ -566,7 +566,7 @@ bool tiny_qualifies(const TcCfg& c) {
            tiny_layout(c, grid_bytes).bytes <= 227u * 1024u;
 }
 
-cudaError_t launch_tiny(const TcCfg& c, size_t, const __half* grid_h, const uint8_t* wblob, QueryBatch& qb,
+cudaError_t launch_tiny(const TcCfg& c, const __half* grid_h, const uint8_t* wblob, QueryBatch& qb,
                         int64_t max_n, int* status, cudaStream_t st, bool pdl) {
     auto kern = c.split ? k_forward_tiny<kOpsBf16x3> : c.f16 ? k_forward_tiny<kOpsFp16> : k_forward_tiny<kOpsBf16>;
     const uint32_t grid_bytes = (uint32_t)c.base.level_res[0] * c.base.level_res[0] * c.base.level_res[0] * 8u;

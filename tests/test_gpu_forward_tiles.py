@@ -1,0 +1,54 @@
+"""The tensor-core forward kernel at the edges of its tiles and groups: one
+query, a tile less or more one, one tile per SM and one more than every tile
+group holds, on networks whose inputs fill the activation columns unevenly
+(an odd number of one-feature levels before the product-mode inputs, an odd
+number of two-feature levels, 128-wide layers, sixteen lobes). Densities at
+the sampled directions against the FP64 oracle: 1e-4 in the FP32-accuracy
+mode, 2e-2 at the 99.9th percentile (the reduced-precision bar, denominator
+floored at 1e-2 / (4 pi)) otherwise."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from gpu_helpers import cuda, host, make_model
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+ODD_ONE = synth.Workload(name="3 levels x 1 feat, product", mode=synth.PRODUCT, level_res=[5, 9, 30], feat=1,
+                         log2_table=12, widths=[24, 16, 8], K=2)
+ODD_TWO = synth.Workload(name="5 levels x 2 feats", mode=synth.RADIANCE, level_res=[4, 7, 12, 25, 40], feat=2,
+                         log2_table=13, widths=[12, 32, 32], K=8)
+LOBES16 = synth.Workload(name="3 levels x 2 feats, product, K=16", mode=synth.PRODUCT, level_res=[6, 11, 40], feat=2,
+                         log2_table=12, widths=[28, 64, 64], K=16)
+WIDE = synth.Workload(name="2 levels x 4 feats, 128 wide", mode=synth.RADIANCE, level_res=[6, 30], feat=4,
+                      log2_table=13, widths=[8, 128, 20], K=5)
+
+
+@pytest.mark.parametrize("precision", [synth.FP32_TC, synth.BF16X3, synth.FP16], ids=["fp32tc", "bf16x3", "fp16"])
+@pytest.mark.parametrize("w", [ODD_ONE, ODD_TWO, LOBES16, WIDE], ids=lambda w: w.name.split(",")[0])
+def test_tile_edges(w, precision):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sizes = [1, 127, 129, sms * 128, 4 * sms * 128 + 1]
+    params = synth.random_params(w, 41)
+    m = make_model(w, params, sizes[-1], precision=precision)
+    for n in sizes:
+        pos, u = synth.positions(n, n), synth.sample_uniforms(n, n)
+        aux = synth.aux_inputs(n, n) if w.mode == synth.PRODUCT else None
+        d, p, _ = m.query_sample(cuda(pos), cuda(u), None if aux is None else cuda(aux))
+        m.check_device_status()
+        # Every query of the small batches; first, last and a seeded subset of
+        # the large ones.
+        pick = np.unique(np.r_[0, n - 1, np.random.default_rng(n).choice(n, min(n, 4096), replace=False)])
+        gd, gp = host(d)[:, pick].astype(np.float64), host(p)[pick]
+        ref = oracle.eval_pdf64(w, params, pos[:, pick], gd, None if aux is None else aux[:, pick])
+        if precision == synth.FP32_TC:
+            assert (np.abs(gp - ref) / ref).max() <= 1e-4, n
+        else:
+            assert np.quantile(np.abs(gp - ref) / np.maximum(ref, 1e-2 / (4 * math.pi)), 0.999) <= 2e-2, n
