@@ -87,7 +87,12 @@ enum { NPM_FP32 = 0, NPM_BF16 = 1, NPM_BF16X3 = 2, NPM_FP16 = 3, NPM_FP32_TC = 4
  *                  features, plus 21 SH/roughness values in product mode,
  *                  zero-padded), widths[n_layers] must equal 4K. Every width
  *                  is a multiple of 4 and at most NPM_MAX_WIDTH.
- *   precision      NPM_FP32: FP32 grid and CUDA-core FP32 MLP.
+ *   precision      NPM_FP32: FP32 grid and FP32 MLP arithmetic. Inference
+ *                  runs on the tensor cores with every activation and weight
+ *                  as three BF16 parts, which hold all 24 bits of an FP32
+ *                  value (products down to 2^-24 kept, FP32 accumulation);
+ *                  networks whose weights do not fit there in that form (more
+ *                  than about 34,000), and training, on the CUDA cores.
  *                  NPM_BF16: FP16 grid copy, BF16 tensor-core MLP (tcgen05)
  *                  with FP32 accumulation; all vMF math stays FP32. Single-
  *                  pass BF16 inference does NOT meet the reduced-precision
@@ -396,11 +401,10 @@ npm_status npm_scene_radiance(int product, uint64_t noise_seed, int64_t n, const
  * Errors: NPM_ERR_INVALID_ARG (configuration or arguments),
  * NPM_ERR_CAPACITY when the padded weights exceed
  * NPM_NOALLOC_MAX_WEIGHT_FLOATS, NPM_ERR_CUDA on a failed launch.
- * Kernel: the FP32 tile-group forward kernel, which has no kernel-internal
- * waits (no mailbox hand-offs between thread groups), so no launch can give
- * up part-way: when the call returns NPM_OK, every pdf_out value is written
- * by the work it queued. (npm_eval_pdf on a handle may run the
- * warp-specialised kernel instead, whose bounded waits report through the
+ * Kernel: the CUDA-core forward kernel, which has no kernel-internal waits,
+ * so no launch can give up part-way: when the call returns NPM_OK, every
+ * pdf_out value is written by the work it queued. (npm_eval_pdf on a handle
+ * runs the tensor-core kernel, whose bounded waits report through the
  * handle's status word; this entry point has no such word.)
  * Set-up: every call looks up the device address of the scratch array on
  * the current device (cudaGetSymbolAddress: no allocation; the first call
@@ -508,19 +512,20 @@ npm_status npm_pdf_integral(npm_handle* h, int64_t n_pos, const float* pos, cons
                             void* stream);
 
 /* Bound of the device-side waits inside the FP32 forward kernel of this
- * handle (its encoder and MLP thread groups hand tiles over through
- * shared-memory mailboxes; failure handling, not part of the method).
+ * handle (its threads wait on mbarriers for the weights' copy and for each
+ * layer's tensor-core instructions; failure handling, not part of the
+ * method).
  *   cycles > 0: a wait gives up after about `cycles` SM clock cycles
  *               (default 2^31, about a second at 2 GHz);
- *   cycles <= 0: every wait is one non-blocking test, so a hand-off that is
- *               not already complete gives up at once (this lets a test
+ *   cycles <= 0: every wait is one non-blocking test, so one for work that
+ *               is not already complete gives up at once (this lets a test
  *               exercise the timeout path without waiting).
  * A wait that gives up ends the kernel early: the outputs of that call are
  * incomplete and npm_check_device_status then returns NPM_ERR_TIMEOUT. The
- * kernel issues no asynchronous copies, so nothing is left in flight and the
- * context stays usable. Applies to launches made after the call; the
- * tensor-core kernels keep their fixed bound. Errors: NPM_ERR_INVALID_ARG
- * (NULL handle). */
+ * kernel first waits again, with a bound of its own, for the copies and
+ * tensor-core instructions it has in flight, so that the context stays
+ * usable. Applies to launches made after the call; the other precisions'
+ * kernels keep their fixed bound. Errors: NPM_ERR_INVALID_ARG (NULL handle). */
 npm_status npm_set_wait_limit(npm_handle* h, int64_t cycles);
 
 /* Debug builds (compiled with NPM_DEBUG_BOUNDS; not a hot call): every

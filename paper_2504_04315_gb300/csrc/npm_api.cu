@@ -153,24 +153,27 @@ npm_status check_call(npm_handle* h, int64_t n, int64_t ld, const void* pos, con
 // Device-side count of completed Adam steps (scalars[16]).
 int* step_dev(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 16); }
 
-// Padded FP32 forward weights of the moving average (inference).
-npm_status arrange_inference_weights(npm_handle* h, cudaStream_t st) {
+// The weights as the kernels read them: the tensor-core operands, and the
+// CUDA-core kernels' padded copies where those serve training or inference
+// (of the moving average too, when inference evaluates it).
+npm_status arrange_all_weights(npm_handle* h, cudaStream_t st) {
+    if (h->tc) {
+        NPM_CUDA(npm::tc_refresh_weights(h, !npm::tc_can_train(h), st), "arrange weights");
+        return NPM_OK;
+    }
+    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, h->wbwd, st), "arrange weights");
     if (h->ema)
         NPM_CUDA(npm::launch_arrange_weights(h->dc, h->ema + h->mlp_off, h->wfwd_inf, nullptr, st),
                  "arrange ema weights");
     return NPM_OK;
 }
 
-// Every copy derived from the parameters: the FP32 kernels' padded weights,
-// the FP16 grid and the tensor-core weights (of the moving average too,
-// when inference evaluates it).
+// Every copy derived from the parameters: the arranged weights and the FP16
+// grid.
 npm_status refresh_derived(npm_handle* h, cudaStream_t st) {
-    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, h->wbwd, st),
-             "arrange weights");
-    npm_status s = arrange_inference_weights(h, st);
+    npm_status s = arrange_all_weights(h, st);
     if (s != NPM_OK) return s;
     if (h->grid_h) NPM_CUDA(npm::launch_to_half(h->ng, inf_params(h), h->grid_h, st), "grid fp16 copy");
-    if (h->tc) NPM_CUDA(npm::tc_refresh_weights(h, st), "bf16 weight copy");
     return NPM_OK;
 }
 
@@ -295,10 +298,13 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
             npm_destroy(h);
             return s;
         }
-        if ((s = npm::tc_create(h)) != NPM_OK) {
-            npm_destroy(h);
-            return s;
-        }
+    }
+    // An FP32 model that the tensor-core forward does not hold runs on the
+    // CUDA-core kernels.
+    s = npm::tc_create(h);
+    if (s != NPM_OK && !(s == NPM_ERR_UNSUPPORTED && cfg->precision == NPM_FP32)) {
+        npm_destroy(h);
+        return s;
     }
     cudaMemset(h->grads, 0, h->n_int * sizeof(float));
     cudaMemset(h->adam_m, 0, h->n_int * sizeof(float));
@@ -501,7 +507,7 @@ npm_status npm_query_sample(npm_handle* h, int64_t n, const float* pos, const fl
     cudaStream_t st = (cudaStream_t)stream;
     if (h->tc) return npm::tc_query(h, n, ld, pos, aux, u, uniform_frac, true, dir_out, pdf_out, mix_out, st);
     NPM_CUDA(npm::launch_forward_fp32(h->dc, inf_params(h), inf_wfwd(h), n, ld, pos, aux, u, uniform_frac,
-                                      true, dir_out, pdf_out, mix_out, st, status_word(h), h->wait_limit),
+                                      true, dir_out, pdf_out, mix_out, st),
              "query_sample launch");
     return NPM_OK;
 }
@@ -578,7 +584,7 @@ npm_status npm_eval_pdf(npm_handle* h, int64_t n, const float* pos, const float*
     cudaStream_t st = (cudaStream_t)stream;
     if (h->tc) return npm::tc_query(h, n, ld, pos, aux, dir, 0.0f, false, nullptr, pdf_out, nullptr, st);
     NPM_CUDA(npm::launch_forward_fp32(h->dc, inf_params(h), inf_wfwd(h), n, ld, pos, aux, dir, 0.0f, false,
-                                      nullptr, pdf_out, nullptr, st, status_word(h), h->wait_limit),
+                                      nullptr, pdf_out, nullptr, st),
              "eval_pdf launch");
     return NPM_OK;
 }
@@ -594,8 +600,7 @@ npm_status npm_eval_log_pdf(npm_handle* h, int64_t n, const float* pos, const fl
     cudaStream_t st = (cudaStream_t)stream;
     if (h->tc) return npm::tc_query(h, n, ld, pos, aux, dir, 0.0f, false, nullptr, logpdf_out, nullptr, st, true);
     NPM_CUDA(npm::launch_forward_fp32(h->dc, inf_params(h), inf_wfwd(h), n, ld, pos, aux, dir, 0.0f, false,
-                                      nullptr, logpdf_out, nullptr, st, status_word(h), h->wait_limit, false,
-                                      true),
+                                      nullptr, logpdf_out, nullptr, st, true),
              "eval_log_pdf launch");
     return NPM_OK;
 }
@@ -625,16 +630,7 @@ static npm_status adam_impl(npm_handle* h, const float* loss, cudaStream_t st) {
                               h->cfg.beta1, h->cfg.beta2, h->cfg.eps, step_dev(h), loss, status,
                               h->grid_h, h->grid_h ? h->ng : 0, h->ema, h->ema_decay, st),
              "adam launch");
-    // The FP32 kernels' padded weights: needed unless the tensor-core
-    // kernels serve both inference and training.
-    if (!(h->tc && npm::tc_can_train(h))) {
-        NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, h->wbwd, st),
-                 "arrange weights");
-        npm_status s = arrange_inference_weights(h, st);
-        if (s != NPM_OK) return s;
-    }
-    if (h->tc) NPM_CUDA(npm::tc_refresh_weights(h, st), "bf16 weight copy");
-    return NPM_OK;
+    return arrange_all_weights(h, st);
 }
 
 npm_status npm_train_step(npm_handle* h, int64_t n, const float* pos, const float* aux,

@@ -401,6 +401,25 @@ __device__ __forceinline__ float inv_minus_coth(float k) {
     return 1.0f / k - 1.0f - 2.0f / expm1f(2.0f * k);
 }
 
+// Arrange layer l of the MLP weights (row-major [out][in] per layer, packed)
+// into the padded forward (W^T [in][np_fwd]) and backward (W [out][np_bwd];
+// may be NULL) blobs of the CUDA-core kernels; thread tid of nt.
+__device__ __forceinline__ void arrange_layer(const DevCfg& cfg, int l, const float* __restrict__ mlp,
+                                              float* __restrict__ wfwd, float* __restrict__ wbwd, int tid, int nt) {
+    for (int m = 0; m < l; ++m) mlp += cfg.widths[m] * cfg.widths[m + 1];
+    const int K = cfg.widths[l], N = cfg.widths[l + 1];
+    const int npf = cfg.np_fwd[l], npb = cfg.np_bwd[l];
+    for (int i = tid; i < K * npf; i += nt) {
+        const int k = i / npf, nn = i % npf;
+        wfwd[cfg.off_fwd[l] + i] = nn < N ? mlp[nn * K + k] : 0.0f;
+    }
+    if (wbwd)  // backward copy (training only)
+        for (int i = tid; i < N * npb; i += nt) {
+            const int nn = i / npb, k = i % npb;
+            wbwd[cfg.off_bwd[l] + i] = k < K ? mlp[nn * K + k] : 0.0f;
+        }
+}
+
 // A batch of query requests served by one launch of a forward kernel: the
 // kernel's tiles are numbered across segments; segment s owns tiles
 // [tile0, tile0 + ceil(n / tile size)). When n_dev is set (one segment),

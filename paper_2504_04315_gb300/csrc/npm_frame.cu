@@ -283,7 +283,7 @@ npm_status enqueue_frame(npm_wavefront* w, cudaStream_t st) {
         q.pdf = s.pdf;
         q.ufrac = w->cfg.uniform_frac;
         cudaError_t e = h->tc ? npm::tc_query_batch(h, qb, s.P, st, true)
-                              : npm::launch_forward_fp32_batch(h->dc, inf_params(h), inf_wfwd(h), qb, s.P, st, status_word(h), h->wait_limit);
+                              : npm::launch_forward_fp32_batch(h->dc, inf_params(h), inf_wfwd(h), qb, s.P, st);
         if (e != cudaSuccess) return npm::set_error(NPM_ERR_CUDA, cudaGetErrorString(e));
         e = npm::launch_maybe_pdl(k_wf_advance, dim3(g), dim3(kAdvanceThreads), 0, st, true, s, b, src);
         if (e != cudaSuccess) return npm::set_error(NPM_ERR_CUDA, cudaGetErrorString(e));

@@ -75,10 +75,12 @@ npm_status make_devcfg(const npm_config* cfg, DevCfg* out, int64_t* ng, int64_t*
 // Records msg as the thread's last error and returns s.
 npm_status set_error(npm_status s, const char* msg);
 
-// Tensor-core (tcgen05, BF16) path, npm_tc.cu.
+// Tensor-core (tcgen05) path, npm_tc.cu. An FP32 model that it does not hold
+// gets NPM_ERR_UNSUPPORTED from tc_create and runs on the CUDA-core kernels.
 npm_status tc_create(npm_handle* h);
 void tc_destroy(npm_handle* h);
-cudaError_t tc_refresh_weights(npm_handle* h, cudaStream_t st);
+// Weights arranged for the MMAs; with cuda_cores also h->wfwd and h->wbwd.
+cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st);
 // pdl: the small networks' kernel may be launched as a programmatic
 // dependent of the stream's previous kernel, which must then not write the
 // model's weights or grid (other kernels launch as usual).

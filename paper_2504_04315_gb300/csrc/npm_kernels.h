@@ -63,34 +63,21 @@ inline int env_override(const char* name, std::atomic<int>& cache) {
     return v;
 }
 
-// Default bound of a kernel-internal wait: 2^31 SM clock cycles (about a
-// second at 2 GHz).
-constexpr long long kDefaultWaitLimit = 1ll << 31;
-
 size_t fwd_smem_bytes(const DevCfg& c);
 // Shared-memory carveout (percent of the maximum) that holds `bytes`.
 int carveout_percent(size_t bytes);
 size_t train_smem_bytes(const DevCfg& c);
 
-// wait_free: use only the tile-group kernel, which has no kernel-internal
-// waits (no mailbox hand-offs), so no launch can end early on a timeout.
 // log_pdf (evaluation only): pdf_out receives log V instead of V.
 cudaError_t launch_forward_fp32(const DevCfg& cfg, const float* grid, const float* wfwd, int64_t n,
                                 int64_t ld, const float* pos, const float* aux, const float* uin,
                                 float ufrac, bool sample, float* dir_out, float* pdf_out,
-                                float* mix_out, cudaStream_t st, int* status = nullptr,
-                                long long wait_limit = kDefaultWaitLimit, bool wait_free = false,
-                                bool log_pdf = false);
+                                float* mix_out, cudaStream_t st, bool log_pdf = false);
 
 // Several requests in one launch (segment table; tile offsets filled in
-// here). max_n bounds the device-side count when qb.n_dev is set. status
-// (device word, or NULL) receives kStatusTimeout if a kernel-internal
-// hand-off gives up after wait_limit SM clock cycles (<= 0: one
-// non-blocking test per wait).
+// here). max_n bounds the device-side count when qb.n_dev is set.
 cudaError_t launch_forward_fp32_batch(const DevCfg& cfg, const float* grid, const float* wfwd,
-                                      QueryBatch& qb, int64_t max_n, cudaStream_t st,
-                                      int* status = nullptr, long long wait_limit = kDefaultWaitLimit,
-                                      bool wait_free = false);
+                                      QueryBatch& qb, int64_t max_n, cudaStream_t st);
 
 cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t mlp_off,
                               const float* wfwd, const float* wbwd, int64_t n, int64_t ld,

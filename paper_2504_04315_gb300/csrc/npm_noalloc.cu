@@ -75,11 +75,11 @@ extern "C" npm_status npm_eval_pdf_noalloc(const npm_config* cfg, const float* p
     k_noalloc_arrange<<<8, 256, 0, st>>>(dc, params + ng, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return npm::set_error(NPM_ERR_CUDA, cudaGetErrorString(e));
-    // The tile-group kernel only: it has no kernel-internal waits, so no
+    // The CUDA-core kernel: it has no kernel-internal waits, so no
     // launch can give up part-way, and with no status word to report such
     // an outcome every pdf_out value is written when the call succeeds.
     e = npm::launch_forward_fp32(dc, params, scratch, n, ld, pos, aux, dir, 0.0f, false, nullptr,
-                                 pdf_out, nullptr, st, nullptr, npm::kDefaultWaitLimit, true);
+                                 pdf_out, nullptr, st);
     if (e != cudaSuccess) return npm::set_error(NPM_ERR_CUDA, cudaGetErrorString(e));
     return NPM_OK;
 }

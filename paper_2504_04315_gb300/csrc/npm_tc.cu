@@ -219,31 +219,39 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
     for (; k < kend; ++k) store_one(sA, tile_off(row, k, kp), 0.0f, lo);
 }
 
-// Master FP32 weights (packed [out][in] per layer) -> BF16 blob in the UMMA
-// K-major layout, zero padded to Np x Kp per layer.
-__global__ void k_tc_weights(TcCfg tc, const float* __restrict__ mlp, uint8_t* __restrict__ blob) {
-    int64_t woff = 0;
-    for (int l = 0; l < tc.base.n_layers; ++l) {
-        const TcLayer& ly = tc.layer[l];
-        const int total = ly.Np * ly.Kp;
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-            const int nn = i / ly.Kp, k = i % ly.Kp;
-            const float v = (nn < ly.N && k < ly.K) ? mlp[woff + (int64_t)nn * ly.K + k] : 0.0f;
-            if (tc.f16) {
-                // FP16 high part and FP16 residual (the weights to ~22 bits)
-                const __half hh = __float2half_rn(v);
-                *reinterpret_cast<__half*>(blob + ly.w_off + tile_off(nn, k, ly.Kp)) = hh;
-                *reinterpret_cast<__half*>(blob + tc.w_bytes + ly.w_off + tile_off(nn, k, ly.Kp)) =
-                    __float2half_rn(v - __half2float(hh));
-                continue;
-            }
-            const __nv_bfloat16 hb = __float2bfloat16_rn(v);
-            *reinterpret_cast<__nv_bfloat16*>(blob + ly.w_off + tile_off(nn, k, ly.Kp)) = hb;
-            if (tc.split)
-                *reinterpret_cast<__nv_bfloat16*>(blob + tc.w_bytes + ly.w_off + tile_off(nn, k, ly.Kp)) =
-                    __float2bfloat16_rn(v - __bfloat162float(hb));
+// Master FP32 weights (packed [out][in] per layer) -> 16-bit operand parts in
+// the UMMA K-major layout, zero padded to Np x Kp per layer; with wfwd also
+// the CUDA-core kernels' padded copies. blockIdx.y: layer (one pass of load
+// latency for all layers instead of one each).
+__global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __restrict__ mlp,
+                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, float* __restrict__ wbwd) {
+    const int l = blockIdx.y;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, wbwd, tid, nt);
+    const TcLayer& ly = tc.layer[l];
+    for (int m = 0; m < l; ++m) mlp += tc.layer[m].K * tc.layer[m].N;
+    for (int i = tid; i < ly.Np * ly.Kp; i += nt) {
+        const int nn = i / ly.Kp, k = i % ly.Kp;
+        const float v = (nn < ly.N && k < ly.K) ? mlp[nn * ly.K + k] : 0.0f;
+        uint8_t* at = blob + ly.w_off + tile_off(nn, k, ly.Kp);
+        if (tc.f16) {
+            // FP16 high part and FP16 residual (the weights to ~22 bits)
+            const __half hh = __float2half_rn(v);
+            *reinterpret_cast<__half*>(at) = hh;
+            *reinterpret_cast<__half*>(at + tc.w_bytes) = __float2half_rn(v - __half2float(hh));
+            continue;
         }
-        woff += (int64_t)ly.K * ly.N;
+        // BF16 parts, each rounded to nearest from what the ones before
+        // leave (three hold all 24 bits). An infinite weight becomes the
+        // largest finite value in FP32 arithmetic, where its residuals
+        // would be NaN.
+        float rest = v;
+        for (int p = 0; p < tc.wparts; ++p) {
+            __nv_bfloat16 b = __float2bfloat16_rn(rest);
+            if (tc.wparts == 3 && __hisinf(b)) b = __float2bfloat16_rz(copysignf(3.38e38f, rest));
+            *reinterpret_cast<__nv_bfloat16*>(at + p * tc.w_bytes) = b;
+            rest -= __bfloat162float(b);
+        }
     }
 }
 
@@ -842,7 +850,8 @@ static int pad16(int v) { return (v + 15) / 16 * 16; }
 
 npm_status tc_create(npm_handle* h) {
     const npm_config& c = h->cfg;
-    if (c.feat_per_level != 1 && c.feat_per_level != 2 && c.feat_per_level != 4 &&
+    const bool fp32 = c.precision == NPM_FP32;
+    if (!fp32 && c.feat_per_level != 1 && c.feat_per_level != 2 && c.feat_per_level != 4 &&
         c.feat_per_level != 8)
         return NPM_ERR_UNSUPPORTED;
     TcState* s = new TcState();
@@ -883,16 +892,21 @@ npm_status tc_create(npm_handle* h) {
     t.a0_bytes = sep0 ? (uint32_t)(kTile * t.layer[0].Kp * 2) : 0u;
     t.split = (c.precision == NPM_BF16X3 || c.precision == NPM_FP32_TC) ? 1 : 0;
     t.f16 = (c.precision == NPM_FP16 || c.precision == NPM_FP32_TC) ? 1 : 0;
-    t.fp32 = c.precision == NPM_FP32_TC ? 1 : 0;
-    const uint32_t nsplit = t.split ? 2u : 1u;
-    const uint32_t nw = (t.split || t.f16) ? 2u : 1u;
+    t.fp32 = (c.precision == NPM_FP32_TC || fp32) ? 1 : 0;
+    t.parts = fp32 ? 3 : t.split ? 2 : 1;
+    t.wparts = fp32 ? 3 : (t.split || t.f16) ? 2 : 1;
+    const uint32_t nsplit = (uint32_t)t.parts, nw = (uint32_t)t.wparts;
     int maxkp = 16;
     for (int l = 0; l < c.n_layers; ++l) maxkp = std::max(maxkp, t.layer[l].Kp);
     t.d_cols = (uint32_t)((maxnp + 31) / 32 * 32);
     t.a_cols = (uint32_t)(maxkp / 2);
     t.g_cols = t.d_cols + nsplit * t.a_cols;
     t.enc_width = enc_width;
-    if (nw * t.w_bytes + nsplit * (t.a0_bytes + t.a_bytes) + 64 > 200 * 1024 || c.K > 16) {
+    // FP32 models that do not fit keep the CUDA-core kernels; in the other
+    // modes the limit (weights and one pair of activation tiles) is part of
+    // the interface.
+    if (fp32 ? nw * t.w_bytes > 200 * 1024 || t.g_cols > 512u
+             : nw * t.w_bytes + nsplit * (t.a0_bytes + t.a_bytes) + 64 > 200 * 1024 || c.K > 16) {
         delete s;
         return NPM_ERR_UNSUPPORTED;
     }
@@ -906,6 +920,7 @@ npm_status tc_create(npm_handle* h) {
         s->train_cfg = t;
         // Training multiplies BF16 operands whatever the inference format.
         s->train_cfg.f16 = 0;
+        s->train_cfg.wparts = 2;
         for (int l = 0; l < c.n_layers; ++l) s->train_cfg.layer[l].idesc |= (1u << 7) | (1u << 10);
         uint32_t off = 2u * t.w_bytes, col0 = 0, cols = 0;
         int64_t wo = 0;
@@ -964,7 +979,7 @@ npm_status tc_create(npm_handle* h) {
         // the shared residual tile.
         s->train_cfg.split = tr.split;
         s->train_cfg.a_bytes = tr.hlo_off - tr.h_off[0];
-        // The FP32-accuracy mode trains with the FP32 kernels.
+        // FP32 and the FP32-accuracy mode train with the FP32 kernels.
         s->can_train = fits && pw <= 512 && tr.smem <= 220 * 1024 && !t.fp32;
     }
     if (device_alloc((void**)&s->wblob, nw * t.w_bytes) != cudaSuccess) {
@@ -1003,18 +1018,21 @@ void tc_destroy(npm_handle* h) {
     h->tc = nullptr;
 }
 
-cudaError_t tc_refresh_weights(npm_handle* h, cudaStream_t st) {
+cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) {
     TcState* s = h->tc;
-    k_tc_weights<<<16, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob);
-    if (s->wblob_train) k_tc_weights<<<16, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train);
+    const dim3 grid(16, h->dc.n_layers);
+    k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr,
+                                       h->wbwd);
+    if (s->wblob_train)
+        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr);
     if (h->ema) {
         if (!s->wblob_inf) {
-            const size_t bytes = ((s->cfg.split || s->cfg.f16) ? 2u : 1u) * (size_t)s->cfg.w_bytes;
+            const size_t bytes = (size_t)s->cfg.wparts * s->cfg.w_bytes;
             cudaError_t e = cudaMalloc(&s->wblob_inf, bytes);
             if (e != cudaSuccess) return e;
             cudaMemsetAsync(s->wblob_inf, 0, bytes, st);
         }
-        k_tc_weights<<<16, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr);
     }
     return cudaGetLastError();
 }
@@ -1086,7 +1104,9 @@ cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStr
     const uint8_t* wb = h->ema ? s->wblob_inf : s->wblob;  // inference weights
     int* status = status_word(h);
     const long long limit = 1ll << 32;  // the tensor-core kernels' fixed bound
-    // The FP32-accuracy mode gathers from the FP32 table.
+    // FP32 and the FP32-accuracy mode gather from the FP32 table.
+    if (c.parts == 3)
+        return launch_fwd_ops<kThreeBf16>(c, inf_params(h), wb, qb, max_n, status, h->wait_limit, false, st);
     if (c.fp32) return launch_fwd_ops<kTwoFp16>(c, inf_params(h), wb, qb, max_n, status, limit, false, st);
     // The small serving networks get their own kernel (npm_tc_tiny.cu);
     // tuning override NPM_TC_TINY=0 selects the general kernel instead.

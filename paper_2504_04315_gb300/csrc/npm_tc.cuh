@@ -34,12 +34,13 @@ struct TcCfg {
     uint32_t a0_bytes; // bytes of the layer-0 input tile when it has its own
                        // buffer (the encoding leaves all-zero 8-column chunks);
                        // 0 when layer 0 shares the buffer of layers >= 1
-    int split;         // 1: BF16 residual operands (three MMAs per K step)
+    int parts, wparts; // 16-bit operand parts of an activation and of a weight
+    int split;         // 1: two BF16 parts (three MMAs per K step)
     int f16;           // 1: FP16 operands: activations rounded to FP16, weights
                        // FP16 plus an FP16 residual (two MMAs per K step);
                        // with split, activations FP16 plus an FP16 residual too
-    int fp32;          // 1: the FP32-accuracy mode (split FP16 operands, FP32
-                       // grid table, the FP32 path's sampler)
+    int fp32;          // 1: FP32 or the FP32-accuracy mode (FP32 grid table, the
+                       // FP32 path's sampler)
     // Tensor-memory columns of a forward tile group: d_cols of accumulator,
     // then one a_cols wide block per activation part (two 16-bit values to a
     // column); g_cols in all.
@@ -387,7 +388,9 @@ cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint8_t* wblo
 //   kOneFp16   activations rounded to FP16, weights FP16 plus residual
 //   kTwoBf16   activations and weights BF16 plus residual
 //   kTwoFp16   activations and weights FP16 plus residual, FP32 grid table
-enum : int { kOneBf16 = 0, kOneFp16 = 1, kTwoBf16 = 2, kTwoFp16 = 3 };
+//   kThreeBf16 activations and weights as three BF16 parts (all 24 bits of an
+//              FP32 value), FP32 grid table: FP32 arithmetic
+enum : int { kOneBf16 = 0, kOneFp16 = 1, kTwoBf16 = 2, kTwoFp16 = 3, kThreeBf16 = 4 };
 
 // Fused forward of the small serving networks (npm_tc_tiny.cu): radiance
 // mode, one dense level of 4 features, three layers of at most 32 outputs

@@ -31,6 +31,16 @@
 // 300,007 queries, 339 -> 140 us (one group -> four); paper-shaped hash grid,
 // FP16, 2,073,600 queries, 869 -> 719 us (three -> four); eight dense levels
 // of four features, split BF16, 250,007 densities, 102 -> 72 us.
+//
+// FP32 models run here too, their values as three BF16 parts: 8 + 8 + 8 bits
+// hold an FP32 value, and six products of parts leave out less than 2^-24 of
+// it. Against the CUDA-core kernel (GB300): paper-shaped hash grid, 2^20
+// queries, 722 -> 567 us, 3,001 log densities 31 -> 23 us; at 2^18 queries
+// eight dense levels of four features 175 -> 115, 96-wide layers 302 -> 133,
+// 128-wide (one group by its tensor-memory columns) 357 -> 222, sixteen lobes
+// 258 -> 176, one level into 32-wide layers 46 -> 44 us. The error against
+// FP64 stays where it was (density 3.6e-6 and 3.7e-6 relative, log density
+// 2.7e-7 and 2.1e-7): the hardware exponentials decide it.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -48,9 +58,10 @@ namespace tc {
 
 template <int OPS>
 struct OpsTraits {
-    static constexpr int parts = OPS == kOneBf16 || OPS == kOneFp16 ? 1 : 2;  // of an activation
-    static constexpr int wparts = OPS == kOneBf16 ? 1 : 2;                    // of a weight
-    static constexpr bool fp32 = OPS == kTwoFp16;  // FP32 grid table and sampler
+    // Parts of an activation and of a weight.
+    static constexpr int parts = OPS == kThreeBf16 ? 3 : OPS == kOneBf16 || OPS == kOneFp16 ? 1 : 2;
+    static constexpr int wparts = OPS == kThreeBf16 ? 3 : OPS == kOneBf16 ? 1 : 2;
+    static constexpr bool fp32 = OPS == kTwoFp16 || OPS == kThreeBf16;  // FP32 grid table and sampler
     using GridT = typename std::conditional<fp32, float, __half>::type;
 };
 
@@ -59,6 +70,25 @@ struct OpsTraits {
 __host__ __device__ constexpr int fwd_groups(int kmax) { return kmax > 8 ? 2 : 4; }
 
 // ----------------------------------------------------------- operands
+
+// Three BF16 parts of a pair: each rounded to nearest from what the ones
+// before leave, so that they add up to all 24 bits of the value. Infinities
+// become the largest finite value (an infinite part would make the others
+// NaN).
+__device__ __forceinline__ uint32_t bf16x2_finite(float a, float b) {
+    uint32_t d;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    return d;
+}
+__device__ __forceinline__ void three_bf16(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+    p0 = bf16x2_finite(a, b);
+    a -= __uint_as_float(p0 << 16);
+    b -= __uint_as_float(p0 & 0xffff0000u);
+    p1 = bf16x2_finite(a, b);
+    a -= __uint_as_float(p1 << 16);
+    b -= __uint_as_float(p1 & 0xffff0000u);
+    p2 = bf16x2_finite(a, b);
+}
 
 // The operand parts of a pair of values (the first in the low half).
 template <int OPS>
@@ -70,6 +100,8 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[OpsTr
     } else if constexpr (OPS == kTwoFp16) {
         p[0] = pack_f16_sat(a, b);
         p[1] = f16_residual(p[0], a, b);
+    } else if constexpr (OPS == kThreeBf16) {
+        three_bf16(a, b, p[0], p[1], p[2]);
     } else {
         p[0] = pack_bf16(a, b);
         p[1] = pack_bf16(a - __uint_as_float(p[0] << 16), b - __uint_as_float(p[0] & 0xffff0000u));
@@ -85,7 +117,7 @@ __device__ __forceinline__ void relu_split_pair(float a, float b, uint32_t (&p)[
         asm("cvt.rn.satfinite.relu.f16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
     } else if constexpr (OPS == kOneBf16) {
         asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
-    } else if constexpr (OPS == kTwoFp16) {
+    } else if constexpr (OPS == kTwoFp16 || OPS == kThreeBf16) {
         split_pair<OPS>(fmaxf(a, 0.0f), fmaxf(b, 0.0f), p);
     } else {
         asm("cvt.rz.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
@@ -232,15 +264,17 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
                 const float2 a = blend_level2(cl, v);
                 row.put(a.x);
                 row.put(a.y);
-            } else {  // F = 1
-                const auto* g = grid + cfg.level_off[l];
+            } else {  // one, or another number that no vector load fits
+                const auto* g = grid + (size_t)cfg.level_off[l] * F;
                 uint32_t idx[8];
                 float w[8];
                 corners8(cfg, l, cl, idx, w);
-                float s = 0.0f;
+                for (int f = 0; f < F; ++f) {
+                    float s = 0.0f;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) s = fmaf(w[c], load_feat(g + idx[c], 0), s);
-                row.put(s);
+                    for (int c = 0; c < 8; ++c) s = fmaf(w[c], load_feat(g + (size_t)idx[c] * F, f), s);
+                    row.put(s);
+                }
             }
         }
         if (cfg.mode != NPM_PRODUCT && (row.k & 1)) row.put(0.0f);
@@ -256,7 +290,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
     }
     uint32_t col = (uint32_t)(cfg.grid_feats + 1) >> 1;
     if (cfg.mode == NPM_PRODUCT) {
-        if (F != 1 && !(FEAT == 0 && F == 2)) {
+        if (FEAT != 0 || F == 4 || F == 8) {
             // An even number of grid features: 21 values and one zero.
             float e[22];
             sh_band4(ax[0], ax[1], ax[2], e);
@@ -513,8 +547,14 @@ __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, 
             accum = 1u;
         }
     };
-    if constexpr (OpsTraits<OPS>::parts == 2) product(1, 0);
-    if constexpr (OpsTraits<OPS>::wparts == 2) product(0, 1);
+    if constexpr (OPS == kThreeBf16) {
+        // (1, 2), (2, 1) and (2, 2) lie 2^-26 and more below the product.
+        product(0, 2);
+        product(2, 0);
+        product(1, 1);
+    }
+    if constexpr (OpsTraits<OPS>::parts >= 2) product(1, 0);
+    if constexpr (OpsTraits<OPS>::wparts >= 2) product(0, 1);
     product(0, 0);
 }
 

@@ -1,0 +1,10 @@
+// npm_tc_fwd_fp32.cu -- the tensor-core forward kernel (npm_tc_forward.cuh) in
+// FP32 arithmetic: every activation and weight as three BF16 parts.
+#include "npm_tc_forward.cuh"
+
+namespace npm {
+namespace tc {
+template cudaError_t launch_fwd_ops<kThreeBf16>(const TcCfg&, const void*, const uint8_t*, QueryBatch&, int64_t, int*,
+                                                long long, bool, cudaStream_t);
+}  // namespace tc
+}  // namespace npm

@@ -2,10 +2,10 @@
 query, a tile less or more one, one tile per SM and one more than every tile
 group holds, on networks whose inputs fill the activation columns unevenly
 (an odd number of one-feature levels before the product-mode inputs, an odd
-number of two-feature levels, 128-wide layers, sixteen lobes). Densities at
-the sampled directions against the FP64 oracle: 1e-4 in the FP32-accuracy
-mode, 2e-2 at the 99.9th percentile (the reduced-precision bar, denominator
-floored at 1e-2 / (4 pi)) otherwise."""
+number of two-feature levels, three-feature levels, 128-wide layers, sixteen
+lobes). Densities at the sampled directions against the FP64 oracle: 1e-4 in
+FP32 and the FP32-accuracy mode, 2e-2 at the 99.9th percentile (the
+reduced-precision bar, denominator floored at 1e-2 / (4 pi)) otherwise."""
 import math
 
 import numpy as np
@@ -29,11 +29,23 @@ WIDE = synth.Workload(name="2 levels x 4 feats, 128 wide", mode=synth.RADIANCE, 
                       log2_table=13, widths=[8, 128, 20], K=5)
 
 
-@pytest.mark.parametrize("precision", [synth.FP32_TC, synth.BF16X3, synth.FP16], ids=["fp32tc", "bf16x3", "fp16"])
-@pytest.mark.parametrize("w", [ODD_ONE, ODD_TWO, LOBES16, WIDE], ids=lambda w: w.name.split(",")[0])
-def test_tile_edges(w, precision):
+THREE = synth.Workload(name="3 levels x 3 feats", mode=synth.RADIANCE, level_res=[6, 11, 40], feat=3,
+                       log2_table=12, widths=[12, 32, 12], K=3)
+
+PRECISIONS = {"fp32": synth.FP32, "fp32tc": synth.FP32_TC, "bf16x3": synth.BF16X3, "fp16": synth.FP16}
+# Three features per level are FP32's alone.
+CASES = [(w, p) for w in (ODD_ONE, ODD_TWO, LOBES16, WIDE) for p in PRECISIONS] + [(THREE, "fp32")]
+
+
+@pytest.fixture(autouse=True)
+def _need_cuda():
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA GPU")
+
+
+@pytest.mark.parametrize("w,precision", CASES, ids=lambda v: v if isinstance(v, str) else v.name.split(",")[0])
+def test_tile_edges(w, precision):
+    precision = PRECISIONS[precision]
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     sizes = [1, 127, 129, sms * 128, 4 * sms * 128 + 1]
     params = synth.random_params(w, 41)
@@ -48,7 +60,25 @@ def test_tile_edges(w, precision):
         pick = np.unique(np.r_[0, n - 1, np.random.default_rng(n).choice(n, min(n, 4096), replace=False)])
         gd, gp = host(d)[:, pick].astype(np.float64), host(p)[pick]
         ref = oracle.eval_pdf64(w, params, pos[:, pick], gd, None if aux is None else aux[:, pick])
-        if precision == synth.FP32_TC:
+        if precision in (synth.FP32, synth.FP32_TC):
             assert (np.abs(gp - ref) / ref).max() <= 1e-4, n
         else:
             assert np.quantile(np.abs(gp - ref) / np.maximum(ref, 1e-2 / (4 * math.pi)), 0.999) <= 2e-2, n
+
+
+def test_fp32_range():
+    # Hidden values around 1e20 and weights around 1e-20: FP32 keeps its
+    # accuracy over the exponents that a 16-bit format of narrower range
+    # would lose.
+    w, n = ODD_TWO, 2000
+    params = synth.random_params(w, 42)
+    ng = sum(synth.grid_sizes(w)) * w.feat
+    k = w.widths[0] * w.widths[1]
+    params[ng:ng + k] *= np.float32(2.0 ** 66)
+    params[ng + k:] *= np.float32(2.0 ** -66)
+    pos, u = synth.positions(5, n), synth.sample_uniforms(5, n)
+    m = make_model(w, params, n, precision=synth.FP32)
+    d, p, _ = m.query_sample(cuda(pos), cuda(u))
+    m.check_device_status()
+    ref = oracle.eval_pdf64(w, params, pos, host(d).astype(np.float64))
+    assert (np.abs(host(p) - ref) / ref).max() <= 1e-4
