@@ -360,7 +360,11 @@ npm_status npm_destroy(npm_handle* h) {
 
 int64_t npm_num_params(const npm_handle* h) { return h ? h->ng + h->nmlp : -1; }
 
-float* npm_params_device(npm_handle* h) { return h ? h->params : nullptr; }
+float* npm_params_device(npm_handle* h) {
+    if (!h) return nullptr;
+    h->params_shared = true;
+    return h->params;
+}
 float* npm_grads_device(npm_handle* h) { return h ? h->grads : nullptr; }
 
 static npm_status copy_public(npm_handle* h, float* dev, float* host, int64_t count, bool to_dev) {

@@ -27,7 +27,11 @@ struct npm_handle {
     float* wfwd = nullptr;     // padded W^T blobs for the FP32 kernels
     float* wbwd = nullptr;     // padded W blobs (backward)
     __half* grid_h = nullptr;  // FP16 grid copy (BF16 precision)
-    float* scalars = nullptr;  // [0] loss accumulator, [8] status word
+    // [0] loss accumulator, [8] status word, [16] Adam steps, [24] version of
+    // the parameters (both counted on the device, so that replayed graphs
+    // count too)
+    float* scalars = nullptr;
+    bool params_shared = false;  // npm_params_device has handed them out
     float* stage = nullptr;    // device staging for the _host entry points
     cudaStream_t side[2] = {nullptr, nullptr};  // internal streams (host staging)
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -50,6 +54,8 @@ inline const float* inf_params(const npm_handle* h) { return h->ema ? h->ema : h
 inline const float* inf_wfwd(const npm_handle* h) { return h->ema ? h->wfwd_inf : h->wfwd; }
 // Device status word (kStatus* bits, read by npm_check_device_status).
 inline int* status_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 8); }
+// Device-side counter of changes to the parameters.
+inline int* version_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 24); }
 
 namespace npm {
 // NVTX range named after an entry point for the lifetime of the object, so

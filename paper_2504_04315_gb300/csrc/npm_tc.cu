@@ -221,11 +221,14 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
 
 // Master FP32 weights (packed [out][in] per layer) -> 16-bit operand parts in
 // the UMMA K-major layout, zero padded to Np x Kp per layer; with wfwd also
-// the CUDA-core kernels' padded copies. blockIdx.y: layer (one pass of load
-// latency for all layers instead of one each).
+// the CUDA-core kernels' padded copies; with version counts a change of the
+// parameters. blockIdx.y: layer (one pass of load latency for all layers
+// instead of one each).
 __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __restrict__ mlp,
-                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, float* __restrict__ wbwd) {
+                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, float* __restrict__ wbwd,
+                             int* __restrict__ version) {
     const int l = blockIdx.y;
+    if (version && l == 0 && blockIdx.x == 0 && threadIdx.x == 0) *version += 1;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, wbwd, tid, nt);
     const TcLayer& ly = tc.layer[l];
@@ -253,6 +256,59 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __re
             rest -= __bfloat162float(b);
         }
     }
+}
+
+// ------------------------------------------------------- corner blocks
+
+// Entries of a chunk of corner blocks (kept up to date as a whole).
+constexpr int kBlkChunk = 1024;
+// Queries from which a batch uses them. Tables in the L2, without and with
+// blocks (GB300; paper-shaped hash grid in FP32 and FP16, eight dense levels
+// of four features in split BF16): 2^17 queries 85 and 83, 55 and 52, 41 and
+// 39 us, about what bringing stale blocks up to date takes (9 us); 2^18 151
+// and 143, 103 and 93, 75 and 67; 2^20 562 and 509, 371 and 326, 260 and 216.
+constexpr int64_t kBlkMinQueries = 1 << 18;
+
+// Rewrites the chunks of corner blocks whose parameters have changed since
+// (built[chunk] != *version), or all (force). Each chunk's mark is set by the
+// thread block that wrote all of it, so that launches on several streams may
+// overlap: they write the same bytes, and a query sees its own stream's
+// launch complete. Bound by its writes: 33 MB for 1.02 M entries.
+template <typename GT, int F>
+__global__ void __launch_bounds__(256) k_corner_blocks(const __grid_constant__ TcCfg tc, const GT* __restrict__ table,
+                                                       uint4* __restrict__ blk, uint32_t total,
+                                                       int* __restrict__ built, const int* __restrict__ version,
+                                                       int force) {
+    constexpr int C = blk_corners(F, sizeof(GT)), V = 8 / C;  // corners, 32-bit values a corner
+    __shared__ int now, stale;
+    if (threadIdx.x == 0) {
+        now = *version;
+        stale = force || built[blockIdx.x] != now;
+    }
+    __syncthreads();
+    if (!stale) return;
+    const DevCfg& cfg = tc.base;
+    const uint32_t* t32 = reinterpret_cast<const uint32_t*>(table);
+    for (uint32_t e = blockIdx.x * kBlkChunk + threadIdx.x; e < min(total, (blockIdx.x + 1) * kBlkChunk);
+         e += blockDim.x) {
+        int l = -1;  // the last level with blocks that starts at or before e
+        for (int m = 0; m < cfg.n_levels; ++m)
+            if (((tc.blk_mask >> m) & 1u) && tc.blk_off[m] <= e) l = m;
+        const uint32_t D = (uint32_t)cfg.level_res[l], i = e - tc.blk_off[l], last = D * D * D - 1u;
+        uint32_t r[8];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            // (entries past the level's end belong to no cell)
+            const uint32_t at = cfg.level_off[l] + min(i + (c & 1) + ((c & 2) ? D : 0u) + ((c & 4) ? D * D : 0u), last);
+#pragma unroll
+            for (int q = 0; q < V; ++q) r[c * V + q] = t32[(size_t)at * V + q];
+        }
+        blk[2 * (size_t)e] = make_uint4(r[0], r[1], r[2], r[3]);
+        blk[2 * (size_t)e + 1] = make_uint4(r[4], r[5], r[6], r[7]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) built[blockIdx.x] = now;
 }
 
 // ----------------------------------------------------------- training
@@ -840,6 +896,11 @@ struct TcState {
     TcCfg train_cfg;     // copy of cfg for training (split operands)
     TcTrain train;
     bool can_train = false;
+    // Corner blocks of the inference table (npm_tc.cuh), the version of the
+    // parameters that each chunk was built from, and their number; NULL: none.
+    uint4* blk = nullptr;
+    int* blk_built = nullptr;
+    uint32_t blk_total = 0;
     // Grid features of a training batch (max_batch x grid_feats FP32) for
     // 2-feature grids, written by k_train_encode; NULL: the training kernel
     // gathers them itself.
@@ -901,7 +962,6 @@ npm_status tc_create(npm_handle* h) {
     t.d_cols = (uint32_t)((maxnp + 31) / 32 * 32);
     t.a_cols = (uint32_t)(maxkp / 2);
     t.g_cols = t.d_cols + nsplit * t.a_cols;
-    t.enc_width = enc_width;
     // FP32 models that do not fit keep the CUDA-core kernels; in the other
     // modes the limit (weights and one pair of activation tiles) is part of
     // the interface.
@@ -1004,6 +1064,31 @@ npm_status tc_create(npm_handle* h) {
             s->enc = nullptr;
         }
     }
+    // Optional too: corner blocks, in level order while they stay a part of
+    // the L2 (64 of 129 MB).
+    if (c.feat_per_level == 2 || c.feat_per_level == 4) {
+        constexpr uint64_t kMost = (64ull << 20) / 32;
+        uint64_t total = 0;
+        for (int l = 0; l < c.n_levels; ++l) {
+            const uint64_t D = (uint64_t)c.level_res[l], entries = D * D * D;
+            if (!((h->dc.dense_mask >> l) & 1u) || total + entries > kMost) continue;
+            t.blk_mask |= 1u << l;
+            t.blk_off[l] = (uint32_t)total;
+            total += entries;
+        }
+        const size_t chunks = (size_t)((total + kBlkChunk - 1) / kBlkChunk);
+        if (tiny_qualifies(t)) total = 0;  // keeps its table in shared memory
+        if (total && device_alloc((void**)&s->blk, 32 * (size_t)total) == cudaSuccess) {
+            if (device_alloc((void**)&s->blk_built, chunks * sizeof(int)) != cudaSuccess) {
+                cudaFree(s->blk);
+                s->blk = nullptr;
+            } else {
+                cudaMemset(s->blk_built, 0, chunks * sizeof(int));
+                s->blk_total = (uint32_t)total;
+            }
+        }
+        cudaGetLastError();
+    }
     h->tc = s;
     return NPM_OK;
 }
@@ -1014,6 +1099,8 @@ void tc_destroy(npm_handle* h) {
     if (h->tc->wblob_inf) cudaFree(h->tc->wblob_inf);
     if (h->tc->wblob_train) cudaFree(h->tc->wblob_train);
     if (h->tc->enc) cudaFree(h->tc->enc);
+    if (h->tc->blk) cudaFree(h->tc->blk);
+    if (h->tc->blk_built) cudaFree(h->tc->blk_built);
     delete h->tc;
     h->tc = nullptr;
 }
@@ -1022,9 +1109,10 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
     TcState* s = h->tc;
     const dim3 grid(16, h->dc.n_layers);
     k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr,
-                                       h->wbwd);
+                                       h->wbwd, version_word(h));
     if (s->wblob_train)
-        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr,
+                                           nullptr);
     if (h->ema) {
         if (!s->wblob_inf) {
             const size_t bytes = (size_t)s->cfg.wparts * s->cfg.w_bytes;
@@ -1032,7 +1120,7 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
             if (e != cudaSuccess) return e;
             cudaMemsetAsync(s->wblob_inf, 0, bytes, st);
         }
-        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr, nullptr);
     }
     return cudaGetLastError();
 }
@@ -1098,28 +1186,54 @@ cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, con
               : launch_train_tc<16, false>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
 }
 
+// The corner blocks of the inference table, brought up to date on st.
+template <typename GT>
+static cudaError_t update_blocks(npm_handle* h, const GT* table, int force, cudaStream_t st) {
+    TcState* s = h->tc;
+    const unsigned chunks = (s->blk_total + kBlkChunk - 1) / kBlkChunk;
+    if (h->cfg.feat_per_level == 2)
+        k_corner_blocks<GT, 2><<<chunks, 256, 0, st>>>(s->cfg, table, s->blk, s->blk_total, s->blk_built,
+                                                       version_word(h), force);
+    else
+        k_corner_blocks<GT, 4><<<chunks, 256, 0, st>>>(s->cfg, table, s->blk, s->blk_total, s->blk_built,
+                                                       version_word(h), force);
+    return cudaGetLastError();
+}
+
 cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStream_t st, bool pdl) {
     const TcState* s = h->tc;
     const TcCfg& c = s->cfg;
     const uint8_t* wb = h->ema ? s->wblob_inf : s->wblob;  // inference weights
     int* status = status_word(h);
-    const long long limit = 1ll << 32;  // the tensor-core kernels' fixed bound
-    // FP32 and the FP32-accuracy mode gather from the FP32 table.
-    if (c.parts == 3)
-        return launch_fwd_ops<kThreeBf16>(c, inf_params(h), wb, qb, max_n, status, h->wait_limit, false, st);
-    if (c.fp32) return launch_fwd_ops<kTwoFp16>(c, inf_params(h), wb, qb, max_n, status, limit, false, st);
     // The small serving networks get their own kernel (npm_tc_tiny.cu);
     // tuning override NPM_TC_TINY=0 selects the general kernel instead.
     static std::atomic<int> env_tiny{INT32_MIN + 1};
     if (tiny_qualifies(c) && env_override("NPM_TC_TINY", env_tiny) != 0)
         return launch_tiny(c, h->grid_h, wb, qb, max_n, status, st, pdl);
+    // Large batches read the dense levels through corner blocks.
+    int64_t queries = 0;
+    for (int i = 0; i < qb.nseg; ++i) queries += qb.seg[i].n;
+    if (qb.n_dev) queries = max_n;
+    const uint4* blk = s->blk && queries >= kBlkMinQueries ? s->blk : nullptr;
+    if (blk) {
+        // FP32 tables are the parameters themselves: a caller that holds
+        // their address may change them unseen.
+        cudaError_t e = c.fp32 ? update_blocks(h, inf_params(h), h->params_shared ? 1 : 0, st)
+                               : update_blocks(h, h->grid_h, 0, st);
+        if (e != cudaSuccess) return e;
+    }
+    const long long limit = 1ll << 32;  // the 16-bit kernels' fixed bound
+    // FP32 and the FP32-accuracy mode gather from the FP32 table.
+    if (c.parts == 3)
+        return launch_fwd_ops<kThreeBf16>(c, inf_params(h), blk, wb, qb, max_n, status, h->wait_limit, false, st);
+    if (c.fp32) return launch_fwd_ops<kTwoFp16>(c, inf_params(h), blk, wb, qb, max_n, status, limit, false, st);
     // Tuning override NPM_TC_DECODE=1: the warp-per-query decode (up to eight
     // lobes).
     static std::atomic<int> env_dec{INT32_MIN + 1};
     const bool warp_decode = c.base.K <= 8 && env_override("NPM_TC_DECODE", env_dec) == 1;
-    if (c.f16) return launch_fwd_ops<kOneFp16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
-    if (c.split) return launch_fwd_ops<kTwoBf16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
-    return launch_fwd_ops<kOneBf16>(c, h->grid_h, wb, qb, max_n, status, limit, warp_decode, st);
+    if (c.f16) return launch_fwd_ops<kOneFp16>(c, h->grid_h, blk, wb, qb, max_n, status, limit, warp_decode, st);
+    if (c.split) return launch_fwd_ops<kTwoBf16>(c, h->grid_h, blk, wb, qb, max_n, status, limit, warp_decode, st);
+    return launch_fwd_ops<kOneBf16>(c, h->grid_h, blk, wb, qb, max_n, status, limit, warp_decode, st);
 }
 
 npm_status tc_query(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,

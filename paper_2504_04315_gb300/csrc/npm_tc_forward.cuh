@@ -31,6 +31,8 @@
 // 300,007 queries, 339 -> 140 us (one group -> four); paper-shaped hash grid,
 // FP16, 2,073,600 queries, 869 -> 719 us (three -> four); eight dense levels
 // of four features, split BF16, 250,007 densities, 102 -> 72 us.
+// Large batches read the dense levels through corner blocks (npm_tc.cuh), one
+// or two 32-byte loads a level.
 //
 // FP32 models run here too, their values as three BF16 parts: 8 + 8 + 8 bits
 // hold an FP32 value, and six products of parts leave out less than 2^-24 of
@@ -142,12 +144,27 @@ __device__ __forceinline__ void put_pairs(uint32_t act, uint32_t part_cols, uint
 
 // ------------------------------------------------------------- encode
 
-// Two levels' corner features are gathered before either is blended, so that
-// 16 loads (F = 2) are in flight.
+// The grid table and, where a level has them, its corner blocks.
 template <typename GT>
-__device__ __forceinline__ void gather_level2(const DevCfg& cfg, const GT* __restrict__ grid, int l, const Cell& cl,
+struct GridView {
+    const GT* table;
+    const uint4* blk;  // NULL: none
+    uint32_t mask;     // levels with blocks
+    __device__ __forceinline__ bool has(int l) const { return (mask >> l) & 1u; }
+};
+
+// Corner features of level l. Two levels are gathered before either is
+// blended, so that up to 16 loads are in flight.
+template <typename GT>
+__device__ __forceinline__ void gather_level2(const TcCfg& tc, const GridView<GT>& grid, int l, const Cell& cl,
                                               float2 (&v)[8]) {
-    const GT* g = grid + (size_t)cfg.level_off[l] * 2;
+    const DevCfg& cfg = tc.base;
+    if (grid.has(l)) {
+        const uint32_t D = (uint32_t)cfg.level_res[l];
+        gather_blocks2(grid.blk, tc.blk_off[l] + corner_idx1(cfg, l, cl, 0), D * D, grid.table, v);
+        return;
+    }
+    const GT* g = grid.table + (size_t)cfg.level_off[l] * 2;
 #pragma unroll
     for (int c = 0; c < 8; c += 2)
         gather_pair2(g, cfg.level_off[l], corner_idx1(cfg, l, cl, c), corner_idx1(cfg, l, cl, c + 1), v[c], v[c + 1]);
@@ -165,16 +182,22 @@ __device__ __forceinline__ float2 blend_level2(const Cell& cl, const float2 (&v)
     return a;
 }
 
-// Features 4h .. 4h + 3 of a level of F = 4 or 8 features.
+// Features 4h .. 4h + 3 of a level of F = 4 or 8 features (blocks: F = 4).
 template <typename GT>
-__device__ __forceinline__ float4 blend_level4(const DevCfg& cfg, const GT* __restrict__ grid, int l, const Cell& cl,
-                                               int F, int h) {
-    const GT* g = grid + (size_t)cfg.level_off[l] * F;
-    uint32_t idx[8];
-    corner_idx8(cfg, l, cl, idx);
-    decltype(load_raw4(g, 0u, F, 0)) raw[8];
+__device__ __forceinline__ float4 blend_level4(const TcCfg& tc, const GridView<GT>& grid, int l, const Cell& cl, int F,
+                                               int h) {
+    const DevCfg& cfg = tc.base;
+    decltype(load_raw4(grid.table, 0u, F, 0)) raw[8];
+    if (grid.has(l)) {
+        const uint32_t D = (uint32_t)cfg.level_res[l];
+        gather_blocks4(grid.blk, tc.blk_off[l] + corner_idx1(cfg, l, cl, 0), D, D * D, grid.table, raw);
+    } else {
+        const GT* g = grid.table + (size_t)cfg.level_off[l] * F;
+        uint32_t idx[8];
+        corner_idx8(cfg, l, cl, idx);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) raw[c] = load_raw4(g, idx[c], F, h);
+        for (int c = 0; c < 8; ++c) raw[c] = load_raw4(g, idx[c], F, h);
+    }
     float w[8];
     corner_w8(cl, w);
     float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -211,7 +234,7 @@ struct RowPacker {
 // columns, padded with zeros to the layer's kp values. FEAT: features per
 // level (2 or 4), or 0 for any.
 template <int FEAT, int OPS>
-__device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTraits<OPS>::GridT* __restrict__ grid,
+__device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typename OpsTraits<OPS>::GridT>& grid,
                                            float x, float y, float z, const float (&ax)[7], uint32_t act) {
     const DevCfg& cfg = tc.base;
     constexpr int P = OpsTraits<OPS>::parts;
@@ -223,8 +246,8 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
         for (; l + 1 < L; l += 2) {
             const Cell c0 = make_cell(x, y, z, cfg.level_res[l]), c1 = make_cell(x, y, z, cfg.level_res[l + 1]);
             float2 v0[8], v1[8];
-            gather_level2(cfg, grid, l, c0, v0);
-            gather_level2(cfg, grid, l + 1, c1, v1);
+            gather_level2(tc, grid, l, c0, v0);
+            gather_level2(tc, grid, l + 1, c1, v1);
             const float2 a = blend_level2(c0, v0), b = blend_level2(c1, v1);
             uint32_t p[2][P];
             split_pair<OPS>(a.x, a.y, p[0]);
@@ -235,7 +258,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
         if (l < L) {
             const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
             float2 v0[8];
-            gather_level2(cfg, grid, l, c0, v0);
+            gather_level2(tc, grid, l, c0, v0);
             const float2 a = blend_level2(c0, v0);
             uint32_t p[1][P];
             split_pair<OPS>(a.x, a.y, p[0]);
@@ -247,7 +270,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
         for (int l = 0; l < L; ++l) {
             const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
             for (int h = 0; h < (F >> 2); ++h) {
-                const float4 a = blend_level4(cfg, grid, l, cl, F, h);
+                const float4 a = blend_level4(tc, grid, l, cl, F, h);
                 uint32_t p[2][P];
                 split_pair<OPS>(a.x, a.y, p[0]);
                 split_pair<OPS>(a.z, a.w, p[1]);
@@ -260,12 +283,12 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const typename OpsTr
             const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
             if (F == 2) {
                 float2 v[8];
-                gather_level2(cfg, grid, l, cl, v);
+                gather_level2(tc, grid, l, cl, v);
                 const float2 a = blend_level2(cl, v);
                 row.put(a.x);
                 row.put(a.y);
             } else {  // one, or another number that no vector load fits
-                const auto* g = grid + (size_t)cfg.level_off[l] * F;
+                const auto* g = grid.table + (size_t)cfg.level_off[l] * F;
                 uint32_t idx[8];
                 float w[8];
                 corners8(cfg, l, cl, idx, w);
@@ -562,8 +585,8 @@ __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, 
 // in shared memory.
 template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
 __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
-    k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ grid,
-                 const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
+    k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ table,
+                 const uint4* __restrict__ blk, const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
                  long long wait_limit) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int G = (int)(blockDim.x >> 7);
@@ -603,6 +626,7 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
     const uint32_t sW_addr = smem_u32(smem);
     const int L = tc.base.n_layers;
     const bool sample = qb.sample != 0;
+    const GridView<typename OpsTraits<OPS>::GridT> grid{table, blk, blk ? tc.blk_mask : 0u};
 
     int64_t ntiles = qb.total_tiles, n0 = qb.seg[0].n;
     if (qb.n_dev) {
@@ -768,7 +792,7 @@ inline int fwd_group_count(const TcCfg& c, int kmax) {
 }
 
 template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
-cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
+cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint4* blk, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
                        int* status, long long wait_limit, cudaStream_t st) {
     auto kern = k_forward_tc<KMAX, FEAT, OPS, WARPDEC>;
     const int G = fwd_group_count(c, KMAX);
@@ -791,21 +815,21 @@ cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint8_t* wblob, Q
     if (blocks > sms) blocks = sms;
     if (blocks < 1) blocks = 1;
     kern<<<(int)blocks, kThreads * G, smem, st>>>(
-        c, static_cast<const typename OpsTraits<OPS>::GridT*>(grid), wblob, qb, status, wait_limit);
+        c, static_cast<const typename OpsTraits<OPS>::GridT*>(grid), blk, wblob, qb, status, wait_limit);
     return cudaGetLastError();
 }
 
 // The instance of an operand format for this model: up to eight lobes with
 // 2, 4 or any features per level, or sixteen lobes.
 template <int OPS>
-cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
+cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint4* blk, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
                            int* status, long long wait_limit, bool warp_decode, cudaStream_t st) {
-    if (c.base.K > 8) return launch_fwd<16, 0, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+    if (c.base.K > 8) return launch_fwd<16, 0, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
     if constexpr (!OpsTraits<OPS>::fp32)
-        if (warp_decode) return launch_fwd<8, 0, OPS, true>(c, grid, wblob, qb, max_n, status, wait_limit, st);
-    if (c.base.feat == 2) return launch_fwd<8, 2, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
-    if (c.base.feat == 4) return launch_fwd<8, 4, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
-    return launch_fwd<8, 0, OPS>(c, grid, wblob, qb, max_n, status, wait_limit, st);
+        if (warp_decode) return launch_fwd<8, 0, OPS, true>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+    if (c.base.feat == 2) return launch_fwd<8, 2, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+    if (c.base.feat == 4) return launch_fwd<8, 4, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+    return launch_fwd<8, 0, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
 }
 
 }  // namespace tc

@@ -4,7 +4,7 @@
 
 namespace npm {
 namespace tc {
-template cudaError_t launch_fwd_ops<kTwoBf16>(const TcCfg&, const void*, const uint8_t*, QueryBatch&, int64_t, int*,
+template cudaError_t launch_fwd_ops<kTwoBf16>(const TcCfg&, const void*, const uint4*, const uint8_t*, QueryBatch&, int64_t, int*,
                                         long long, bool, cudaStream_t);
 }  // namespace tc
 }  // namespace npm

@@ -1,0 +1,61 @@
+"""Corner blocks of the dense levels (read by batches of 2^18 queries and
+more): the same bytes as the table, so a large batch gives exactly what the
+table gives its two halves, on every table format, with levels of the
+smallest resolutions and hashed levels between; and they follow the
+parameters through set_params, a training step, the weight average and a
+write through npm_params_device."""
+import numpy as np
+import pytest
+
+import synth
+from gpu_helpers import cuda, make_model
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+N = 1 << 18
+TWO = synth.Workload(name="6 levels x 2 feats", mode=synth.RADIANCE, level_res=[2, 3, 40, 10, 17, 25], feat=2,
+                     log2_table=14, widths=[12, 32, 16], K=4, n_train=4096)
+FOUR = synth.Workload(name="4 levels x 4 feats", mode=synth.RADIANCE, level_res=[30, 2, 9, 20], feat=4,
+                      log2_table=13, widths=[16, 32, 16], K=4, n_train=4096)
+
+
+def _same(m, pos, u):
+    d, p, _ = m.query_sample(pos, u, n=N)
+    for a, b in ((0, N // 2), (N // 2, N)):
+        dh, ph, _ = m.query_sample(pos[:, a:b].contiguous(), u[:, a:b].contiguous())
+        assert torch.equal(d[:, a:b], dh) and torch.equal(p[a:b], ph), (a, b)
+
+
+@pytest.mark.parametrize("precision", [synth.FP32, synth.FP32_TC, synth.BF16X3, synth.FP16],
+                         ids=["fp32", "fp32tc", "bf16x3", "fp16"])
+@pytest.mark.parametrize("w", [TWO, FOUR], ids=lambda w: w.name)
+def test_blocks_equal_the_table(w, precision):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    x = synth.positions(3, N)
+    x[:, :8] = np.array([[0, 1, 0.5, 1, 0, 0.9999999, 1e-7, 0.25]] * 3, dtype=np.float32)  # edges of the box
+    pos, u = cuda(x), cuda(synth.sample_uniforms(3, N))
+    m = make_model(w, synth.random_params(w, 51), N, precision=precision)
+    _same(m, pos, u)
+    m.set_params(synth.random_params(w, 52))
+    _same(m, pos, u)
+    b = synth.train_batch_uniform(w, w.n_train, seed=51)
+    m.train_step(cuda(b.pos), cuda(b.dir), cuda(b.radiance), cuda(b.pdf))
+    _same(m, pos, u)
+    m.set_ema(0.5)
+    m.train_step(cuda(b.pos), cuda(b.dir), cuda(b.radiance), cuda(b.pdf))
+    _same(m, pos, u)
+    m.set_ema(0.0)
+    # The FP32 tables are the parameters: a write through their address counts.
+    ptr = m._L.npm_params_device(m.handle)
+    ng = sum(synth.grid_sizes(w)) * w.feat
+
+    class Grid:
+        __cuda_array_interface__ = {"shape": (ng,), "typestr": "<f4", "data": (ptr, False), "version": 2}
+
+    torch.as_tensor(Grid(), device="cuda").mul_(0.5)
+    _same(m, pos, u)
+    m.check_device_status()
+    m.close()
