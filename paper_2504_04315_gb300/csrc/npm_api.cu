@@ -126,17 +126,26 @@ npm_status validate(const npm_config* c) {
     return NPM_OK;
 }
 
+// A device buffer whose first element lies `shift` elements into its
+// allocation (freed by dfree); a mirror of the parameters ends the next
+// multiple of 4 elements behind its last one.
 template <typename T>
-npm_status dalloc(T** p, size_t count, const char* what) {
+npm_status dalloc(T** p, size_t count, const char* what, size_t shift = 0) {
     *p = nullptr;
     if (count == 0) count = 1;
-    cudaError_t e = npm::device_alloc((void**)p, count * sizeof(T));
+    cudaError_t e = npm::device_alloc((void**)p, (shift ? (shift + count + 3) / 4 * 4 : count) * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
         return fail(NPM_ERR_OOM, std::string("cudaMalloc failed for ") + what);
     }
+    *p += shift;
     return NPM_OK;
+}
+
+template <typename T>
+void dfree(T* p, size_t shift) {
+    if (p) cudaFree(p - shift);
 }
 
 npm_status check_call(npm_handle* h, int64_t n, int64_t ld, const void* pos, const void* aux) {
@@ -149,6 +158,10 @@ npm_status check_call(npm_handle* h, int64_t n, int64_t ld, const void* pos, con
         return fail(NPM_ERR_INVALID_ARG, "product mode needs aux [7][ld]");
     return NPM_OK;
 }
+
+// Values that Adam runs over: the parameters from the 16-byte boundary before
+// them to the one behind.
+int64_t adam_count(const npm_handle* h) { return round_up(2 * (int64_t)h->dc.grid_shift + h->n_int, 4); }
 
 // Device-side count of completed Adam steps (scalars[16]).
 int* step_dev(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 16); }
@@ -268,14 +281,25 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
     const int of = d.fwd_floats, ob = d.bwd_floats;
     h->mlp_off = round_up(h->ng, 64);
     h->n_int = round_up(h->mlp_off + h->nmlp, 64);
+    // Tables of 2 features start so that the first hashed level (and with it,
+    // where they follow one another, every hashed level) starts on a 32-byte
+    // (FP32) or 16-byte (FP16) boundary: half of its x-neighbours then share
+    // a 16-byte FP32 load, three quarters a 16-byte FP16 one.
+    if (d.feat == 2)
+        for (int l = 0; l < d.n_levels; ++l)
+            if (!((d.dense_mask >> l) & 1u)) {
+                h->dc.grid_shift = (4u - (d.level_off[l] & 3u)) & 3u;
+                break;
+            }
+    const size_t sh = 2 * (size_t)d.grid_shift;  // in values
     h->fwd_smem = npm::fwd_smem_bytes(d);
     h->train_smem = npm::train_smem_bytes(d);
 
     size_t nb = (size_t)(cfg->max_batch > 0 ? cfg->max_batch : 1);
-    if ((s = dalloc(&h->params, h->n_int, "params")) != NPM_OK ||
-        (s = dalloc(&h->grads, h->n_int, "grads")) != NPM_OK ||
-        (s = dalloc(&h->adam_m, h->n_int, "adam m")) != NPM_OK ||
-        (s = dalloc(&h->adam_v, h->n_int, "adam v")) != NPM_OK ||
+    if ((s = dalloc(&h->params, h->n_int, "params", sh)) != NPM_OK ||
+        (s = dalloc(&h->grads, h->n_int, "grads", sh)) != NPM_OK ||
+        (s = dalloc(&h->adam_m, h->n_int, "adam m", sh)) != NPM_OK ||
+        (s = dalloc(&h->adam_v, h->n_int, "adam v", sh)) != NPM_OK ||
         (s = dalloc(&h->wfwd, (size_t)of, "forward weights")) != NPM_OK ||
         (s = dalloc(&h->wbwd, (size_t)ob, "backward weights")) != NPM_OK ||
         (s = dalloc(&h->scalars, 64, "scalars")) != NPM_OK ||
@@ -294,7 +318,7 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
             return fail(NPM_ERR_CUDA, "cannot create internal events");
         }
     if (cfg->precision != NPM_FP32) {
-        if ((s = dalloc(&h->grid_h, (size_t)h->ng, "grid fp16")) != NPM_OK) {
+        if ((s = dalloc(&h->grid_h, (size_t)h->ng, "grid fp16", sh)) != NPM_OK) {
             npm_destroy(h);
             return s;
         }
@@ -306,9 +330,9 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
         npm_destroy(h);
         return s;
     }
-    cudaMemset(h->grads, 0, h->n_int * sizeof(float));
-    cudaMemset(h->adam_m, 0, h->n_int * sizeof(float));
-    cudaMemset(h->adam_v, 0, h->n_int * sizeof(float));
+    // (whole allocations: Adam runs over the values before and behind too)
+    for (float* b : {h->params, h->grads, h->adam_m, h->adam_v})
+        cudaMemset(b - sh, 0, adam_count(h) * sizeof(float));
     cudaMemset(h->scalars, 0, 64 * sizeof(float));
     // Seeded initialisation: grid U[-1e-4, 1e-4], MLP Glorot-uniform.
     std::vector<float> init(h->n_int, 0.0f);
@@ -346,10 +370,12 @@ npm_status npm_destroy(npm_handle* h) {
     if (!h) return NPM_OK;
     cudaDeviceSynchronize();
     if (h->tc) npm::tc_destroy(h);
-    void* ptrs[] = {h->params, h->grads, h->adam_m, h->adam_v,   h->wfwd,  h->wbwd,
-                    h->scalars, h->stage, h->grid_h, h->ema, h->wfwd_inf};
+    void* ptrs[] = {h->wfwd, h->wbwd, h->scalars, h->stage, h->wfwd_inf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    const size_t sh = 2 * (size_t)h->dc.grid_shift;
+    for (float* p : {h->params, h->grads, h->adam_m, h->adam_v, h->ema}) dfree(p, sh);
+    dfree(h->grid_h, sh);
     for (int i = 0; i < 2; ++i)
         if (h->side[i]) cudaStreamDestroy(h->side[i]);
     for (int i = 0; i < 3; ++i)
@@ -434,7 +460,7 @@ npm_status npm_set_ema(npm_handle* h, float decay, void* stream) {
     if (decay == 0.0f) {
         if (h->ema) {
             NPM_CUDA(cudaStreamSynchronize(st), "synchronise");
-            cudaFree(h->ema);
+            dfree(h->ema, 2 * (size_t)h->dc.grid_shift);
             cudaFree(h->wfwd_inf);
             h->ema = h->wfwd_inf = nullptr;
         }
@@ -446,13 +472,15 @@ npm_status npm_set_ema(npm_handle* h, float decay, void* stream) {
     }
     if (!h->ema) {
         npm_status s;
-        if ((s = dalloc(&h->ema, h->n_int, "ema")) != NPM_OK) return s;
+        if ((s = dalloc(&h->ema, h->n_int, "ema", 2 * (size_t)h->dc.grid_shift)) != NPM_OK) return s;
         if ((s = dalloc(&h->wfwd_inf, (size_t)h->dc.fwd_floats, "ema forward weights")) != NPM_OK) {
-            cudaFree(h->ema);
+            dfree(h->ema, 2 * (size_t)h->dc.grid_shift);
             h->ema = nullptr;
             return s;
         }
-        NPM_CUDA(cudaMemcpyAsync(h->ema, h->params, h->n_int * sizeof(float), cudaMemcpyDeviceToDevice, st),
+        const size_t sh = 2 * (size_t)h->dc.grid_shift;
+        NPM_CUDA(cudaMemcpyAsync(h->ema - sh, h->params - sh, adam_count(h) * sizeof(float),
+                                 cudaMemcpyDeviceToDevice, st),
                  "start ema");
     }
     h->ema_decay = decay;
@@ -630,9 +658,11 @@ static npm_status backward_impl(npm_handle* h, int64_t n, const float* pos, cons
 static npm_status adam_impl(npm_handle* h, const float* loss, cudaStream_t st) {
     h->step += 1;
     int* status = reinterpret_cast<int*>(h->scalars + 8);
-    NPM_CUDA(npm::launch_adam(h->n_int, h->params, h->grads, h->adam_m, h->adam_v, h->cfg.lr,
-                              h->cfg.beta1, h->cfg.beta2, h->cfg.eps, step_dev(h), loss, status,
-                              h->grid_h, h->grid_h ? h->ng : 0, h->ema, h->ema_decay, st),
+    const int64_t sh = 2 * (int64_t)h->dc.grid_shift;
+    NPM_CUDA(npm::launch_adam(adam_count(h), h->params - sh, h->grads - sh, h->adam_m - sh, h->adam_v - sh,
+                              h->cfg.lr, h->cfg.beta1, h->cfg.beta2, h->cfg.eps, step_dev(h), loss, status,
+                              h->grid_h ? h->grid_h - sh : nullptr, h->grid_h ? sh + h->ng : 0,
+                              h->ema ? h->ema - sh : nullptr, h->ema_decay, st),
              "adam launch");
     return arrange_all_weights(h, st);
 }

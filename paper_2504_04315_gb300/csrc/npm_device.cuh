@@ -29,6 +29,10 @@ struct DevCfg {
     int widths[NPM_MAX_LAYERS + 1];
     int level_res[NPM_MAX_LEVELS];
     uint32_t level_off[NPM_MAX_LEVELS];  // first entry of each level
+    // Entries by which the tables (2 features; parameters, gradient, moments,
+    // average and FP16 copy alike) start past a 32-byte (FP32) or 16-byte
+    // (FP16) boundary, so that the hashed levels start on one.
+    uint32_t grid_shift;
     // FP32 fused kernels: per layer, padded output count (multiple of 16)
     // and float offsets of the pre-arranged weight blobs.
     int np_fwd[NPM_MAX_LAYERS];   // padded N of W^T [K][np] (forward)
@@ -150,8 +154,8 @@ __device__ __forceinline__ void corners8(const DevCfg& cfg, int l, const Cell& c
 }
 
 // Features of two x-adjacent corners (entries a, b of a 2-feature level
-// starting at entry level_off; gl points at the level): one 16-byte load
-// (FP32) or 8-byte load (FP16) when the two entries form an aligned pair,
+// whose first entry lies level_off entries past a 16-byte boundary; gl points
+// at the level): one 16-byte load when the two entries form an aligned pair,
 // else one load each. Random gathers cost the L1 a wavefront per lane and
 // load, so the paired lanes halve their share.
 __device__ __forceinline__ void gather_pair2(const float* gl, uint32_t level_off, uint32_t a, uint32_t b,
@@ -167,26 +171,9 @@ __device__ __forceinline__ void gather_pair2(const float* gl, uint32_t level_off
         vb = __ldg(reinterpret_cast<const float2*>(gl) + b);
     }
 }
-__device__ __forceinline__ void gather_pair2(const __half* gl, uint32_t level_off, uint32_t a, uint32_t b,
-                                             float2& va, float2& vb) {
-    const uint32_t lo = a < b ? a : b;
-    if ((a > b ? a - b : b - a) == 1u && ((level_off + lo) & 1u) == 0u) {
-        const uint2 raw = __ldg(reinterpret_cast<const uint2*>(gl + (size_t)lo * 2));
-        const float2 v0 = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-        const float2 v1 = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-        va = a < b ? v0 : v1;
-        vb = a < b ? v1 : v0;
-    } else {
-        const unsigned int ra = __ldg(reinterpret_cast<const unsigned int*>(gl) + a);
-        const unsigned int rb = __ldg(reinterpret_cast<const unsigned int*>(gl) + b);
-        va = __half22float2(*reinterpret_cast<const __half2*>(&ra));
-        vb = __half22float2(*reinterpret_cast<const __half2*>(&rb));
-    }
-}
-
 // Grid-gradient scatter of two x-adjacent corners (entries a, b of a level
-// starting at entry level_off, 2 features each; gl points at the level):
-// when the two entries form one 16-byte aligned pair, one 4-wide atomic add
+// whose first entry lies level_off entries past a 16-byte boundary, 2 features
+// each; gl points at the level): when the two entries form one 16-byte aligned pair, one 4-wide atomic add
 // serves both (the L2 atomic units are limited by operations, not bytes).
 __device__ __forceinline__ void scatter_pair2(float* gl, uint32_t level_off, uint32_t a, uint32_t b, float wa,
                                               float wb, float d0, float d1) {

@@ -193,7 +193,7 @@ __device__ __forceinline__ void gather_level(const DevCfg& cfg, const float* __r
     if (F == 2) {
         float2 v[8];
 #pragma unroll
-        for (int c = 0; c < 8; c += 2) gather_pair2(gl, cfg.level_off[l], idx[c], idx[c + 1], v[c], v[c + 1]);
+        for (int c = 0; c < 8; c += 2) gather_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], v[c], v[c + 1]);
         corner_w8(cl, w);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -258,7 +258,7 @@ __device__ __forceinline__ void encode_tile(int t, const DevCfg& cfg, const floa
                 const float* gr = grid + (size_t)cfg.level_off[l + 2 * r] * 2;
 #pragma unroll
                 for (int c = 0; c < 8; c += 2)
-                    gather_pair2(gr, cfg.level_off[l + 2 * r], idx[r][c], idx[r][c + 1], v[r][c], v[r][c + 1]);
+                    gather_pair2(gr, cfg.level_off[l + 2 * r] + cfg.grid_shift, idx[r][c], idx[r][c + 1], v[r][c], v[r][c + 1]);
             }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -708,9 +708,10 @@ __device__ __forceinline__ void weight_grad(const float* dl, const float* h, int
 #pragma unroll
             for (int r = 0; r < 8; ++r)
                 if (n0 + r < N) {
+                    // (8-byte aligned: the gradient shares the tables' shift)
                     float* dst = gW + (size_t)(n0 + r) * K + k0;
-                    atomicAdd(reinterpret_cast<float4*>(dst),
-                              make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]));
+                    atomicAdd(reinterpret_cast<float2*>(dst), make_float2(acc[r][0], acc[r][1]));
+                    atomicAdd(reinterpret_cast<float2*>(dst) + 1, make_float2(acc[r][2], acc[r][3]));
                 }
         }
 }
@@ -737,7 +738,7 @@ __device__ __forceinline__ void grid_scatter(const DevCfg& cfg, const float* den
         if (F == 2) {
 #pragma unroll
             for (int c = 0; c < 8; c += 2)
-                scatter_pair2(gl, cfg.level_off[l], idx[c], idx[c + 1], ws[c], ws[c + 1], dg[0], dg[1]);
+                scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1], dg[0], dg[1]);
             continue;
         }
 #pragma unroll

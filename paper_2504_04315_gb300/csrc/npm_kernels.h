@@ -89,8 +89,10 @@ cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* w
                                    cudaStream_t st);
 
 // Adam at step *steps + 1 (device counter, advanced on the stream after the
-// update). ema (or NULL): moving average updated with ema_decay; the FP16
-// copy is then taken from it.
+// update). The buffers are those of the parameters and what mirrors them from
+// the 16-byte boundary before their first value on (n a multiple of 4).
+// ema (or NULL): moving average updated with ema_decay; the FP16 copy is then
+// taken from it.
 cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float lr, float b1,
                         float b2, float eps, int* steps, const float* loss, int* status,
                         __half* half_copy, int64_t n_half, float* ema, float ema_decay,

@@ -119,9 +119,9 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
             float2 v0[8], v1[8];
 #pragma unroll
             for (int c = 0; c < 8; c += 2) {
-                gather_pair2(g0, cfg.level_off[l], corner_idx1(cfg, l, c0, c), corner_idx1(cfg, l, c0, c + 1),
+                gather_pair2(g0, cfg.level_off[l] + cfg.grid_shift, corner_idx1(cfg, l, c0, c), corner_idx1(cfg, l, c0, c + 1),
                              v0[c], v0[c + 1]);
-                gather_pair2(g1, cfg.level_off[l + 1], corner_idx1(cfg, l + 1, c1, c),
+                gather_pair2(g1, cfg.level_off[l + 1] + cfg.grid_shift, corner_idx1(cfg, l + 1, c1, c),
                              corner_idx1(cfg, l + 1, c1, c + 1), v1[c], v1[c + 1]);
             }
             float w0s[8], w1s[8];
@@ -462,7 +462,7 @@ __device__ __forceinline__ void scatter_levels(const DevCfg& cfg, float* __restr
                     atomicAdd(e, wc * dg[q]);
                 } else if constexpr (FF == 2) {
                     if (c & 1) continue;  // corners c, c + 1 (along x) together
-                    scatter_pair2(gl, cfg.level_off[l], idx[c], idx[c + 1], ws[c], ws[c + 1], dg[2 * q],
+                    scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1], dg[2 * q],
                                   dg[2 * q + 1]);
                 } else {
 #pragma unroll
@@ -497,34 +497,17 @@ __global__ void __launch_bounds__(256) k_train_encode(const __grid_constant__ De
         const int l0 = (int)(i - j * ng) * LPT;
         const float x = pos[j], y = pos[ld + j], z = pos[2 * ld + j];
         Cell cs[LPT];
-        float2 v[LPT][8];
+        Level2<float> v[LPT];
 #pragma unroll
-        for (int r = 0; r < LPT; ++r) {
-            const int l = l0 + r;
-            if (l < cfg.n_levels) {
-                cs[r] = make_cell(x, y, z, cfg.level_res[l]);
-                const float* gr = grid32 + (size_t)cfg.level_off[l] * 2;
-#pragma unroll
-                for (int c = 0; c < 8; c += 2)
-                    gather_pair2(gr, cfg.level_off[l], corner_idx1(cfg, l, cs[r], c), corner_idx1(cfg, l, cs[r], c + 1),
-                                 v[r][c], v[r][c + 1]);
+        for (int r = 0; r < LPT; ++r)
+            if (l0 + r < cfg.n_levels) {
+                cs[r] = make_cell(x, y, z, cfg.level_res[l0 + r]);
+                v[r].load_table(cfg, grid32, l0 + r, cs[r]);
             }
-        }
 #pragma unroll
-        for (int r = 0; r < LPT; ++r) {
-            const int l = l0 + r;
-            if (l < cfg.n_levels) {
-                float ws[8];
-                corner_w8(cs[r], ws);
-                float a0 = 0.0f, a1 = 0.0f;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    a0 = fmaf(ws[c], v[r][c].x, a0);
-                    a1 = fmaf(ws[c], v[r][c].y, a1);
-                }
-                *reinterpret_cast<float2*>(enc + j * G + 2 * l) = make_float2(a0, a1);
-            }
-        }
+        for (int r = 0; r < LPT; ++r)
+            if (l0 + r < cfg.n_levels)
+                *reinterpret_cast<float2*>(enc + j * G + 2 * (l0 + r)) = v[r].blend(cs[r]);
     }
 }
 
@@ -611,7 +594,7 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
                 corners8(cfg, l, cl, idx, ws);
 #pragma unroll
                 for (int c = 0; c < 8; c += 2)
-                    scatter_pair2(gl, cfg.level_off[l], idx[c], idx[c + 1], ws[c], ws[c + 1], pdg[0], pdg[1]);
+                    scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1], pdg[0], pdg[1]);
             }
 #pragma unroll
             for (int i = 0; i < 14; ++i) pdg[i] = pdg[i + 2];

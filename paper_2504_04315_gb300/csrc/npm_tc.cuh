@@ -162,6 +162,11 @@ __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[2]) 
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(r[0]), "r"(r[1])
                  : "memory");
 }
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[3]) {
+    const uint32_t a[2] = {r[0], r[1]}, b[1] = {r[2]};
+    tmem_st(taddr, a);
+    tmem_st(taddr + 2u, b);
+}
 __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[4]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
                  "r"(r[2]), "r"(r[3])
@@ -333,11 +338,7 @@ __device__ __forceinline__ void vmf_sample_rp(const Lobe& L, float u1, float u2,
 
 // ------------------------------------------------------------ grid gathers
 
-// Table entry loads: FP16 copy (inference) or FP32 master (training).
-__device__ __forceinline__ float2 load_feat2(const __half* g, uint32_t idx) {
-    const uint32_t raw = __ldg(reinterpret_cast<const unsigned int*>(g) + idx);
-    return __half22float2(*reinterpret_cast<const __half2*>(&raw));
-}
+// Table entry loads of the FP32 table.
 __device__ __forceinline__ float2 load_feat2(const float* g, uint32_t idx) {
     return __ldg(reinterpret_cast<const float2*>(g) + idx);
 }
@@ -378,21 +379,117 @@ __device__ __forceinline__ Block32 load_block(const uint4* __restrict__ blk, uin
     return b;
 }
 
-// The 8 corners (2 features each) of a cell with lowest block e; DD = D^2.
-__device__ __forceinline__ void gather_blocks2(const uint4* __restrict__ blk, uint32_t e, uint32_t, const __half*,
-                                               float2 (&v)[8]) {
-    const Block32 b = load_block(blk, e);
+// Corner features of one level of 2 features as loaded: nothing here waits
+// for the loads, so that several levels' are in flight before the first is
+// blended (a select on a loaded value, or a branch around one, would wait).
+//
+// From the table: a pair of x-neighbours in one load of twice the width where
+// they form an aligned pair (half of a level's; it may come swapped), else in
+// two.
+template <typename GT>
+struct Level2;
+
+__device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const Cell& cl, int c);
+
+template <>
+struct Level2<float> {
+    float r[16];
+    uint32_t swap;  // bit i: pair i swapped
+    __device__ __forceinline__ void load_blocks(const uint4* __restrict__ blk, uint32_t e, uint32_t DD) {
+        const Block32 b[2] = {load_block(blk, e), load_block(blk, e + DD)};
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = __half22float2(*reinterpret_cast<const __half2*>(&b.r[c]));
-}
-__device__ __forceinline__ void gather_blocks2(const uint4* __restrict__ blk, uint32_t e, uint32_t DD, const float*,
-                                               float2 (&v)[8]) {
-    const Block32 b[2] = {load_block(blk, e), load_block(blk, e + DD)};
+        for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(b[i >> 3].r[i & 7]);
+        swap = 0u;
+    }
+    __device__ __forceinline__ void load_table(const DevCfg& cfg, const float* __restrict__ table, int l,
+                                               const Cell& cl) {
+        const uint32_t off = cfg.level_off[l];
+        const float* g = table + (size_t)off * 2;
+        const uint32_t odd = (off + cfg.grid_shift) & 1u;
+        swap = 0u;
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-        v[c] = make_float2(__uint_as_float(b[c >> 2].r[2 * (c & 3)]), __uint_as_float(b[c >> 2].r[2 * (c & 3) + 1]));
-}
-// The same for 4 features.
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t a = corner_idx1(cfg, l, cl, 2 * i), b = corner_idx1(cfg, l, cl, 2 * i + 1);
+            const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
+            const uint32_t pair = (hi - lo == 1u && (lo & 1u) == odd) ? 1u : 0u;
+            swap |= (pair && a > b ? 1u : 0u) << i;
+            asm("{\n\t.reg .pred p;\n\t"
+                "setp.ne.u32 p, %6, 0;\n\t"
+                "@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t"
+                "@!p ld.global.nc.v2.f32 {%0, %1}, [%4];\n\t"
+                "@!p ld.global.nc.v2.f32 {%2, %3}, [%5];\n\t}\n"
+                : "=f"(r[4 * i]), "=f"(r[4 * i + 1]), "=f"(r[4 * i + 2]), "=f"(r[4 * i + 3])
+                : "l"(g + 2 * (size_t)(pair ? lo : a)), "l"(g + 2 * (size_t)b), "r"(pair));
+        }
+    }
+    __device__ __forceinline__ float2 blend(const Cell& cl) const {
+        float w[8];
+        corner_w8(cl, w);
+        float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool sw = (swap >> i) & 1u;
+            const float wa = sw ? w[2 * i + 1] : w[2 * i], wb = sw ? w[2 * i] : w[2 * i + 1];
+            s.x = fmaf(wa, r[4 * i], s.x);
+            s.y = fmaf(wa, r[4 * i + 1], s.y);
+            s.x = fmaf(wb, r[4 * i + 2], s.x);
+            s.y = fmaf(wb, r[4 * i + 3], s.y);
+        }
+        return s;
+    }
+};
+
+template <>
+struct Level2<__half> {
+    uint32_t r[8];  // corners; from the table pair i may come swapped
+    uint32_t swap;
+    __device__ __forceinline__ void load_blocks(const uint4* __restrict__ blk, uint32_t e, uint32_t) {
+        const Block32 b = load_block(blk, e);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = b.r[i];
+        swap = 0u;
+    }
+    __device__ __forceinline__ void load_table(const DevCfg& cfg, const __half* __restrict__ table, int l,
+                                               const Cell& cl) {
+        const uint32_t off = cfg.level_off[l];
+        const uint32_t* g = reinterpret_cast<const uint32_t*>(table) + off;
+        const uint32_t odd = (off + cfg.grid_shift) & 1u;
+        swap = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t a = corner_idx1(cfg, l, cl, 2 * i), b = corner_idx1(cfg, l, cl, 2 * i + 1);
+            const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
+            const uint32_t pair = (hi - lo == 1u && (lo & 1u) == odd) ? 1u : 0u;
+            swap |= (pair && a > b ? 1u : 0u) << i;
+            asm("{\n\t.reg .pred p;\n\t"
+                "setp.ne.u32 p, %4, 0;\n\t"
+                "@p ld.global.nc.v2.b32 {%0, %1}, [%2];\n\t"
+                "@!p ld.global.nc.b32 %0, [%2];\n\t"
+                "@!p ld.global.nc.b32 %1, [%3];\n\t}\n"
+                : "=r"(r[2 * i]), "=r"(r[2 * i + 1])
+                : "l"(g + (pair ? lo : a)), "l"(g + b), "r"(pair));
+        }
+    }
+    __device__ __forceinline__ float2 blend(const Cell& cl) const {
+        float w[8];
+        corner_w8(cl, w);
+        float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool sw = (swap >> i) & 1u;
+            const float wa = sw ? w[2 * i + 1] : w[2 * i], wb = sw ? w[2 * i] : w[2 * i + 1];
+            const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&r[2 * i]));
+            const float2 fb = __half22float2(*reinterpret_cast<const __half2*>(&r[2 * i + 1]));
+            s.x = fmaf(wa, fa.x, s.x);
+            s.y = fmaf(wa, fa.y, s.y);
+            s.x = fmaf(wb, fb.x, s.x);
+            s.y = fmaf(wb, fb.y, s.y);
+        }
+        return s;
+    }
+};
+
+// Corner features of 4 features of a cell with lowest block e; DD = D^2.
 __device__ __forceinline__ void gather_blocks4(const uint4* __restrict__ blk, uint32_t e, uint32_t, uint32_t DD,
                                                const __half*, uint2 (&v)[8]) {
     const Block32 b[2] = {load_block(blk, e), load_block(blk, e + DD)};

@@ -68,8 +68,12 @@ struct OpsTraits {
 };
 
 // Tile groups a CTA is compiled for: four at 128 registers; two for up to
-// sixteen lobes, whose raw outputs alone take 64.
-__host__ __device__ constexpr int fwd_groups(int kmax) { return kmax > 8 ? 2 : 4; }
+// sixteen lobes, whose raw outputs alone take 64; three at 168 for FP32 on
+// 2-feature grids (three is what the columns of 64-wide layers allow there,
+// and two levels' FP32 gathers in flight take the registers).
+__host__ __device__ constexpr int fwd_groups(int kmax, int feat, int ops) {
+    return kmax > 8 ? 2 : (ops == kThreeBf16 && feat == 2) ? 3 : 4;
+}
 
 // ----------------------------------------------------------- operands
 
@@ -153,33 +157,17 @@ struct GridView {
     __device__ __forceinline__ bool has(int l) const { return (mask >> l) & 1u; }
 };
 
-// Corner features of level l. Two levels are gathered before either is
-// blended, so that up to 16 loads are in flight.
+// Corner features of level l (2 features).
 template <typename GT>
 __device__ __forceinline__ void gather_level2(const TcCfg& tc, const GridView<GT>& grid, int l, const Cell& cl,
-                                              float2 (&v)[8]) {
+                                              Level2<GT>& v) {
     const DevCfg& cfg = tc.base;
     if (grid.has(l)) {
         const uint32_t D = (uint32_t)cfg.level_res[l];
-        gather_blocks2(grid.blk, tc.blk_off[l] + corner_idx1(cfg, l, cl, 0), D * D, grid.table, v);
-        return;
+        v.load_blocks(grid.blk, tc.blk_off[l] + corner_idx1(cfg, l, cl, 0), D * D);
+    } else {
+        v.load_table(cfg, grid.table, l, cl);
     }
-    const GT* g = grid.table + (size_t)cfg.level_off[l] * 2;
-#pragma unroll
-    for (int c = 0; c < 8; c += 2)
-        gather_pair2(g, cfg.level_off[l], corner_idx1(cfg, l, cl, c), corner_idx1(cfg, l, cl, c + 1), v[c], v[c + 1]);
-}
-
-__device__ __forceinline__ float2 blend_level2(const Cell& cl, const float2 (&v)[8]) {
-    float w[8];
-    corner_w8(cl, w);
-    float2 a = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        a.x = fmaf(w[c], v[c].x, a.x);
-        a.y = fmaf(w[c], v[c].y, a.y);
-    }
-    return a;
 }
 
 // Features 4h .. 4h + 3 of a level of F = 4 or 8 features (blocks: F = 4).
@@ -230,39 +218,63 @@ struct RowPacker {
     }
 };
 
-// The network input of query (x, y, z): this thread's row of the activation
+// Product-mode inputs of query j (Sec. 4.3): SH of the outgoing direction and
+// of the normal, roughness.
+__device__ __forceinline__ void product_inputs(const QuerySeg& S, uint32_t j, bool valid, float (&e)[22]) {
+    float ax[7] = {0.0f, 0.0f, 1.0f, 0.0f, 0.0f, 1.0f, 0.0f};
+    if (valid)
+#pragma unroll
+        for (int i = 0; i < 7; ++i) ax[i] = S.aux[i * S.ld + j];
+    __syncwarp();
+    sh_band4(ax[0], ax[1], ax[2], e);
+    sh_band2(ax[3], ax[4], ax[5], e + 16);
+    e[20] = ax[6];
+    e[21] = 0.0f;
+}
+
+// The network input of query j at (x, y, z): this thread's row of the activation
 // columns, padded with zeros to the layer's kp values. FEAT: features per
 // level (2 or 4), or 0 for any.
 template <int FEAT, int OPS>
 __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typename OpsTraits<OPS>::GridT>& grid,
-                                           float x, float y, float z, const float (&ax)[7], uint32_t act) {
+                                           float x, float y, float z, const QuerySeg& S, uint32_t j, bool valid,
+                                           uint32_t act) {
     const DevCfg& cfg = tc.base;
     constexpr int P = OpsTraits<OPS>::parts;
     const uint32_t pc = tc.a_cols;
     __syncwarp();
     const int L = cfg.n_levels, F = FEAT ? FEAT : cfg.feat;
     if constexpr (FEAT == 2) {
+        // NF levels' gathers in flight before the first is blended: what the
+        // registers hold without spilling (2^20 queries of the paper-shaped
+        // grid, FP16 with 2, 3, 4: 302, 290, 327 us, four spilling 116 bytes;
+        // FP32 accuracy with 1, 2: 377, 407 us, two spilling 120 bytes; FP32
+        // with 2, 3: 461, 469 us).
+        constexpr int NF = OPS == kTwoFp16 ? 1 : OPS == kThreeBf16 ? 2 : 3;
         int l = 0;
-        for (; l + 1 < L; l += 2) {
-            const Cell c0 = make_cell(x, y, z, cfg.level_res[l]), c1 = make_cell(x, y, z, cfg.level_res[l + 1]);
-            float2 v0[8], v1[8];
-            gather_level2(tc, grid, l, c0, v0);
-            gather_level2(tc, grid, l + 1, c1, v1);
-            const float2 a = blend_level2(c0, v0), b = blend_level2(c1, v1);
-            uint32_t p[2][P];
-            split_pair<OPS>(a.x, a.y, p[0]);
-            split_pair<OPS>(b.x, b.y, p[1]);
-            __syncwarp();
-            put_pairs<OPS, 2>(act, pc, (uint32_t)l, p);
+        for (; l + NF <= L; l += NF) {
+            Cell cl[NF];
+            Level2<typename OpsTraits<OPS>::GridT> v[NF];
+#pragma unroll
+            for (int i = 0; i < NF; ++i) {
+                cl[i] = make_cell(x, y, z, cfg.level_res[l + i]);
+                gather_level2(tc, grid, l + i, cl[i], v[i]);
+            }
+            uint32_t p[NF][P];
+#pragma unroll
+            for (int i = 0; i < NF; ++i) {
+                const float2 a = v[i].blend(cl[i]);
+                split_pair<OPS>(a.x, a.y, p[i]);
+            }
+            put_pairs<OPS, NF>(act, pc, (uint32_t)l, p);
         }
-        if (l < L) {
-            const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
-            float2 v0[8];
-            gather_level2(tc, grid, l, c0, v0);
-            const float2 a = blend_level2(c0, v0);
+        for (; l < L; ++l) {
+            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            Level2<typename OpsTraits<OPS>::GridT> v;
+            gather_level2(tc, grid, l, cl, v);
+            const float2 a = v.blend(cl);
             uint32_t p[1][P];
             split_pair<OPS>(a.x, a.y, p[0]);
-            __syncwarp();
             put_pairs<OPS, 1>(act, pc, (uint32_t)l, p);
         }
     } else if (FEAT == 4 || F == 4 || F == 8) {
@@ -282,9 +294,9 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
         for (int l = 0; l < L; ++l) {
             const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
             if (F == 2) {
-                float2 v[8];
+                Level2<typename OpsTraits<OPS>::GridT> v;
                 gather_level2(tc, grid, l, cl, v);
-                const float2 a = blend_level2(cl, v);
+                const float2 a = v.blend(cl);
                 row.put(a.x);
                 row.put(a.y);
             } else {  // one, or another number that no vector load fits
@@ -302,10 +314,8 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
         }
         if (cfg.mode != NPM_PRODUCT && (row.k & 1)) row.put(0.0f);
         if (cfg.mode == NPM_PRODUCT) {
-            float e[21];
-            sh_band4(ax[0], ax[1], ax[2], e);
-            sh_band2(ax[3], ax[4], ax[5], e + 16);
-            e[20] = ax[6];
+            float e[22];
+            product_inputs(S, j, valid, e);
 #pragma unroll
             for (int i = 0; i < 21; ++i) row.put(e[i]);
             if (row.k & 1) row.put(0.0f);
@@ -316,10 +326,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
         if (FEAT != 0 || F == 4 || F == 8) {
             // An even number of grid features: 21 values and one zero.
             float e[22];
-            sh_band4(ax[0], ax[1], ax[2], e);
-            sh_band2(ax[3], ax[4], ax[5], e + 16);
-            e[20] = ax[6];
-            e[21] = 0.0f;
+            product_inputs(S, j, valid, e);
 #pragma unroll
             for (int i = 0; i < 22; i += 2) {
                 uint32_t p[1][P];
@@ -342,19 +349,10 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
 // outputs. Only the chosen lobe is decoded for the sample; the density then
 // decodes lobe by lobe, so that no array of decoded lobes stays live (nine
 // lobe decodes instead of eight, half the registers).
-struct QueryIo {
-    int64_t j, ld;
-    bool valid;
-    float u[4];  // uniforms when sampling, direction when evaluating
-    float ufrac;
-    float* dir;
-    float* pdf;
-    float* mix;
-};
-
+// u: uniforms when sampling, direction when evaluating.
 template <int KMAX, bool FP32>
-__device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&rawu)[KMAX / 4][16], const QueryIo& q,
-                                           bool sample, bool log_pdf) {
+__device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&rawu)[KMAX / 4][16], const QuerySeg& S,
+                                           uint32_t j, bool valid, const float (&u)[4], bool sample, bool log_pdf) {
     const int K = cfg.K;
     auto raw = [&](int i) { return __uint_as_float(rawu[i >> 4][i & 15]); };
     float mx = -INFINITY;
@@ -372,7 +370,7 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
 #pragma unroll
     for (int i = 0; i < KMAX; ++i)
         if (i < K) lam[i] *= inv;
-    float w[3] = {q.u[0], q.u[1], q.u[2]};
+    float w[3] = {u[0], u[1], u[2]};
     if (sample) {
         // Smallest lobe i with u0 < lambda_0 + ... + lambda_i (last if none).
         float cum = 0.0f, rk = raw(1), rt = raw(2), rp = raw(3);
@@ -386,15 +384,15 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
                     rt = raw(4 * i + 2);
                     rp = raw(4 * i + 3);
                 }
-                found = found || q.u[0] < cum;
+                found = found || u[0] < cum;
             }
-        if (q.ufrac > 0.0f && q.u[3] < q.ufrac) {
-            uniform_sphere(q.u[1], q.u[2], w);
+        if (S.ufrac > 0.0f && u[3] < S.ufrac) {
+            uniform_sphere(u[1], u[2], w);
         } else {
             Lobe sl;
             decode_lobe_fast(cfg.kappa_act, rk, rt, rp, sl, nullptr, nullptr);
-            if (FP32) vmf_sample(sl, q.u[1], q.u[2], w);
-            else vmf_sample_rp(sl, q.u[1], q.u[2], w);
+            if (FP32) vmf_sample(sl, u[1], u[2], w);
+            else vmf_sample_rp(sl, u[1], u[2], w);
         }
     }
     float pv = 0.0f;
@@ -424,24 +422,24 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
                 Lobe lb;
                 float th, ph;
                 decode_lobe_fast(cfg.kappa_act, raw(4 * i + 1), raw(4 * i + 2), raw(4 * i + 3), lb, &th, &ph);
-                if (q.mix && q.valid) {
-                    float* mo = q.mix + (int64_t)(4 * i) * q.ld + q.j;
+                if (S.mix && valid) {
+                    float* mo = S.mix + (int64_t)(4 * i) * S.ld + j;
                     mo[0] = lam[i];
-                    mo[q.ld] = lb.kap;
-                    mo[2 * q.ld] = th;
-                    mo[3 * q.ld] = ph;
+                    mo[S.ld] = lb.kap;
+                    mo[2 * S.ld] = th;
+                    mo[3 * S.ld] = ph;
                 }
                 pv += lam[i] * vmf_eval_fast(lb, vmf_scaled_norm_fast(lb.kap), w[0], w[1], w[2]);
             }
-        if (sample && q.ufrac > 0.0f) pv = q.ufrac * kInv4Pi + (1.0f - q.ufrac) * pv;
+        if (sample && S.ufrac > 0.0f) pv = S.ufrac * kInv4Pi + (1.0f - S.ufrac) * pv;
     }
-    if (q.valid) {
+    if (valid) {
         if (sample) {
-            q.dir[q.j] = w[0];
-            q.dir[q.ld + q.j] = w[1];
-            q.dir[2 * q.ld + q.j] = w[2];
+            S.dir[j] = w[0];
+            S.dir[S.ld + j] = w[1];
+            S.dir[2 * S.ld + j] = w[2];
         }
-        q.pdf[q.j] = pv;
+        S.pdf[j] = pv;
     }
 }
 
@@ -584,7 +582,7 @@ __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, 
 // WARPDEC: the warp-per-query decode (tc_decode_warp) from raw outputs staged
 // in shared memory.
 template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
-__global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
+__global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
     k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ table,
                  const uint4* __restrict__ blk, const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
                  long long wait_limit) {
@@ -628,63 +626,53 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
     const bool sample = qb.sample != 0;
     const GridView<typename OpsTraits<OPS>::GridT> grid{table, blk, blk ? tc.blk_mask : 0u};
 
-    int64_t ntiles = qb.total_tiles, n0 = qb.seg[0].n;
+    // Tiles and queries of a segment in 32 bits: batches hold at most 2^31
+    // queries.
+    uint32_t ntiles = (uint32_t)qb.total_tiles, n0 = (uint32_t)qb.seg[0].n;
     if (qb.n_dev) {
-        n0 = *qb.n_dev;
-        ntiles = (n0 + kTile - 1) / kTile;
+        n0 = (uint32_t)*qb.n_dev;
+        ntiles = (n0 + (kTile - 1)) / kTile;
     }
     bool ok = true, issued = false;
     uint32_t phase = 0;
     // Tiles are dealt to the CTAs first and to a CTA's groups second, so a
     // batch of fewer tiles than groups spreads over as many SMs as it can.
-    const int64_t stride = (int64_t)gridDim.x * G;
-    for (int64_t tile = blockIdx.x + (int64_t)g * gridDim.x; tile < ntiles; tile += stride) {
+    const uint32_t stride = gridDim.x * (uint32_t)G;
+    for (uint32_t tile = blockIdx.x + (uint32_t)g * gridDim.x; tile < ntiles; tile += stride) {
         int sg = 0;
-        while (sg + 1 < qb.nseg && tile >= qb.seg[sg + 1].tile0) ++sg;
+        while (sg + 1 < qb.nseg && tile >= (uint32_t)qb.seg[sg + 1].tile0) ++sg;
         const QuerySeg& S = qb.seg[sg];
-        const int64_t n = (sg == 0 && qb.n_dev) ? n0 : S.n;
-        const int64_t ld = S.ld;
-        QueryIo q;
-        q.j = (tile - S.tile0) * kTile + t;
-        q.ld = ld;
-        q.valid = q.j < n;
-        q.ufrac = S.ufrac;
-        q.dir = S.dir;
-        q.pdf = S.pdf;
-        q.mix = S.mix;
+        const uint32_t n = (sg == 0 && qb.n_dev) ? n0 : (uint32_t)S.n;
+        const uint32_t base = (tile - (uint32_t)S.tile0) * kTile, j = base + t;
+        const bool valid = j < n;
         float x = 0.0f, y = 0.0f, z = 0.0f;
-        float ax[7] = {0.0f, 0.0f, 1.0f, 0.0f, 0.0f, 1.0f, 0.0f};
-        if (q.valid) {
-            x = S.pos[q.j];
-            y = S.pos[ld + q.j];
-            z = S.pos[2 * ld + q.j];
-            if (tc.base.mode == NPM_PRODUCT)
-#pragma unroll
-                for (int i = 0; i < 7; ++i) ax[i] = S.aux[i * ld + q.j];
+        if (valid) {
+            x = S.pos[j];
+            y = S.pos[S.ld + j];
+            z = S.pos[2 * S.ld + j];
         }
         if (warp == 3) {
             // The group's next tile's positions into L2 (three 512-byte rows).
             const int lane = t & 31, r = lane >> 2;
-            const int64_t nt = tile + stride;
+            const uint32_t nt = tile + stride;
             if (r < 3 && nt < ntiles) {
                 int s2 = sg;
-                while (s2 + 1 < qb.nseg && nt >= qb.seg[s2 + 1].tile0) ++s2;
+                while (s2 + 1 < qb.nseg && nt >= (uint32_t)qb.seg[s2 + 1].tile0) ++s2;
                 const QuerySeg& S2 = qb.seg[s2];
-                const int64_t b2 = (nt - S2.tile0) * kTile + 32 * (lane & 3);
-                const int64_t n2 = (s2 == 0 && qb.n_dev) ? n0 : S2.n;
+                const uint32_t b2 = (nt - (uint32_t)S2.tile0) * kTile + 32 * (lane & 3);
+                const uint32_t n2 = (s2 == 0 && qb.n_dev) ? n0 : (uint32_t)S2.n;
                 if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + r * S2.ld + b2));
             }
         }
-        encode_row<FEAT, OPS>(tc, grid, x, y, z, ax, act + lanes);
+        encode_row<FEAT, OPS>(tc, grid, x, y, z, S, j, valid, act + lanes);
         // The uniforms (or the direction), loaded now so that their latency
         // passes during the layers.
-        q.u[0] = q.u[1] = q.u[3] = 0.0f;
-        q.u[2] = sample ? 0.0f : 1.0f;
-        if (q.valid) {
-            q.u[0] = S.uin[q.j];
-            q.u[1] = S.uin[ld + q.j];
-            q.u[2] = S.uin[2 * ld + q.j];
-            if (q.ufrac > 0.0f) q.u[3] = S.uin[3 * ld + q.j];
+        float u[4] = {0.0f, 0.0f, sample ? 0.0f : 1.0f, 0.0f};
+        if (valid) {
+            u[0] = S.uin[j];
+            u[1] = S.uin[S.ld + j];
+            u[2] = S.uin[2 * S.ld + j];
+            if (S.ufrac > 0.0f) u[3] = S.uin[3 * S.ld + j];
         }
         __syncwarp();
         tmem_wait_st();
@@ -757,10 +745,11 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
                         *reinterpret_cast<uint4*>(sRaw + t * RS + 16 * c + 4 * i) =
                             make_uint4(raw[c][4 * i], raw[c][4 * i + 1], raw[c][4 * i + 2], raw[c][4 * i + 3]);
             tc_group_sync(g);
-            tc_decode_warp<KMAX>(tc, sRaw, warp, t & 31, (tile - S.tile0) * kTile, n, ld, S.uin, S.ufrac, sample, S.dir,
-                                 S.pdf, S.mix, qb.log_pdf != 0);
+            tc_decode_warp<KMAX>(tc, sRaw, warp, t & 31, base, n, S.ld, S.uin, S.ufrac, sample, S.dir, S.pdf, S.mix,
+                                 qb.log_pdf != 0);
         } else {
-            if (ok) decode_row<KMAX, OpsTraits<OPS>::fp32>(tc.base, raw, q, sample, qb.log_pdf != 0);
+            if (ok)
+                decode_row<KMAX, OpsTraits<OPS>::fp32>(tc.base, raw, S, j, valid, u, sample, qb.log_pdf != 0);
         }
     }
     if (!ok && (t & 31) == 0) atomicOr(status, kStatusTimeout);
@@ -781,8 +770,8 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX), 1)
 
 // Tile groups of a CTA: as many as the instance is compiled for and the
 // 512 tensor-memory columns hold.
-inline int fwd_group_count(const TcCfg& c, int kmax) {
-    int G = fwd_groups(kmax);
+inline int fwd_group_count(const TcCfg& c, int most) {
+    int G = most;
     for (; G > 1; --G) {
         uint32_t cols = 32;
         while (cols < (uint32_t)G * c.g_cols) cols <<= 1;
@@ -795,7 +784,7 @@ template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
 cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint4* blk, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
                        int* status, long long wait_limit, cudaStream_t st) {
     auto kern = k_forward_tc<KMAX, FEAT, OPS, WARPDEC>;
-    const int G = fwd_group_count(c, KMAX);
+    const int G = fwd_group_count(c, fwd_groups(KMAX, FEAT, OPS));
     const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * c.w_bytes;
     size_t smem = fwd_stage_off(wbytes, G);
     if (WARPDEC) smem += (size_t)G * kTile * (4 * KMAX + 4) * sizeof(float);
