@@ -167,16 +167,16 @@ int64_t adam_count(const npm_handle* h) { return round_up(2 * (int64_t)h->dc.gri
 int* step_dev(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 16); }
 
 // The weights as the kernels read them: the tensor-core operands, and the
-// CUDA-core kernels' padded copies where those serve training or inference
+// CUDA-core kernels' padded copy where those serve training or inference
 // (of the moving average too, when inference evaluates it).
 npm_status arrange_all_weights(npm_handle* h, cudaStream_t st) {
     if (h->tc) {
         NPM_CUDA(npm::tc_refresh_weights(h, !npm::tc_can_train(h), st), "arrange weights");
         return NPM_OK;
     }
-    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, h->wbwd, st), "arrange weights");
+    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, st), "arrange weights");
     if (h->ema)
-        NPM_CUDA(npm::launch_arrange_weights(h->dc, h->ema + h->mlp_off, h->wfwd_inf, nullptr, st),
+        NPM_CUDA(npm::launch_arrange_weights(h->dc, h->ema + h->mlp_off, h->wfwd_inf, st),
                  "arrange ema weights");
     return NPM_OK;
 }
@@ -222,7 +222,7 @@ npm_status make_devcfg(const npm_config* cfg, DevCfg* out, int64_t* ng, int64_t*
             return fail(NPM_ERR_INVALID_ARG, "grid larger than 2^32 values");
     }
     *ng = (int64_t)off * cfg->feat_per_level;
-    int maxw = 0, of = 0, ob = 0;
+    int maxw = 0, of = 0;
     *nmlp = 0;
     for (int l = 0; l <= cfg->n_layers; ++l) {
         d.widths[l] = cfg->widths[l];
@@ -231,15 +231,11 @@ npm_status make_devcfg(const npm_config* cfg, DevCfg* out, int64_t* ng, int64_t*
     for (int l = 0; l < cfg->n_layers; ++l) {
         const int K = cfg->widths[l], N = cfg->widths[l + 1];
         d.np_fwd[l] = pad_np(N);
-        d.np_bwd[l] = pad_np(K);
         d.off_fwd[l] = of;
-        d.off_bwd[l] = ob;
         of += K * d.np_fwd[l];
-        ob += N * d.np_bwd[l];
         *nmlp += (int64_t)K * N;
     }
     d.fwd_floats = of;
-    d.bwd_floats = ob;
     d.max_width = maxw;
     if (fwd_smem_bytes(d) > 227 * 1024)
         return fail(NPM_ERR_UNSUPPORTED, "MLP weights do not fit in shared memory");
@@ -278,7 +274,7 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
         return s;
     }
     const npm::DevCfg& d = h->dc;
-    const int of = d.fwd_floats, ob = d.bwd_floats;
+    const int of = d.fwd_floats;
     h->mlp_off = round_up(h->ng, 64);
     h->n_int = round_up(h->mlp_off + h->nmlp, 64);
     // Tables of 2 features start so that the first hashed level (and with it,
@@ -301,7 +297,6 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
         (s = dalloc(&h->adam_m, h->n_int, "adam m", sh)) != NPM_OK ||
         (s = dalloc(&h->adam_v, h->n_int, "adam v", sh)) != NPM_OK ||
         (s = dalloc(&h->wfwd, (size_t)of, "forward weights")) != NPM_OK ||
-        (s = dalloc(&h->wbwd, (size_t)ob, "backward weights")) != NPM_OK ||
         (s = dalloc(&h->scalars, 64, "scalars")) != NPM_OK ||
         (s = dalloc(&h->stage, nb * (3 + 7 + 4 + 3 + 1), "host staging")) != NPM_OK) {
         npm_destroy(h);
@@ -370,7 +365,7 @@ npm_status npm_destroy(npm_handle* h) {
     if (!h) return NPM_OK;
     cudaDeviceSynchronize();
     if (h->tc) npm::tc_destroy(h);
-    void* ptrs[] = {h->wfwd, h->wbwd, h->scalars, h->stage, h->wfwd_inf};
+    void* ptrs[] = {h->wfwd, h->scalars, h->stage, h->wfwd_inf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     const size_t sh = 2 * (size_t)h->dc.grid_shift;
@@ -642,20 +637,20 @@ static npm_status backward_impl(npm_handle* h, int64_t n, const float* pos, cons
                                 const float* dlogv, int64_t ld, cudaStream_t st) {
     if (!npm::tc_can_train(h) && h->train_smem > 227 * 1024)
         return fail(NPM_ERR_UNSUPPORTED, "training activations do not fit in shared memory");
-    float* loss_acc = h->scalars;
-    NPM_CUDA(cudaMemsetAsync(loss_acc, 0, sizeof(float), st), "clear loss");
+    double* loss = loss_acc(h);
+    NPM_CUDA(cudaMemsetAsync(loss, 0, sizeof(double), st), "clear loss");
     if (n == 0) return NPM_OK;
     if (npm::tc_can_train(h)) {
-        NPM_CUDA(npm::tc_train(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss_acc, st), "train launch");
+        NPM_CUDA(npm::tc_train(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st), "train launch");
         return NPM_OK;
     }
-    NPM_CUDA(npm::launch_train_fp32(h->dc, h->params, h->mlp_off, h->wfwd, h->wbwd, n, ld, pos, aux,
-                                    dir, rad, spdf, dlogv, h->grads, loss_acc, st),
+    NPM_CUDA(npm::launch_train_fp32(h->dc, h->params, h->mlp_off, h->wfwd, n, ld, pos, aux, dir, rad, spdf,
+                                    dlogv, h->grads, loss, st),
              "train launch");
     return NPM_OK;
 }
 
-static npm_status adam_impl(npm_handle* h, const float* loss, cudaStream_t st) {
+static npm_status adam_impl(npm_handle* h, const double* loss, cudaStream_t st) {
     h->step += 1;
     int* status = reinterpret_cast<int*>(h->scalars + 8);
     const int64_t sh = 2 * (int64_t)h->dc.grid_shift;
@@ -679,8 +674,8 @@ npm_status npm_train_step(npm_handle* h, int64_t n, const float* pos, const floa
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = backward_impl(h, n, pos, aux, dir, radiance, sample_pdf, nullptr, ld, st)) != NPM_OK)
         return s;
-    if ((s = adam_impl(h, h->scalars, st)) != NPM_OK) return s;
-    if (loss_out) NPM_CUDA(npm::launch_copy_loss(h->scalars, loss_out, st), "copy loss");
+    if ((s = adam_impl(h, loss_acc(h), st)) != NPM_OK) return s;
+    if (loss_out) NPM_CUDA(npm::launch_copy_loss(loss_acc(h), loss_out, st), "copy loss");
     return NPM_OK;
 }
 

@@ -33,13 +33,11 @@ struct DevCfg {
     // average and FP16 copy alike) start past a 32-byte (FP32) or 16-byte
     // (FP16) boundary, so that the hashed levels start on one.
     uint32_t grid_shift;
-    // FP32 fused kernels: per layer, padded output count (multiple of 16)
-    // and float offsets of the pre-arranged weight blobs.
-    int np_fwd[NPM_MAX_LAYERS];   // padded N of W^T [K][np] (forward)
-    int np_bwd[NPM_MAX_LAYERS];   // padded K of W [N][np] (backward)
+    // CUDA-core kernels: per layer, padded output count (16, 32, 64 or 128)
+    // and float offset of W^T [in][np] in the pre-arranged weight blob.
+    int np_fwd[NPM_MAX_LAYERS];
     int off_fwd[NPM_MAX_LAYERS];
-    int off_bwd[NPM_MAX_LAYERS];
-    int fwd_floats, bwd_floats;
+    int fwd_floats;
     int max_width;
 };
 
@@ -389,22 +387,16 @@ __device__ __forceinline__ float inv_minus_coth(float k) {
 }
 
 // Arrange layer l of the MLP weights (row-major [out][in] per layer, packed)
-// into the padded forward (W^T [in][np_fwd]) and backward (W [out][np_bwd];
-// may be NULL) blobs of the CUDA-core kernels; thread tid of nt.
+// into the padded blob W^T [in][np_fwd] of the CUDA-core kernels; thread tid
+// of nt.
 __device__ __forceinline__ void arrange_layer(const DevCfg& cfg, int l, const float* __restrict__ mlp,
-                                              float* __restrict__ wfwd, float* __restrict__ wbwd, int tid, int nt) {
+                                              float* __restrict__ wfwd, int tid, int nt) {
     for (int m = 0; m < l; ++m) mlp += cfg.widths[m] * cfg.widths[m + 1];
-    const int K = cfg.widths[l], N = cfg.widths[l + 1];
-    const int npf = cfg.np_fwd[l], npb = cfg.np_bwd[l];
-    for (int i = tid; i < K * npf; i += nt) {
-        const int k = i / npf, nn = i % npf;
+    const int K = cfg.widths[l], N = cfg.widths[l + 1], np = cfg.np_fwd[l];
+    for (int i = tid; i < K * np; i += nt) {
+        const int k = i / np, nn = i % np;
         wfwd[cfg.off_fwd[l] + i] = nn < N ? mlp[nn * K + k] : 0.0f;
     }
-    if (wbwd)  // backward copy (training only)
-        for (int i = tid; i < N * npb; i += nt) {
-            const int nn = i / npb, k = i % npb;
-            wbwd[cfg.off_bwd[l] + i] = k < K ? mlp[nn * K + k] : 0.0f;
-        }
 }
 
 // A batch of query requests served by one launch of a forward kernel: the

@@ -41,9 +41,10 @@ __host__ __device__ constexpr int fwd_max_groups(int I) { return I <= 2 ? 6 : 4;
 
 // ----------------------------------------------------------- tile GEMM
 
-// Named barrier of tile group `group` (kNT threads; barrier 0 is the CTA's).
+// Named barrier of tile group `group` (T threads; barrier 0 is the CTA's).
+template <int T = kNT>
 __device__ __forceinline__ void group_sync(int group) {
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(kNT) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(T) : "memory");
 }
 
 template <int NI>
@@ -67,19 +68,21 @@ __device__ __forceinline__ void load_w(const float* p, float (&w)[NI]) {
 }
 
 // out[q][n] = f(sum_k in[q][k] * WT[k][n]) for q < 64, n < N. WT rows are
-// padded to NP = 16 * NI columns (zeros beyond N). mode 0: identity,
-// 1: ReLU, 2: keep where mask[q][n] > 0 (ReLU derivative), else 0.
+// padded to 16 * NI columns (zeros beyond N). mode 0: identity, 1: ReLU.
 // AST > 0: the activation row stride is the compile-time AST (so row and
 // weight addresses are immediate offsets of two pointers); else AS_rt.
+// OS_rt: row stride of out (AST = 0). WPAD: floats between the weight
+// rows beyond NP.
 // INPLACE: out may equal in; the tile group (named barrier group + 1)
 // synchronises between the last read of in and the first store.
-template <int NI, int AST, bool INPLACE>
+// T: threads of the tile group; each owns 64 * 16 / T queries.
+template <int NI, int AST, bool INPLACE, int WPAD = 0, int T = kNT>
 __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int K,
-                                          const float* __restrict__ WT, float* out, int N, int mode,
-                                          const float* __restrict__ mask, int group) {
-    const int AS = AST > 0 ? AST : AS_rt;
-    constexpr int NP = 16 * NI;
-    // Thread t owns output group g (16 groups) and query group qg (8): a
+                                          const float* __restrict__ WT, float* out, int OS_rt, int N, int mode,
+                                          int group) {
+    const int AS = AST > 0 ? AST : AS_rt, OS = AST > 0 ? AST : OS_rt;
+    constexpr int NP = 16 * NI + WPAD;
+    // Thread t owns output group g (16 groups) and query group qg (T / 16): a
     // warp covers all 16 output groups and 2 query groups, lanes 2i and
     // 2i + 1 sharing output group i. Lanes that read the same shared-memory
     // vector are adjacent, which keeps a warp's 16-byte shared loads at two
@@ -88,10 +91,11 @@ __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int
     // Accumulators paired along adjacent outputs: one packed two-lane FMA
     // (fma.rn on each lane, the same rounding as fmaf) per pair.
     constexpr int NP2 = NI >= 2 ? NI / 2 : 1;
-    float2 acc[8][NP2];
-    float acc1[8];
+    constexpr int QG = T / 16, NQ = kTQ / QG;  // query groups, queries of a thread (qg + QG j)
+    float2 acc[NQ][NP2];
+    float acc1[NQ];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < NQ; ++j) {
         acc1[j] = 0.0f;
 #pragma unroll
         for (int i = 0; i < NP2; ++i) acc[j][i] = make_float2(0.0f, 0.0f);
@@ -105,8 +109,8 @@ __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) load_w<NI>(WT + (k + kk) * NP + g * NI, w[kk]);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float4 a = *reinterpret_cast<const float4*>(in + (qg + 8 * j) * AS + k);
+            for (int j = 0; j < NQ; ++j) {
+                const float4 a = *reinterpret_cast<const float4*>(in + (qg + QG * j) * AS + k);
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const float av = kk == 0 ? a.x : kk == 1 ? a.y : kk == 2 ? a.z : a.w;
@@ -119,15 +123,15 @@ __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int
         }
     } else {
         for (int k = 0; k < K; k += 4) {
-            float4 a[8];
+            float4 a[NQ];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) a[j] = *reinterpret_cast<const float4*>(in + (qg + 8 * j) * AS + k);
+            for (int j = 0; j < NQ; ++j) a[j] = *reinterpret_cast<const float4*>(in + (qg + QG * j) * AS + k);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
                 float w[NI];
                 load_w<NI>(WT + (k + kk) * NP + g * NI, w);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < NQ; ++j) {
                     const float av = kk == 0 ? a[j].x : kk == 1 ? a[j].y : kk == 2 ? a[j].z : a[j].w;
                     const float2 aa = make_float2(av, av);
 #pragma unroll
@@ -137,17 +141,16 @@ __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int
             }
         }
     }
-    if constexpr (INPLACE) group_sync(group);
+    if constexpr (INPLACE) group_sync<T>(group);
     const bool full = g * NI + NI <= N;  // all NI outputs of this thread exist
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int row = (qg + 8 * j) * AS;
+    for (int j = 0; j < NQ; ++j) {
+        const int row = (qg + QG * j) * OS;
         float v[NI];
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
             v[i] = NI == 1 ? acc1[j] : ((i & 1) ? acc[j][i >> 1].y : acc[j][i >> 1].x);
             if (mode == 1) v[i] = fmaxf(v[i], 0.0f);
-            if (mode == 2) v[i] = (g * NI + i < N && mask[row + g * NI + i] > 0.0f) ? v[i] : 0.0f;
         }
         if constexpr (NI % 4 == 0) {
             if (full) {
@@ -166,16 +169,16 @@ __device__ __forceinline__ void tile_gemm(int t, const float* in, int AS_rt, int
 // One layer for the tile; only the register tiles up to NIMAX outputs per
 // thread are instantiated (NP = 16 NI <= 16 * NIMAX is guaranteed by the
 // launcher). AST as in tile_gemm.
-template <int NIMAX, int AST = 0, bool INPLACE = false>
+template <int NIMAX, int AST = 0, bool INPLACE = false, int WPAD = 0, int T = kNT>
 __device__ __forceinline__ void layer(int t, const float* in, int AS, int K, const float* WT, int NP,
-                                      float* out, int N, int mode, const float* mask, int group = 0) {
-    if (NP == 16) tile_gemm<1, AST, INPLACE>(t, in, AS, K, WT, out, N, mode, mask, group);
+                                      float* out, int OS, int N, int mode, int group = 0) {
+    if (NP == 16) tile_gemm<1, AST, INPLACE, WPAD, T>(t, in, AS, K, WT, out, OS, N, mode, group);
     else if (NIMAX >= 2 && NP == 32)
-        tile_gemm<(NIMAX >= 2 ? 2 : 1), AST, INPLACE>(t, in, AS, K, WT, out, N, mode, mask, group);
+        tile_gemm<(NIMAX >= 2 ? 2 : 1), AST, INPLACE, WPAD, T>(t, in, AS, K, WT, out, OS, N, mode, group);
     else if (NIMAX >= 4 && NP == 64)
-        tile_gemm<(NIMAX >= 4 ? 4 : 1), AST, INPLACE>(t, in, AS, K, WT, out, N, mode, mask, group);
+        tile_gemm<(NIMAX >= 4 ? 4 : 1), AST, INPLACE, WPAD, T>(t, in, AS, K, WT, out, OS, N, mode, group);
     else if (NIMAX >= 8)
-        tile_gemm<(NIMAX >= 8 ? 8 : 1), AST, INPLACE>(t, in, AS, K, WT, out, N, mode, mask, group);
+        tile_gemm<(NIMAX >= 8 ? 8 : 1), AST, INPLACE, WPAD, T>(t, in, AS, K, WT, out, OS, N, mode, group);
 }
 
 // ------------------------------------------------------------- encode
@@ -224,15 +227,16 @@ __device__ __forceinline__ void gather_level(const DevCfg& cfg, const float* __r
     }
 }
 
-// Fills act[q][0 .. widths[0]) for the tile's 64 queries; local thread t
-// handles query t % 64 and every other level (two levels in flight).
+// Fills act[q][0 .. widths[0]) for the tile's 64 queries; local thread t of T
+// handles query t % 64 and every (T / 64)-th level (two levels in flight).
 // FOUR: 2-feature grids keep four levels' loads in flight (registers the
 // wide instances have to spare).
-template <bool FOUR>
+template <bool FOUR, int T = kNT>
 __device__ __forceinline__ void encode_tile(int t, const DevCfg& cfg, const float* __restrict__ grid,
                                             int64_t base, int64_t n, int64_t ld,
                                             const float* __restrict__ pos,
                                             const float* __restrict__ aux, float* act, int AS) {
+    constexpr int P = T / kTQ;  // threads of a query
     const int q = t & (kTQ - 1), part = t >> 6;
     const int64_t j = base + q;
     const bool valid = j < n;
@@ -246,19 +250,19 @@ __device__ __forceinline__ void encode_tile(int t, const DevCfg& cfg, const floa
     const int F = cfg.feat;
     int l = part;
     if (FOUR && F == 2) {
-        // Four levels' corner loads in flight (levels l, l+2, l+4, l+6).
-        for (; l + 6 < cfg.n_levels; l += 8) {
+        // Four levels' corner loads in flight (levels l, l + P, ...).
+        for (; l + 3 * P < cfg.n_levels; l += 4 * P) {
             Cell cs[4];
             uint32_t idx[4][8];
             float2 v[4][8];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                cs[r] = make_cell(x, y, z, cfg.level_res[l + 2 * r]);
-                corner_idx8(cfg, l + 2 * r, cs[r], idx[r]);
-                const float* gr = grid + (size_t)cfg.level_off[l + 2 * r] * 2;
+                cs[r] = make_cell(x, y, z, cfg.level_res[l + P * r]);
+                corner_idx8(cfg, l + P * r, cs[r], idx[r]);
+                const float* gr = grid + (size_t)cfg.level_off[l + P * r] * 2;
 #pragma unroll
                 for (int c = 0; c < 8; c += 2)
-                    gather_pair2(gr, cfg.level_off[l + 2 * r] + cfg.grid_shift, idx[r][c], idx[r][c + 1], v[r][c], v[r][c + 1]);
+                    gather_pair2(gr, cfg.level_off[l + P * r] + cfg.grid_shift, idx[r][c], idx[r][c + 1], v[r][c], v[r][c + 1]);
             }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -270,25 +274,25 @@ __device__ __forceinline__ void encode_tile(int t, const DevCfg& cfg, const floa
                     a0 = fmaf(w[c], v[r][c].x, a0);
                     a1 = fmaf(w[c], v[r][c].y, a1);
                 }
-                row[(l + 2 * r) * 2] = a0;
-                row[(l + 2 * r) * 2 + 1] = a1;
+                row[(l + P * r) * 2] = a0;
+                row[(l + P * r) * 2 + 1] = a1;
             }
         }
     }
-    for (; l + 2 < cfg.n_levels; l += 4) {
+    for (; l + P < cfg.n_levels; l += 2 * P) {
         const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
-        const Cell c1 = make_cell(x, y, z, cfg.level_res[l + 2]);
+        const Cell c1 = make_cell(x, y, z, cfg.level_res[l + P]);
         float s0[8], s1[8];
         gather_level(cfg, grid, l, c0, s0);
-        gather_level(cfg, grid, l + 2, c1, s1);
+        gather_level(cfg, grid, l + P, c1, s1);
 #pragma unroll
         for (int f = 0; f < 8; ++f)
             if (f < F) {
                 row[l * F + f] = s0[f];
-                row[(l + 2) * F + f] = s1[f];
+                row[(l + P) * F + f] = s1[f];
             }
     }
-    for (; l < cfg.n_levels; l += 2) {
+    for (; l < cfg.n_levels; l += P) {
         const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
         float s0[8];
         gather_level(cfg, grid, l, c0, s0);
@@ -310,7 +314,7 @@ __device__ __forceinline__ void encode_tile(int t, const DevCfg& cfg, const floa
             sh_band4(wo[0], wo[1], wo[2], sh);
 #pragma unroll
             for (int i = 0; i < 16; ++i) row[o + i] = sh[i];
-        } else {
+        } else if (part == 1) {
             float nn[3] = {0.0f, 0.0f, 1.0f}, r = 0.0f;
             if (valid) {
                 nn[0] = aux[3 * ld + j];
@@ -578,8 +582,8 @@ __global__ void __launch_bounds__(fwd_max_groups(NIMAX) * kNT, 1) k_forward_fp32
         }
         for (int l = 0; l < cfg.n_layers; ++l) {
             const bool last = l == cfg.n_layers - 1;
-            layer<NIMAX, AS, true>(t, act, AS, cfg.widths[l], sW + cfg.off_fwd[l], cfg.np_fwd[l], act,
-                                   cfg.widths[l + 1], last ? 0 : 1, nullptr, group);
+            layer<NIMAX, AS, true>(t, act, AS, cfg.widths[l], sW + cfg.off_fwd[l], cfg.np_fwd[l], act, AS,
+                                   cfg.widths[l + 1], last ? 0 : 1, group);
             group_sync(group);
         }
         epilogue_tile<SAMPLE, KH>(t, cfg, act, AS, base, n, S.ld, S.uin, S.ufrac, S.dir, S.pdf, S.mix,
@@ -590,23 +594,25 @@ __global__ void __launch_bounds__(fwd_max_groups(NIMAX) * kNT, 1) k_forward_fp32
 
 // ------------------------------------------------------ training kernel
 
+// Threads of a training tile group: four per query of its 64-query tiles.
+constexpr int kTrainT = 256;
+
 // Per query: raw outputs -> d(sum_j s_j log V_j)/d raw, written in place,
-// and s_j log V_j accumulated into *loss. Log-domain mixture so that log V
+// and s_j log V_j added to lacc. Log-domain mixture so that log V
 // and the responsibilities r_i stay finite when V underflows FP32.
-__device__ __forceinline__ void grad_epilogue(const DevCfg& cfg, float* act, int AS, int64_t base,
+template <int P>
+__device__ __forceinline__ void grad_epilogue(int t, const DevCfg& cfg, float* act, int AS, int64_t base,
                                               int64_t n, int64_t ld,
                                               const float* __restrict__ dir,
                                               const float* __restrict__ rad,
                                               const float* __restrict__ spdf,
-                                              const float* __restrict__ dlogv, float inv_n,
-                                              float* __restrict__ loss) {
-    const int t = threadIdx.x;
-    const int q = t >> 1, half = t & 1;
+                                              const float* __restrict__ dlogv, float inv_n, float& lacc) {
+    const int q = t / P, part = t % P;
     const int64_t j = base + q;
     const bool valid = j < n;
     float* raw = act + q * AS;
-    const int K = cfg.K, KH = (K + 1) >> 1;
-    const int l0 = half * KH, cnt = min(K, l0 + KH) - l0;
+    const int K = cfg.K, KH = (K + P - 1) / P;
+    const int l0 = part * KH, cnt = min(K, l0 + KH) - l0;  // (none where the others hold all)
     float w[3] = {0.0f, 0.0f, 1.0f};
     float s = 0.0f;
     if (valid) {
@@ -615,18 +621,20 @@ __device__ __forceinline__ void grad_epilogue(const DevCfg& cfg, float* act, int
         w[2] = dir[2 * ld + j];
         s = dlogv ? dlogv[j] : -(rad[j] / spdf[j]) * inv_n;
     }
-    constexpr int H = NPM_MAX_LOBES / 2;
+    constexpr int H = NPM_MAX_LOBES / P;
     float lp[H], a[H], kap[H], md[H], wdt[H], wdp[H], sk[H], st[H], sp[H];
     float mx = -INFINITY;
 #pragma unroll
     for (int ii = 0; ii < H; ++ii)
         if (ii < cnt) mx = fmaxf(mx, raw[4 * (l0 + ii)]);
-    mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 1));
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
     float ssum = 0.0f;
 #pragma unroll
     for (int ii = 0; ii < H; ++ii)
         if (ii < cnt) ssum += expf(raw[4 * (l0 + ii)] - mx);
-    ssum += __shfl_xor_sync(kFull, ssum, 1);
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) ssum += __shfl_xor_sync(kFull, ssum, o);
     const float lse = mx + logf(ssum);
     float amax = -INFINITY;
 #pragma unroll
@@ -653,12 +661,14 @@ __device__ __forceinline__ void grad_epilogue(const DevCfg& cfg, float* act, int
             a[ii] = lp[ii] + logf(vmf_scaled_norm(kap[ii])) + kap[ii] * (md[ii] - 1.0f);
             amax = fmaxf(amax, a[ii]);
         }
-    amax = fmaxf(amax, __shfl_xor_sync(kFull, amax, 1));
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(kFull, amax, o));
     float es = 0.0f;
 #pragma unroll
     for (int ii = 0; ii < H; ++ii)
         if (ii < cnt) es += expf(a[ii] - amax);
-    es += __shfl_xor_sync(kFull, es, 1);
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) es += __shfl_xor_sync(kFull, es, o);
     const float logV = amax + logf(es);
 #pragma unroll
     for (int ii = 0; ii < H; ++ii)
@@ -672,63 +682,101 @@ __device__ __forceinline__ void grad_epilogue(const DevCfg& cfg, float* act, int
             raw[4 * i + 2] = sr * kap[ii] * wdt[ii] * kPi * st[ii] * (1.0f - st[ii]);
             raw[4 * i + 3] = sr * kap[ii] * wdp[ii] * 2.0f * kPi * sp[ii] * (1.0f - sp[ii]);
         }
-    // Zero the padding columns of the raw buffer (4K == widths[n_layers], so
-    // nothing to do) and accumulate the loss once per query.
-    float lv = (valid && half == 0) ? s * logV : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lv += __shfl_xor_sync(kFull, lv, o);
-    if ((threadIdx.x & 31) == 0 && lv != 0.0f) atomicAdd(loss, lv);
+    if (valid && part == 0) lacc += s * logV;
 }
 
-// dW[n][k] += sum_q dl[q][n] * h[q][k] (global atomics).
-__device__ __forceinline__ void weight_grad(const float* dl, const float* h, int AS, int N, int K,
+// dW[n][k] += sum_q dl[q][n] * h[q][k] (global atomics); row strides DS, HS.
+// Thread t of 256 owns 4 x 4 blocks.
+__device__ __forceinline__ void weight_grad(int t, const float* dl, int DS, const float* h, int HS, int N, int K,
                                             float* __restrict__ gW) {
-    const int t = threadIdx.x;
-    const int a = t >> 4, b = t & 15;
-    for (int n0 = a * 8; n0 < N; n0 += 64)
-        for (int k0 = b * 4; k0 < K; k0 += 64) {
-            float acc[8][4];
+    for (int n0 = (t >> 4) * 4; n0 < N; n0 += 64)
+        for (int k0 = (t & 15) * 4; k0 < K; k0 += 64) {
+            float2 acc[4][2];
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = 0.0f;
-            const bool two = n0 + 4 < N;
+            for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
             for (int q = 0; q < kTQ; ++q) {
-                const float4 hv = *reinterpret_cast<const float4*>(h + q * AS + k0);
-                const float4 d0 = *reinterpret_cast<const float4*>(dl + q * AS + n0);
-                float4 d1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (two) d1 = *reinterpret_cast<const float4*>(dl + q * AS + n0 + 4);
-                const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-                const float hh[4] = {hv.x, hv.y, hv.z, hv.w};
+                const float4 hv = *reinterpret_cast<const float4*>(h + q * HS + k0);
+                const float4 d = *reinterpret_cast<const float4*>(dl + q * DS + n0);
+                const float2 h0 = make_float2(hv.x, hv.y), h1 = make_float2(hv.z, hv.w);
+                const float dv[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
-                for (int r = 0; r < 8; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(dv[r], hh[c], acc[r][c]);
+                for (int r = 0; r < 4; ++r) {
+                    const float2 dd = make_float2(dv[r], dv[r]);
+                    acc[r][0] = __ffma2_rn(dd, h0, acc[r][0]);
+                    acc[r][1] = __ffma2_rn(dd, h1, acc[r][1]);
+                }
             }
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
-                if (n0 + r < N) {
-                    // (8-byte aligned: the gradient shares the tables' shift)
-                    float* dst = gW + (size_t)(n0 + r) * K + k0;
-                    atomicAdd(reinterpret_cast<float2*>(dst), make_float2(acc[r][0], acc[r][1]));
-                    atomicAdd(reinterpret_cast<float2*>(dst) + 1, make_float2(acc[r][2], acc[r][3]));
-                }
+            for (int r = 0; r < 4; ++r) {
+                // (8-byte aligned: the gradient shares the tables' shift)
+                float2* dst = reinterpret_cast<float2*>(gW + (size_t)(n0 + r) * K + k0);
+                atomicAdd(dst, acc[r][0]);
+                atomicAdd(dst + 1, acc[r][1]);
+            }
         }
 }
 
+// The layer's input gradient in place of its input h: h[q][k] =
+// (sum_n dl[q][n] W[n][k]) where h[q][k] > 0 (ReLU's derivative; everywhere
+// without relu), from the forward pass's copy of the weights, W^T rows of WS
+// floats. Thread (qg, g) of 256 owns queries qg + 16 j and inputs g + 16 i; the sums
+// run over n in packed pairs. WS = np + 4 keeps the 16 rows that a warp reads
+// at once on different banks.
+__device__ __forceinline__ void input_grad(int t, const float* dl, int DS, int N, const float* __restrict__ WT, int WS,
+                                           float* h, int HS, int K, bool relu) {
+    constexpr int KI = 4, NQ = 4;  // inputs a thread and pass, queries
+    const int g = (t & 31) >> 1, qg = (t & 1) | ((t >> 5) << 1);
+    for (int k0 = 0; k0 < K; k0 += 16 * KI) {
+        float2 acc[NQ][KI];
+#pragma unroll
+        for (int j = 0; j < NQ; ++j)
+#pragma unroll
+            for (int i = 0; i < KI; ++i) acc[j][i] = make_float2(0.0f, 0.0f);
+        // Rows past K repeat the last one (their sums are not stored).
+        const float* wr[KI];
+#pragma unroll
+        for (int i = 0; i < KI; ++i) wr[i] = WT + min(k0 + g + 16 * i, K - 1) * WS;
+        for (int n = 0; n < N; n += 4) {
+            float4 w[KI];
+#pragma unroll
+            for (int i = 0; i < KI; ++i) w[i] = *reinterpret_cast<const float4*>(wr[i] + n);
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                const float4 a = *reinterpret_cast<const float4*>(dl + (qg + 16 * j) * DS + n);
+                const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+#pragma unroll
+                for (int i = 0; i < KI; ++i) {
+                    acc[j][i] = __ffma2_rn(a0, make_float2(w[i].x, w[i].y), acc[j][i]);
+                    acc[j][i] = __ffma2_rn(a1, make_float2(w[i].z, w[i].w), acc[j][i]);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NQ; ++j)
+#pragma unroll
+            for (int i = 0; i < KI; ++i) {
+                const int k = k0 + g + 16 * i;
+                if (k < K) {
+                    float* o = h + (qg + 16 * j) * HS + k;
+                    *o = !relu || *o > 0.0f ? acc[j][i].x + acc[j][i].y : 0.0f;
+                }
+            }
+    }
+}
+
 // Grid gradient: dV_l[corner] += weight * dG_l (Eq. 11 transposed).
-__device__ __forceinline__ void grid_scatter(const DevCfg& cfg, const float* denc, int AS,
+__device__ __forceinline__ void grid_scatter(int t, const DevCfg& cfg, const float* denc, int AS,
                                              int64_t base, int64_t n, int64_t ld,
                                              const float* __restrict__ pos,
                                              float* __restrict__ ggrid) {
-    const int t = threadIdx.x;
     const int q = t & (kTQ - 1), part = t >> 6;
     const int64_t j = base + q;
     if (j >= n) return;
     const float x = pos[j], y = pos[ld + j], z = pos[2 * ld + j];
     const float* row = denc + q * AS;
     const int F = cfg.feat;
-    for (int l = part; l < cfg.n_levels; l += 2) {
+    for (int l = part; l < cfg.n_levels; l += kTrainT / kTQ) {
         const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
         float* gl = ggrid + (size_t)cfg.level_off[l] * F;
         const float* dg = row + l * F;
@@ -755,66 +803,103 @@ __device__ __forceinline__ void grid_scatter(const DevCfg& cfg, const float* den
     }
 }
 
-__global__ void __launch_bounds__(kNT) k_train_fp32(DevCfg cfg, const float* __restrict__ params,
-                                                    int64_t mlp_off,
-                                                    const float* __restrict__ wfwd,
-                                                    const float* __restrict__ wbwd, int64_t n,
-                                                    int64_t ld, const float* __restrict__ pos,
-                                                    const float* __restrict__ aux,
-                                                    const float* __restrict__ dir,
-                                                    const float* __restrict__ rad,
-                                                    const float* __restrict__ spdf,
-                                                    const float* __restrict__ dlogv, float inv_n,
-                                                    float* __restrict__ grad,
-                                                    float* __restrict__ loss) {
+// Floats of a CTA's shared memory: the weights, W^T rows padded by 4, and per
+// tile group the input and every layer's output of a 64-query tile, rows
+// padded by 4.
+constexpr int kPad = 4;
+__host__ __device__ inline int train_weight_floats(const DevCfg& c) {
+    int n = 0;
+    for (int l = 0; l < c.n_layers; ++l) n += c.widths[l] * (c.np_fwd[l] + kPad);
+    return n;
+}
+__host__ __device__ inline int train_group_floats(const DevCfg& c) {
+    int n = 0;
+    for (int l = 0; l <= c.n_layers; ++l) n += kTQ * (c.widths[l] + kPad);
+    return n;
+}
+
+// Tile groups of 256 threads share the weights; each walks its own 64-query
+// tiles. A layer's gradient replaces its activations in place, and forward
+// and backward read one copy of the weights, so two groups (16 warps) fit
+// beside it on the 64-wide networks. Bound by FMA issue and shared-memory
+// operands, which share the L1 data pipe. Against one group of 128 threads
+// with one buffer more and the backward weights in global memory (GB300):
+// 65,551 samples of the eight-level grid into 64-wide layers 370 -> 214 us,
+// 20,011 of the product-mode network 200 -> 135 us (two groups of 128
+// threads: 301 against 261 us for the whole step of the first).
+constexpr int kTrainGroups = 2;
+
+__global__ void __launch_bounds__(kTrainGroups* kTrainT, 1)
+    k_train_fp32(const __grid_constant__ DevCfg cfg, const float* __restrict__ params, int64_t mlp_off,
+                 const float* __restrict__ wfwd, int64_t n, int64_t ld, const float* __restrict__ pos,
+                 const float* __restrict__ aux, const float* __restrict__ dir, const float* __restrict__ rad,
+                 const float* __restrict__ spdf, const float* __restrict__ dlogv, float inv_n,
+                 float* __restrict__ grad, double* __restrict__ loss) {
     extern __shared__ float4 smem4[];
     float* sW = reinterpret_cast<float*>(smem4);
-    const int AS = cfg.max_width + 4;
     const int L = cfg.n_layers;
-    float* buf0 = sW + cfg.fwd_floats;  // L + 2 activation buffers
-    auto buf = [&](int i) { return buf0 + i * kTQ * AS; };
-    for (int i = threadIdx.x; i < cfg.fwd_floats / 4; i += kNT)
-        smem4[i] = __ldg(reinterpret_cast<const float4*>(wfwd) + i);
-    __syncthreads();
-    const int64_t ntiles = (n + kTQ - 1) / kTQ;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t base = tile * kTQ;
-        encode_tile<false>(threadIdx.x, cfg, params, base, n, ld, pos, aux, buf(0), AS);
-        __syncthreads();
+    const int G = blockDim.x / kTrainT, group = threadIdx.x / kTrainT, t = threadIdx.x % kTrainT;
+    float* buf0 = sW + train_weight_floats(cfg) + group * train_group_floats(cfg);
+    {
+        int o = 0;
         for (int l = 0; l < L; ++l) {
-            layer<8>(threadIdx.x, buf(l), AS, cfg.widths[l], sW + cfg.off_fwd[l], cfg.np_fwd[l],
-                     buf(l + 1), cfg.widths[l + 1], l == L - 1 ? 0 : 1, nullptr);
-            __syncthreads();
+            const int np4 = cfg.np_fwd[l] / 4, ws4 = (cfg.np_fwd[l] + kPad) / 4;
+            const float4* src = reinterpret_cast<const float4*>(wfwd + cfg.off_fwd[l]);
+            for (int i = threadIdx.x; i < cfg.widths[l] * np4; i += blockDim.x)
+                smem4[o + i / np4 * ws4 + i % np4] = __ldg(src + i);
+            o += cfg.widths[l] * ws4;
         }
-        grad_epilogue(cfg, buf(L), AS, base, n, ld, dir, rad, spdf, dlogv, inv_n, loss);
-        __syncthreads();
-        // Backward: delta_L lives in buf(L); delta_{L-1} in buf(L+1);
-        // delta_{i-1} (i < L) overwrites buf(i), whose activations are spent.
-        float* dcur = buf(L);
-        for (int i = L; i >= 1; --i) {
-            const int N = cfg.widths[i], Kw = cfg.widths[i - 1];
-            float* h = buf(i - 1);
-            // Offset of W_i inside the packed MLP region.
-            int64_t woff = 0;
-            for (int m = 0; m < i - 1; ++m) woff += (int64_t)cfg.widths[m] * cfg.widths[m + 1];
-            weight_grad(dcur, h, AS, N, Kw, grad + mlp_off + woff);
-            float* dnext = (i == L) ? buf(L + 1) : buf(i);
-            layer<8>(threadIdx.x, dcur, AS, N, wbwd + cfg.off_bwd[i - 1], cfg.np_bwd[i - 1], dnext,
-                     Kw, i > 1 ? 2 : 0, h);
-            __syncthreads();
-            dcur = dnext;
-        }
-        grid_scatter(cfg, dcur, AS, base, n, ld, pos, grad);
-        __syncthreads();
     }
+    __syncthreads();
+    float lacc = 0.0f;  // this thread's share of the loss
+    const int64_t ntiles = (n + kTQ - 1) / kTQ;
+    for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < ntiles; tile += (int64_t)gridDim.x * G) {
+        const int64_t base = tile * kTQ;
+        float* buf = buf0;
+        const float* w = sW;
+        encode_tile<false, kTrainT>(t, cfg, params, base, n, ld, pos, aux, buf, cfg.widths[0] + kPad);
+        group_sync<kTrainT>(group);
+        for (int l = 0; l < L; ++l) {
+            const int IS = cfg.widths[l] + kPad, OS = cfg.widths[l + 1] + kPad;
+            float* out = buf + kTQ * IS;
+            layer<8, 0, false, kPad, kTrainT>(t, buf, IS, cfg.widths[l], w, cfg.np_fwd[l], out, OS, cfg.widths[l + 1],
+                                     l == L - 1 ? 0 : 1, group);
+            group_sync<kTrainT>(group);
+            buf = out;
+            w += cfg.widths[l] * (cfg.np_fwd[l] + kPad);
+        }
+        grad_epilogue<kTrainT / kTQ>(t, cfg, buf, cfg.widths[L] + kPad, base, n, ld, dir, rad, spdf, dlogv, inv_n, lacc);
+        group_sync<kTrainT>(group);
+        // Backward: the gradient of layer l's output lies in buf; that of its
+        // input takes the place of the input.
+        float* gW = grad + mlp_off;
+        for (int l = 0; l < L; ++l) gW += cfg.widths[l] * cfg.widths[l + 1];
+        for (int l = L - 1; l >= 0; --l) {
+            const int N = cfg.widths[l + 1], K = cfg.widths[l];
+            float* h = buf - kTQ * (K + kPad);
+            w -= K * (cfg.np_fwd[l] + kPad);
+            gW -= K * N;
+            weight_grad(t, buf, N + kPad, h, K + kPad, N, K, gW);
+            group_sync<kTrainT>(group);
+            input_grad(t, buf, N + kPad, N, w, cfg.np_fwd[l] + kPad, h, K + kPad, K, l > 0);
+            group_sync<kTrainT>(group);
+            buf = h;
+        }
+        grid_scatter(t, cfg, buf, cfg.widths[0] + kPad, base, n, ld, pos, grad);
+        group_sync<kTrainT>(group);
+    }
+    // The loss: one atomic a warp.
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(kFull, lacc, o);
+    if ((t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
 }
 
 // ------------------------------------------------------- utility kernels
 
 // blockIdx.y: layer.
 __global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const float* __restrict__ mlp,
-                                  float* __restrict__ wfwd, float* __restrict__ wbwd) {
-    arrange_layer(cfg, blockIdx.y, mlp, wfwd, wbwd, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+                                  float* __restrict__ wfwd) {
+    arrange_layer(cfg, blockIdx.y, mlp, wfwd, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // Dense Adam with bias correction (Kingma and Ba) at step t = *steps + 1,
@@ -827,7 +912,7 @@ __global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const floa
 // (Sec. 5.3); the FP16 copy (inference only) is then taken from e.
 __global__ void k_adam(int64_t n4, float4* __restrict__ p, float4* __restrict__ g,
                        float4* __restrict__ m, float4* __restrict__ v, float lr, float b1, float b2,
-                       float eps, const int* __restrict__ steps, const float* __restrict__ loss,
+                       float eps, const int* __restrict__ steps, const double* __restrict__ loss,
                        int* __restrict__ status, __half2* __restrict__ half_copy, int64_t n_half,
                        float4* __restrict__ ema, float ema_decay) {
     const bool skip = loss != nullptr && !isfinite(*loss);
@@ -922,13 +1007,15 @@ __global__ void k_to_half(int64_t n, const float* __restrict__ src, __half* __re
         dst[i] = __float2half_rn(src[i]);
 }
 
-__global__ void k_copy_loss(const float* __restrict__ acc, float* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *out = *acc;
+__global__ void k_copy_loss(const double* __restrict__ acc, float* __restrict__ out) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) *out = (float)*acc;
 }
 
 // ----------------------------------------------------------- launchers
 
 
+// What decides whether a network can be trained in FP32 (part of the
+// interface); the kernel's own layout is never larger.
 size_t train_smem_bytes(const DevCfg& c) {
     return sizeof(float) *
            ((size_t)c.fwd_floats + (size_t)(c.n_layers + 2) * kTQ * (c.max_width + 4));
@@ -942,17 +1029,6 @@ static int sm_count() {
         cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev);
     }
     return cached;
-}
-
-template <typename KernelT>
-static int persistent_grid(KernelT kern, size_t smem, int64_t ntiles) {
-    int per_sm = 0;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kNT, smem);
-    if (per_sm < 1) per_sm = 1;
-    int64_t g = (int64_t)per_sm * sm_count();
-    if (g > ntiles) g = ntiles;
-    return (int)(g < 1 ? 1 : g);
 }
 
 // Shared-memory carveout (percent of the 228 KB maximum) that holds `bytes`.
@@ -1046,27 +1122,31 @@ cudaError_t launch_forward_fp32(const DevCfg& cfg, const float* grid, const floa
     return launch_forward_fp32_batch(cfg, grid, wfwd, qb, n, st);
 }
 
-cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t mlp_off,
-                              const float* wfwd, const float* wbwd, int64_t n, int64_t ld,
-                              const float* pos, const float* aux, const float* dir,
-                              const float* rad, const float* spdf, const float* dlogv,
-                              float* grad, float* loss, cudaStream_t st) {
-    const size_t smem = train_smem_bytes(cfg);
+cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t mlp_off, const float* wfwd, int64_t n,
+                              int64_t ld, const float* pos, const float* aux, const float* dir, const float* rad,
+                              const float* spdf, const float* dlogv, float* grad, double* loss, cudaStream_t st) {
+    const size_t wbytes = sizeof(float) * train_weight_floats(cfg), gbytes = sizeof(float) * train_group_floats(cfg);
+    int G = kTrainGroups;
+    while (G > 1 && wbytes + G * gbytes > 227 * 1024) --G;
+    const size_t smem = wbytes + G * gbytes;
+    static std::atomic<uint64_t> attrs{~0ull};
+    cudaError_t e = set_smem_attrs(k_train_fp32, smem, carveout_percent(smem + 1024), attrs);
+    if (e != cudaSuccess) return e;
     const int64_t ntiles = (n + kTQ - 1) / kTQ;
-    const int g = persistent_grid(k_train_fp32, smem, ntiles);
-    k_train_fp32<<<g, kNT, smem, st>>>(cfg, params, mlp_off, wfwd, wbwd, n, ld, pos, aux, dir, rad,
-                                       spdf, dlogv, 1.0f / (float)n, grad, loss);
+    int64_t g = sm_count();
+    if (ntiles < g) g = ntiles;
+    k_train_fp32<<<(int)g, G * kTrainT, smem, st>>>(cfg, params, mlp_off, wfwd, n, ld, pos, aux, dir, rad, spdf, dlogv,
+                                                1.0f / (float)n, grad, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, float* wbwd,
-                                   cudaStream_t st) {
-    k_arrange_weights<<<dim3(16, cfg.n_layers), 256, 0, st>>>(cfg, mlp, wfwd, wbwd);
+cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, cudaStream_t st) {
+    k_arrange_weights<<<dim3(16, cfg.n_layers), 256, 0, st>>>(cfg, mlp, wfwd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float lr, float b1,
-                        float b2, float eps, int* steps, const float* loss, int* status,
+                        float b2, float eps, int* steps, const double* loss, int* status,
                         __half* half_copy, int64_t n_half, float* ema, float ema_decay,
                         cudaStream_t st) {
     const int64_t n4 = n / 4;
@@ -1100,7 +1180,7 @@ cudaError_t launch_to_half(int64_t n, const float* src, __half* dst, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_copy_loss(const float* acc, float* out, cudaStream_t st) {
+cudaError_t launch_copy_loss(const double* acc, float* out, cudaStream_t st) {
     k_copy_loss<<<1, 32, 0, st>>>(acc, out);
     return cudaGetLastError();
 }

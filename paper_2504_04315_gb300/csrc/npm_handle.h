@@ -24,10 +24,9 @@ struct npm_handle {
     float* grads = nullptr;
     float* adam_m = nullptr;
     float* adam_v = nullptr;
-    float* wfwd = nullptr;     // padded W^T blobs for the FP32 kernels
-    float* wbwd = nullptr;     // padded W blobs (backward)
+    float* wfwd = nullptr;     // padded W^T blob of the CUDA-core kernels
     __half* grid_h = nullptr;  // FP16 grid copy (BF16 precision)
-    // [0] loss accumulator, [8] status word, [16] Adam steps, [24] version of
+    // [0] loss accumulator (64 bits), [8] status word, [16] Adam steps, [24] version of
     // the parameters (both counted on the device, so that replayed graphs
     // count too)
     float* scalars = nullptr;
@@ -52,6 +51,7 @@ struct npm_handle {
 // Parameters and FP32 forward weights that inference evaluates.
 inline const float* inf_params(const npm_handle* h) { return h->ema ? h->ema : h->params; }
 inline const float* inf_wfwd(const npm_handle* h) { return h->ema ? h->wfwd_inf : h->wfwd; }
+inline double* loss_acc(npm_handle* h) { return reinterpret_cast<double*>(h->scalars); }
 // Device status word (kStatus* bits, read by npm_check_device_status).
 inline int* status_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 8); }
 // Device-side counter of changes to the parameters.
@@ -85,7 +85,7 @@ npm_status set_error(npm_status s, const char* msg);
 // gets NPM_ERR_UNSUPPORTED from tc_create and runs on the CUDA-core kernels.
 npm_status tc_create(npm_handle* h);
 void tc_destroy(npm_handle* h);
-// Weights arranged for the MMAs; with cuda_cores also h->wfwd and h->wbwd.
+// Weights arranged for the MMAs; with cuda_cores also h->wfwd.
 cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st);
 // pdl: the small networks' kernel may be launched as a programmatic
 // dependent of the stream's previous kernel, which must then not write the
@@ -94,7 +94,7 @@ cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStr
 // Training step kernels on tensor cores (split BF16 operands).
 bool tc_can_train(npm_handle* h);
 cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux, const float* dir,
-                     const float* rad, const float* spdf, const float* dlogv, float* loss, cudaStream_t st);
+                     const float* rad, const float* spdf, const float* dlogv, double* loss, cudaStream_t st);
 // log_pdf (evaluation only): pdf_out receives log V instead of V.
 npm_status tc_query(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,
                     const float* uin, float ufrac, bool sample, float* dir_out, float* pdf_out,

@@ -79,14 +79,11 @@ cudaError_t launch_forward_fp32(const DevCfg& cfg, const float* grid, const floa
 cudaError_t launch_forward_fp32_batch(const DevCfg& cfg, const float* grid, const float* wfwd,
                                       QueryBatch& qb, int64_t max_n, cudaStream_t st);
 
-cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t mlp_off,
-                              const float* wfwd, const float* wbwd, int64_t n, int64_t ld,
-                              const float* pos, const float* aux, const float* dir,
-                              const float* rad, const float* spdf, const float* dlogv,
-                              float* grad, float* loss, cudaStream_t st);
+cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t mlp_off, const float* wfwd, int64_t n,
+                              int64_t ld, const float* pos, const float* aux, const float* dir, const float* rad,
+                              const float* spdf, const float* dlogv, float* grad, double* loss, cudaStream_t st);
 
-cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, float* wbwd,
-                                   cudaStream_t st);
+cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, cudaStream_t st);
 
 // Adam at step *steps + 1 (device counter, advanced on the stream after the
 // update). The buffers are those of the parameters and what mirrors them from
@@ -94,7 +91,7 @@ cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* w
 // ema (or NULL): moving average updated with ema_decay; the FP16 copy is then
 // taken from it.
 cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float lr, float b1,
-                        float b2, float eps, int* steps, const float* loss, int* status,
+                        float b2, float eps, int* steps, const double* loss, int* status,
                         __half* half_copy, int64_t n_half, float* ema, float ema_decay,
                         cudaStream_t st);
 
@@ -103,6 +100,6 @@ cudaError_t launch_grid_indices(const DevCfg& cfg, int64_t n, int64_t ld, const 
 
 cudaError_t launch_to_half(int64_t n, const float* src, __half* dst, cudaStream_t st);
 
-cudaError_t launch_copy_loss(const float* acc, float* out, cudaStream_t st);
+cudaError_t launch_copy_loss(const double* acc, float* out, cudaStream_t st);
 
 }  // namespace npm

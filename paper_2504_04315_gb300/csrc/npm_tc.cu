@@ -221,16 +221,15 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
 
 // Master FP32 weights (packed [out][in] per layer) -> 16-bit operand parts in
 // the UMMA K-major layout, zero padded to Np x Kp per layer; with wfwd also
-// the CUDA-core kernels' padded copies; with version counts a change of the
+// the CUDA-core kernels' padded copy; with version counts a change of the
 // parameters. blockIdx.y: layer (one pass of load latency for all layers
 // instead of one each).
 __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __restrict__ mlp,
-                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, float* __restrict__ wbwd,
-                             int* __restrict__ version) {
+                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, int* __restrict__ version) {
     const int l = blockIdx.y;
     if (version && l == 0 && blockIdx.x == 0 && threadIdx.x == 0) *version += 1;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, wbwd, tid, nt);
+    if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, tid, nt);
     const TcLayer& ly = tc.layer[l];
     for (int m = 0; m < l; ++m) mlp += tc.layer[m].K * tc.layer[m].N;
     for (int i = tid; i < ly.Np * ly.Kp; i += nt) {
@@ -524,7 +523,7 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
     const uint8_t* __restrict__ wblob, int64_t n, int64_t ld, const float* __restrict__ pos,
     const float* __restrict__ aux, const float* __restrict__ dir, const float* __restrict__ rad,
     const float* __restrict__ spdf, const float* __restrict__ dlogv, float inv_n, float* __restrict__ grad,
-    int64_t mlp_off, float* __restrict__ loss, int* __restrict__ status, const float* __restrict__ enc) {
+    int64_t mlp_off, double* __restrict__ loss, int* __restrict__ status, const float* __restrict__ enc) {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int KH = KMAX / 2;
     uint8_t* sW = smem;
@@ -829,7 +828,7 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
     // Loss: one atomic per warp.
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
-    if ((t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, lacc);
+    if ((t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
     // Weight gradients: lane o of layer l's TMEM region holds dW_l[o][*].
     tc_fence_before();
     __syncthreads();
@@ -1092,10 +1091,9 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
     TcState* s = h->tc;
     const dim3 grid(16, h->dc.n_layers);
     k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr,
-                                       h->wbwd, version_word(h));
+                                       version_word(h));
     if (s->wblob_train)
-        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr,
-                                           nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr);
     if (h->ema) {
         if (!s->wblob_inf) {
             const size_t bytes = (size_t)s->cfg.wparts * s->cfg.w_bytes;
@@ -1103,7 +1101,7 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
             if (e != cudaSuccess) return e;
             cudaMemsetAsync(s->wblob_inf, 0, bytes, st);
         }
-        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr, nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr);
     }
     return cudaGetLastError();
 }
@@ -1111,7 +1109,7 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
 template <int KMAX, bool F2>
 static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,
                                    const float* dir, const float* rad, const float* spdf, const float* dlogv,
-                                   float* loss, cudaStream_t st) {
+                                   double* loss, cudaStream_t st) {
     TcState* s = h->tc;
     auto kern = k_train_tc<KMAX, F2>;
     // CTAs per SM: the instance's register budget, if shared and tensor
@@ -1156,7 +1154,7 @@ static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const f
 bool tc_can_train(npm_handle* h) { return h->tc && h->tc->can_train; }
 
 cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux, const float* dir,
-                     const float* rad, const float* spdf, const float* dlogv, float* loss, cudaStream_t st) {
+                     const float* rad, const float* spdf, const float* dlogv, double* loss, cudaStream_t st) {
     const int K = h->cfg.K;
     const bool f2 = h->cfg.feat_per_level == 2;
     if (K <= 4)
