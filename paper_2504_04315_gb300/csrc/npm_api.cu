@@ -169,22 +169,24 @@ int* step_dev(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 16); }
 // The weights as the kernels read them: the tensor-core operands, and the
 // CUDA-core kernels' padded copy where those serve training or inference
 // (of the moving average too, when inference evaluates it).
-npm_status arrange_all_weights(npm_handle* h, cudaStream_t st) {
+npm_status arrange_all_weights(npm_handle* h, const npm::UpdateEnd& end, cudaStream_t st) {
     if (h->tc) {
-        NPM_CUDA(npm::tc_refresh_weights(h, !npm::tc_can_train(h), st), "arrange weights");
+        NPM_CUDA(npm::tc_refresh_weights(h, !npm::tc_can_train(h), end, st), "arrange weights");
         return NPM_OK;
     }
-    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, st), "arrange weights");
     if (h->ema)
-        NPM_CUDA(npm::launch_arrange_weights(h->dc, h->ema + h->mlp_off, h->wfwd_inf, st),
+        NPM_CUDA(npm::launch_arrange_weights(h->dc, h->ema + h->mlp_off, h->wfwd_inf, npm::UpdateEnd{}, st),
                  "arrange ema weights");
+    NPM_CUDA(npm::launch_arrange_weights(h->dc, h->params + h->mlp_off, h->wfwd, end, st), "arrange weights");
     return NPM_OK;
 }
 
 // Every copy derived from the parameters: the arranged weights and the FP16
 // grid.
 npm_status refresh_derived(npm_handle* h, cudaStream_t st) {
-    npm_status s = arrange_all_weights(h, st);
+    npm::UpdateEnd end{};
+    end.version = version_word(h);
+    npm_status s = arrange_all_weights(h, end, st);
     if (s != NPM_OK) return s;
     if (h->grid_h) NPM_CUDA(npm::launch_to_half(h->ng, inf_params(h), h->grid_h, st), "grid fp16 copy");
     return NPM_OK;
@@ -637,9 +639,8 @@ static npm_status backward_impl(npm_handle* h, int64_t n, const float* pos, cons
                                 const float* dlogv, int64_t ld, cudaStream_t st) {
     if (!npm::tc_can_train(h) && h->train_smem > 227 * 1024)
         return fail(NPM_ERR_UNSUPPORTED, "training activations do not fit in shared memory");
-    double* loss = loss_acc(h);
-    NPM_CUDA(cudaMemsetAsync(loss, 0, sizeof(double), st), "clear loss");
     if (n == 0) return NPM_OK;
+    double* loss = dlogv ? nullptr : loss_acc(h);  // a training step's
     if (npm::tc_can_train(h)) {
         NPM_CUDA(npm::tc_train(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st), "train launch");
         return NPM_OK;
@@ -650,16 +651,24 @@ static npm_status backward_impl(npm_handle* h, int64_t n, const float* pos, cons
     return NPM_OK;
 }
 
-static npm_status adam_impl(npm_handle* h, const double* loss, cudaStream_t st) {
+// loss: whether a training step's loss is checked and cleared (and copied to
+// loss_out).
+static npm_status adam_impl(npm_handle* h, bool loss, float* loss_out, cudaStream_t st) {
     h->step += 1;
     int* status = reinterpret_cast<int*>(h->scalars + 8);
     const int64_t sh = 2 * (int64_t)h->dc.grid_shift;
     NPM_CUDA(npm::launch_adam(adam_count(h), h->params - sh, h->grads - sh, h->adam_m - sh, h->adam_v - sh,
-                              h->cfg.lr, h->cfg.beta1, h->cfg.beta2, h->cfg.eps, step_dev(h), loss, status,
+                              h->cfg.lr, h->cfg.beta1, h->cfg.beta2, h->cfg.eps, step_dev(h),
+                              loss ? loss_acc(h) : nullptr, status,
                               h->grid_h ? h->grid_h - sh : nullptr, h->grid_h ? sh + h->ng : 0,
                               h->ema ? h->ema - sh : nullptr, h->ema_decay, st),
              "adam launch");
-    return arrange_all_weights(h, st);
+    npm::UpdateEnd end{};
+    end.version = version_word(h);
+    end.steps = step_dev(h);
+    if (loss) end.loss_acc = loss_acc(h);
+    end.loss_out = loss_out;
+    return arrange_all_weights(h, end, st);
 }
 
 npm_status npm_train_step(npm_handle* h, int64_t n, const float* pos, const float* aux,
@@ -674,9 +683,7 @@ npm_status npm_train_step(npm_handle* h, int64_t n, const float* pos, const floa
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = backward_impl(h, n, pos, aux, dir, radiance, sample_pdf, nullptr, ld, st)) != NPM_OK)
         return s;
-    if ((s = adam_impl(h, loss_acc(h), st)) != NPM_OK) return s;
-    if (loss_out) NPM_CUDA(npm::launch_copy_loss(loss_acc(h), loss_out, st), "copy loss");
-    return NPM_OK;
+    return adam_impl(h, true, loss_out, st);
 }
 
 npm_status npm_backward(npm_handle* h, int64_t n, const float* pos, const float* aux,
@@ -694,7 +701,7 @@ npm_status npm_backward(npm_handle* h, int64_t n, const float* pos, const float*
 npm_status npm_adam_step(npm_handle* h, void* stream) {
     npm::CallRange range("npm_adam_step");
     if (!h) return fail(NPM_ERR_INVALID_ARG, "handle is NULL");
-    return adam_impl(h, nullptr, (cudaStream_t)stream);
+    return adam_impl(h, false, nullptr, (cudaStream_t)stream);
 }
 
 npm_status npm_grid_indices(npm_handle* h, int64_t n, const float* pos, int64_t ld, int32_t* out,

@@ -386,6 +386,23 @@ __device__ __forceinline__ float inv_minus_coth(float k) {
     return 1.0f / k - 1.0f - 2.0f / expm1f(2.0f * k);
 }
 
+// What the last kernel of a parameter update does besides arranging the
+// weights, by one thread: counts the change of the parameters, and after an
+// Adam step counts that, hands out the loss and clears its accumulator for
+// the next step. NULL fields are left out.
+struct UpdateEnd {
+    int* version;
+    int* steps;
+    double* loss_acc;
+    float* loss_out;
+};
+__device__ __forceinline__ void end_update(const UpdateEnd& e) {
+    if (e.version) *e.version += 1;
+    if (e.steps) *e.steps += 1;
+    if (e.loss_out) *e.loss_out = (float)*e.loss_acc;
+    if (e.loss_acc) *e.loss_acc = 0.0;
+}
+
 // Arrange layer l of the MLP weights (row-major [out][in] per layer, packed)
 // into the padded blob W^T [in][np_fwd] of the CUDA-core kernels; thread tid
 // of nt.

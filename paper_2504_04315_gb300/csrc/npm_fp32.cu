@@ -891,20 +891,21 @@ __global__ void __launch_bounds__(kTrainGroups* kTrainT, 1)
     // The loss: one atomic a warp.
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(kFull, lacc, o);
-    if ((t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
+    if (loss && (t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
 }
 
 // ------------------------------------------------------- utility kernels
 
 // blockIdx.y: layer.
 __global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const float* __restrict__ mlp,
-                                  float* __restrict__ wfwd) {
+                                  float* __restrict__ wfwd, UpdateEnd end) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) end_update(end);
     arrange_layer(cfg, blockIdx.y, mlp, wfwd, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // Dense Adam with bias correction (Kingma and Ba) at step t = *steps + 1,
 // c1 = 1 - b1^t, c2 = 1 - b2^t; the step count lives in device memory so that
-// captured graphs replay correctly (k_step_done advances it afterwards).
+// captured graphs replay correctly (end_update advances it afterwards).
 // Skips the update when *loss is not finite and flags it. Clears the
 // gradient. Optionally refreshes an FP16 copy of the first n_half parameters
 // (the grid). With ema set, also the exponential moving average
@@ -915,7 +916,7 @@ __global__ void k_adam(int64_t n4, float4* __restrict__ p, float4* __restrict__ 
                        float eps, const int* __restrict__ steps, const double* __restrict__ loss,
                        int* __restrict__ status, __half2* __restrict__ half_copy, int64_t n_half,
                        float4* __restrict__ ema, float ema_decay) {
-    const bool skip = loss != nullptr && !isfinite(*loss);
+    const bool skip = loss != nullptr && !isfinite((float)*loss);
     if (skip && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kStatusNumeric);
     const float t = (float)(*steps + 1);
     const float c1 = 1.0f - powf(b1, t), c2 = 1.0f - powf(b2, t);
@@ -981,10 +982,6 @@ __global__ void k_adam(int64_t n4, float4* __restrict__ p, float4* __restrict__ 
     }
 }
 
-__global__ void k_step_done(int* steps) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *steps += 1;
-}
-
 __global__ void k_grid_indices(DevCfg cfg, int64_t n, int64_t ld, const float* __restrict__ pos,
                                int32_t* __restrict__ out) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
@@ -1005,10 +1002,6 @@ __global__ void k_to_half(int64_t n, const float* __restrict__ src, __half* __re
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         dst[i] = __float2half_rn(src[i]);
-}
-
-__global__ void k_copy_loss(const double* __restrict__ acc, float* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *out = (float)*acc;
 }
 
 // ----------------------------------------------------------- launchers
@@ -1140,8 +1133,9 @@ cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t ml
     return cudaGetLastError();
 }
 
-cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, cudaStream_t st) {
-    k_arrange_weights<<<dim3(16, cfg.n_layers), 256, 0, st>>>(cfg, mlp, wfwd);
+cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, const UpdateEnd& end,
+                                   cudaStream_t st) {
+    k_arrange_weights<<<dim3(16, cfg.n_layers), 256, 0, st>>>(cfg, mlp, wfwd, end);
     return cudaGetLastError();
 }
 
@@ -1159,9 +1153,6 @@ cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float
                                  b2, eps, steps, loss, status,
                                  reinterpret_cast<__half2*>(half_copy), n_half,
                                  reinterpret_cast<float4*>(ema), ema_decay);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_step_done<<<1, 32, 0, st>>>(steps);
     return cudaGetLastError();
 }
 
@@ -1177,11 +1168,6 @@ cudaError_t launch_to_half(int64_t n, const float* src, __half* dst, cudaStream_
     int grid = (int)((n + 255) / 256);
     if (grid > 4096) grid = 4096;
     k_to_half<<<grid, 256, 0, st>>>(n, src, dst);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_copy_loss(const double* acc, float* out, cudaStream_t st) {
-    k_copy_loss<<<1, 32, 0, st>>>(acc, out);
     return cudaGetLastError();
 }
 

@@ -26,7 +26,8 @@ struct npm_handle {
     float* adam_v = nullptr;
     float* wfwd = nullptr;     // padded W^T blob of the CUDA-core kernels
     __half* grid_h = nullptr;  // FP16 grid copy (BF16 precision)
-    // [0] loss accumulator (64 bits), [8] status word, [16] Adam steps, [24] version of
+    // [0] loss accumulator (64 bits; zero between training steps), [8] status
+    // word, [16] Adam steps, [24] version of
     // the parameters (both counted on the device, so that replayed graphs
     // count too)
     float* scalars = nullptr;
@@ -86,12 +87,13 @@ npm_status set_error(npm_status s, const char* msg);
 npm_status tc_create(npm_handle* h);
 void tc_destroy(npm_handle* h);
 // Weights arranged for the MMAs; with cuda_cores also h->wfwd.
-cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st);
+cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, const UpdateEnd& end, cudaStream_t st);
 // pdl: the small networks' kernel may be launched as a programmatic
 // dependent of the stream's previous kernel, which must then not write the
 // model's weights or grid (other kernels launch as usual).
 cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStream_t st, bool pdl = false);
-// Training step kernels on tensor cores (split BF16 operands).
+// Training step kernels on tensor cores (split BF16 operands); loss: 64-bit
+// accumulator or NULL.
 bool tc_can_train(npm_handle* h);
 cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux, const float* dir,
                      const float* rad, const float* spdf, const float* dlogv, double* loss, cudaStream_t st);

@@ -83,10 +83,11 @@ cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t ml
                               int64_t ld, const float* pos, const float* aux, const float* dir, const float* rad,
                               const float* spdf, const float* dlogv, float* grad, double* loss, cudaStream_t st);
 
-cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, cudaStream_t st);
+cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, const UpdateEnd& end,
+                                   cudaStream_t st);
 
-// Adam at step *steps + 1 (device counter, advanced on the stream after the
-// update). The buffers are those of the parameters and what mirrors them from
+// Adam at step *steps + 1 (device counter, advanced by the arrangement of the
+// weights that follows). The buffers are those of the parameters and what mirrors them from
 // the 16-byte boundary before their first value on (n a multiple of 4).
 // ema (or NULL): moving average updated with ema_decay; the FP16 copy is then
 // taken from it.
@@ -99,7 +100,5 @@ cudaError_t launch_grid_indices(const DevCfg& cfg, int64_t n, int64_t ld, const 
                                 int32_t* out, cudaStream_t st);
 
 cudaError_t launch_to_half(int64_t n, const float* src, __half* dst, cudaStream_t st);
-
-cudaError_t launch_copy_loss(const double* acc, float* out, cudaStream_t st);
 
 }  // namespace npm

@@ -221,13 +221,12 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
 
 // Master FP32 weights (packed [out][in] per layer) -> 16-bit operand parts in
 // the UMMA K-major layout, zero padded to Np x Kp per layer; with wfwd also
-// the CUDA-core kernels' padded copy; with version counts a change of the
-// parameters. blockIdx.y: layer (one pass of load latency for all layers
+// the CUDA-core kernels' padded copy. blockIdx.y: layer (one pass of load latency for all layers
 // instead of one each).
 __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __restrict__ mlp,
-                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, int* __restrict__ version) {
+                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, UpdateEnd end) {
     const int l = blockIdx.y;
-    if (version && l == 0 && blockIdx.x == 0 && threadIdx.x == 0) *version += 1;
+    if (l == 0 && blockIdx.x == 0 && threadIdx.x == 0) end_update(end);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, tid, nt);
     const TcLayer& ly = tc.layer[l];
@@ -828,7 +827,7 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
     // Loss: one atomic per warp.
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
-    if ((t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
+    if (loss && (t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
     // Weight gradients: lane o of layer l's TMEM region holds dW_l[o][*].
     tc_fence_before();
     __syncthreads();
@@ -1087,13 +1086,12 @@ void tc_destroy(npm_handle* h) {
     h->tc = nullptr;
 }
 
-cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) {
+cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, const UpdateEnd& end, cudaStream_t st) {
     TcState* s = h->tc;
+    // The launch that ends the update comes last.
     const dim3 grid(16, h->dc.n_layers);
-    k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr,
-                                       version_word(h));
     if (s->wblob_train)
-        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, UpdateEnd{});
     if (h->ema) {
         if (!s->wblob_inf) {
             const size_t bytes = (size_t)s->cfg.wparts * s->cfg.w_bytes;
@@ -1101,8 +1099,9 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, cudaStream_t st) 
             if (e != cudaSuccess) return e;
             cudaMemsetAsync(s->wblob_inf, 0, bytes, st);
         }
-        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, nullptr);
+        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, UpdateEnd{});
     }
+    k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr, end);
     return cudaGetLastError();
 }
 
