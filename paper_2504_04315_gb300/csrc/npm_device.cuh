@@ -169,6 +169,31 @@ __device__ __forceinline__ void gather_pair2(const float* gl, uint32_t level_off
         vb = __ldg(reinterpret_cast<const float2*>(gl) + b);
     }
 }
+// Atomic adds to global memory without a return value, one operation for 1, 2
+// or 4 consecutive values (4-, 8- or 16-byte aligned). The L2 is limited by
+// operations per slice, not bytes, and a reduction, unlike atomicAdd on a
+// vector, leaves no result for a warp to wait on.
+__device__ __forceinline__ void red_add(float* p, float a) {
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory");
+}
+__device__ __forceinline__ void red_add(float* p, float a, float b) {
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ void red_add(float* p, float a, float b, float c, float d) {
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+// Four values at an 8-byte aligned address: one operation where it is 16-byte
+// aligned (wide, the same for all threads), else two.
+__device__ __forceinline__ void red_add4(float* p, bool wide, float a, float b, float c, float d) {
+    if (wide) {
+        red_add(p, a, b, c, d);
+    } else {
+        red_add(p, a, b);
+        red_add(p + 2, c, d);
+    }
+}
+
 // Grid-gradient scatter of two x-adjacent corners (entries a, b of a level
 // whose first entry lies level_off entries past a 16-byte boundary, 2 features
 // each; gl points at the level): when the two entries form one 16-byte aligned pair, one 4-wide atomic add
@@ -177,12 +202,11 @@ __device__ __forceinline__ void scatter_pair2(float* gl, uint32_t level_off, uin
                                               float wb, float d0, float d1) {
     const uint32_t lo = a < b ? a : b;
     if ((a > b ? a - b : b - a) == 1u && ((level_off + lo) & 1u) == 0u) {
-        const float4 v = a < b ? make_float4(wa * d0, wa * d1, wb * d0, wb * d1)
-                               : make_float4(wb * d0, wb * d1, wa * d0, wa * d1);
-        atomicAdd(reinterpret_cast<float4*>(gl + (size_t)lo * 2), v);
+        const float wl = a < b ? wa : wb, wh = a < b ? wb : wa;
+        red_add(gl + (size_t)lo * 2, wl * d0, wl * d1, wh * d0, wh * d1);
     } else {
-        atomicAdd(reinterpret_cast<float2*>(gl + (size_t)a * 2), make_float2(wa * d0, wa * d1));
-        atomicAdd(reinterpret_cast<float2*>(gl + (size_t)b * 2), make_float2(wb * d0, wb * d1));
+        red_add(gl + (size_t)a * 2, wa * d0, wa * d1);
+        red_add(gl + (size_t)b * 2, wb * d0, wb * d1);
     }
 }
 

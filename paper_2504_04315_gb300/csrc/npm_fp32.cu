@@ -689,6 +689,7 @@ __device__ __forceinline__ void grad_epilogue(int t, const DevCfg& cfg, float* a
 // Thread t of 256 owns 4 x 4 blocks.
 __device__ __forceinline__ void weight_grad(int t, const float* dl, int DS, const float* h, int HS, int N, int K,
                                             float* __restrict__ gW) {
+    const bool wide = (reinterpret_cast<uintptr_t>(gW) & 15u) == 0;
     for (int n0 = (t >> 4) * 4; n0 < N; n0 += 64)
         for (int k0 = (t & 15) * 4; k0 < K; k0 += 64) {
             float2 acc[4][2];
@@ -710,9 +711,7 @@ __device__ __forceinline__ void weight_grad(int t, const float* dl, int DS, cons
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 // (8-byte aligned: the gradient shares the tables' shift)
-                float2* dst = reinterpret_cast<float2*>(gW + (size_t)(n0 + r) * K + k0);
-                atomicAdd(dst, acc[r][0]);
-                atomicAdd(dst + 1, acc[r][1]);
+                red_add4(gW + (size_t)(n0 + r) * K + k0, wide, acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
             }
         }
 }
@@ -794,10 +793,9 @@ __device__ __forceinline__ void grid_scatter(int t, const DevCfg& cfg, const flo
             const float w = ws[c];
             float* e = gl + (size_t)idx[c] * F;
             if (F == 4) {
-                atomicAdd(reinterpret_cast<float4*>(e),
-                          make_float4(w * dg[0], w * dg[1], w * dg[2], w * dg[3]));
+                red_add(e, w * dg[0], w * dg[1], w * dg[2], w * dg[3]);
             } else {
-                for (int f = 0; f < F; ++f) atomicAdd(e + f, w * dg[f]);
+                for (int f = 0; f < F; ++f) red_add(e + f, w * dg[f]);
             }
         }
     }

@@ -28,25 +28,27 @@ using namespace tc;
 
 namespace {
 
+// Training operand tiles (128 samples x columns, BF16) are stored in planes of
+// 8 columns: 2048 bytes a plane, 16 bytes a row. Core matrices (8 rows x 16
+// bytes) then lie 128 bytes apart along the rows and 2048 along the columns
+// in every tile, whatever its width, so that a tile and the residual tile
+// behind it are one operand of twice the columns.
+constexpr uint32_t kPlane = kTile * 16;
+__device__ __forceinline__ uint32_t plane_off(int row, int col) {
+    return (uint32_t)(col >> 3) * kPlane + (uint32_t)row * 16u + (uint32_t)(col & 7) * 2u;
+}
+
 // --------------------------------------------------------------- encode
 
-// Thread t writes row t of A (BF16, kp columns) for its query.
-// F2: the grid has 2 features per level (compile-time), so two levels' 16
-// corner loads can be in flight before blending; other grids take the
-// generic per-level path (fewer registers).
-// Levels [lbeg, lend) are encoded; tail: also the product-mode inputs and
-// the zero padding. lo: byte offset of the residual tile (0 without split).
-// pad_all: write zeros up to kp; otherwise only up to the next 8-column
-// chunk (the caller keeps the all-zero chunks beyond it written).
-template <bool F2, typename GT>
-__device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict__ grid_h,
-                                          int64_t j, bool valid, int64_t ld,
-                                          const float* __restrict__ pos,
-                                          const float* __restrict__ aux, uint8_t* sA, int row,
-                                          uint32_t lo, bool pad_all, int lbeg, int lend, bool tail) {
+// The inputs of one training sample from the FP32 table: row `row` of the
+// tile at sA, residuals lo bytes further. F2: 2 features per level
+// (compile-time). Levels [lbeg, lend) are encoded; tail: also the
+// product-mode inputs and the zero padding to kp columns.
+template <bool F2>
+__device__ __forceinline__ void tc_encode(const TcCfg& tc, const float* __restrict__ grid32, int64_t j, bool valid,
+                                          int64_t ld, const float* __restrict__ pos, const float* __restrict__ aux,
+                                          uint8_t* sA, int row, uint32_t lo, int lbeg, int lend, bool tail) {
     const DevCfg& cfg = tc.base;
-    const int kp = tc.layer[0].Kp;
-    const bool f16 = tc.f16 != 0;
     float x = 0.0f, y = 0.0f, z = 0.0f;
     if (valid) {
         x = pos[j];
@@ -54,144 +56,44 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
         z = pos[2 * ld + j];
     }
     const int F = F2 ? 2 : cfg.feat;
-    int l = lbeg;
-    if (!F2 && (F == 4 || F == 8) && lbeg == 0 && lend == 1 && tail && cfg.mode != NPM_PRODUCT) {
-        // A single level of 4 or 8 features fills the first 8-column chunk
-        // (features, then zeros): one 16-byte store (and one for residuals);
-        // with pad_all, zero chunks follow up to kp.
-        const Cell cl = make_cell(x, y, z, cfg.level_res[0]);
-        uint32_t idx[8];
-        corner_idx8(cfg, 0, cl, idx);
-        float ws[8];
-        corner_w8(cl, ws);
-        float e[8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (h == 0 || F == 8) {
-                decltype(load_raw4(grid_h, 0u, F, 0)) raw[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) raw[c] = load_raw4(grid_h, idx[c], F, h);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float4 v = widen4(raw[c]);
-                    acc.x = fmaf(ws[c], v.x, acc.x);
-                    acc.y = fmaf(ws[c], v.y, acc.y);
-                    acc.z = fmaf(ws[c], v.z, acc.z);
-                    acc.w = fmaf(ws[c], v.w, acc.w);
-                }
-            }
-            e[4 * h] = acc.x;
-            e[4 * h + 1] = acc.y;
-            e[4 * h + 2] = acc.z;
-            e[4 * h + 3] = acc.w;
-        }
-        uint32_t hw[4], lw[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (f16) {
-                hw[i] = pack_f16_sat(e[2 * i], e[2 * i + 1]);
-                lw[i] = lo ? f16_residual(hw[i], e[2 * i], e[2 * i + 1]) : 0u;
-            } else {
-                __nv_bfloat162 hb = __floats2bfloat162_rn(e[2 * i], e[2 * i + 1]);
-                hw[i] = *reinterpret_cast<uint32_t*>(&hb);
-                const float2 hf = __bfloat1622float2(hb);
-                lw[i] = pack_bf16(e[2 * i] - hf.x, e[2 * i + 1] - hf.y);
-            }
-        }
-        const uint32_t off = tile_off(row, 0, kp);
-        *reinterpret_cast<uint4*>(sA + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        if (lo) *reinterpret_cast<uint4*>(sA + lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-        if (pad_all)
-            for (int c = 8; c < kp; c += 8) {
-                const uint32_t oz = tile_off(row, c, kp);
-                *reinterpret_cast<uint4*>(sA + oz) = make_uint4(0u, 0u, 0u, 0u);
-                if (lo) *reinterpret_cast<uint4*>(sA + lo + oz) = make_uint4(0u, 0u, 0u, 0u);
-            }
-        return;
-    }
-    if constexpr (F2) {
-        for (; l + 1 < lend; l += 2) {
-            const Cell c0 = make_cell(x, y, z, cfg.level_res[l]);
-            const Cell c1 = make_cell(x, y, z, cfg.level_res[l + 1]);
-            const GT* g0 = grid_h + (size_t)cfg.level_off[l] * 2;
-            const GT* g1 = grid_h + (size_t)cfg.level_off[l + 1] * 2;
-            float2 v0[8], v1[8];
-#pragma unroll
-            for (int c = 0; c < 8; c += 2) {
-                gather_pair2(g0, cfg.level_off[l] + cfg.grid_shift, corner_idx1(cfg, l, c0, c), corner_idx1(cfg, l, c0, c + 1),
-                             v0[c], v0[c + 1]);
-                gather_pair2(g1, cfg.level_off[l + 1] + cfg.grid_shift, corner_idx1(cfg, l + 1, c1, c),
-                             corner_idx1(cfg, l + 1, c1, c + 1), v1[c], v1[c + 1]);
-            }
-            float w0s[8], w1s[8];
-            corner_w8(c0, w0s);
-            corner_w8(c1, w1s);
-            float a0 = 0.0f, a1 = 0.0f, b0 = 0.0f, b1 = 0.0f;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float w0 = w0s[c], w1 = w1s[c];
-                a0 = fmaf(w0, v0[c].x, a0);
-                a1 = fmaf(w0, v0[c].y, a1);
-                b0 = fmaf(w1, v1[c].x, b0);
-                b1 = fmaf(w1, v1[c].y, b1);
-            }
-            store_pair(sA, tile_off(row, 2 * l, kp), a0, a1, lo, f16);
-            store_pair(sA, tile_off(row, 2 * l + 2, kp), b0, b1, lo, f16);
-        }
-    }
-    for (; l < lend; ++l) {
+    for (int l = lbeg; l < lend; ++l) {
         const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
-        const GT* gl = grid_h + (size_t)cfg.level_off[l] * F;
-        if (F2) {  // F = 2 (F2 kernels serve exactly the 2-feature grids)
-            float s0 = 0.0f, s1 = 0.0f;
-            uint32_t idx[8];
-            corner_idx8(cfg, l, cl, idx);
-            float2 v[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) v[c] = load_feat2(gl, idx[c]);
-            float ws[8];
-            corner_w8(cl, ws);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float w = ws[c];
-                s0 = fmaf(w, v[c].x, s0);
-                s1 = fmaf(w, v[c].y, s1);
-            }
-            store_pair(sA, tile_off(row, 2 * l, kp), s0, s1, lo, f16);
-        } else if (F == 4 || F == 8) {
+        if (F2) {
+            Level2<float> v;
+            v.load_table(cfg, grid32, l, cl);
+            const float2 a = v.blend(cl);
+            store_pair(sA, plane_off(row, 2 * l), a.x, a.y, lo);
+            continue;
+        }
+        const float* gl = grid32 + (size_t)cfg.level_off[l] * F;
+        uint32_t idx[8];
+        corner_idx8(cfg, l, cl, idx);
+        if (F == 4 || F == 8) {
             // One vector load per corner and group of 4 features.
-            uint32_t idx[8];
-            corner_idx8(cfg, l, cl, idx);
-            float ws[8];
-            corner_w8(cl, ws);
             for (int h = 0; h < (F >> 2); ++h) {
-                decltype(load_raw4(gl, 0u, F, 0)) raw[8];
+                float4 raw[8];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) raw[c] = load_raw4(gl, idx[c], F, h);
+                float ws[8];
+                corner_w8(cl, ws);
                 float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const float w = ws[c];
-                    const float4 v = widen4(raw[c]);
-                    acc.x = fmaf(w, v.x, acc.x);
-                    acc.y = fmaf(w, v.y, acc.y);
-                    acc.z = fmaf(w, v.z, acc.z);
-                    acc.w = fmaf(w, v.w, acc.w);
+                    acc.x = fmaf(ws[c], raw[c].x, acc.x);
+                    acc.y = fmaf(ws[c], raw[c].y, acc.y);
+                    acc.z = fmaf(ws[c], raw[c].z, acc.z);
+                    acc.w = fmaf(ws[c], raw[c].w, acc.w);
                 }
                 const int k = l * F + 4 * h;
-                store_pair(sA, tile_off(row, k, kp), acc.x, acc.y, lo, f16);
-                store_pair(sA, tile_off(row, k + 2, kp), acc.z, acc.w, lo, f16);
+                store_pair(sA, plane_off(row, k), acc.x, acc.y, lo);
+                store_pair(sA, plane_off(row, k + 2), acc.z, acc.w, lo);
             }
-        } else {
-            // F = 1
-            float s = 0.0f;
-            uint32_t idx[8];
-            float ws[8];
-            corners8(cfg, l, cl, idx, ws);
+        } else {  // F = 1
+            float ws[8], s = 0.0f;
+            corner_w8(cl, ws);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) s = fmaf(ws[c], load_feat(gl + idx[c], 0), s);
-            store_one(sA, tile_off(row, l, kp), s, lo, f16);
+            for (int c = 0; c < 8; ++c) s = fmaf(ws[c], __ldg(gl + idx[c]), s);
+            store_one(sA, plane_off(row, l), s, lo);
         }
     }
     if (!tail) return;
@@ -212,11 +114,10 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const GT* __restrict_
         sh_band2(nn[0], nn[1], nn[2], e + 16);
         e[20] = r;
 #pragma unroll
-        for (int i = 0; i < 21; ++i) store_one(sA, tile_off(row, k + i, kp), e[i], lo, f16);
+        for (int i = 0; i < 21; ++i) store_one(sA, plane_off(row, k + i), e[i], lo);
         k += 21;
     }
-    const int kend = pad_all ? kp : min(kp, (k + 7) & ~7);
-    for (; k < kend; ++k) store_one(sA, tile_off(row, k, kp), 0.0f, lo);
+    for (; k < tc.layer[0].Kp; ++k) store_one(sA, plane_off(row, k), 0.0f, lo);
 }
 
 // Master FP32 weights (packed [out][in] per layer) -> 16-bit operand parts in
@@ -311,28 +212,84 @@ __global__ void __launch_bounds__(256) k_corner_blocks(const __grid_constant__ T
 
 // ----------------------------------------------------------- training
 
-// Training layout: per layer the input activation tile H_l (BF16, K-major,
-// 128 x Kp_l) at h_off, the delta tile D (BF16, K-major, 128 samples x
-// d_cols, the widest layer) at d_off; TMEM columns [0, c0) hold the forward / input-gradient
-// accumulator and [dw_col_l, dw_col_l + Kp_l) the weight gradient of
-// layer l, accumulated over all tiles of the CTA.
+// Training layout. A CTA holds G tile groups of 256 threads that share the
+// weights and the weight-gradient accumulators; each group walks its own
+// 128-sample tiles. A group's shared memory is one slot per layer, slot l with
+// the BF16 high parts of layer l's input (kPlane layout), and a last slot L:
+//   forward  : slot L holds the residuals of the current layer's input;
+//   loss     : the loss gradient, high parts and residuals, goes to slot L;
+//   backward : the gradient of layer l's input replaces that input in slot l,
+//              its residuals follow in slot l + 1, whose contents (the
+//              gradient of layer l's output) the finished MMAs have read.
+// So a gradient and its residuals are always adjacent, and where both fit 128
+// rows one MMA per K step forms D_hi^T H and D_lo^T H in lanes o and Np + o of
+// the layer's accumulator. (The MMA reads 128 rows: what lies behind the
+// tiles, at most 32 KB from a slot's start, ends in lanes never read.)
+// Tensor memory: every layer's weight gradient (Kp_l columns, all tiles of the
+// CTA), then per group an accumulator and the parked encoder gradient.
 struct TcTrain {
-    uint32_t h_off[NPM_MAX_LAYERS];
+    uint32_t slot[NPM_MAX_LAYERS + 1];  // byte offsets within a group's tiles
     uint32_t dw_col[NPM_MAX_LAYERS];
     uint32_t idesc_dw[NPM_MAX_LAYERS];  // A MN-major, B MN-major, N = Kp_l
     uint32_t idesc_dx[NPM_MAX_LAYERS];  // A K-major,  B MN-major, N = Kp_l
-    uint32_t d_off, x_off, bar_off, smem, tmem_cols;
-    uint32_t d_cols;                    // columns of the delta tile
+    uint32_t g_bytes;                   // a group's tiles
+    uint32_t x_off, w_off, bar_off, smem;
+    uint32_t acc_col, acc_cols, park_col, tmem_cols;
     int64_t woff[NPM_MAX_LAYERS];       // packed offset of W_l in the MLP region
-    int split;                          // BF16 residual operands (three MMAs per K step)
-    uint32_t hlo_off;                   // residual of the current layer's input tile
-    uint32_t dlo_off;                   // residual of the delta tile
+    int groups;
+    int park;                           // encoder gradients wait in tensor memory (2-feature grids)
 };
 
-// Training runs two threads per sample row: thread t serves row t & 127 and
-// half t >> 7 of the row's work (grid levels, epilogue column chunks,
-// lobes). Warps w and w + 4 read the same TMEM lane quarter.
+// Training runs two threads per sample row: thread t of a group serves row
+// t & 127 and half t >> 7 of the row's work (grid levels, epilogue column
+// chunks, lobes). Warps w and w + 4 read the same TMEM lane quarter.
 constexpr int kTrainThreads = 2 * kTile;
+
+// Named barrier of training group g (id 0 is the CTA's), and its form that
+// also ORs a predicate.
+__device__ __forceinline__ void train_sync(int g) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kTrainThreads) : "memory");
+}
+__device__ __forceinline__ bool train_sync_or(int g, bool p) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred q, o;\n\t"
+        "setp.ne.u32 q, %3, 0;\n\t"
+        "bar.red.or.pred o, %1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, o;\n\t}\n"
+        : "=r"(r)
+        : "r"(1 + g), "r"(kTrainThreads), "r"((uint32_t)p)
+        : "memory");
+    return r != 0;
+}
+
+// Turns at the shared weight-gradient accumulators: MMAs of two threads are
+// not ordered by themselves, so a group's thread takes the turn, waits for the
+// completion of the batch before (its commit's phase of `bar`), issues and
+// commits its own, and passes the turn on without waiting for it.
+struct DwTurn {
+    uint32_t taken;    // 0 or 1
+    uint32_t batches;  // batches issued so far
+};
+__device__ __forceinline__ bool take_turn(DwTurn* turn, uint32_t bar) {
+    const long long t0 = clock64();
+    while (atomicCAS(&turn->taken, 0u, 1u) != 0u) {
+        if (clock64() - t0 > (1ll << 32)) return false;
+        __nanosleep(20);
+    }
+    __threadfence_block();
+    const uint32_t b = *reinterpret_cast<volatile uint32_t*>(&turn->batches);
+    if (b > 0 && !mbar_wait_bounded(bar, (b - 1) & 1u)) {
+        atomicExch(&turn->taken, 0u);
+        return false;
+    }
+    return true;
+}
+__device__ __forceinline__ void pass_turn(DwTurn* turn) {
+    *reinterpret_cast<volatile uint32_t*>(&turn->batches) += 1u;
+    __threadfence_block();
+    atomicExch(&turn->taken, 0u);
+}
 
 // Half h of the lobes of one sample, lobes i = h KMAX/2 + q. Pass 1 forms
 // each lobe's terms and the half's partial log-sum-exps of the softmax
@@ -418,10 +375,10 @@ __device__ __forceinline__ float lse_combine(float ma, float sa, float mb, float
     return m + __logf(t);
 }
 
-// NC (a multiple of 8) values as BF16 at row t, columns c0 .. c0+NC of a
-// K-major tile, with their residuals lo_off bytes on when lo_off != 0.
+// NC (a multiple of 8) values as BF16 at row t, columns c0 .. c0+NC of a tile
+// in planes, with their residuals lo_off bytes on.
 template <int NC>
-__device__ __forceinline__ void store_cols(uint8_t* base, int t, int c0, int kp, const float* v, uint32_t lo_off) {
+__device__ __forceinline__ void store_cols(uint8_t* base, int t, int c0, const float* v, uint32_t lo_off) {
 #pragma unroll
     for (int c = 0; c < NC; c += 8) {
         uint32_t hw[4], lw[4];
@@ -432,9 +389,9 @@ __device__ __forceinline__ void store_cols(uint8_t* base, int t, int c0, int kp,
             const float2 hf = __bfloat1622float2(hb);
             lw[i] = pack_bf16(v[c + 2 * i] - hf.x, v[c + 2 * i + 1] - hf.y);
         }
-        const uint32_t off = tile_off(t, c0 + c, kp);
+        const uint32_t off = plane_off(t, c0 + c);
         *reinterpret_cast<uint4*>(base + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        if (lo_off) *reinterpret_cast<uint4*>(base + lo_off + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+        *reinterpret_cast<uint4*>(base + lo_off + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
 }
 
@@ -457,7 +414,7 @@ __device__ __forceinline__ void scatter_levels(const DevCfg& cfg, float* __restr
                 const float wc = ws[c];
                 float* e = gl + (size_t)idx[c] * FF;
                 if constexpr (FF == 1) {
-                    atomicAdd(e, wc * dg[q]);
+                    red_add(e, wc * dg[q]);
                 } else if constexpr (FF == 2) {
                     if (c & 1) continue;  // corners c, c + 1 (along x) together
                     scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1], dg[2 * q],
@@ -465,9 +422,8 @@ __device__ __forceinline__ void scatter_levels(const DevCfg& cfg, float* __restr
                 } else {
 #pragma unroll
                     for (int f = 0; f < FF; f += 4)
-                        atomicAdd(reinterpret_cast<float4*>(e + f),
-                                  make_float4(wc * dg[FF * q + f], wc * dg[FF * q + f + 1], wc * dg[FF * q + f + 2],
-                                              wc * dg[FF * q + f + 3]));
+                        red_add(e + f, wc * dg[FF * q + f], wc * dg[FF * q + f + 1], wc * dg[FF * q + f + 2],
+                                wc * dg[FF * q + f + 3]);
                 }
             }
         }
@@ -509,15 +465,22 @@ __global__ void __launch_bounds__(256) k_train_encode(const __grid_constant__ De
     }
 }
 
-// The small four-lobe instance (single-level grids) is compiled for three
-// CTAs per SM (80 registers without spills; its delta tiles are only as
-// wide as its layers, 53 KB a CTA): its tile chain of MMA round trips is
-// latency-bound, and the other CTAs overlap it. (Four CTAs at 64 registers
-// measured slower.)
-__host__ __device__ constexpr int train_ctas_per_sm(int kmax, bool f2) { return (kmax == 4 && !f2) ? 3 : 1; }
+// CTAs per SM of the one-group instances: three for the small four-lobe one
+// (single-level grids; 80 registers without spills, 53 KB a CTA), whose tile
+// chain of MMA round trips is latency-bound and overlapped by the other CTAs.
+// (Four CTAs at 64 registers measured slower.) The multi-level networks
+// overlap two tiles in one CTA instead: two groups share the weights.
+// Measured against one tile of 256 threads a CTA (GB300): product-mode
+// network, 2^19 samples, kernel 610 -> 451 us, with vector reductions in the
+// place of atomics on vectors (which return their result; 972 us with them)
+// and the flush of the weight gradients below; small network, 2^18 samples,
+// 100 -> 82 us (165 us with one scalar atomic per weight and share).
+__host__ __device__ constexpr int train_ctas_per_sm(int kmax, bool f2, int g) {
+    return g == 1 && kmax == 4 && !f2 ? 3 : 1;
+}
 
-template <int KMAX, bool F2>
-__global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_train_tc(
+template <int KMAX, bool F2, int G>
+__global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, G)) k_train_tc(
     const __grid_constant__ TcCfg tc, const __grid_constant__ TcTrain tt, const float* __restrict__ grid32,
     const uint8_t* __restrict__ wblob, int64_t n, int64_t ld, const float* __restrict__ pos,
     const float* __restrict__ aux, const float* __restrict__ dir, const float* __restrict__ rad,
@@ -525,66 +488,75 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
     int64_t mlp_off, double* __restrict__ loss, int* __restrict__ status, const float* __restrict__ enc) {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int KH = KMAX / 2;
-    uint8_t* sW = smem;
-    uint8_t* sD = smem + tt.d_off;
-    float4* xch = reinterpret_cast<float4*>(smem + tt.x_off);  // [2][kTile] partial log-sum-exps
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + tt.bar_off);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
-    const int t = threadIdx.x, warp = t >> 5;
-    const int row = t & (kTile - 1), half = t >> 7;
-    const uint32_t bar_mma = smem_u32(&bars[0]), bar_w = smem_u32(&bars[1]);
+    const int g = G > 1 ? (int)(threadIdx.x >> 8) : 0;
+    const int t = G > 1 ? (int)(threadIdx.x & 255) : (int)threadIdx.x;
+    const int warp = t >> 5, row = t & (kTile - 1), half = t >> 7;
+    uint8_t* tiles = smem + g * tt.g_bytes;
+    float4* xch = reinterpret_cast<float4*>(smem + tt.x_off) + g * 2 * kTile;  // [2][kTile] partial log-sum-exps
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + tt.bar_off);  // weights, weight gradients, MMAs of each group
+    DwTurn* turn = reinterpret_cast<DwTurn*>(bars + 2 + G);
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(turn + 1);
+    const uint32_t bar_w = smem_u32(&bars[0]), bar_dw = smem_u32(&bars[1]), bar_mma = smem_u32(&bars[2 + g]);
     const DevCfg& cfg = tc.base;
     const int L = cfg.n_layers;
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(tt.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (t == 0) {
-        mbar_init(bar_mma, 1);
-        mbar_init(bar_w, 1);
+    const uint32_t wbytes = 2u * tc.w_bytes;
+    if (threadIdx.x == 32) {
+        for (int i = 0; i < 2 + G; ++i) mbar_init(smem_u32(&bars[i]), 1);
+        turn->taken = turn->batches = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_w), "r"(wbytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         smem_u32(smem + tt.w_off)),
+                     "l"(wblob), "r"(wbytes), "r"(bar_w)
+                     : "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    const uint32_t wbytes = (tt.split ? 2u : 1u) * tc.w_bytes;
-    if (t == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_w), "r"(wbytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                         smem_u32(sW)),
-                     "l"(wblob), "r"(wbytes), "r"(bar_w)
-                     : "memory");
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    {
+        // The weight-gradient accumulators start at zero.
+        const uint32_t z[8] = {};
+        for (uint32_t c = 8u * (threadIdx.x >> 7); c < tt.acc_col; c += 8u * (kTrainThreads * G / 128)) tmem_st(tmem + lanes + c, z);
+        tmem_wait_st();
+        tc_fence_before();
     }
-    bool ok = !__syncthreads_or(warp == 0 && !mbar_wait_bounded(bar_w, 0));
+    bool ok = !__syncthreads_or(threadIdx.x < 32 && !mbar_wait_bounded(bar_w, 0));
+    tc_fence_after();
     uint32_t phase = 0;
-    const uint32_t sW_addr = smem_u32(sW), sD_addr = smem_u32(sD), base_addr = smem_u32(smem);
-    const uint32_t wlo = tc.w_bytes;                      // residual weights follow the high parts
-    const uint32_t hlo_addr = base_addr + tt.hlo_off, dlo_addr = base_addr + tt.dlo_off;
-    const uint32_t drg = tt.d_cols * 16u;  // bytes per 8-sample row group of the delta tile
-    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    bool issued = false;
+    const uint32_t acc = tmem + tt.acc_col + (uint32_t)g * tt.acc_cols;
+    const uint32_t park = tmem + tt.park_col + 32u * (uint32_t)g + 16u * (uint32_t)half + lanes;
+    const uint32_t sW_addr = smem_u32(smem + tt.w_off), tile_addr = smem_u32(tiles);
+    const uint32_t wlo = tc.w_bytes;  // residual weights follow the high parts
     // Grid levels of this half: [lv0, lv1); the second half also encodes the
     // product-mode inputs and the padding.
     const int nl0 = (cfg.n_levels + 1) / 2;
     const int lv0 = half ? nl0 : 0, lv1 = half ? cfg.n_levels : nl0;
     float lacc = 0.0f;
-    bool first = true;
     // Deferred grid scatter (2-feature grids): a tile's encoder gradient of
-    // this thread's eight levels (pdg, two columns per level, the next
-    // level's first) and the sample position wait for the next tile, whose
-    // eight MMA waits each issue one level's atomics: the L2 atomics then
+    // this thread's eight levels waits in tensor memory for the next tile,
+    // whose MMA waits each issue one level's atomics: the L2 atomics then
     // overlap the tensor-core work instead of following it.
-    float pdg[16];
     float px = 0.0f, py = 0.0f, pz = 0.0f;
-    bool pend = false;
+    bool pend = false, pvalid = false;
     int pq = 0;  // pending levels already issued
     auto scatter_next = [&]() {
         if (F2 && pend && pq < 8) {
+            uint32_t r[2];
+            __syncwarp();
+            tmem_ld2(park + 2u * (uint32_t)pq, r);
+            tmem_wait2(r);
             const int l = 8 * half + pq;
-            if (l < cfg.n_levels) {
+            if (pvalid && l < cfg.n_levels) {
                 const Cell cl = make_cell(px, py, pz, cfg.level_res[l]);
                 float* gl = grad + (size_t)cfg.level_off[l] * 2;
                 uint32_t idx[8];
@@ -592,44 +564,41 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
                 corners8(cfg, l, cl, idx, ws);
 #pragma unroll
                 for (int c = 0; c < 8; c += 2)
-                    scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1], pdg[0], pdg[1]);
+                    scatter_pair2(gl, cfg.level_off[l] + cfg.grid_shift, idx[c], idx[c + 1], ws[c], ws[c + 1],
+                                  __uint_as_float(r[0]), __uint_as_float(r[1]));
             }
-#pragma unroll
-            for (int i = 0; i < 14; ++i) pdg[i] = pdg[i + 2];
+            __syncwarp();
             ++pq;
         }
     };
-    const int64_t ntiles = (n + kTile - 1) / kTile;
-    // This half's grid features (two per level, at most 8 levels) of row
-    // `row` of tile tl from k_train_encode, loaded one tile ahead.
-    float2 ev[8];
-    auto load_enc = [&](int64_t tl) {
-        const int64_t jj = tl * kTile + row;
-        const bool v = tl < ntiles && jj < n;
-        const float* er = enc + (v ? jj : 0) * (int64_t)cfg.grid_feats;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            ev[q] = (v && lv0 + q < lv1) ? __ldg(reinterpret_cast<const float2*>(er + 2 * (lv0 + q)))
-                                         : make_float2(0.0f, 0.0f);
+    // Waits for this group's MMAs; a wait that gives up is made known to the
+    // group at its next barrier.
+    auto wait_mma = [&]() {
+        ok = __all_sync(0xffffffffu, ok && mbar_wait_bounded(bar_mma, phase));
+        phase ^= 1u;
+        tc_fence_after();
     };
-    if (F2 && enc) load_enc(blockIdx.x);
-    for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+    const int64_t ntiles = (n + kTile - 1) / kTile;
+    // (a wait that gave up ends the loop at the group's next barrier, for all)
+    for (int64_t tile = blockIdx.x + (int64_t)g * gridDim.x; tile < ntiles; tile += (int64_t)gridDim.x * G) {
         const int64_t j = tile * kTile + row;
         const bool valid = j < n;
+        uint8_t* rest = tiles + tt.slot[L];
         if (F2 && enc) {
-            // This half's grid features, then the product-mode inputs and
-            // the padding; the next tile's features are loaded meanwhile.
-            const int kp0 = tc.layer[0].Kp;
-            const uint32_t lo = tc.split ? tc.a_bytes : 0u;
+            // This half's grid features (k_train_encode), then the
+            // product-mode inputs and the padding.
+            const float* er = enc + (valid ? j : 0) * (int64_t)cfg.grid_feats;
+            float2 ev[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (lv0 + q < lv1) store_pair(smem + tt.h_off[0], tile_off(row, 2 * (lv0 + q), kp0), ev[q].x, ev[q].y, lo);
-            load_enc(tile + gridDim.x);
-            tc_encode<F2>(tc, grid32, j, valid, ld, pos, aux, smem + tt.h_off[0], row, lo, true, lv1, lv1,
-                          half == 1);
+                ev[q] = (valid && lv0 + q < lv1) ? __ldg(reinterpret_cast<const float2*>(er + 2 * (lv0 + q)))
+                                                 : make_float2(0.0f, 0.0f);
+            tc_encode<F2>(tc, grid32, j, valid, ld, pos, aux, tiles, row, tt.slot[L], lv1, lv1, half == 1);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (lv0 + q < lv1) store_pair(tiles, plane_off(row, 2 * (lv0 + q)), ev[q].x, ev[q].y, tt.slot[L]);
         } else {
-            tc_encode<F2>(tc, grid32, j, valid, ld, pos, aux, smem + tt.h_off[0], row, tc.split ? tc.a_bytes : 0u,
-                          true, lv0, lv1, half == 1);
+            tc_encode<F2>(tc, grid32, j, valid, ld, pos, aux, tiles, row, tt.slot[L], lv0, lv1, half == 1);
         }
         // The loss inputs of this row, loaded now so that their latency
         // passes during the forward layers' tensor-core round trips.
@@ -642,174 +611,198 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
         }
         fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        if (train_sync_or(g, !ok)) {
+            ok = false;
+            break;
+        }
         float raw[4 * KH];
         // Forward, keeping every layer's input tile.
-        for (int l = 0; l < L && ok; ++l) {
+        for (int l = 0; l < L; ++l) {
             const TcLayer& ly = tc.layer[l];
             if (t == 0) {
                 tc_fence_after();
-                // The descriptors of K step s are those of step 0 with the
-                // start address 256 bytes (16 units) further.
+                // K step s starts two planes (256 units of 16 bytes) further.
                 const uint32_t sbo = (uint32_t)(ly.Kp >> 3) * 128u;
-                const uint64_t ad0 = umma_desc(base_addr + tt.h_off[l], 128u, sbo);
+                const uint64_t ad0 = umma_desc(tile_addr + tt.slot[l], kPlane, 128u);
+                const uint64_t al0 = umma_desc(tile_addr + tt.slot[L], kPlane, 128u);
                 const uint64_t bd0 = umma_desc(sW_addr + ly.w_off, 128u, sbo);
                 const uint64_t bl0 = umma_desc(sW_addr + wlo + ly.w_off, 128u, sbo);
-                const uint64_t al0 = umma_desc(hlo_addr, 128u, sbo);
                 for (int s = 0; s < (ly.Kp >> 4); ++s) {
-                    const uint64_t o = (uint64_t)(16 * s);
-                    mma_bf16(tmem, ad0 + o, bd0 + o, ly.idesc, s > 0 ? 1u : 0u);
-                    if (tt.split) {
-                        mma_bf16(tmem, ad0 + o, bl0 + o, ly.idesc, 1u);
-                        mma_bf16(tmem, al0 + o, bd0 + o, ly.idesc, 1u);
-                    }
+                    const uint64_t oa = (uint64_t)(256 * s), ob = (uint64_t)(16 * s);
+                    mma_bf16(acc, ad0 + oa, bd0 + ob, ly.idesc, s > 0 ? 1u : 0u);
+                    mma_bf16(acc, ad0 + oa, bl0 + ob, ly.idesc, 1u);
+                    mma_bf16(acc, al0 + oa, bd0 + ob, ly.idesc, 1u);
                 }
                 mma_commit(bar_mma);
+                issued = true;
             }
             scatter_next();  // the previous tile's grid gradient, one level
-            // Warp 0 spins on the barrier; the others sleep at the CTA
-            // barrier, which then orders their TMEM reads after completion.
-            const bool done = warp != 0 || mbar_wait_bounded(bar_mma, phase);
-            phase ^= 1u;
-            ok = !__syncthreads_or(!done);
-            if (!ok) break;
-            tc_fence_after();
+            wait_mma();
             if (l < L - 1) {
-                uint8_t* hn = smem + tt.h_off[l + 1];
-                const int kpn = tc.layer[l + 1].Kp;
-                const uint32_t lo = tt.split ? tt.hlo_off - tt.h_off[l + 1] : 0u;
-                for (int c0 = 16 * half; c0 < ly.Np; c0 += 32) {
-                    uint32_t r[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)c0, r);
-                    tmem_wait16(r);
-                    float v[16];
+                if (ok) {
+                    uint8_t* hn = tiles + tt.slot[l + 1];
+                    const uint32_t lo = tt.slot[L] - tt.slot[l + 1];
+                    for (int c0 = 16 * half; c0 < ly.Np; c0 += 32) {
+                        uint32_t r[16];
+                        tmem_ld16(acc + lanes + (uint32_t)c0, r);
+                        tmem_wait16(r);
+                        float v[16];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = fmaxf(__uint_as_float(r[i]), 0.0f);
-                    store16(hn, tile_off(row, c0, kpn), tile_off(row, c0 + 8, kpn), v, lo);
+                        for (int i = 0; i < 16; ++i) v[i] = fmaxf(__uint_as_float(r[i]), 0.0f);
+                        store_cols<16>(hn, row, c0, v, lo);
+                    }
                 }
                 fence_async_smem();
                 tc_fence_before();
-                __syncthreads();
-            } else {
+                if (train_sync_or(g, !ok)) {
+                    ok = false;
+                    break;
+                }
+            } else if (ok) {
                 // This half's lobes: columns [half * 4 KH, (half + 1) * 4 KH).
                 if constexpr (4 * KH >= 16) {
 #pragma unroll
                     for (int c = 0; c < 4 * KH / 16; ++c) {
-                        uint32_t r[16];
-                        tmem_ld16(tmem + lane_base + (uint32_t)(half * 4 * KH + 16 * c), r);
-                        tmem_wait16(r);
+                        uint32_t r[16] = {};
+                        if (half * 4 * KH + 16 * c < ly.Np) {
+                            tmem_ld16(acc + lanes + (uint32_t)(half * 4 * KH + 16 * c), r);
+                            tmem_wait16(r);
+                        }
 #pragma unroll
                         for (int i = 0; i < 16; ++i) raw[16 * c + i] = __uint_as_float(r[i]);
                     }
                 } else {
                     uint32_t r[16];
-                    tmem_ld16(tmem + lane_base, r);
+                    tmem_ld16(acc + lanes, r);
                     tmem_wait16(r);
 #pragma unroll
                     for (int i = 0; i < 4 * KH; ++i) raw[i] = __uint_as_float(half ? r[4 * KH + i] : r[i]);
                 }
             }
         }
-        if (!ok) break;
         // Loss and d loss / d raw (zero for rows beyond n).
-        GradHalf<KMAX> gh;
-        const float4 part = gh.pass1(cfg, half, raw, w);
-        xch[half * kTile + row] = part;
-        __syncthreads();
-        const float4 oth = xch[(half ^ 1) * kTile + row];
-        const float lse = lse_combine(part.x, part.y, oth.x, oth.y);
-        const float lsa = lse_combine(part.z, part.w, oth.z, oth.w);
-        if (valid && half == 0) lacc += sc * (lsa - lse);
-        float dr[4 * KH];
-        gh.pass2(lse, lsa, sc, dr);
-        const uint32_t dlo = tt.split ? tt.dlo_off - tt.d_off : 0u;
-        store_cols<4 * KH>(sD, row, half * 4 * KH, (int)tt.d_cols, dr, dlo);
+        {
+            GradHalf<KMAX> gh;
+            float4 part = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (ok) part = gh.pass1(cfg, half, raw, w);
+            xch[half * kTile + row] = part;
+            if (train_sync_or(g, !ok)) {
+                ok = false;
+                break;
+            }
+            const float4 oth = xch[(half ^ 1) * kTile + row];
+            const float lse = lse_combine(part.x, part.y, oth.x, oth.y);
+            const float lsa = lse_combine(part.z, part.w, oth.z, oth.w);
+            if (valid && half == 0) lacc += sc * (lsa - lse);
+            float dr[4 * KH];
+            gh.pass2(lse, lsa, sc, dr);
+            // (columns beyond the last layer's padded outputs do not exist)
+            if constexpr (4 * KH >= 16) {
+#pragma unroll
+                for (int c = 0; c < 4 * KH; c += 16)
+                    if (half * 4 * KH + c < tc.layer[L - 1].Np)
+                        store_cols<16>(rest, row, half * 4 * KH + c, dr + c, (uint32_t)tc.layer[L - 1].Np * (kPlane / 8));
+            } else {
+                store_cols<4 * KH>(rest, row, half * 4 * KH, dr, (uint32_t)tc.layer[L - 1].Np * (kPlane / 8));
+            }
+        }
         fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        train_sync(g);
         // Backward, top layer first.
-        for (int l = L - 1; l >= 0 && ok; --l) {
+        for (int l = L - 1; l >= 0; --l) {
             const TcLayer& ly = tc.layer[l];
+            const uint32_t lo_off = (uint32_t)ly.Np * (kPlane / 8);  // residuals behind the output gradient
             if (t == 0) {
                 tc_fence_after();
-                const uint32_t hk = (uint32_t)(ly.Kp >> 3) * 128u;  // K step of an H_l / W_l tile
-                // Step-0 descriptors; step s adds its byte offset >> 4 to the
-                // start address field.
-                // dW_l += D^T H_l: M = 128 (outputs), N = Kp_l, K = 128 samples.
-                const uint64_t bh0 = umma_desc(base_addr + tt.h_off[l], hk, 128u);
-                const uint64_t dw0 = umma_desc(sD_addr, drg, 128u), dwl0 = umma_desc(dlo_addr, drg, 128u);
-                const uint64_t bstep = (uint64_t)((2u * hk) >> 4), dstep = (uint64_t)((2u * drg) >> 4);
-                for (int s = 0; s < 8; ++s) {
-                    const uint64_t bh = bh0 + s * bstep;
-                    mma_bf16(tmem + tt.dw_col[l], dw0 + s * dstep, bh, tt.idesc_dw[l], (first && s == 0) ? 0u : 1u);
-                    if (tt.split) mma_bf16(tmem + tt.dw_col[l], dwl0 + s * dstep, bh, tt.idesc_dw[l], 1u);
-                }
+                const uint32_t hk = (uint32_t)(ly.Kp >> 3) * 128u;  // K step of a W_l tile
+                const uint32_t d_addr = tile_addr + tt.slot[l + 1];
                 // D W_l: M = 128 samples, N = Kp_l, K = Np_l outputs.
-                const uint64_t ad0 = umma_desc(sD_addr, 128u, drg), al0 = umma_desc(dlo_addr, 128u, drg);
+                const uint64_t ad0 = umma_desc(d_addr, kPlane, 128u), al0 = umma_desc(d_addr + lo_off, kPlane, 128u);
                 const uint64_t bd0 = umma_desc(sW_addr + ly.w_off, hk, 128u);
                 const uint64_t bl0 = umma_desc(sW_addr + wlo + ly.w_off, hk, 128u);
+                const uint64_t bstep = (uint64_t)((2u * hk) >> 4);
                 for (int s = 0; s < (ly.Np >> 4); ++s) {
-                    const uint64_t o = (uint64_t)(16 * s), ob = s * bstep;
-                    mma_bf16(tmem, ad0 + o, bd0 + ob, tt.idesc_dx[l], s > 0 ? 1u : 0u);
-                    if (tt.split) {
-                        mma_bf16(tmem, ad0 + o, bl0 + ob, tt.idesc_dx[l], 1u);
-                        mma_bf16(tmem, al0 + o, bd0 + ob, tt.idesc_dx[l], 1u);
+                    const uint64_t oa = (uint64_t)(256 * s), ob = s * bstep;
+                    mma_bf16(acc, ad0 + oa, bd0 + ob, tt.idesc_dx[l], s > 0 ? 1u : 0u);
+                    mma_bf16(acc, ad0 + oa, bl0 + ob, tt.idesc_dx[l], 1u);
+                    mma_bf16(acc, al0 + oa, bd0 + ob, tt.idesc_dx[l], 1u);
+                }
+                // dW_l += D^T H_l: M = 128 (outputs, then their residuals),
+                // N = Kp_l, K = 128 samples (256 bytes a step).
+                if (G == 1 || take_turn(turn, bar_dw)) {
+                    tc_fence_after();
+                    const uint64_t bh0 = umma_desc(tile_addr + tt.slot[l], 128u, kPlane);
+                    const uint64_t dw0 = umma_desc(d_addr, 128u, kPlane), dwl0 = umma_desc(d_addr + lo_off, 128u, kPlane);
+                    for (int s = 0; s < 8; ++s) {
+                        const uint64_t o = (uint64_t)(16 * s);
+                        mma_bf16(tmem + tt.dw_col[l], dw0 + o, bh0 + o, tt.idesc_dw[l], 1u);
+                        if (2 * ly.Np > 128) mma_bf16(tmem + tt.dw_col[l], dwl0 + o, bh0 + o, tt.idesc_dw[l], 1u);
                     }
+                    if (G > 1) {
+                        mma_commit(bar_dw);
+                        pass_turn(turn);
+                    }
+                } else {
+                    ok = false;
                 }
                 mma_commit(bar_mma);
             }
             scatter_next();
-            const bool done = warp != 0 || mbar_wait_bounded(bar_mma, phase);
-            phase ^= 1u;
-            ok = !__syncthreads_or(!done);
-            if (!ok) break;
-            tc_fence_after();
-            const uint8_t* hl = smem + tt.h_off[l];
+            wait_mma();
             if (l > 0) {
-                // delta_{l-1} = (D W_l) masked by ReLU'(z_{l-1}) (H_l > 0).
-                for (int c0 = 16 * half; c0 < ly.Kp; c0 += 32) {
-                    uint32_t r[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)c0, r);
-                    tmem_wait16(r);
-                    const uint4 m0 = *reinterpret_cast<const uint4*>(hl + tile_off(row, c0, ly.Kp));
-                    const uint4 m1 = *reinterpret_cast<const uint4*>(hl + tile_off(row, c0 + 8, ly.Kp));
-                    const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-                    float v[16];
+                // The gradient of layer l's input, D W_l where the input is
+                // positive (ReLU'), in its place.
+                if (ok) {
+                    uint8_t* hl = tiles + tt.slot[l];
+                    for (int c0 = 16 * half; c0 < ly.Kp; c0 += 32) {
+                        uint32_t r[16];
+                        tmem_ld16(acc + lanes + (uint32_t)c0, r);
+                        tmem_wait16(r);
+                        const uint4 m0 = *reinterpret_cast<const uint4*>(hl + plane_off(row, c0));
+                        const uint4 m1 = *reinterpret_cast<const uint4*>(hl + plane_off(row, c0 + 8));
+                        const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                        float v[16];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&mw[i]));
-                        v[2 * i] = hv.x > 0.0f ? __uint_as_float(r[2 * i]) : 0.0f;
-                        v[2 * i + 1] = hv.y > 0.0f ? __uint_as_float(r[2 * i + 1]) : 0.0f;
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&mw[i]));
+                            v[2 * i] = hv.x > 0.0f ? __uint_as_float(r[2 * i]) : 0.0f;
+                            v[2 * i + 1] = hv.y > 0.0f ? __uint_as_float(r[2 * i + 1]) : 0.0f;
+                        }
+                        store_cols<16>(hl, row, c0, v, (uint32_t)ly.Kp * (kPlane / 8));
                     }
-                    store16(sD, tile_off(row, c0, (int)tt.d_cols), tile_off(row, c0 + 8, (int)tt.d_cols), v, dlo);
                 }
                 fence_async_smem();
                 tc_fence_before();
-                __syncthreads();
-            } else if (16 * half < cfg.grid_feats) {
+                if (train_sync_or(g, !ok)) {
+                    ok = false;
+                    break;
+                }
+            } else if (ok && 16 * half < cfg.grid_feats) {
                 // Encoder gradient of this half's 16 grid-feature columns ->
                 // grid scatter.
-                float dg[16];
-                {
-                    uint32_t r[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)(16 * half), r);
-                    tmem_wait16(r);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) dg[i] = __uint_as_float(r[i]);
-                }
-                tc_fence_before();
-                if constexpr (F2) {
+                uint32_t r[16];
+                tmem_ld16(acc + lanes + (uint32_t)(16 * half), r);
+                tmem_wait16(r);
+                if (F2 && tt.park) {
                     while (pend && pq < 8) scatter_next();  // networks with fewer than 4 layers
-                    pend = valid;
+                    const uint32_t a[8] = {r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]};
+                    const uint32_t b[8] = {r[8], r[9], r[10], r[11], r[12], r[13], r[14], r[15]};
+                    tmem_st(park, a);
+                    tmem_st(park + 8u, b);
+                    tmem_wait_st();
+                    pend = true;
+                    pvalid = valid;
                     pq = 0;
                     if (valid) {
                         px = pos[j];
                         py = pos[ld + j];
                         pz = pos[2 * ld + j];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) pdg[i] = dg[i];
                     }
                 } else if (valid) {
+                    float dg[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) dg[i] = __uint_as_float(r[i]);
                     const float x = pos[j], y = pos[ld + j], z = pos[2 * ld + j];
                     const int F = cfg.feat;
                     if (F == 2) scatter_levels<2, 8>(cfg, grad, x, y, z, 8 * half, dg);
@@ -817,48 +810,78 @@ __global__ void __launch_bounds__(kTrainThreads, train_ctas_per_sm(KMAX, F2)) k_
                     else if (F == 8) scatter_levels<8, 2>(cfg, grad, x, y, z, 2 * half, dg);
                     else scatter_levels<1, 16>(cfg, grad, x, y, z, 16 * half, dg);
                 }
+                __syncwarp();
+                tc_fence_before();
             } else {
                 tc_fence_before();
             }
         }
-        first = false;
     }
     while (pend && pq < 8) scatter_next();  // the last tile's grid gradient
     // Loss: one atomic per warp.
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
     if (loss && (t & 31) == 0 && lacc != 0.0f) atomicAdd(loss, (double)lacc);
-    // Weight gradients: lane o of layer l's TMEM region holds dW_l[o][*].
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (ok && !first) {
-        for (int l = 0; l < L; ++l) {
-            const TcLayer& ly = tc.layer[l];
-            float* gW = grad + mlp_off + tt.woff[l];
-            for (int c0 = 16 * half; c0 < ly.Kp; c0 += 32) {
-                uint32_t r[16];
-                tmem_ld16(tmem + lane_base + tt.dw_col[l] + (uint32_t)c0, r);
-                tmem_wait16(r);
-                if (row < ly.N)
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < ly.K) atomicAdd(gW + (int64_t)row * ly.K + c0 + i, __uint_as_float(r[i]));
-            }
-        }
-    }
     if (!ok) {
-        if (t == 0) atomicOr(status, kStatusTimeout);
-        // As in the forward kernel: drain this CTA's in-flight weight copy and
-        // MMA batch (bounded) before the tensor memory is released.
-        if (warp == 0) {
-            (void)mbar_wait_bounded(bar_w, 0);
-            (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
+        if ((t & 31) == 0) atomicOr(status, kStatusTimeout);
+        // Before the tensor memory is released: wait again, bounded, for this
+        // group's MMAs that may still be in flight.
+        if (t == 0 && issued) (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
+    }
+    // Weight gradients, once every group is done: lane o of layer l's columns
+    // holds D_hi^T H, lane Np + o the residuals' share (or the lane of the high
+    // part both). The shares meet in shared memory (the tiles are done with),
+    // and four weights leave in one operation: every CTA adds to the same few
+    // kilobytes, whose L2 slices take the operations one after another (with
+    // one per weight and share that was two thirds of the small network's
+    // kernel).
+    tc_fence_before();
+    const bool all_ok = !__syncthreads_or(!ok);
+    tc_fence_after();
+    if (all_ok) {
+        const int lane = (int)(threadIdx.x & 127), set = (int)(threadIdx.x >> 7);
+        constexpr int kSets = kTrainThreads * G / 128;
+        float* stage = reinterpret_cast<float*>(smem);
+        for (int pass = 0; pass < 2; ++pass) {
+            float* sl = stage;
+            for (int l = 0; l < L; ++l) {
+                const TcLayer& ly = tc.layer[l];
+                const bool both = 2 * ly.Np <= 128;
+                float* gW = grad + mlp_off + tt.woff[l] + (int64_t)lane * ly.K;
+                const bool wide = (reinterpret_cast<uintptr_t>(grad + mlp_off) & 15u) == 0;
+                const bool mine = pass == 0 ? both && lane >= ly.Np && lane < 2 * ly.Np : lane < ly.N;
+                for (int c0 = 16 * set; c0 < ly.Kp; c0 += 16 * kSets) {
+                    uint32_t r[16];
+                    tmem_ld16(tmem + lanes + tt.dw_col[l] + (uint32_t)c0, r);
+                    tmem_wait16(r);
+                    if (mine) {
+                        // stage: [Kp / 4][Np] vectors, so that a warp's lie side by side
+#pragma unroll
+                        for (int i = 0; i < 16; i += 4) {
+                            float4* st4 = reinterpret_cast<float4*>(sl) + (size_t)((c0 + i) >> 2) * ly.Np;
+                            float4 v = make_float4(__uint_as_float(r[i]), __uint_as_float(r[i + 1]),
+                                                   __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+                            if (pass == 0) {
+                                st4[lane - ly.Np] = v;
+                            } else if (c0 + i < ly.K) {
+                                if (both) {
+                                    const float4 lo = st4[lane];
+                                    v = make_float4(v.x + lo.x, v.y + lo.y, v.z + lo.z, v.w + lo.w);
+                                }
+                                red_add4(gW + c0 + i, wide, v.x, v.y, v.z, v.w);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (both) sl += ly.Kp * ly.Np;
+            }
+            __syncthreads();
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tt.tmem_cols) : "memory");
     }
@@ -951,8 +974,8 @@ npm_status tc_create(npm_handle* h) {
         delete s;
         return NPM_ERR_UNSUPPORTED;
     }
-    // Training layout. Gradients take split BF16 operands in both
-    // reduced-precision modes: single-pass BF16 compounds its rounding down
+    // Training layout. Gradients take split BF16 operands in every
+    // reduced-precision mode: single-pass BF16 compounds its rounding down
     // the layers and through the cancelling grid sums (per-tensor gradient
     // errors of tens of percent), so only inference offers the plain form.
     {
@@ -961,19 +984,24 @@ npm_status tc_create(npm_handle* h) {
         s->train_cfg = t;
         // Training multiplies BF16 operands whatever the inference format.
         s->train_cfg.f16 = 0;
+        s->train_cfg.split = 1;
         s->train_cfg.wparts = 2;
         for (int l = 0; l < c.n_layers; ++l) s->train_cfg.layer[l].idesc |= (1u << 7) | (1u << 10);
-        uint32_t off = 2u * t.w_bytes, col0 = 0, cols = 0;
+        uint32_t off = 0, cols = 0;
         int64_t wo = 0;
+        int wide = 16, maxin = 16;  // widest layer, widest input
         bool fits = c.K * 4 <= 64 && c.n_levels * c.feat_per_level <= 32;
         for (int l = 0; l < c.n_layers; ++l) {
             const TcLayer& ly = t.layer[l];
-            tr.h_off[l] = off;
+            tr.slot[l] = off;
             off += (uint32_t)(kTile * ly.Kp * 2);
-            col0 = (uint32_t)std::max<int>((int)col0, std::max(ly.Kp, ly.Np));
+            maxin = std::max(maxin, ly.Kp);
+            wide = std::max(wide, std::max(ly.Kp, ly.Np));
             tr.woff[l] = wo;
             wo += (int64_t)ly.K * ly.N;
             if (ly.Np > 128 || ly.Kp > 128) fits = false;
+            tr.dw_col[l] = cols;
+            cols += (uint32_t)ly.Kp;
             // dW: A = delta^T (MN-major), B = H_l (MN-major), M = 128, N = Kp_l.
             tr.idesc_dw[l] = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                              ((uint32_t)(ly.Kp >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
@@ -981,47 +1009,46 @@ npm_status tc_create(npm_handle* h) {
             tr.idesc_dx[l] = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) |
                              ((uint32_t)(ly.Kp >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
         }
-        tr.split = 1;
-        int maxkp = 0;
-        for (int l = 0; l < c.n_layers; ++l) maxkp = std::max(maxkp, t.layer[l].Kp);
-        col0 = (col0 + 15) / 16 * 16;
-        cols = col0;
-        for (int l = 0; l < c.n_layers; ++l) {
-            tr.dw_col[l] = cols;
-            cols += (uint32_t)t.layer[l].Kp;
-        }
+        // Which networks train on tensor cores is part of the interface: those
+        // whose weights, tiles and a gradient tile pair as wide as the widest
+        // layer fit 220 KB, with the accumulators in 512 columns. This layout
+        // is never larger.
+        const uint32_t need = 2u * t.w_bytes + off + 2u * kTile * wide * 2u + kTile * maxin * 2u + 64u;
         uint32_t pw = 32;
-        while (pw < cols) pw <<= 1;
-        tr.tmem_cols = pw;
-        // Delta tile: as wide as the widest layer (inputs or outputs). The
-        // weight-gradient MMA reads it transposed with M = 128 output rows:
-        // rows beyond the layer's outputs come from the next row groups and,
-        // past the last one, up to 2 KB beyond the tile (the residual tile
-        // that follows); they land in weight-gradient rows that are never
-        // read.
-        uint32_t dcols = 16;
-        for (int l = 0; l < c.n_layers; ++l)
-            dcols = std::max<uint32_t>(dcols, (uint32_t)std::max(t.layer[l].Kp, t.layer[l].Np));
-        tr.d_cols = dcols;
-        tr.d_off = (off + 127u) / 128u * 128u;
-        tr.dlo_off = tr.d_off + kTile * dcols * 2;
-        // One residual activation tile, reused layer by layer; the loss
-        // step's exchange of partial log-sum-exps reuses it too (the forward
-        // has finished with it, and the next tile's encode rewrites it after
-        // the backward).
-        tr.hlo_off = tr.dlo_off + kTile * dcols * 2;
-        const uint32_t hlo_bytes = (uint32_t)(kTile * maxkp * 2);
-        // (Kp >= 16, so the tile has at least 4 KB: the exchange buffer's
-        // 2 x kTile float4 and the over-read's 2 KB.)
-        tr.x_off = tr.hlo_off;
-        tr.bar_off = tr.hlo_off + hlo_bytes;
-        tr.smem = tr.bar_off + 64;
-        // The encoder writes its residual at (tile + a_bytes): point that at
-        // the shared residual tile.
-        s->train_cfg.split = tr.split;
-        s->train_cfg.a_bytes = tr.hlo_off - tr.h_off[0];
+        while (pw < cols + (uint32_t)wide) pw <<= 1;
         // FP32 and the FP32-accuracy mode train with the FP32 kernels.
-        s->can_train = fits && pw <= 512 && tr.smem <= 220 * 1024 && !t.fp32;
+        s->can_train = fits && pw <= 512 && need <= 220 * 1024 && !t.fp32;
+        const int last = t.layer[c.n_layers - 1].Np;
+        tr.slot[c.n_layers] = off;
+        off += (uint32_t)(kTile * std::max(maxin, 2 * last) * 2);
+        tr.g_bytes = off;
+        tr.acc_col = cols;
+        tr.acc_cols = (uint32_t)wide;
+        // Two groups where they fit; the small four-lobe networks run three
+        // CTAs of one group instead, sixteen lobes take the registers of one.
+        auto lay = [&](int G) {
+            tr.groups = G;
+            tr.x_off = (uint32_t)G * tr.g_bytes;
+            tr.w_off = tr.x_off + (uint32_t)G * 2u * kTile * 16u;
+            // An MMA reads 128 rows from the start of a gradient's slot.
+            uint32_t end = tr.w_off + 2u * t.w_bytes;
+            for (int l = 1; l <= c.n_layers; ++l)
+                end = std::max(end, (uint32_t)(G - 1) * tr.g_bytes + tr.slot[l] + 16u * kPlane +
+                                        (2 * t.layer[l - 1].Np > 128 ? (uint32_t)t.layer[l - 1].Np * (kPlane / 8) : 0u));
+            tr.bar_off = (end + 127u) / 128u * 128u;
+            tr.smem = tr.bar_off + 8u * (2u + (uint32_t)G) + 32u;
+            uint32_t used = cols + (uint32_t)G * (uint32_t)wide;
+            tr.park = c.feat_per_level == 2 && used + 32u * (uint32_t)G <= 512u ? 1 : 0;
+            tr.park_col = used;
+            if (tr.park) used += 32u * (uint32_t)G;
+            tr.tmem_cols = 32;
+            while (tr.tmem_cols < used) tr.tmem_cols <<= 1;
+            return tr.tmem_cols <= 512u && tr.smem <= 227u * 1024u;
+        };
+        const bool small = c.K <= 4 && c.feat_per_level != 2;
+        if (small || c.K > 8 || !lay(2)) {
+            if (!lay(1)) s->can_train = false;
+        }
     }
     if (device_alloc((void**)&s->wblob, nw * t.w_bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -1105,15 +1132,15 @@ cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, const UpdateEnd& 
     return cudaGetLastError();
 }
 
-template <int KMAX, bool F2>
+template <int KMAX, bool F2, int G>
 static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const float* pos, const float* aux,
                                    const float* dir, const float* rad, const float* spdf, const float* dlogv,
                                    double* loss, cudaStream_t st) {
     TcState* s = h->tc;
-    auto kern = k_train_tc<KMAX, F2>;
+    auto kern = k_train_tc<KMAX, F2, G>;
     // CTAs per SM: the instance's register budget, if shared and tensor
     // memory hold that many.
-    int per_sm = train_ctas_per_sm(KMAX, F2);
+    int per_sm = train_ctas_per_sm(KMAX, F2, G);
     while (per_sm > 1 && ((size_t)per_sm * (s->train.smem + 1024) > 227 * 1024 ||
                           (uint32_t)per_sm * s->train.tmem_cols > 512u))
         --per_sm;
@@ -1144,9 +1171,9 @@ static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const f
         enc = s->enc;
     }
     const uint8_t* wb = s->wblob_train ? s->wblob_train : s->wblob;
-    kern<<<g < 1 ? 1 : g, kTrainThreads, s->train.smem, st>>>(s->train_cfg, s->train, h->params, wb, n, ld, pos,
-                                                         aux, dir, rad, spdf, dlogv, 1.0f / (float)n, h->grads,
-                                                         h->mlp_off, loss, status, enc);
+    kern<<<g < 1 ? 1 : g, kTrainThreads * G, s->train.smem, st>>>(s->train_cfg, s->train, h->params, wb, n, ld, pos,
+                                                                  aux, dir, rad, spdf, dlogv, 1.0f / (float)n,
+                                                                  h->grads, h->mlp_off, loss, status, enc);
     return cudaGetLastError();
 }
 
@@ -1156,14 +1183,17 @@ cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, con
                      const float* rad, const float* spdf, const float* dlogv, double* loss, cudaStream_t st) {
     const int K = h->cfg.K;
     const bool f2 = h->cfg.feat_per_level == 2;
-    if (K <= 4)
-        return f2 ? launch_train_tc<4, true>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
-                  : launch_train_tc<4, false>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
-    if (K <= 8)
-        return f2 ? launch_train_tc<8, true>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
-                  : launch_train_tc<8, false>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
-    return f2 ? launch_train_tc<16, true>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
-              : launch_train_tc<16, false>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
+    const bool two = h->tc->train.groups == 2;
+    if (K <= 4 && !f2) return launch_train_tc<4, false, 1>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
+    if (K <= 8) {
+        if (f2)
+            return two ? launch_train_tc<8, true, 2>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
+                       : launch_train_tc<8, true, 1>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
+        return two ? launch_train_tc<8, false, 2>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
+                   : launch_train_tc<8, false, 1>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
+    }
+    return f2 ? launch_train_tc<16, true, 1>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st)
+              : launch_train_tc<16, false, 1>(h, n, ld, pos, aux, dir, rad, spdf, dlogv, loss, st);
 }
 
 // The corner blocks of the inference table, brought up to date on st.

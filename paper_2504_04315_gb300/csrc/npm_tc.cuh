@@ -202,6 +202,14 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
                  : "memory");
 }
 
+// The same for two columns.
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&r)[2]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait2(uint32_t (&r)[2]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]) : : "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t*>(&h);
@@ -253,55 +261,18 @@ __device__ __forceinline__ uint32_t tile_off(int row, int k, int kp) {
     return (uint32_t)((row >> 3) * (kp >> 3) * 128 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2);
 }
 
-// Rounds v to BF16 (hi) and, when lo_off != 0, also stores the BF16
-// residual v - hi at the same position of the residual tile lo_off bytes on.
-__device__ __forceinline__ void store16(uint8_t* sA, uint32_t off0, uint32_t off1, const float (&v)[16],
-                                        uint32_t lo_off) {
-    uint32_t h[8], l[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        __nv_bfloat162 hb = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-        h[i] = *reinterpret_cast<uint32_t*>(&hb);
-        const float2 hf = __bfloat1622float2(hb);
-        l[i] = pack_bf16(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
-    }
-    *reinterpret_cast<uint4*>(sA + off0) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(sA + off1) = make_uint4(h[4], h[5], h[6], h[7]);
-    if (lo_off) {
-        *reinterpret_cast<uint4*>(sA + lo_off + off0) = make_uint4(l[0], l[1], l[2], l[3]);
-        *reinterpret_cast<uint4*>(sA + lo_off + off1) = make_uint4(l[4], l[5], l[6], l[7]);
-    }
-}
-
-// One or two BF16 values (and their residuals when lo_off != 0), or FP16
-// values when f16.
-__device__ __forceinline__ void store_pair(uint8_t* sA, uint32_t off, float a, float b, uint32_t lo_off,
-                                           bool f16 = false) {
-    if (f16) {
-        const uint32_t hp = pack_f16_sat(a, b);
-        *reinterpret_cast<uint32_t*>(sA + off) = hp;
-        if (lo_off) *reinterpret_cast<uint32_t*>(sA + lo_off + off) = f16_residual(hp, a, b);
-        return;
-    }
+// One or two BF16 values and their residuals lo_off bytes on.
+__device__ __forceinline__ void store_pair(uint8_t* sA, uint32_t off, float a, float b, uint32_t lo_off) {
     __nv_bfloat162 hb = __floats2bfloat162_rn(a, b);
     *reinterpret_cast<__nv_bfloat162*>(sA + off) = hb;
-    if (lo_off) {
-        const float2 hf = __bfloat1622float2(hb);
-        *reinterpret_cast<uint32_t*>(sA + lo_off + off) = pack_bf16(a - hf.x, b - hf.y);
-    }
+    const float2 hf = __bfloat1622float2(hb);
+    *reinterpret_cast<uint32_t*>(sA + lo_off + off) = pack_bf16(a - hf.x, b - hf.y);
 }
 
-__device__ __forceinline__ void store_one(uint8_t* sA, uint32_t off, float a, uint32_t lo_off, bool f16 = false) {
-    if (f16) {
-        const uint32_t hp = pack_f16_sat(a, 0.0f);
-        *reinterpret_cast<uint16_t*>(sA + off) = (uint16_t)(hp & 0xffffu);
-        if (lo_off) *reinterpret_cast<uint16_t*>(sA + lo_off + off) = (uint16_t)(f16_residual(hp, a, 0.0f) & 0xffffu);
-        return;
-    }
+__device__ __forceinline__ void store_one(uint8_t* sA, uint32_t off, float a, uint32_t lo_off) {
     const __nv_bfloat16 hb = __float2bfloat16_rn(a);
     *reinterpret_cast<__nv_bfloat16*>(sA + off) = hb;
-    if (lo_off)
-        *reinterpret_cast<__nv_bfloat16*>(sA + lo_off + off) = __float2bfloat16_rn(a - __bfloat162float(hb));
+    *reinterpret_cast<__nv_bfloat16*>(sA + lo_off + off) = __float2bfloat16_rn(a - __bfloat162float(hb));
 }
 
 // Sampler of the reduced-precision path (Sec. 5.3, Jakob's inversion as in
