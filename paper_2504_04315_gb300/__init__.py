@@ -20,9 +20,15 @@ SOFTPLUS, EXP = 0, 1
 FP32, BF16, BF16X3, FP16, FP32_TC = 0, 1, 2, 3, 4
 
 
+_TORCH = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _TORCH
+    if _TORCH is None:
+        import torch
+        _TORCH = torch
+    return _TORCH
 
 
 def make_config(mode: int, level_res: Sequence[int], feat: int, log2_table: int,
@@ -64,21 +70,31 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+_raw_stream = None  # (device index) -> cudaStream_t of its current stream
+
+
 def _stream_ptr(stream) -> Optional[int]:
-    if stream is None:
-        torch = _torch()
-        return torch.cuda.current_stream().cuda_stream
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # The current stream's handle without a torch.cuda.Stream object around it
+    # (4 us of a small call's 20 us on the host).
+    global _raw_stream
+    torch = _torch()
+    if _raw_stream is None:
+        ptr = torch.cuda.current_stream().cuda_stream  # initialises CUDA in torch
+        _raw_stream = torch._C._cuda_getCurrentRawStream
+        return ptr
+    return _raw_stream(torch._C._cuda_getDevice())
 
 
 def _soa(t, rows: int, name: str):
     """Validate a [rows][ld] float32 CUDA tensor; returns ld."""
-    torch = _torch()
-    if t.dtype != torch.float32 or not t.is_cuda:
+    if t.dtype != _torch().float32 or not t.is_cuda:
         raise TypeError(f"{name} must be a float32 CUDA tensor")
-    if t.dim() != 2 or t.shape[0] < rows or not t.is_contiguous():
+    shape = t.shape
+    if len(shape) != 2 or shape[0] < rows or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous [{rows}][ld] tensor")
-    return t.shape[1]
+    return shape[1]
 
 
 class NPM:
@@ -115,12 +131,12 @@ class NPM:
                      want_mix: bool = False, out=None, stream=None):
         """Guided directions and densities. pos [3][ld], u [3 or 4][ld],
         aux [7][ld] (product mode). Returns (dir [3][ld], pdf [ld], mix)."""
-        torch = _torch()
         ld = _soa(pos, 3, "pos")
         n = ld if n is None else n
         _soa(u, 4 if uniform_frac > 0 else 3, "u")
         if aux is not None:
             _soa(aux, 7, "aux")
+        torch = _torch()
         if out is None:
             d = torch.empty((3, ld), device=pos.device, dtype=torch.float32)
             p = torch.empty((ld,), device=pos.device, dtype=torch.float32)
@@ -173,7 +189,7 @@ class NPM:
         torch = _torch()
         ld = _soa(pos, 3, "pos")
         n = ld if n is None else n
-        loss = torch.zeros((1,), device=pos.device, dtype=torch.float32) if loss_out is None else loss_out
+        loss = torch.empty((1,), device=pos.device, dtype=torch.float32) if loss_out is None else loss_out
         _lib.check(self._L.npm_train_step(self._h, n, _ptr(pos), _ptr(aux), _ptr(dirs),
                                           _ptr(radiance), _ptr(sample_pdf), ld, _ptr(loss),
                                           _stream_ptr(stream)), "npm_train_step")

@@ -427,10 +427,8 @@ npm_status npm_set_params_device(npm_handle* h, const float* dev, int64_t count,
     if (!h || !dev) return fail(NPM_ERR_INVALID_ARG, "NULL argument");
     if (count != h->ng + h->nmlp) return fail(NPM_ERR_INVALID_ARG, "count != npm_num_params");
     cudaStream_t st = (cudaStream_t)stream;
-    NPM_CUDA(cudaMemcpyAsync(h->params, dev, h->ng * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy grid");
-    NPM_CUDA(cudaMemcpyAsync(h->params + h->mlp_off, dev + h->ng, h->nmlp * sizeof(float),
-                             cudaMemcpyDeviceToDevice, st),
-             "copy mlp");
+    NPM_CUDA(npm::launch_copy_params(dev, h->params, h->ng, dev + h->ng, h->params + h->mlp_off, h->nmlp, st),
+             "copy parameters");
     if (h->ema)
         NPM_CUDA(cudaMemcpyAsync(h->ema, h->params, h->n_int * sizeof(float), cudaMemcpyDeviceToDevice, st),
                  "reset ema");
@@ -442,10 +440,8 @@ npm_status npm_get_grads_device(npm_handle* h, float* dev, int64_t count, void* 
     if (!h || !dev) return fail(NPM_ERR_INVALID_ARG, "NULL argument");
     if (count != h->ng + h->nmlp) return fail(NPM_ERR_INVALID_ARG, "count != npm_num_params");
     cudaStream_t st = (cudaStream_t)stream;
-    NPM_CUDA(cudaMemcpyAsync(dev, h->grads, h->ng * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy grid");
-    NPM_CUDA(cudaMemcpyAsync(dev + h->ng, h->grads + h->mlp_off, h->nmlp * sizeof(float),
-                             cudaMemcpyDeviceToDevice, st),
-             "copy mlp");
+    NPM_CUDA(npm::launch_copy_params(h->grads, dev, h->ng, h->grads + h->mlp_off, dev + h->ng, h->nmlp, st),
+             "copy gradient");
     return NPM_OK;
 }
 

@@ -21,6 +21,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "npm_device.cuh"
 #include "npm_kernels.h"
 
@@ -996,6 +998,28 @@ __global__ void k_grid_indices(DevCfg cfg, int64_t n, int64_t ld, const float* _
     }
 }
 
+// dst0[i] = src0[i] for i < n0 in vectors V, dst1[i] = src1[i] for i < n1: the
+// grid and the MLP between the public layout and the library's, in one launch
+// at any alignment (a copy call each cost the host two to three times that,
+// and ran at half the bandwidth where the two sides' alignments differ).
+template <typename V>
+__global__ void __launch_bounds__(256) k_copy_params(const V* __restrict__ src0, V* __restrict__ dst0, int64_t n0,
+                                                     const float* __restrict__ src1, float* __restrict__ dst1,
+                                                     int64_t n1) {
+    constexpr int U = 4;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < n0; i += U * stride) {
+        V v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * stride < n0) v[u] = src0[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * stride < n0) dst0[i + u * stride] = v[u];
+    }
+    for (int64_t i = i0; i < n1; i += stride) dst1[i] = src1[i];
+}
+
 __global__ void k_to_half(int64_t n, const float* __restrict__ src, __half* __restrict__ dst) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -1159,6 +1183,25 @@ cudaError_t launch_grid_indices(const DevCfg& cfg, int64_t n, int64_t ld, const 
     int grid = (int)((n + 255) / 256);
     if (grid > 4096) grid = 4096;
     k_grid_indices<<<grid, 256, 0, st>>>(cfg, n, ld, pos, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_params(const float* src0, float* dst0, int64_t n0, const float* src1, float* dst1, int64_t n1,
+                               cudaStream_t st) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src0) | reinterpret_cast<uintptr_t>(dst0) |
+                        (uintptr_t)(n0 * (int64_t)sizeof(float));
+    const int64_t cap = (int64_t)sm_count() * 8;
+    auto launch = [&](auto* v) {
+        using V = std::remove_pointer_t<decltype(v)>;
+        const int64_t n = n0 * (int64_t)sizeof(float) / (int64_t)sizeof(V);
+        int64_t blocks = (n / 4 + n1 / 4 + 255) / 256;
+        blocks = blocks < 1 ? 1 : blocks > cap ? cap : blocks;
+        k_copy_params<V><<<(int)blocks, 256, 0, st>>>(reinterpret_cast<const V*>(src0), reinterpret_cast<V*>(dst0), n,
+                                                      src1, dst1, n1);
+    };
+    if (a % 16 == 0) launch(static_cast<float4*>(nullptr));
+    else if (a % 8 == 0) launch(static_cast<float2*>(nullptr));
+    else launch(static_cast<float*>(nullptr));
     return cudaGetLastError();
 }
 

@@ -99,6 +99,10 @@ cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float
 cudaError_t launch_grid_indices(const DevCfg& cfg, int64_t n, int64_t ld, const float* pos,
                                 int32_t* out, cudaStream_t st);
 
+// Two device-to-device copies in one launch.
+cudaError_t launch_copy_params(const float* src0, float* dst0, int64_t n0, const float* src1, float* dst1, int64_t n1,
+                               cudaStream_t st);
+
 cudaError_t launch_to_half(int64_t n, const float* src, __half* dst, cudaStream_t st);
 
 }  // namespace npm
