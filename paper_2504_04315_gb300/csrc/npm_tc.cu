@@ -942,19 +942,6 @@ npm_status tc_create(npm_handle* h) {
         maxnp = ly.Np > maxnp ? ly.Np : maxnp;
     }
     t.w_bytes = (off + 127u) / 128u * 128u;
-    // Layer 0 gets its own input buffer only when the encoding leaves whole
-    // zero chunks to write once; otherwise it shares the buffer of the
-    // hidden layers (less shared memory, more L1 for the grid gathers).
-    const int enc_width = c.n_levels * c.feat_per_level + (c.mode == NPM_PRODUCT ? 21 : 0);
-    // A single small grid level (the tiny models) shares the buffer anyway:
-    // its zero chunk costs one store per tile, and the smaller CTA lets eight
-    // of them share an SM instead of six.
-    const bool single_small = c.n_levels == 1 && c.feat_per_level <= 8 && c.mode != NPM_PRODUCT;
-    const bool sep0 = (enc_width + 7) / 8 * 8 < t.layer[0].Kp && !single_small;
-    int maxkp1 = 16;  // widest input of the layers sharing the buffer
-    for (int l = sep0 ? 1 : 0; l < c.n_layers; ++l) maxkp1 = std::max(maxkp1, t.layer[l].Kp);
-    t.a_bytes = (uint32_t)(kTile * maxkp1 * 2);
-    t.a0_bytes = sep0 ? (uint32_t)(kTile * t.layer[0].Kp * 2) : 0u;
     t.split = (c.precision == NPM_BF16X3 || c.precision == NPM_FP32_TC) ? 1 : 0;
     t.f16 = (c.precision == NPM_FP16 || c.precision == NPM_FP32_TC) ? 1 : 0;
     t.fp32 = (c.precision == NPM_FP32_TC || fp32) ? 1 : 0;
@@ -966,11 +953,18 @@ npm_status tc_create(npm_handle* h) {
     t.d_cols = (uint32_t)((maxnp + 31) / 32 * 32);
     t.a_cols = (uint32_t)(maxkp / 2);
     t.g_cols = t.d_cols + nsplit * t.a_cols;
-    // FP32 models that do not fit keep the CUDA-core kernels; in the other
-    // modes the limit (weights and one pair of activation tiles) is part of
-    // the interface.
+    // FP32 models that do not fit keep the CUDA-core kernels. In the other
+    // modes the limit is part of the interface: 200 KB for the weights and one
+    // activation tile per part (two where the encoding leaves whole 8-column
+    // chunks of a multi-level network's first layer empty).
+    const int enc_width = c.n_levels * c.feat_per_level + (c.mode == NPM_PRODUCT ? 21 : 0);
+    const bool one_level = c.n_levels == 1 && c.feat_per_level <= 8 && c.mode != NPM_PRODUCT;
+    const bool sep0 = (enc_width + 7) / 8 * 8 < t.layer[0].Kp && !one_level;
+    int hidden = 16;  // widest input of the layers that share a tile
+    for (int l = sep0 ? 1 : 0; l < c.n_layers; ++l) hidden = std::max(hidden, t.layer[l].Kp);
+    const uint32_t tile_bytes = (uint32_t)(kTile * (hidden + (sep0 ? t.layer[0].Kp : 0)) * 2);
     if (fp32 ? nw * t.w_bytes > 200 * 1024 || t.g_cols > 512u
-             : nw * t.w_bytes + nsplit * (t.a0_bytes + t.a_bytes) + 64 > 200 * 1024 || c.K > 16) {
+             : nw * t.w_bytes + nsplit * tile_bytes + 64 > 200 * 1024 || c.K > 16) {
         delete s;
         return NPM_ERR_UNSUPPORTED;
     }

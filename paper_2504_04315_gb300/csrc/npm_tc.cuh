@@ -30,10 +30,6 @@ struct TcCfg {
     TcLayer layer[NPM_MAX_LAYERS];
     uint32_t w_bytes;  // bytes of one weight blob (multiple of 128); the
                        // residual (lo) blob follows when split
-    uint32_t a_bytes;  // bytes of one activation tile; the lo tile follows
-    uint32_t a0_bytes; // bytes of the layer-0 input tile when it has its own
-                       // buffer (the encoding leaves all-zero 8-column chunks);
-                       // 0 when layer 0 shares the buffer of layers >= 1
     int parts, wparts; // 16-bit operand parts of an activation and of a weight
     int split;         // 1: two BF16 parts (three MMAs per K step)
     int f16;           // 1: FP16 operands: activations rounded to FP16, weights

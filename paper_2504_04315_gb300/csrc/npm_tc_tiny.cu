@@ -4,7 +4,7 @@
 // accumulation in tensor memory) and K = 4 vMF lobes (the reduced-precision
 // serving workload).
 //
-// The general kernel (npm_tc.cu) serves every shape; this one trims the
+// The general kernel (npm_tc_forward.cuh) serves every shape; this one trims the
 // per-query instruction count of the shape the serving loop runs, where the
 // kernel is bound by instruction issue rather than memory or tensor work:
 //   - encode: the level's 8 corners as 8-byte FP16 loads at 32-bit indices,
@@ -16,9 +16,11 @@
 //     logarithm, reciprocal, sine and cosine on arguments kept in their
 //     accurate ranges; the sampler itself (Sec. 5.3, Jakob's inversion) is
 //     the general kernel's vmf_sample_rp.
-// Tiles, weights, shared-memory layout and the bounded waits are those of
-// the general kernel: thread t owns query t of a 128-query tile and lane t
-// of tensor memory; one elected thread issues the MMAs.
+// Tiles, weights, activations in tensor memory and the bounded waits are those
+// of the general kernel: thread t owns query t of a 128-query tile and lane t
+// of tensor memory; one elected thread issues the MMAs. Against activation
+// tiles in shared memory with one warp waiting for the MMAs and a second group
+// barrier a layer (GB300, 2^22 queries): split BF16 165 -> 146 us.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -152,7 +154,7 @@ __device__ __forceinline__ float2 norm_pair(float2 kap) {
 // mix (or NULL): rows (lambda, kappa, theta, phi) of lobes i, i + 1 of
 // query j are written.
 __device__ __forceinline__ void decode_pair(float2 lam, float2 rk, float2 rt, float2 rp, LobePair& L,
-                                            float* __restrict__ mix, int i, int64_t ld, int64_t j) {
+                                            float* __restrict__ mix, int i, int64_t ld, uint32_t j) {
     L.lam = lam;
     // kappa = softplus(k') = max(k', 0) + ln(1 + e^{-|k'|})
     const float2 q = ex2x2(mul2(make_float2(fabsf(rk.x), fabsf(rk.y)), f2(-kL2E)));
@@ -208,43 +210,24 @@ __device__ __forceinline__ float2 pair_log_terms(const LobePair& L, float2 logit
 }
 
 // Tile groups per CTA: one CTA per SM, each group of 128 threads walks its
-// own tiles with its own activation tile, tensor-memory columns, MMA
-// barrier and named CTA barrier, sharing one copy of the weights and of the
-// grid table in shared memory.
+// own tiles with its own tensor-memory columns, MMA barrier and named CTA
+// barrier, sharing one copy of the weights and of the grid table in shared
+// memory. A group's columns: 32 of accumulator, then the activations' high
+// parts and residuals (16 each: 32 values of 16 bits).
 constexpr int kGroups = 8;
-
-// Named barrier of group g (id 0 is the CTA-wide __syncthreads).
-__device__ __forceinline__ void group_sync(int g) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kThreads) : "memory");
-}
-// Barrier of group g that also ORs a predicate over its threads.
-__device__ __forceinline__ bool group_sync_or(int g, bool p) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred q, o;\n\t"
-        "setp.ne.u32 q, %3, 0;\n\t"
-        "bar.red.or.pred o, %1, %2, q;\n\t"
-        "selp.u32 %0, 1, 0, o;\n\t}\n"
-        : "=r"(r)
-        : "r"(1 + g), "r"(kThreads), "r"((uint32_t)p)
-        : "memory");
-    return r != 0;
-}
+constexpr uint32_t kGroupCols = 64;
 
 // Shared-memory layout of the CTA (byte offsets).
 struct TinyLayout {
-    uint32_t grid, a, a_stride, bars, bytes;
+    uint32_t grid, bars, bytes;
 };
 
 __host__ __device__ inline TinyLayout tiny_layout(const TcCfg& c, uint32_t grid_bytes) {
     TinyLayout L;
-    const uint32_t nw = (c.split || c.f16) ? 2u : 1u;       // weight blobs
-    const uint32_t na = c.split ? 2u : 1u;                  // activation tiles
-    L.grid = nw * c.w_bytes;                                // weights first (hi, then lo)
-    L.a = (L.grid + grid_bytes + 1023u) & ~1023u;           // per-group activation tiles
-    L.a_stride = na * c.a_bytes;                            // hi tile, then its residual
-    L.bars = L.a + (uint32_t)kGroups * L.a_stride;          // [0] weights + grid, [1 + g] MMA
-    L.bytes = L.bars + 8u * (1u + kGroups) + 16u;           // + tensor-memory slot
+    const uint32_t nw = (c.split || c.f16) ? 2u : 1u;  // weight blobs
+    L.grid = nw * c.w_bytes;                           // weights first (hi, then lo)
+    L.bars = (L.grid + grid_bytes + 15u) & ~15u;       // [0] weights + grid, [1 + g] MMA
+    L.bytes = L.bars + 8u * (1u + kGroups) + 16u;      // + tensor-memory slot
     return L;
 }
 
@@ -264,7 +247,6 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
     const int warp = t >> 5;             // warp within the group (its TMEM lane quarter)
     uint8_t* sW = smem;
     const uint2* sG = reinterpret_cast<const uint2*>(smem + lay.grid);
-    uint8_t* sA = smem + lay.a + (uint32_t)g * lay.a_stride;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.bars);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 1 + kGroups);
     const uint32_t bar_w = smem_u32(&bars[0]);
@@ -272,7 +254,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
 
     if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(32u * kGroups)
+                     "r"(kGroupCols * kGroups)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -284,8 +266,8 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // This group's 32 tensor-memory columns.
-    const uint32_t tmem = *tslot + 32u * (uint32_t)g;
+    // This group's tensor-memory columns: accumulator, activations.
+    const uint32_t tmem = *tslot + kGroupCols * (uint32_t)g, act = tmem + 32u;
     if (threadIdx.x == 0) {
         // Weights and grid table: two bulk copies on one barrier.
         const uint32_t wb = (uint32_t)nw * tc.w_bytes;
@@ -310,54 +292,51 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
     grid_dep_launch();
     bool ok = !__syncthreads_or(threadIdx.x < 32 && !mbar_wait_bounded(bar_w, 0));
     uint32_t phase = 0;
+    bool issued = false;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    // This thread's row in the K-major activation tile: 16-column layout
-    // (layer 0) and 32-column layout (layers 1 and 2); chunk c of 8 columns
-    // is 128 bytes further.
-    const uint32_t row16 = (uint32_t)((t >> 3) * 256 + (t & 7) * 16);
-    const uint32_t row32 = (uint32_t)((t >> 3) * 512 + (t & 7) * 16);
-    const uint32_t lo_off = SPLIT ? tc.a_bytes : 0u;
     const int D = tc.base.level_res[0];
     const uint32_t uD = (uint32_t)D, uD2 = uD * uD;
     const int np0 = tc.layer[0].Np, np1 = tc.layer[1].Np;
 
-    int64_t ntiles = qb.total_tiles, n0 = qb.seg[0].n;
+    // Tiles and queries of a segment in 32 bits: batches hold at most 2^31
+    // queries.
+    uint32_t ntiles = (uint32_t)qb.total_tiles, n0 = (uint32_t)qb.seg[0].n;
     if (qb.n_dev) {
-        n0 = *qb.n_dev;
-        ntiles = (n0 + kTile - 1) / kTile;
+        n0 = (uint32_t)*qb.n_dev;
+        ntiles = (n0 + (kTile - 1)) / kTile;
     }
-    const int64_t stride = (int64_t)gridDim.x * kGroups;
-    for (int64_t tile = (int64_t)blockIdx.x * kGroups + g; ok && tile < ntiles; tile += stride) {
+    const uint32_t stride = gridDim.x * (uint32_t)kGroups;
+    // Tiles are dealt to the CTAs first and to a CTA's groups second.
+    for (uint32_t tile = blockIdx.x + (uint32_t)g * gridDim.x; tile < ntiles; tile += stride) {
         int sg = 0;
-        while (sg + 1 < qb.nseg && tile >= qb.seg[sg + 1].tile0) ++sg;
+        while (sg + 1 < qb.nseg && tile >= (uint32_t)qb.seg[sg + 1].tile0) ++sg;
         const QuerySeg& S = qb.seg[sg];
-        const int64_t n = (sg == 0 && qb.n_dev) ? n0 : S.n;
+        const uint32_t n = (sg == 0 && qb.n_dev) ? n0 : (uint32_t)S.n;
         const int64_t ld = S.ld;
-        const int64_t j = (tile - S.tile0) * kTile + t;
+        const uint32_t base = (tile - (uint32_t)S.tile0) * kTile, j = base + t;
         const bool valid = j < n;
         if (warp == 3) {
             // Into L2 while this tile is encoded and run through the MLP: its
             // uniforms (or directions) and the group's next tile's positions.
             const int lane = t & 31, r = lane >> 2;
-            const int64_t b0 = (tile - S.tile0) * kTile + 32 * (lane & 3);
+            const uint32_t b0 = base + 32 * (lane & 3);
             if (r < 4) {
                 if ((r < 3 || S.ufrac > 0.0f) && b0 < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.uin + r * ld + b0));
             } else if (r < 7) {
-                const int64_t nt = tile + stride;
+                const uint32_t nt = tile + stride;
                 if (nt < ntiles) {
                     int s2 = sg;
-                    while (s2 + 1 < qb.nseg && nt >= qb.seg[s2 + 1].tile0) ++s2;
+                    while (s2 + 1 < qb.nseg && nt >= (uint32_t)qb.seg[s2 + 1].tile0) ++s2;
                     const QuerySeg& S2 = qb.seg[s2];
-                    const int64_t b2 = (nt - S2.tile0) * kTile + 32 * (lane & 3);
-                    const int64_t n2 = (s2 == 0 && qb.n_dev) ? n0 : S2.n;
+                    const uint32_t b2 = (nt - (uint32_t)S2.tile0) * kTile + 32 * (lane & 3);
+                    const uint32_t n2 = (s2 == 0 && qb.n_dev) ? n0 : (uint32_t)S2.n;
                     if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + (r - 4) * S2.ld + b2));
                 }
             }
         }
         // ---- encode (Sec. 5.1, Eq. 11): the 8 corners of the cell from the
-        // shared-memory table, blended in FP32, written as this row's first
-        // 8-column chunk (4 features, 4 zeros); the second chunk of the
-        // 16-column input is zero.
+        // shared-memory table, blended in FP32, stored as this lane's 16-value
+        // input (4 features, 12 zeros).
         {
             float x = 0.0f, y = 0.0f, z = 0.0f;
             if (valid) {
@@ -387,48 +366,51 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
             uint32_t h01, h23, l01 = 0u, l23 = 0u;
             feat_pair<OPS>(a01.x, a01.y, h01, l01);
             feat_pair<OPS>(a23.x, a23.y, h23, l23);
-            *reinterpret_cast<uint4*>(sA + row16) = make_uint4(h01, h23, 0u, 0u);
-            *reinterpret_cast<uint4*>(sA + row16 + 128) = make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t h[8] = {h01, h23, 0u, 0u, 0u, 0u, 0u, 0u};
+            __syncwarp();
+            tmem_st(act + lane_base, h);
             if (SPLIT) {
-                *reinterpret_cast<uint4*>(sA + lo_off + row16) = make_uint4(l01, l23, 0u, 0u);
-                *reinterpret_cast<uint4*>(sA + lo_off + row16 + 128) = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t lo[8] = {l01, l23, 0u, 0u, 0u, 0u, 0u, 0u};
+                tmem_st(act + 16u + lane_base, lo);
             }
+            tmem_wait_st();
         }
-        fence_async_smem();
         tc_fence_before();
-        group_sync(g);
+        if (tc_group_sync_or(g, !ok)) {
+            ok = false;
+            break;
+        }
         uint32_t rawu[16];
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
             const TcLayer& ly = tc.layer[l];
             if (t == 0) {
                 tc_fence_after();
-                // Descriptors of K step s are those of step 0 with the start
-                // address 256 bytes (16 units) further.
-                const uint64_t ad = umma_desc(smem_u32(sA), 128u, (uint32_t)(ly.Kp >> 3) * 128u);
+                // K step s: eight activation columns on, weight descriptors
+                // with the start address 256 bytes (16 units) further.
                 const uint64_t bd = umma_desc(smem_u32(sW) + ly.w_off, 128u, (uint32_t)(ly.Kp >> 3) * 128u);
-                const uint64_t bl = bd + (uint64_t)(tc.w_bytes >> 4), al = ad + (uint64_t)(lo_off >> 4);
+                const uint64_t bl = bd + (uint64_t)(tc.w_bytes >> 4);
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
                     if (s < (ly.Kp >> 4)) {
                         const uint64_t o = (uint64_t)(16 * s);
-                        mma_bf16(tmem, ad + o, bd + o, ly.idesc, s > 0 ? 1u : 0u);
-                        if (OPS != kOpsBf16) mma_bf16(tmem, ad + o, bl + o, ly.idesc, 1u);
-                        if (SPLIT) mma_bf16(tmem, al + o, bd + o, ly.idesc, 1u);
+                        const uint32_t a = act + 8u * (uint32_t)s;
+                        mma_tmem_a(tmem, a, bd + o, ly.idesc, s > 0 ? 1u : 0u);
+                        if (OPS != kOpsBf16) mma_tmem_a(tmem, a, bl + o, ly.idesc, 1u);
+                        if (SPLIT) mma_tmem_a(tmem, a + 16u, bd + o, ly.idesc, 1u);
                     }
                 }
                 mma_commit(bar_mma);
             }
-            // Warp 0 of the group waits on the MMA barrier; the group's other
-            // warps wait in its named barrier, which also passes the outcome.
-            const bool done = warp != 0 || mbar_wait_bounded(bar_mma, phase);
+            issued = true;
+            // Every warp waits on the MMAs' barrier; a wait that gives up is
+            // made known to the group at its next barrier.
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_limit(bar_mma, phase, 1ll << 32));
             phase ^= 1u;
-            ok = !group_sync_or(g, !done);
-            if (!ok) break;
             tc_fence_after();
             if (l < 2) {
                 // ReLU, BF16 high part and residual of this row's outputs,
-                // as the next layer's input (32-column layout).
+                // as the next layer's input.
                 const int np = l == 0 ? np0 : np1;
 #pragma unroll
                 for (int c0 = 0; c0 < 32; c0 += 16) {
@@ -440,25 +422,23 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
                             relu_pair<OPS>(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), hi[i], lo[i]);
-                        const uint32_t o = row32 + (uint32_t)(c0 >> 3) * 128u;
-                        *reinterpret_cast<uint4*>(sA + o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                        *reinterpret_cast<uint4*>(sA + o + 128) = make_uint4(hi[4], hi[5], hi[6], hi[7]);
-                        if (SPLIT) {
-                            *reinterpret_cast<uint4*>(sA + lo_off + o) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                            *reinterpret_cast<uint4*>(sA + lo_off + o + 128) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
-                        }
+                        tmem_st(act + lane_base + (uint32_t)(c0 >> 1), hi);
+                        if (SPLIT) tmem_st(act + 16u + lane_base + (uint32_t)(c0 >> 1), lo);
                     }
                 }
-                fence_async_smem();
+                tmem_wait_st();
                 tc_fence_before();
-                group_sync(g);
+                if (tc_group_sync_or(g, !ok)) {
+                    ok = false;
+                    break;
+                }
             } else {
                 tmem_ld16(tmem + lane_base, rawu);
                 tmem_wait16(rawu);
                 tc_fence_before();
             }
         }
-        if (!ok) break;
+        // (after a wait that gave up the loop ends at the next barrier)
         // ---- decode (Table 1), sample (Sec. 5.3) and density (Eq. 4).
         float r[16];
 #pragma unroll
@@ -542,14 +522,14 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
         // for group 0, the weights' and grid's bulk copies).
         if (warp == 0) {
             if (g == 0) (void)mbar_wait_bounded(bar_w, 0);
-            (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
+            if (issued) (void)mbar_wait_bounded(bar_mma, phase ^ 1u);
         }
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x < 32) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(32u * kGroups)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(kGroupCols * kGroups)
                      : "memory");
     }
 }
@@ -559,11 +539,13 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
 bool tiny_qualifies(const TcCfg& c) {
     const DevCfg& d = c.base;
     const uint32_t grid_bytes = (uint32_t)d.level_res[0] * d.level_res[0] * d.level_res[0] * 8u;
+    // Grids up to the size at which this kernel has been compared with the
+    // general one (90 KB of table with two activation parts, 154 with one).
+    const uint32_t most = (227u - 64u * (uint32_t)c.parts) * 1024u - 88u;
     return !c.fp32 && d.mode == NPM_RADIANCE && d.n_levels == 1 && d.feat == 4 && (d.dense_mask & 1u) && d.n_layers == 3 &&
            d.K == 4 && d.kappa_act == NPM_SOFTPLUS && c.layer[0].Kp == 16 && c.layer[0].Np <= 32 &&
            c.layer[1].Kp == 32 && c.layer[1].Np <= 32 && c.layer[2].Kp == 32 && c.layer[2].Np == 16 &&
-           c.a0_bytes == 0 && c.a_bytes == (uint32_t)(kTile * 32 * 2) && grid_bytes % 16u == 0 &&
-           tiny_layout(c, grid_bytes).bytes <= 227u * 1024u;
+           grid_bytes % 16u == 0 && ((c.wparts * c.w_bytes + grid_bytes + 1023u) & ~1023u) <= most;
 }
 
 cudaError_t launch_tiny(const TcCfg& c, const __half* grid_h, const uint8_t* wblob, QueryBatch& qb,
@@ -587,7 +569,7 @@ cudaError_t launch_tiny(const TcCfg& c, const __half* grid_h, const uint8_t* wbl
     }
     qb.total_tiles = t0;
     const int64_t hint = qb.n_dev ? (max_n + kTile - 1) / kTile : t0;
-    int64_t g = (hint + kGroups - 1) / kGroups;
+    int64_t g = hint;  // fewer tiles than SMs: one each
     if (g > sms) g = sms;
     if (g < 1) g = 1;
     return launch_maybe_pdl(kern, dim3((unsigned)g), dim3(kThreads * kGroups), smem, st, pdl, c,
