@@ -431,38 +431,37 @@ __device__ __forceinline__ void scatter_levels(const DevCfg& cfg, float* __restr
 }
 
 // Grid features of a training batch for 2-feature grids (Sec. 5.1, Eq. 11):
-// enc[j][2l + f] = sum_corners w_c V_l[corner][f] from the FP32 master
-// table, in the FP32 arithmetic of tc_encode (same corners, weights and FMA
-// order). One thread per (sample, group of LPT levels), all of a group's
-// corner loads in flight; a full-occupancy kernel without shared memory
-// keeps the whole L1 and many warps for these random L2 reads, which the
-// training kernel (one CTA per SM holding most of the shared memory) cannot.
-template <int LPT>
+// enc[l][j] = sum_corners w_c V_l[corner] (two values) from the FP32 master
+// table. One thread per sample and kEncLevels levels (blockIdx.y: level
+// group), so that a warp reads and writes one level at a time; a
+// full-occupancy kernel without shared memory keeps the whole L1 and many
+// warps for these random L2 reads, which the training kernel (one CTA per SM
+// holding most of the shared memory) cannot. Bound by the L1's one request
+// per lane and cycle. 2^19 samples of the 16-level grid (GB300): 138 us with
+// 2 levels a thread, 139 with 1, 150 with 4; 174 with a warp's lanes spread
+// over the levels of four samples; whole 32-byte sectors per pair (5 instead
+// of 6 requests a level, more registers) 154.
+constexpr int kEncLevels = 2;
+
 __global__ void __launch_bounds__(256) k_train_encode(const __grid_constant__ DevCfg cfg,
                                                       const float* __restrict__ grid32, int64_t n,
                                                       int64_t ld, const float* __restrict__ pos,
-                                                      float* __restrict__ enc) {
-    const int ng = (cfg.n_levels + LPT - 1) / LPT;
-    const int G = cfg.grid_feats;
-    const int64_t total = n * ng;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = i / ng;
-        const int l0 = (int)(i - j * ng) * LPT;
-        const float x = pos[j], y = pos[ld + j], z = pos[2 * ld + j];
-        Cell cs[LPT];
-        Level2<float> v[LPT];
+                                                      float2* __restrict__ enc) {
+    const int l0 = (int)blockIdx.y * kEncLevels;
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const float x = pos[j], y = pos[ld + j], z = pos[2 * ld + j];
+    Cell cs[kEncLevels];
+    Level2<float> v[kEncLevels];
 #pragma unroll
-        for (int r = 0; r < LPT; ++r)
-            if (l0 + r < cfg.n_levels) {
-                cs[r] = make_cell(x, y, z, cfg.level_res[l0 + r]);
-                v[r].load_table(cfg, grid32, l0 + r, cs[r]);
-            }
+    for (int r = 0; r < kEncLevels; ++r)
+        if (l0 + r < cfg.n_levels) {
+            cs[r] = make_cell(x, y, z, cfg.level_res[l0 + r]);
+            v[r].load_table(cfg, grid32, l0 + r, cs[r]);
+        }
 #pragma unroll
-        for (int r = 0; r < LPT; ++r)
-            if (l0 + r < cfg.n_levels)
-                *reinterpret_cast<float2*>(enc + j * G + 2 * (l0 + r)) = v[r].blend(cs[r]);
-    }
+    for (int r = 0; r < kEncLevels; ++r)
+        if (l0 + r < cfg.n_levels) enc[(int64_t)(l0 + r) * n + j] = v[r].blend(cs[r]);
 }
 
 // CTAs per SM of the one-group instances: three for the small four-lobe one
@@ -485,7 +484,7 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
     const uint8_t* __restrict__ wblob, int64_t n, int64_t ld, const float* __restrict__ pos,
     const float* __restrict__ aux, const float* __restrict__ dir, const float* __restrict__ rad,
     const float* __restrict__ spdf, const float* __restrict__ dlogv, float inv_n, float* __restrict__ grad,
-    int64_t mlp_off, double* __restrict__ loss, int* __restrict__ status, const float* __restrict__ enc) {
+    int64_t mlp_off, double* __restrict__ loss, int* __restrict__ status, const float2* __restrict__ enc) {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int KH = KMAX / 2;
     const int g = G > 1 ? (int)(threadIdx.x >> 8) : 0;
@@ -587,12 +586,10 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
         if (F2 && enc) {
             // This half's grid features (k_train_encode), then the
             // product-mode inputs and the padding.
-            const float* er = enc + (valid ? j : 0) * (int64_t)cfg.grid_feats;
             float2 ev[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                ev[q] = (valid && lv0 + q < lv1) ? __ldg(reinterpret_cast<const float2*>(er + 2 * (lv0 + q)))
-                                                 : make_float2(0.0f, 0.0f);
+                ev[q] = (valid && lv0 + q < lv1) ? __ldg(enc + (int64_t)(lv0 + q) * n + j) : make_float2(0.0f, 0.0f);
             tc_encode<F2>(tc, grid32, j, valid, ld, pos, aux, tiles, row, tt.slot[L], lv1, lv1, half == 1);
 #pragma unroll
             for (int q = 0; q < 8; ++q)
@@ -908,7 +905,7 @@ struct TcState {
     // Grid features of a training batch (max_batch x grid_feats FP32) for
     // 2-feature grids, written by k_train_encode; NULL: the training kernel
     // gathers them itself.
-    float* enc = nullptr;
+    float2* enc = nullptr;
 };
 
 static int pad16(int v) { return (v + 15) / 16 * 16; }
@@ -1149,17 +1146,10 @@ static cudaError_t launch_train_tc(npm_handle* h, int64_t n, int64_t ld, const f
     const int64_t slots = (int64_t)per_sm * sms;
     const int g = (int)(ntiles < slots ? ntiles : slots);
     int* status = reinterpret_cast<int*>(h->scalars + 8);
-    const float* enc = nullptr;
+    const float2* enc = nullptr;
     if (F2 && s->enc && n <= h->cfg.max_batch) {
-        // Levels per thread: two (64 registers, more warps) measured a little
-        // faster than four; tuning override NPM_ENC_LPT (2 or 4).
-        static std::atomic<int> env_lpt{INT32_MIN + 1};
-        const int lpt = env_override("NPM_ENC_LPT", env_lpt) == 4 ? 4 : 2;
-        const int64_t items = n * ((h->dc.n_levels + lpt - 1) / lpt);
-        int64_t eg = (items + 255) / 256;
-        if (eg > (int64_t)sms * 16) eg = (int64_t)sms * 16;
-        if (lpt == 2) k_train_encode<2><<<(int)eg, 256, 0, st>>>(h->dc, h->params, n, ld, pos, s->enc);
-        else k_train_encode<4><<<(int)eg, 256, 0, st>>>(h->dc, h->params, n, ld, pos, s->enc);
+        const dim3 grid((unsigned)((n + 255) / 256), (unsigned)((h->dc.n_levels + kEncLevels - 1) / kEncLevels));
+        k_train_encode<<<grid, 256, 0, st>>>(h->dc, h->params, n, ld, pos, s->enc);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         enc = s->enc;
