@@ -81,15 +81,18 @@ __device__ __forceinline__ int64_t bounded_slot(int64_t j, int64_t) { return j; 
 
 // ------------------------------------------------------ lattice (Eq. 11)
 
-// Cell and fraction along one axis: x clamped to [0,1] (NaN -> 0),
-// p = x * (D - 1) with one round-to-nearest multiply, cell = min(floor p, D-2).
-__device__ __forceinline__ void lattice_axis(float x, int D, uint32_t& cell, float& frac) {
-    float xa = fminf(fmaxf(x, 0.0f), 1.0f);
-    float p = __fmul_rn(xa, (float)(D - 1));
-    int c = (int)floorf(p);
-    c = c > D - 2 ? D - 2 : c;
-    cell = (uint32_t)c;
-    frac = __fsub_rn(p, (float)c);
+// A coordinate clamped to [0,1] (NaN -> 0).
+__device__ __forceinline__ float clamp01(float x) { return fminf(fmaxf(x, 0.0f), 1.0f); }
+
+// Cell and fraction along one axis at xa in [0,1]: p = xa * (D - 1) with one
+// round-to-nearest multiply, cell = min(floor p, D - 2). Adding 2^23 rounded
+// down leaves floor p (below 2^23) in the significand: floor and both
+// conversions in full-rate additions.
+__device__ __forceinline__ void lattice_axis(float xa, int D, uint32_t& cell, float& frac) {
+    const float p = __fmul_rn(xa, (float)(D - 1));
+    const float t = fminf(__fadd_rd(p, 8388608.0f), __uint_as_float(0x4b000000u + (uint32_t)(D - 2)));
+    cell = __float_as_uint(t) - 0x4b000000u;
+    frac = __fsub_rn(p, __fsub_rn(t, 8388608.0f));
 }
 
 // Cell of a point at one level: lower lattice point and fractions.
@@ -98,12 +101,16 @@ struct Cell {
     float f[3];
 };
 
-__device__ __forceinline__ Cell make_cell(float x, float y, float z, int D) {
+// (x, y, z) clamped to [0,1]: once per point, not per level.
+__device__ __forceinline__ Cell make_cell_in(float x, float y, float z, int D) {
     Cell cl;
     lattice_axis(x, D, cl.c[0], cl.f[0]);
     lattice_axis(y, D, cl.c[1], cl.f[1]);
     lattice_axis(z, D, cl.c[2], cl.f[2]);
     return cl;
+}
+__device__ __forceinline__ Cell make_cell(float x, float y, float z, int D) {
+    return make_cell_in(clamp01(x), clamp01(y), clamp01(z), D);
 }
 
 // The 8 corners of a cell at level l (corner c: bit0 = +x, bit1 = +y,

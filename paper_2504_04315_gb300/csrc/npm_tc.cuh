@@ -271,6 +271,28 @@ __device__ __forceinline__ void store_one(uint8_t* sA, uint32_t off, float a, ui
     *reinterpret_cast<__nv_bfloat16*>(sA + lo_off + off) = __float2bfloat16_rn(a - __bfloat162float(hb));
 }
 
+constexpr float kL2E = 1.4426950408889634f;  // log2(e)
+constexpr float kLn2 = 0.69314718055994531f;
+
+// Hardware approximations (PTX ex2/lg2/rcp/sin/cos .approx): e^x is
+// evaluated as 2^(x log2 e) with the scaling folded into the caller's FMA.
+__device__ __forceinline__ float hw_ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float hw_lg2(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float hw_rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+
 // Sampler of the reduced-precision path (Sec. 5.3, Jakob's inversion as in
 // vmf_sample) on the hardware approximations: 1 - e^{-2k} and log(1 + y) by
 // their series where the direct forms lose relative accuracy (2k < 0.1,
@@ -351,10 +373,44 @@ __device__ __forceinline__ Block32 load_block(const uint4* __restrict__ blk, uin
 // blended (a select on a loaded value, or a branch around one, would wait).
 //
 // From the table: a pair of x-neighbours in one load of twice the width where
-// they form an aligned pair (half of a level's; it may come swapped), else in
-// two.
+// they form an aligned pair (half of a level's), else in two.
 template <typename GT>
 struct Level2;
+
+// The four pairs of x-neighbours of a cell: entries a, b, whether they form an
+// aligned pair (then a is its first entry) and whether that comes swapped. On
+// a hashed level the neighbours i, i + 1 differ in bit 0 alone exactly when i
+// is even, for all four pairs alike; on a dense one they are always adjacent.
+struct Pairs {
+    uint32_t a[4], b[4], pair[4], swap;
+    __device__ __forceinline__ Pairs(const DevCfg& cfg, int l, const Cell& cl) {
+        const uint32_t odd = (cfg.level_off[l] + cfg.grid_shift) & 1u;
+        swap = 0u;
+        if ((cfg.dense_mask >> l) & 1u) {
+            const uint32_t D = (uint32_t)cfg.level_res[l];
+            const uint32_t e = bounded_index(cl.c[0] + D * (cl.c[1] + D * cl.c[2]), D * D * D - D * D - D - 1u);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = e + ((i & 1) ? D : 0u) + ((i & 2) ? D * D : 0u);
+                b[i] = a[i] + 1u;
+                pair[i] = (a[i] ^ odd ^ 1u) & 1u;
+            }
+        } else {
+            const uint32_t hy0 = cl.c[1] * 2654435761u, hz0 = cl.c[2] * 805459861u;
+            const uint32_t hy[2] = {hy0, hy0 + 2654435761u}, hz[2] = {hz0, hz0 + 805459861u};
+            const uint32_t even = (cl.c[0] & 1u) == 0u && odd == 0u ? 1u : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t h = hy[i & 1] ^ hz[i >> 1];
+                const uint32_t e = (cl.c[0] ^ h) & cfg.table_mask;
+                b[i] = ((cl.c[0] + 1u) ^ h) & cfg.table_mask;
+                swap |= (e & even) << i;
+                a[i] = e & ~even;
+                pair[i] = even;
+            }
+        }
+    }
+};
 
 __device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const Cell& cl, int c);
 
@@ -370,24 +426,18 @@ struct Level2<float> {
     }
     __device__ __forceinline__ void load_table(const DevCfg& cfg, const float* __restrict__ table, int l,
                                                const Cell& cl) {
-        const uint32_t off = cfg.level_off[l];
-        const float* g = table + (size_t)off * 2;
-        const uint32_t odd = (off + cfg.grid_shift) & 1u;
-        swap = 0u;
+        const float* g = table + (size_t)cfg.level_off[l] * 2;
+        const Pairs p(cfg, l, cl);
+        swap = p.swap;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = corner_idx1(cfg, l, cl, 2 * i), b = corner_idx1(cfg, l, cl, 2 * i + 1);
-            const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
-            const uint32_t pair = (hi - lo == 1u && (lo & 1u) == odd) ? 1u : 0u;
-            swap |= (pair && a > b ? 1u : 0u) << i;
+        for (int i = 0; i < 4; ++i)
             asm("{\n\t.reg .pred p;\n\t"
                 "setp.ne.u32 p, %6, 0;\n\t"
                 "@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t"
                 "@!p ld.global.nc.v2.f32 {%0, %1}, [%4];\n\t"
                 "@!p ld.global.nc.v2.f32 {%2, %3}, [%5];\n\t}\n"
                 : "=f"(r[4 * i]), "=f"(r[4 * i + 1]), "=f"(r[4 * i + 2]), "=f"(r[4 * i + 3])
-                : "l"(g + 2 * (size_t)(pair ? lo : a)), "l"(g + 2 * (size_t)b), "r"(pair));
-        }
+                : "l"(g + 2 * (size_t)p.a[i]), "l"(g + 2 * (size_t)p.b[i]), "r"(p.pair[i]));
     }
     __device__ __forceinline__ float2 blend(const Cell& cl) const {
         float w[8];
@@ -418,24 +468,18 @@ struct Level2<__half> {
     }
     __device__ __forceinline__ void load_table(const DevCfg& cfg, const __half* __restrict__ table, int l,
                                                const Cell& cl) {
-        const uint32_t off = cfg.level_off[l];
-        const uint32_t* g = reinterpret_cast<const uint32_t*>(table) + off;
-        const uint32_t odd = (off + cfg.grid_shift) & 1u;
-        swap = 0u;
+        const uint32_t* g = reinterpret_cast<const uint32_t*>(table) + cfg.level_off[l];
+        const Pairs p(cfg, l, cl);
+        swap = p.swap;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = corner_idx1(cfg, l, cl, 2 * i), b = corner_idx1(cfg, l, cl, 2 * i + 1);
-            const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
-            const uint32_t pair = (hi - lo == 1u && (lo & 1u) == odd) ? 1u : 0u;
-            swap |= (pair && a > b ? 1u : 0u) << i;
+        for (int i = 0; i < 4; ++i)
             asm("{\n\t.reg .pred p;\n\t"
                 "setp.ne.u32 p, %4, 0;\n\t"
                 "@p ld.global.nc.v2.b32 {%0, %1}, [%2];\n\t"
                 "@!p ld.global.nc.b32 %0, [%2];\n\t"
                 "@!p ld.global.nc.b32 %1, [%3];\n\t}\n"
                 : "=r"(r[2 * i]), "=r"(r[2 * i + 1])
-                : "l"(g + (pair ? lo : a)), "l"(g + b), "r"(pair));
-        }
+                : "l"(g + p.a[i]), "l"(g + p.b[i]), "r"(p.pair[i]));
     }
     __device__ __forceinline__ float2 blend(const Cell& cl) const {
         float w[8];

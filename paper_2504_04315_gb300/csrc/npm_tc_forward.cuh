@@ -232,7 +232,7 @@ __device__ __forceinline__ void product_inputs(const QuerySeg& S, uint32_t j, bo
     e[21] = 0.0f;
 }
 
-// The network input of query j at (x, y, z): this thread's row of the activation
+// The network input of query j at (x, y, z) in the unit box: this thread's row of the activation
 // columns, padded with zeros to the layer's kp values. FEAT: features per
 // level (2 or 4), or 0 for any.
 template <int FEAT, int OPS>
@@ -257,7 +257,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             Level2<typename OpsTraits<OPS>::GridT> v[NF];
 #pragma unroll
             for (int i = 0; i < NF; ++i) {
-                cl[i] = make_cell(x, y, z, cfg.level_res[l + i]);
+                cl[i] = make_cell_in(x, y, z, cfg.level_res[l + i]);
                 gather_level2(tc, grid, l + i, cl[i], v[i]);
             }
             uint32_t p[NF][P];
@@ -269,7 +269,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             put_pairs<OPS, NF>(act, pc, (uint32_t)l, p);
         }
         for (; l < L; ++l) {
-            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
             Level2<typename OpsTraits<OPS>::GridT> v;
             gather_level2(tc, grid, l, cl, v);
             const float2 a = v.blend(cl);
@@ -280,7 +280,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
     } else if (FEAT == 4 || F == 4 || F == 8) {
 #pragma unroll(FEAT == 4 ? 2 : 1)
         for (int l = 0; l < L; ++l) {
-            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
             for (int h = 0; h < (F >> 2); ++h) {
                 const float4 a = blend_level4(tc, grid, l, cl, F, h);
                 uint32_t p[2][P];
@@ -292,7 +292,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
     } else {
         RowPacker<OPS> row{act, pc, 0, 0.0f};
         for (int l = 0; l < L; ++l) {
-            const Cell cl = make_cell(x, y, z, cfg.level_res[l]);
+            const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
             if (F == 2) {
                 Level2<typename OpsTraits<OPS>::GridT> v;
                 gather_level2(tc, grid, l, cl, v);
@@ -345,10 +345,73 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
 
 // --------------------------------------------------------------- decode
 
+// Two lobes decoded (Table 1) for the density in packed FP32, two lobes an
+// instruction, in the arithmetic of decode_lobe_fast, vmf_scaled_norm_fast and
+// vmf_eval_fast: hardware exponential, logarithm, reciprocal, sine and cosine
+// on arguments in their accurate ranges. theta = pi s(t'), phi = pi + ph with
+// ph = pi (2 s(p') - 1); the mean is (-nx, -ny, -nz).
+struct LobePair2 {
+    float2 kap, th, ph, nx, ny, nz;
+
+    template <typename Raw>
+    __device__ __forceinline__ void decode(int kappa_act, const Raw& raw, int i) {
+        const float2 rk = make_float2(raw(4 * i + 1), raw(4 * i + 5)), rt = make_float2(raw(4 * i + 2), raw(4 * i + 6)),
+                     rp = make_float2(raw(4 * i + 3), raw(4 * i + 7));
+        if (kappa_act == NPM_EXP) {
+            const float2 e = __fmul2_rn(rk, f2(kL2E));
+            kap = make_float2(hw_ex2(e.x), hw_ex2(e.y));
+        } else {
+            // max(t, 0) + ln(1 + e^{-|t|})
+            const float2 e = __fmul2_rn(make_float2(fabsf(rk.x), fabsf(rk.y)), f2(-kL2E));
+            const float2 q = __fadd2_rn(make_float2(hw_ex2(e.x), hw_ex2(e.y)), f2(1.0f));
+            kap = __ffma2_rn(make_float2(hw_lg2(q.x), hw_lg2(q.y)), f2(kLn2),
+                             make_float2(fmaxf(rk.x, 0.0f), fmaxf(rk.y, 0.0f)));
+        }
+        const float2 st = logistic2(rt), sp = logistic2(rp);
+        th = __fmul2_rn(st, f2(kPi));
+        ph = __fmul2_rn(__ffma2_rn(sp, f2(2.0f), f2(-1.0f)), f2(kPi));
+        const float2 a = __fadd2_rn(th, f2(-0.5f * kPi));  // sin(th) = cos(a), cos(th) = -sin(a)
+        float sa0, ca0, sa1, ca1, sb0, cb0, sb1, cb1;
+        __sincosf(a.x, &sa0, &ca0);
+        __sincosf(a.y, &sa1, &ca1);
+        __sincosf(ph.x, &sb0, &cb0);
+        __sincosf(ph.y, &sb1, &cb1);
+        const float2 sth = make_float2(ca0, ca1);
+        nx = __fmul2_rn(sth, make_float2(cb0, cb1));
+        ny = __fmul2_rn(sth, make_float2(sb0, sb1));
+        nz = make_float2(sa0, sa1);
+    }
+    __device__ __forceinline__ static float2 logistic2(float2 t) {
+        const float2 e = __fmul2_rn(t, f2(-kL2E));
+        const float2 q = __fadd2_rn(make_float2(hw_ex2(e.x), hw_ex2(e.y)), f2(1.0f));
+        return make_float2(hw_rcp(q.x), hw_rcp(q.y));
+    }
+    // kappa (mu . w - 1) log2(e)
+    __device__ __forceinline__ float2 exponent(const float (&w)[3]) const {
+        const float2 d = __ffma2_rn(nz, f2(w[2]), __ffma2_rn(ny, f2(w[1]), __fmul2_rn(nx, f2(w[0]))));  // -mu . w
+        return __fmul2_rn(__fmul2_rn(kap, __fadd2_rn(d, f2(1.0f))), f2(-kL2E));
+    }
+    // c(kappa) = kappa / (2 pi (1 - e^{-2 kappa}))
+    __device__ __forceinline__ float2 norm() const {
+        const float2 k = kap;
+        float2 s = __ffma2_rn(k, f2(4.0f / 15.0f), f2(-2.0f / 3.0f));
+        s = __ffma2_rn(k, s, f2(4.0f / 3.0f));
+        s = __ffma2_rn(k, s, f2(-2.0f));
+        s = __fmul2_rn(k, __ffma2_rn(k, s, f2(2.0f)));
+        const float2 x = __fmul2_rn(k, f2(-2.0f * kL2E));
+        const float2 e = __ffma2_rn(make_float2(hw_ex2(x.x), hw_ex2(x.y)), f2(-1.0f), f2(1.0f));
+        const float2 em = __fmul2_rn(make_float2(k.x < 0.05f ? s.x : e.x, k.y < 0.05f ? s.y : e.y), f2(2.0f * kPi));
+        const float2 c = __fmul2_rn(k, make_float2(hw_rcp(em.x), hw_rcp(em.y)));
+        const float2 c0 = __ffma2_rn(k, f2(kInv4Pi), f2(kInv4Pi));  // kappa -> 0
+        return make_float2(k.x < 1e-6f ? c0.x : c.x, k.y < 1e-6f ? c0.y : c.y);
+    }
+};
+
 // Table 1, sampling (Sec. 5.3) and density (Eq. 4) of one query from its raw
 // outputs. Only the chosen lobe is decoded for the sample; the density then
-// decodes lobe by lobe, so that no array of decoded lobes stays live (nine
-// lobe decodes instead of eight, half the registers).
+// decodes pair by pair, so that no array of decoded lobes stays live (nine
+// lobe decodes instead of eight, half the registers). Pairs past the last
+// lobe read the zeros of the padded last layer.
 // u: uniforms when sampling, direction when evaluating.
 template <int KMAX, bool FP32>
 __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&rawu)[KMAX / 4][16], const QuerySeg& S,
@@ -402,13 +465,16 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
         const float lnorm = mx + __logf(ssum);
         float m = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < KMAX; ++i)
+        for (int i = 0; i < KMAX; i += 2)
             if (i < K) {
-                Lobe lb;
-                decode_lobe_fast(cfg.kappa_act, raw(4 * i + 1), raw(4 * i + 2), raw(4 * i + 3), lb, nullptr, nullptr);
-                const float d = lb.mu[0] * w[0] + lb.mu[1] * w[1] + lb.mu[2] * w[2];
-                lam[i] = (raw(4 * i) - lnorm) + __logf(vmf_scaled_norm_fast(lb.kap)) + lb.kap * (d - 1.0f);
+                LobePair2 p;
+                p.decode(cfg.kappa_act, raw, i);
+                const float2 e = p.exponent(w), c = p.norm();
+                lam[i] = (raw(4 * i) - lnorm) + kLn2 * (hw_lg2(c.x) + e.x);
                 m = fmaxf(m, lam[i]);
+                lam[i + 1] = -INFINITY;
+                if (i + 1 < K) lam[i + 1] = (raw(4 * i + 4) - lnorm) + kLn2 * (hw_lg2(c.y) + e.y);
+                m = fmaxf(m, lam[i + 1]);
             }
         float s = 0.0f;
 #pragma unroll
@@ -417,19 +483,30 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
         pv = m + __logf(s);
     } else {
 #pragma unroll
-        for (int i = 0; i < KMAX; ++i)
+        for (int i = 0; i < KMAX; i += 2)
             if (i < K) {
-                Lobe lb;
-                float th, ph;
-                decode_lobe_fast(cfg.kappa_act, raw(4 * i + 1), raw(4 * i + 2), raw(4 * i + 3), lb, &th, &ph);
+                LobePair2 p;
+                p.decode(cfg.kappa_act, raw, i);
+                const bool two = i + 1 < K;
+                const float2 l = make_float2(lam[i], two ? lam[i + 1] : 0.0f);
                 if (S.mix && valid) {
                     float* mo = S.mix + (int64_t)(4 * i) * S.ld + j;
-                    mo[0] = lam[i];
-                    mo[S.ld] = lb.kap;
-                    mo[2 * S.ld] = th;
-                    mo[3 * S.ld] = ph;
+                    mo[0] = l.x;
+                    mo[S.ld] = p.kap.x;
+                    mo[2 * S.ld] = p.th.x;
+                    mo[3 * S.ld] = p.ph.x + kPi;
+                    if (two) {
+                        mo += 4 * S.ld;
+                        mo[0] = l.y;
+                        mo[S.ld] = p.kap.y;
+                        mo[2 * S.ld] = p.th.y;
+                        mo[3 * S.ld] = p.ph.y + kPi;
+                    }
                 }
-                pv += lam[i] * vmf_eval_fast(lb, vmf_scaled_norm_fast(lb.kap), w[0], w[1], w[2]);
+                const float2 e = p.exponent(w);
+                const float2 v = __fmul2_rn(l, __fmul2_rn(p.norm(), make_float2(hw_ex2(e.x), hw_ex2(e.y))));
+                pv += v.x;
+                if (two) pv += v.y;
             }
         if (sample && S.ufrac > 0.0f) pv = S.ufrac * kInv4Pi + (1.0f - S.ufrac) * pv;
     }
@@ -647,9 +724,9 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
         const bool valid = j < n;
         float x = 0.0f, y = 0.0f, z = 0.0f;
         if (valid) {
-            x = S.pos[j];
-            y = S.pos[S.ld + j];
-            z = S.pos[2 * S.ld + j];
+            x = clamp01(S.pos[j]);
+            y = clamp01(S.pos[S.ld + j]);
+            z = clamp01(S.pos[2 * S.ld + j]);
         }
         if (warp == 3) {
             // The group's next tile's positions into L2 (three 512-byte rows).

@@ -36,29 +36,8 @@ namespace tc {
 
 namespace {
 
-constexpr float kL2E = 1.4426950408889634f;  // log2(e)
-constexpr float kLn2 = 0.69314718055994531f;
-
-// Hardware approximations (PTX ex2/lg2/rcp/sin/cos .approx): e^x is
-// evaluated as 2^(x log2 e) with the scaling folded into the caller's FMA.
-__device__ __forceinline__ float hw_ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float hw_lg2(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float hw_rcp(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float2 ex2x2(float2 x) { return make_float2(hw_ex2(x.x), hw_ex2(x.y)); }
 __device__ __forceinline__ float2 rcpx2(float2 x) { return make_float2(hw_rcp(x.x), hw_rcp(x.y)); }
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
