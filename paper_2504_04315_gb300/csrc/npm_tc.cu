@@ -28,12 +28,8 @@ using namespace tc;
 
 namespace {
 
-// Training operand tiles (128 samples x columns, BF16) are stored in planes of
-// 8 columns: 2048 bytes a plane, 16 bytes a row. Core matrices (8 rows x 16
-// bytes) then lie 128 bytes apart along the rows and 2048 along the columns
-// in every tile, whatever its width, so that a tile and the residual tile
-// behind it are one operand of twice the columns.
-constexpr uint32_t kPlane = kTile * 16;
+// Place of a value in an operand tile stored in planes (kPlane): a tile and the
+// residual tile behind it are one operand of twice the columns.
 __device__ __forceinline__ uint32_t plane_off(int row, int col) {
     return (uint32_t)(col >> 3) * kPlane + (uint32_t)row * 16u + (uint32_t)(col & 7) * 2u;
 }
@@ -949,7 +945,6 @@ npm_status tc_create(npm_handle* h) {
     for (int l = 0; l < c.n_layers; ++l) maxkp = std::max(maxkp, t.layer[l].Kp);
     t.d_cols = (uint32_t)((maxnp + 31) / 32 * 32);
     t.a_cols = (uint32_t)(maxkp / 2);
-    t.g_cols = t.d_cols + nsplit * t.a_cols;
     // FP32 models that do not fit keep the CUDA-core kernels. In the other
     // modes the limit is part of the interface: 200 KB for the weights and one
     // activation tile per part (two where the encoding leaves whole 8-column
@@ -960,7 +955,7 @@ npm_status tc_create(npm_handle* h) {
     int hidden = 16;  // widest input of the layers that share a tile
     for (int l = sep0 ? 1 : 0; l < c.n_layers; ++l) hidden = std::max(hidden, t.layer[l].Kp);
     const uint32_t tile_bytes = (uint32_t)(kTile * (hidden + (sep0 ? t.layer[0].Kp : 0)) * 2);
-    if (fp32 ? nw * t.w_bytes > 200 * 1024 || t.g_cols > 512u
+    if (fp32 ? nw * t.w_bytes + (uint32_t)(kTile * maxkp * 2) > 224 * 1024
              : nw * t.w_bytes + nsplit * tile_bytes + 64 > 200 * 1024 || c.K > 16) {
         delete s;
         return NPM_ERR_UNSUPPORTED;

@@ -16,6 +16,11 @@ namespace npm {
 namespace tc {
 
 constexpr int kTile = 128;
+// Operand tiles in shared memory that the kernels write (128 rows x columns,
+// 16 bits) are stored in planes of 8 columns: kPlane bytes a plane, 16 bytes
+// a row. Core matrices (8 rows x 16 bytes) then lie 128 bytes apart along the
+// rows and kPlane along the columns in every tile, whatever its width.
+constexpr uint32_t kPlane = kTile * 16;
 constexpr int kThreads = 128;
 
 struct TcLayer {
@@ -39,7 +44,8 @@ struct TcCfg {
                        // FP32 path's sampler)
     // Tensor-memory columns of a forward tile group: d_cols of accumulator,
     // then one a_cols wide block per activation part (two 16-bit values to a
-    // column); g_cols in all.
+    // column; an instance may keep a third part in shared memory instead),
+    // g_cols in all (set per launch).
     uint32_t d_cols, a_cols, g_cols;
     // Corner blocks (below): bit l set where level l has them, and the level's
     // first block.
@@ -533,10 +539,11 @@ __device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const 
 
 // ------------------------------------------------------- forward kernels
 
-// Byte offset of the staging space behind the weights, the barriers and the
-// tensor-memory slot of a forward CTA of G tile groups.
+// Byte offset of the space behind the weights, the barriers and the
+// tensor-memory slot of a forward CTA of G tile groups (third activation
+// parts; staged raw outputs).
 __host__ __device__ inline uint32_t fwd_stage_off(uint32_t wbytes, int G) {
-    return (wbytes + 8u * (1u + (uint32_t)G) + 16u + 15u) & ~15u;
+    return (wbytes + 8u * (1u + (uint32_t)G) + 16u + 127u) & ~127u;
 }
 
 // The general forward in one operand format (npm_tc_forward.cuh; one

@@ -68,12 +68,9 @@ struct OpsTraits {
 };
 
 // Tile groups a CTA is compiled for: four at 128 registers; two for up to
-// sixteen lobes, whose raw outputs alone take 64; three at 168 for FP32 on
-// 2-feature grids (three is what the columns of 64-wide layers allow there,
-// and two levels' FP32 gathers in flight take the registers).
-__host__ __device__ constexpr int fwd_groups(int kmax, int feat, int ops) {
-    return kmax > 8 ? 2 : (ops == kThreeBf16 && feat == 2) ? 3 : 4;
-}
+// sixteen lobes, whose raw outputs alone take 64. FP32 on 2-feature grids also
+// has an instance of three at 168 (launch_fwd_ops).
+__host__ __device__ constexpr int fwd_groups(int kmax) { return kmax > 8 ? 2 : 4; }
 
 // ----------------------------------------------------------- operands
 
@@ -132,17 +129,38 @@ __device__ __forceinline__ void relu_split_pair(float a, float b, uint32_t (&p)[
     }
 }
 
-// N (1, 2, 4 or 8) operand pairs of this thread's row into the activation
-// columns col .. col + N of every part. All 32 lanes take part.
-template <int OPS, int N>
-__device__ __forceinline__ void put_pairs(uint32_t act, uint32_t part_cols, uint32_t col,
-                                          const uint32_t (&v)[N][OpsTraits<OPS>::parts]) {
+// Where a thread's row of the activations goes: its lane of the tensor-memory
+// columns, and (THIRD) its row of the third part's tile in shared memory, in
+// planes (kPlane): four 64-wide groups' accumulators and two parts fill the 512
+// columns.
+template <bool THIRD>
+struct ActRow {
+    uint32_t tmem, part_cols;
+    uint8_t* third;
+};
+
+// N operand pairs of this thread's row into the activation columns (two
+// values each) col .. col + N of every part. All 32 lanes take part.
+template <int OPS, bool THIRD, int N>
+__device__ __forceinline__ void put_pairs(const ActRow<THIRD>& act, uint32_t col, const uint32_t (&v)[N][OpsTraits<OPS>::parts]) {
 #pragma unroll
     for (int p = 0; p < OpsTraits<OPS>::parts; ++p) {
+        if (THIRD && p == 2) {
+            if constexpr (N == 8) {  // col is a multiple of 8
+                uint8_t* at = act.third + (col >> 2) * kPlane;
+                *reinterpret_cast<uint4*>(at) = make_uint4(v[0][p], v[1][p], v[2][p], v[3][p]);
+                *reinterpret_cast<uint4*>(at + kPlane) = make_uint4(v[4][p], v[5][p], v[6][p], v[7][p]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+                    *reinterpret_cast<uint32_t*>(act.third + ((col + i) >> 2) * kPlane + ((col + i) & 3u) * 4u) = v[i][p];
+            }
+            continue;
+        }
         uint32_t r[N];
 #pragma unroll
         for (int i = 0; i < N; ++i) r[i] = v[i][p];
-        tmem_st(act + p * part_cols + col, r);
+        tmem_st(act.tmem + p * act.part_cols + col, r);
     }
 }
 
@@ -201,9 +219,9 @@ __device__ __forceinline__ float4 blend_level4(const TcCfg& tc, const GridView<G
 }
 
 // Values of a row one after another, stored in pairs.
-template <int OPS>
+template <int OPS, bool THIRD>
 struct RowPacker {
-    uint32_t act, part_cols;
+    ActRow<THIRD> act;
     int k;
     float prev;
     __device__ __forceinline__ void put(float v) {
@@ -211,7 +229,7 @@ struct RowPacker {
             uint32_t p[1][OpsTraits<OPS>::parts];
             split_pair<OPS>(prev, v, p[0]);
             __syncwarp();
-            put_pairs<OPS, 1>(act, part_cols, (uint32_t)(k >> 1), p);
+            put_pairs<OPS, THIRD, 1>(act, (uint32_t)(k >> 1), p);
         }
         prev = v;
         ++k;
@@ -235,22 +253,16 @@ __device__ __forceinline__ void product_inputs(const QuerySeg& S, uint32_t j, bo
 // The network input of query j at (x, y, z) in the unit box: this thread's row of the activation
 // columns, padded with zeros to the layer's kp values. FEAT: features per
 // level (2 or 4), or 0 for any.
-template <int FEAT, int OPS>
+template <int FEAT, int OPS, int NF, bool THIRD>
 __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typename OpsTraits<OPS>::GridT>& grid,
                                            float x, float y, float z, const QuerySeg& S, uint32_t j, bool valid,
-                                           uint32_t act) {
+                                           const ActRow<THIRD>& act) {
     const DevCfg& cfg = tc.base;
     constexpr int P = OpsTraits<OPS>::parts;
-    const uint32_t pc = tc.a_cols;
     __syncwarp();
     const int L = cfg.n_levels, F = FEAT ? FEAT : cfg.feat;
     if constexpr (FEAT == 2) {
-        // NF levels' gathers in flight before the first is blended: what the
-        // registers hold without spilling (2^20 queries of the paper-shaped
-        // grid, FP16 with 2, 3, 4: 302, 290, 327 us, four spilling 116 bytes;
-        // FP32 accuracy with 1, 2: 377, 407 us, two spilling 120 bytes; FP32
-        // with 2, 3: 461, 469 us).
-        constexpr int NF = OPS == kTwoFp16 ? 1 : OPS == kThreeBf16 ? 2 : 3;
+        // NF levels' gathers in flight before the first is blended.
         int l = 0;
         for (; l + NF <= L; l += NF) {
             Cell cl[NF];
@@ -266,7 +278,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
                 const float2 a = v[i].blend(cl[i]);
                 split_pair<OPS>(a.x, a.y, p[i]);
             }
-            put_pairs<OPS, NF>(act, pc, (uint32_t)l, p);
+            put_pairs<OPS, THIRD, NF>(act, (uint32_t)l, p);
         }
         for (; l < L; ++l) {
             const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
@@ -275,7 +287,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             const float2 a = v.blend(cl);
             uint32_t p[1][P];
             split_pair<OPS>(a.x, a.y, p[0]);
-            put_pairs<OPS, 1>(act, pc, (uint32_t)l, p);
+            put_pairs<OPS, THIRD, 1>(act, (uint32_t)l, p);
         }
     } else if (FEAT == 4 || F == 4 || F == 8) {
 #pragma unroll(FEAT == 4 ? 2 : 1)
@@ -286,11 +298,11 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
                 uint32_t p[2][P];
                 split_pair<OPS>(a.x, a.y, p[0]);
                 split_pair<OPS>(a.z, a.w, p[1]);
-                put_pairs<OPS, 2>(act, pc, (uint32_t)((l * F + 4 * h) >> 1), p);
+                put_pairs<OPS, THIRD, 2>(act, (uint32_t)((l * F + 4 * h) >> 1), p);
             }
         }
     } else {
-        RowPacker<OPS> row{act, pc, 0, 0.0f};
+        RowPacker<OPS, THIRD> row{act, 0, 0.0f};
         for (int l = 0; l < L; ++l) {
             const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
             if (F == 2) {
@@ -331,7 +343,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             for (int i = 0; i < 22; i += 2) {
                 uint32_t p[1][P];
                 split_pair<OPS>(e[i], e[i + 1], p[0]);
-                put_pairs<OPS, 1>(act, pc, col + (uint32_t)(i >> 1), p);
+                put_pairs<OPS, THIRD, 1>(act, col + (uint32_t)(i >> 1), p);
             }
         }
         col = (uint32_t)(cfg.grid_feats + 22) >> 1;
@@ -339,7 +351,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
     const uint32_t end = (uint32_t)tc.layer[0].Kp >> 1;
     for (; col < end; ++col) {
         const uint32_t p[1][P] = {};
-        put_pairs<OPS, 1>(act, pc, col, p);
+        put_pairs<OPS, THIRD, 1>(act, col, p);
     }
 }
 
@@ -628,12 +640,18 @@ __device__ __forceinline__ void tc_decode_warp(const TcCfg& tc, const float* __r
 
 // --------------------------------------------------------------- kernel
 
+// Bytes of a group's third activation part in shared memory.
+template <bool THIRD>
+__host__ __device__ inline uint32_t fwd_third_bytes(const TcCfg& tc) {
+    return THIRD ? tc.a_cols / 4u * kPlane : 0u;
+}
+
 // The MMAs of one layer: every K step of each product of parts, the smallest
 // products first, so that the large ones meet the accumulator's rounding only
 // Kp / 16 times. Issued by one thread.
-template <int OPS>
+template <int OPS, bool THIRD>
 __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, uint32_t acc, uint32_t act,
-                                            uint32_t sW_addr) {
+                                            uint32_t third, uint32_t sW_addr) {
     const uint64_t b0 = umma_desc(sW_addr + ly.w_off, 128u, (uint32_t)(ly.Kp >> 3) * 128u);
     const int nk = ly.Kp >> 4;
     uint32_t accum = 0u;
@@ -648,7 +666,13 @@ __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, 
     if constexpr (OPS == kThreeBf16) {
         // (1, 2), (2, 1) and (2, 2) lie 2^-26 and more below the product.
         product(0, 2);
-        product(2, 0);
+        if constexpr (THIRD) {
+            const uint64_t a2 = umma_desc(third, kPlane, 128u);
+            for (int s = 0; s < nk; ++s)
+                mma_bf16(acc, a2 + (uint64_t)(2 * (kPlane >> 4) * s), b0 + (uint64_t)(16 * s), ly.idesc, 1u);
+        } else {
+            product(2, 0);
+        }
         product(1, 1);
     }
     if constexpr (OpsTraits<OPS>::parts >= 2) product(1, 0);
@@ -657,13 +681,20 @@ __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, 
 }
 
 // WARPDEC: the warp-per-query decode (tc_decode_warp) from raw outputs staged
-// in shared memory.
-template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
-__global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
+// in shared memory. THIRD: the third activation part lies in shared memory.
+template <int KMAX, int FEAT, int OPS, bool WARPDEC = false, int GMAX = fwd_groups(KMAX),
+          bool THIRD = (OPS == kThreeBf16)>
+__global__ void __launch_bounds__(kThreads * GMAX, 1)
     k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ table,
                  const uint4* __restrict__ blk, const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
                  long long wait_limit) {
     extern __shared__ __align__(1024) uint8_t smem[];
+    // Levels of 2-feature grids gathered before the first is blended: what the
+    // registers hold without spilling (2^20 queries of the paper-shaped grid,
+    // FP16 with 2, 3, 4: 302, 290, 327 us, four spilling 116 bytes; FP32
+    // accuracy with 1, 2: 377, 407 us, two spilling 120 bytes; FP32, three
+    // groups, with 2, 3: 461, 469 us).
+    constexpr int NF = GMAX == 3 ? 2 : OpsTraits<OPS>::fp32 ? 1 : 3;
     const int G = (int)(blockDim.x >> 7);
     const int g = (int)(threadIdx.x >> 7);   // tile group
     const int t = (int)(threadIdx.x & 127);  // row of the group's tile
@@ -695,9 +726,12 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // This group's columns: the accumulator, then the activations' parts.
+    // This group's columns: the accumulator, then the activations' parts; the
+    // third part's tile.
     const uint32_t acc = *tslot + (uint32_t)g * tc.g_cols, act = acc + tc.d_cols;
+    uint8_t* third = smem + fwd_stage_off(wbytes, G) + (uint32_t)g * fwd_third_bytes<THIRD>(tc);
     const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+    const ActRow<THIRD> row{act + lanes, tc.a_cols, third + t * 16};
     const uint32_t sW_addr = smem_u32(smem);
     const int L = tc.base.n_layers;
     const bool sample = qb.sample != 0;
@@ -741,7 +775,7 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
                 if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + r * S2.ld + b2));
             }
         }
-        encode_row<FEAT, OPS>(tc, grid, x, y, z, S, j, valid, act + lanes);
+        encode_row<FEAT, OPS, NF, THIRD>(tc, grid, x, y, z, S, j, valid, row);
         // The uniforms (or the direction), loaded now so that their latency
         // passes during the layers.
         float u[4] = {0.0f, 0.0f, sample ? 0.0f : 1.0f, 0.0f};
@@ -753,6 +787,7 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
         }
         __syncwarp();
         tmem_wait_st();
+        if constexpr (THIRD) fence_async_smem();
         tc_fence_before();
         if (tc_group_sync_or(g, !ok)) {
             ok = false;
@@ -766,7 +801,7 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
                 if (!issued) ok = mbar_wait_limit(bar_w, 0, wait_limit);
                 if (ok) {
                     tc_fence_after();
-                    issue_layer<OPS>(tc, ly, acc, act, sW_addr);
+                    issue_layer<OPS, THIRD>(tc, ly, acc, act, smem_u32(third), sW_addr);
                     mma_commit(bar_mma);
                     issued = true;
                 }
@@ -787,10 +822,11 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
                             relu_split_pair<OPS>(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), p[i]);
-                        put_pairs<OPS, 8>(act + lanes, tc.a_cols, (uint32_t)(c0 >> 1), p);
+                        put_pairs<OPS, THIRD, 8>(row, (uint32_t)(c0 >> 1), p);
                     }
                     tmem_wait_st();
                 }
+                if constexpr (THIRD) fence_async_smem();
                 tc_fence_before();
                 if (tc_group_sync_or(g, !ok)) {
                     ok = false;
@@ -845,25 +881,32 @@ __global__ void __launch_bounds__(kThreads * fwd_groups(KMAX, FEAT, OPS), 1)
 
 // ------------------------------------------------------------- launcher
 
-// Tile groups of a CTA: as many as the instance is compiled for and the
-// 512 tensor-memory columns hold.
-inline int fwd_group_count(const TcCfg& c, int most) {
+// Columns of a tile group, and the groups of a CTA: as many as the instance is
+// compiled for and the 512 tensor-memory columns and the shared memory hold.
+template <int OPS, bool THIRD>
+uint32_t fwd_group_cols(const TcCfg& c) {
+    return c.d_cols + (uint32_t)(OpsTraits<OPS>::parts - (THIRD ? 1 : 0)) * c.a_cols;
+}
+template <int OPS, bool THIRD>
+int fwd_group_count(const TcCfg& c, int most) {
+    const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * c.w_bytes;
     int G = most;
-    for (; G > 1; --G) {
-        uint32_t cols = 32;
-        while (cols < (uint32_t)G * c.g_cols) cols <<= 1;
-        if (cols <= 512u) break;
-    }
+    while (G > 1 && ((uint32_t)G * fwd_group_cols<OPS, THIRD>(c) > 512u ||
+                     fwd_stage_off(wbytes, G) + (uint32_t)G * fwd_third_bytes<THIRD>(c) > 226u * 1024u))
+        --G;
     return G;
 }
 
-template <int KMAX, int FEAT, int OPS, bool WARPDEC = false>
-cudaError_t launch_fwd(const TcCfg& c, const void* grid, const uint4* blk, const uint8_t* wblob, QueryBatch& qb, int64_t max_n,
-                       int* status, long long wait_limit, cudaStream_t st) {
-    auto kern = k_forward_tc<KMAX, FEAT, OPS, WARPDEC>;
-    const int G = fwd_group_count(c, fwd_groups(KMAX, FEAT, OPS));
+template <int KMAX, int FEAT, int OPS, bool WARPDEC = false, int GMAX = fwd_groups(KMAX),
+          bool THIRD = (OPS == kThreeBf16)>
+cudaError_t launch_fwd(const TcCfg& cfg, const void* grid, const uint4* blk, const uint8_t* wblob, QueryBatch& qb,
+                       int64_t max_n, int* status, long long wait_limit, cudaStream_t st) {
+    auto kern = k_forward_tc<KMAX, FEAT, OPS, WARPDEC, GMAX, THIRD>;
+    TcCfg c = cfg;
+    c.g_cols = fwd_group_cols<OPS, THIRD>(c);
+    const int G = fwd_group_count<OPS, THIRD>(c, GMAX);
     const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * c.w_bytes;
-    size_t smem = fwd_stage_off(wbytes, G);
+    size_t smem = fwd_stage_off(wbytes, G) + (size_t)G * fwd_third_bytes<THIRD>(c);
     if (WARPDEC) smem += (size_t)G * kTile * (4 * KMAX + 4) * sizeof(float);
     static std::atomic<uint64_t> attrs{~0ull};
     cudaError_t e = set_smem_attrs(kern, smem, carveout_percent(smem + 1024), attrs);
@@ -893,6 +936,30 @@ cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint4* blk, c
     if (c.base.K > 8) return launch_fwd<16, 0, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
     if constexpr (!OpsTraits<OPS>::fp32)
         if (warp_decode) return launch_fwd<8, 0, OPS, true>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+    if constexpr (OPS == kThreeBf16) {
+        // FP32 has instances that keep the third part in tensor memory too.
+        // 4-feature grids take theirs where its columns suffice for four
+        // groups (2^18 queries of a 16-wide network: 44 us, with the part in
+        // shared memory 47). 2-feature grids' has three groups with two
+        // levels' gathers in flight, against four with one, whose rounds of
+        // tiles take 1.37 times as long: whichever needs less for the rounds
+        // of this batch (paper-shaped grid, three and four groups: 3,000
+        // queries 20 and 21 us; 2^16 50 and 42; 2^17 78 and 71; 2^18 128 and
+        // 132; 2^20 449 and 461).
+        if (c.base.feat == 4 && 4u * fwd_group_cols<OPS, false>(c) <= 512u)
+            return launch_fwd<8, 4, OPS, false, 4, false>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+        if (c.base.feat == 2 && fwd_group_count<OPS, false>(c, 3) == 3) {
+            int dev = 0, sms = 1;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            int64_t tiles = 0;
+            for (int i = 0; i < qb.nseg; ++i) tiles += (qb.seg[i].n + kTile - 1) / kTile;
+            if (qb.n_dev) tiles = (max_n + kTile - 1) / kTile;
+            const int64_t r3 = (tiles + 3 * sms - 1) / (3 * sms), r4 = (tiles + 4 * sms - 1) / (4 * sms);
+            if (137 * r4 >= 100 * r3)
+                return launch_fwd<8, 2, OPS, false, 3, false>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
+        }
+    }
     if (c.base.feat == 2) return launch_fwd<8, 2, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
     if (c.base.feat == 4) return launch_fwd<8, 4, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
     return launch_fwd<8, 0, OPS>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);

@@ -1,6 +1,6 @@
 """The tensor-core forward kernel at the edges of its tiles and groups: one
-query, a tile less or more one, one tile per SM and one more than every tile
-group holds, on networks whose inputs fill the activation columns unevenly
+query, a tile less or more one, one tile per SM, as many as four tile groups
+per SM hold and one query more, on networks whose inputs fill the activation columns unevenly
 (an odd number of one-feature levels before the product-mode inputs, an odd
 number of two-feature levels, three-feature levels, 128-wide layers, sixteen
 lobes). Densities at the sampled directions against the FP64 oracle: 1e-4 in
@@ -27,14 +27,15 @@ LOBES16 = synth.Workload(name="3 levels x 2 feats, product, K=16", mode=synth.PR
                          log2_table=12, widths=[28, 64, 64], K=16)
 WIDE = synth.Workload(name="2 levels x 4 feats, 128 wide", mode=synth.RADIANCE, level_res=[6, 30], feat=4,
                       log2_table=13, widths=[8, 128, 20], K=5)
-
+WIDE_TWO = synth.Workload(name="2 levels x 2 feats, 96 wide", mode=synth.RADIANCE, level_res=[6, 30], feat=2,
+                          log2_table=13, widths=[4, 96, 20], K=5)
 
 THREE = synth.Workload(name="3 levels x 3 feats", mode=synth.RADIANCE, level_res=[6, 11, 40], feat=3,
                        log2_table=12, widths=[12, 32, 12], K=3)
 
 PRECISIONS = {"fp32": synth.FP32, "fp32tc": synth.FP32_TC, "bf16x3": synth.BF16X3, "fp16": synth.FP16}
 # Three features per level are FP32's alone.
-CASES = [(w, p) for w in (ODD_ONE, ODD_TWO, LOBES16, WIDE) for p in PRECISIONS] + [(THREE, "fp32")]
+CASES = [(w, p) for w in (ODD_ONE, ODD_TWO, LOBES16, WIDE, WIDE_TWO) for p in PRECISIONS] + [(THREE, "fp32")]
 
 
 @pytest.fixture(autouse=True)
@@ -47,7 +48,7 @@ def _need_cuda():
 def test_tile_edges(w, precision):
     precision = PRECISIONS[precision]
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    sizes = [1, 127, 129, sms * 128, 4 * sms * 128 + 1]
+    sizes = [1, 127, 129, sms * 128, 4 * sms * 128, 4 * sms * 128 + 1]
     params = synth.random_params(w, 41)
     m = make_model(w, params, sizes[-1], precision=precision)
     for n in sizes:
