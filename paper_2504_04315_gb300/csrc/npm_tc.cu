@@ -483,9 +483,9 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
     int64_t mlp_off, double* __restrict__ loss, int* __restrict__ status, const float2* __restrict__ enc) {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int KH = KMAX / 2;
-    const int g = G > 1 ? (int)(threadIdx.x >> 8) : 0;
+    const int g = G > 1 ? (int)warp_uniform(threadIdx.x >> 8) : 0;
     const int t = G > 1 ? (int)(threadIdx.x & 255) : (int)threadIdx.x;
-    const int warp = t >> 5, row = t & (kTile - 1), half = t >> 7;
+    const int warp = (int)warp_uniform((uint32_t)t >> 5), row = t & (kTile - 1), half = warp >> 2;
     uint8_t* tiles = smem + g * tt.g_bytes;
     float4* xch = reinterpret_cast<float4*>(smem + tt.x_off) + g * 2 * kTile;  // [2][kTile] partial log-sum-exps
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + tt.bar_off);  // weights, weight gradients, MMAs of each group
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = warp_uniform(*tslot);
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
     {
         // The weight-gradient accumulators start at zero.
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
         // Forward, keeping every layer's input tile.
         for (int l = 0; l < L; ++l) {
             const TcLayer& ly = tc.layer[l];
-            if (t == 0) {
+            if (warp == 0) {
                 tc_fence_after();
                 // K step s starts two planes (256 units of 16 bytes) further.
                 const uint32_t sbo = (uint32_t)(ly.Kp >> 3) * 128u;
@@ -620,13 +620,16 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
                 const uint64_t al0 = umma_desc(tile_addr + tt.slot[L], kPlane, 128u);
                 const uint64_t bd0 = umma_desc(sW_addr + ly.w_off, 128u, sbo);
                 const uint64_t bl0 = umma_desc(sW_addr + wlo + ly.w_off, 128u, sbo);
-                for (int s = 0; s < (ly.Kp >> 4); ++s) {
-                    const uint64_t oa = (uint64_t)(256 * s), ob = (uint64_t)(16 * s);
-                    mma_bf16(acc, ad0 + oa, bd0 + ob, ly.idesc, s > 0 ? 1u : 0u);
-                    mma_bf16(acc, ad0 + oa, bl0 + ob, ly.idesc, 1u);
-                    mma_bf16(acc, al0 + oa, bd0 + ob, ly.idesc, 1u);
+                if (elect_one()) {
+                    for (int s = 0; s < (ly.Kp >> 4); ++s) {
+                        const uint64_t oa = (uint64_t)(256 * s), ob = (uint64_t)(16 * s);
+                        mma_bf16(acc, ad0 + oa, bd0 + ob, ly.idesc, s > 0 ? 1u : 0u);
+                        mma_bf16(acc, ad0 + oa, bl0 + ob, ly.idesc, 1u);
+                        mma_bf16(acc, al0 + oa, bd0 + ob, ly.idesc, 1u);
+                    }
+                    mma_commit(bar_mma);
                 }
-                mma_commit(bar_mma);
+                __syncwarp();
                 issued = true;
             }
             scatter_next();  // the previous tile's grid gradient, one level
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
         for (int l = L - 1; l >= 0; --l) {
             const TcLayer& ly = tc.layer[l];
             const uint32_t lo_off = (uint32_t)ly.Np * (kPlane / 8);  // residuals behind the output gradient
-            if (t == 0) {
+            if (warp == 0) {
                 tc_fence_after();
                 const uint32_t hk = (uint32_t)(ly.Kp >> 3) * 128u;  // K step of a W_l tile
                 const uint32_t d_addr = tile_addr + tt.slot[l + 1];
@@ -715,31 +718,34 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
                 const uint64_t bd0 = umma_desc(sW_addr + ly.w_off, hk, 128u);
                 const uint64_t bl0 = umma_desc(sW_addr + wlo + ly.w_off, hk, 128u);
                 const uint64_t bstep = (uint64_t)((2u * hk) >> 4);
-                for (int s = 0; s < (ly.Np >> 4); ++s) {
-                    const uint64_t oa = (uint64_t)(256 * s), ob = s * bstep;
-                    mma_bf16(acc, ad0 + oa, bd0 + ob, tt.idesc_dx[l], s > 0 ? 1u : 0u);
-                    mma_bf16(acc, ad0 + oa, bl0 + ob, tt.idesc_dx[l], 1u);
-                    mma_bf16(acc, al0 + oa, bd0 + ob, tt.idesc_dx[l], 1u);
-                }
                 // dW_l += D^T H_l: M = 128 (outputs, then their residuals),
                 // N = Kp_l, K = 128 samples (256 bytes a step).
-                if (G == 1 || take_turn(turn, bar_dw)) {
-                    tc_fence_after();
-                    const uint64_t bh0 = umma_desc(tile_addr + tt.slot[l], 128u, kPlane);
-                    const uint64_t dw0 = umma_desc(d_addr, 128u, kPlane), dwl0 = umma_desc(d_addr + lo_off, 128u, kPlane);
-                    for (int s = 0; s < 8; ++s) {
-                        const uint64_t o = (uint64_t)(16 * s);
-                        mma_bf16(tmem + tt.dw_col[l], dw0 + o, bh0 + o, tt.idesc_dw[l], 1u);
-                        if (2 * ly.Np > 128) mma_bf16(tmem + tt.dw_col[l], dwl0 + o, bh0 + o, tt.idesc_dw[l], 1u);
+                const uint64_t bh0 = umma_desc(tile_addr + tt.slot[l], 128u, kPlane);
+                const uint64_t dw0 = umma_desc(d_addr, 128u, kPlane), dwl0 = umma_desc(d_addr + lo_off, 128u, kPlane);
+                if (elect_one()) {
+                    for (int s = 0; s < (ly.Np >> 4); ++s) {
+                        const uint64_t oa = (uint64_t)(256 * s), ob = s * bstep;
+                        mma_bf16(acc, ad0 + oa, bd0 + ob, tt.idesc_dx[l], s > 0 ? 1u : 0u);
+                        mma_bf16(acc, ad0 + oa, bl0 + ob, tt.idesc_dx[l], 1u);
+                        mma_bf16(acc, al0 + oa, bd0 + ob, tt.idesc_dx[l], 1u);
                     }
-                    if (G > 1) {
-                        mma_commit(bar_dw);
-                        pass_turn(turn);
+                    if (G == 1 || take_turn(turn, bar_dw)) {
+                        tc_fence_after();
+                        for (int s = 0; s < 8; ++s) {
+                            const uint64_t o = (uint64_t)(16 * s);
+                            mma_bf16(tmem + tt.dw_col[l], dw0 + o, bh0 + o, tt.idesc_dw[l], 1u);
+                            if (2 * ly.Np > 128) mma_bf16(tmem + tt.dw_col[l], dwl0 + o, bh0 + o, tt.idesc_dw[l], 1u);
+                        }
+                        if (G > 1) {
+                            mma_commit(bar_dw);
+                            pass_turn(turn);
+                        }
+                    } else {
+                        ok = false;
                     }
-                } else {
-                    ok = false;
+                    mma_commit(bar_mma);
                 }
-                mma_commit(bar_mma);
+                __syncwarp();
             }
             scatter_next();
             wait_mma();

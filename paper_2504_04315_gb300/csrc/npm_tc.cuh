@@ -92,6 +92,26 @@ __device__ __forceinline__ void mma_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uin
         : "memory");
 }
 
+// One thread of a converged warp, for the MMAs and their commit. Their operands
+// are warp-uniform and computed by the whole warp from uniform values
+// (warp_uniform, parameters), and the branch is taken by an elected thread: an
+// MMA then issues every 80 cycles or so, against 210-250 under `t == 0`, where
+// the operands of each are moved from the thread's registers first. Issue was a
+// third of a tile's time (GB300, per tile of the paper-shaped grid, FP32: 12,600
+// of 44,500 cycles, now 4,800 of 33,000). A predicate on each instruction, steps
+// unrolled in full, or another warp of each group issuing all measured slower
+// (2^20 queries: 410, 416 and 382 us against 360).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)

@@ -696,9 +696,9 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
     // groups, with 2, 3: 461, 469 us).
     constexpr int NF = GMAX == 3 ? 2 : OpsTraits<OPS>::fp32 ? 1 : 3;
     const int G = (int)(blockDim.x >> 7);
-    const int g = (int)(threadIdx.x >> 7);   // tile group
-    const int t = (int)(threadIdx.x & 127);  // row of the group's tile
-    const int warp = t >> 5;                 // warp of the group (its tensor-memory lane quarter)
+    const int g = (int)warp_uniform(threadIdx.x >> 7);  // tile group
+    const int t = (int)(threadIdx.x & 127);             // row of the group's tile
+    const int warp = (int)warp_uniform((threadIdx.x >> 5) & 3u);                 // warp of the group (its tensor-memory lane quarter)
     const uint32_t wbytes = (uint32_t)OpsTraits<OPS>::wparts * tc.w_bytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + wbytes);  // [0] weights, [1 + g] MMAs
     uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 1 + G);
@@ -728,7 +728,7 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
     tc_fence_after();
     // This group's columns: the accumulator, then the activations' parts; the
     // third part's tile.
-    const uint32_t acc = *tslot + (uint32_t)g * tc.g_cols, act = acc + tc.d_cols;
+    const uint32_t acc = warp_uniform(*tslot) + (uint32_t)g * tc.g_cols, act = acc + tc.d_cols;
     uint8_t* third = smem + fwd_stage_off(wbytes, G) + (uint32_t)g * fwd_third_bytes<THIRD>(tc);
     const uint32_t lanes = (uint32_t)(warp * 32) << 16;
     const ActRow<THIRD> row{act + lanes, tc.a_cols, third + t * 16};
@@ -796,13 +796,16 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
         uint32_t raw[KMAX / 4][16];
         for (int l = 0; l < L; ++l) {
             const TcLayer& ly = tc.layer[l];
-            if (t == 0) {
+            if (warp == 0) {
                 // The weights have arrived (once per CTA).
-                if (!issued) ok = mbar_wait_limit(bar_w, 0, wait_limit);
+                if (!issued) ok = __all_sync(0xffffffffu, mbar_wait_limit(bar_w, 0, wait_limit));
                 if (ok) {
                     tc_fence_after();
-                    issue_layer<OPS, THIRD>(tc, ly, acc, act, smem_u32(third), sW_addr);
-                    mma_commit(bar_mma);
+                    if (elect_one()) {
+                        issue_layer<OPS, THIRD>(tc, ly, acc, act, smem_u32(third), sW_addr);
+                        mma_commit(bar_mma);
+                    }
+                    __syncwarp();
                     issued = true;
                 }
             }

@@ -20,7 +20,8 @@
 // of the general kernel: thread t owns query t of a 128-query tile and lane t
 // of tensor memory; one elected thread issues the MMAs. Against activation
 // tiles in shared memory with one warp waiting for the MMAs and a second group
-// barrier a layer (GB300, 2^22 queries): split BF16 165 -> 146 us.
+// barrier a layer (GB300, 2^22 queries): split BF16 165 -> 146 us; with the
+// MMAs' operands in uniform registers 129 us.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -221,9 +222,9 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
     constexpr bool SPLIT = OPS == kOpsBf16x3;
     constexpr int nw = OPS == kOpsBf16 ? 1 : 2;  // weight blobs (hi, residual)
     const TinyLayout lay = tiny_layout(tc, grid_bytes);
-    const int g = threadIdx.x >> 7;      // tile group
-    const int t = threadIdx.x & 127;     // row of the group's tile
-    const int warp = t >> 5;             // warp within the group (its TMEM lane quarter)
+    const int g = (int)warp_uniform(threadIdx.x >> 7);  // tile group
+    const int t = threadIdx.x & 127;                   // row of the group's tile
+    const int warp = (int)warp_uniform((threadIdx.x >> 5) & 3u);  // warp within the group (its TMEM lane quarter)
     uint8_t* sW = smem;
     const uint2* sG = reinterpret_cast<const uint2*>(smem + lay.grid);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.bars);
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
     __syncthreads();
     tc_fence_after();
     // This group's tensor-memory columns: accumulator, activations.
-    const uint32_t tmem = *tslot + kGroupCols * (uint32_t)g, act = tmem + 32u;
+    const uint32_t tmem = warp_uniform(*tslot) + kGroupCols * (uint32_t)g, act = tmem + 32u;
     if (threadIdx.x == 0) {
         // Weights and grid table: two bulk copies on one barrier.
         const uint32_t wb = (uint32_t)nw * tc.w_bytes;
@@ -363,23 +364,26 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
             const TcLayer& ly = tc.layer[l];
-            if (t == 0) {
+            if (warp == 0) {
                 tc_fence_after();
                 // K step s: eight activation columns on, weight descriptors
                 // with the start address 256 bytes (16 units) further.
                 const uint64_t bd = umma_desc(smem_u32(sW) + ly.w_off, 128u, (uint32_t)(ly.Kp >> 3) * 128u);
                 const uint64_t bl = bd + (uint64_t)(tc.w_bytes >> 4);
+                if (elect_one()) {
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    if (s < (ly.Kp >> 4)) {
-                        const uint64_t o = (uint64_t)(16 * s);
-                        const uint32_t a = act + 8u * (uint32_t)s;
-                        mma_tmem_a(tmem, a, bd + o, ly.idesc, s > 0 ? 1u : 0u);
-                        if (OPS != kOpsBf16) mma_tmem_a(tmem, a, bl + o, ly.idesc, 1u);
-                        if (SPLIT) mma_tmem_a(tmem, a + 16u, bd + o, ly.idesc, 1u);
+                    for (int s = 0; s < 2; ++s) {
+                        if (s < (ly.Kp >> 4)) {
+                            const uint64_t o = (uint64_t)(16 * s);
+                            const uint32_t a = act + 8u * (uint32_t)s;
+                            mma_tmem_a(tmem, a, bd + o, ly.idesc, s > 0 ? 1u : 0u);
+                            if (OPS != kOpsBf16) mma_tmem_a(tmem, a, bl + o, ly.idesc, 1u);
+                            if (SPLIT) mma_tmem_a(tmem, a + 16u, bd + o, ly.idesc, 1u);
+                        }
                     }
+                    mma_commit(bar_mma);
                 }
-                mma_commit(bar_mma);
+                __syncwarp();
             }
             issued = true;
             // Every warp waits on the MMAs' barrier; a wait that gives up is
