@@ -653,31 +653,35 @@ template <int OPS, bool THIRD>
 __device__ __forceinline__ void issue_layer(const TcCfg& tc, const TcLayer& ly, uint32_t acc, uint32_t act,
                                             uint32_t third, uint32_t sW_addr) {
     const uint64_t b0 = umma_desc(sW_addr + ly.w_off, 128u, (uint32_t)(ly.Kp >> 3) * 128u);
-    const int nk = ly.Kp >> 4;
-    uint32_t accum = 0u;
-    auto product = [&](int ap, int wp) {
-        const uint64_t b = b0 + (uint64_t)wp * (tc.w_bytes >> 4);
-        const uint32_t a = act + (uint32_t)ap * tc.a_cols;
-        for (int s = 0; s < nk; ++s) {
-            mma_tmem_a(acc, a + 8u * (uint32_t)s, b + (uint64_t)(16 * s), ly.idesc, accum);
-            accum = 1u;
+    with_steps(ly.Kp >> 4, [&](auto steps) {
+        constexpr int NK = decltype(steps)::count;
+        const int nk = NK ? NK : ly.Kp >> 4;
+        bool first = true;
+        auto product = [&](int ap, int wp) {
+            const uint64_t b = b0 + (uint64_t)wp * (tc.w_bytes >> 4);
+            const uint32_t a = act + (uint32_t)ap * tc.a_cols;
+            mma_tmem_a(acc, a, b, ly.idesc, first ? 0u : 1u);
+            first = false;
+#pragma unroll(NK ? NK : 1)
+            for (int s = 1; s < nk; ++s) mma_tmem_a(acc, a + 8u * (uint32_t)s, b + (uint64_t)(16 * s), ly.idesc, 1u);
+        };
+        if constexpr (OPS == kThreeBf16) {
+            // (1, 2), (2, 1) and (2, 2) lie 2^-26 and more below the product.
+            product(0, 2);
+            if constexpr (THIRD) {
+                const uint64_t a2 = umma_desc(third, kPlane, 128u);
+#pragma unroll(NK ? NK : 1)
+                for (int s = 0; s < nk; ++s)
+                    mma_bf16(acc, a2 + (uint64_t)(2 * (kPlane >> 4) * s), b0 + (uint64_t)(16 * s), ly.idesc, 1u);
+            } else {
+                product(2, 0);
+            }
+            product(1, 1);
         }
-    };
-    if constexpr (OPS == kThreeBf16) {
-        // (1, 2), (2, 1) and (2, 2) lie 2^-26 and more below the product.
-        product(0, 2);
-        if constexpr (THIRD) {
-            const uint64_t a2 = umma_desc(third, kPlane, 128u);
-            for (int s = 0; s < nk; ++s)
-                mma_bf16(acc, a2 + (uint64_t)(2 * (kPlane >> 4) * s), b0 + (uint64_t)(16 * s), ly.idesc, 1u);
-        } else {
-            product(2, 0);
-        }
-        product(1, 1);
-    }
-    if constexpr (OpsTraits<OPS>::parts >= 2) product(1, 0);
-    if constexpr (OpsTraits<OPS>::wparts >= 2) product(0, 1);
-    product(0, 0);
+        if constexpr (OpsTraits<OPS>::parts >= 2) product(1, 0);
+        if constexpr (OpsTraits<OPS>::wparts >= 2) product(0, 1);
+        product(0, 0);
+    });
 }
 
 // WARPDEC: the warp-per-query decode (tc_decode_warp) from raw outputs staged
