@@ -635,10 +635,11 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
                     mma_commit(bar_mma);
                 }
                 __syncwarp();
+                issued = true;
             } else {
                 scatter_next();  // the previous tile's grid gradient, one level
+                if (F2) issued = true;  // (by any warp)
             }
-            issued = true;
             wait_mma();
             if (l < L - 1) {
                 if (ok) {
