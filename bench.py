@@ -125,9 +125,9 @@ def mlp_flops(w):
     return 2 * sum(a * b for a, b in zip(w.widths[:-1], w.widths[1:]))
 
 
-# DRAM bytes of one k_forward_fp32_ws launch on the paper-shaped workload
+# DRAM bytes of one FP32 k_forward_tc launch on the paper-shaped workload
 # (2^20 queries) from the ncu capture summarised in profiles/.
-FP32_FORWARD_DRAM_BYTES = 66753024 + 8907520
+FP32_FORWARD_DRAM_BYTES = 147034880 + 17128704
 
 # Algorithmic work per query of the tensor-core forward on the tiny model
 # (K = 4): transcendentals of the vMF decode, sample and pdf (softmax 4,
@@ -181,11 +181,13 @@ def scatter_atomic_counts(model, w, pos_dev):
     return n4, n2
 
 
-def gather_sector_counts(model, w, pos_dev):
+def gather_sector_counts(model, w, pos_dev, blocks=False):
     """32-byte L2 sectors that a batch's grid gathers must touch: per query
     and level, the distinct sectors holding the 8 corners' FP32 entries
     (feat x 4 bytes each, at the level's table offset), counted from the
-    corner indices the library forms (npm_grid_indices)."""
+    corner indices the library forms (npm_grid_indices). blocks:
+    dense levels of 2 and 4 features through corner blocks, as batches of
+    2^18 queries and more read them: at most feat sectors."""
     import torch
     idx = model.grid_indices(pos_dev).to(torch.int64)  # [L][8][n], entry within the level
     offs = torch.tensor(np.cumsum([0] + synth.grid_sizes(w)[:-1]), dtype=torch.int64,
@@ -195,13 +197,18 @@ def gather_sector_counts(model, w, pos_dev):
     last = ((offs + idx) * fb + fb - 1) // 32           # and of its last byte
     sec = torch.cat([first, last], 1).sort(1).values    # [L][16][n]
     distinct = 1 + (sec[:, 1:, :] != sec[:, :-1, :]).sum(1)
+    if blocks and w.feat in (2, 4):
+        for l, d in enumerate(w.level_res):
+            if d ** 3 <= 1 << w.log2_table:
+                distinct[l].clamp_(max=w.feat)
     return int(distinct.sum())
 
 
 def gather_roofline(qps, sectors_per_query, up):
-    """Forward bound of the FP32-accuracy tensor-core mode: its grid gathers
-    at the measured random 32-byte L2 sector rate (the MLP's tensor work and
-    the table, resident in L2, are far below their own limits)."""
+    """Forward bound of the FP32-table modes on hash grids: every query's
+    corners at the measured random 32-byte L2 sector rate (the MLP's tensor
+    work and the table, resident in L2, are far below their own limits; the
+    coarse levels' L1 hits are not counted off)."""
     peak = up["l2_sector_read_gbs"] * 1e9 / (32.0 * sectors_per_query)
     return {"bound": "l2", "achieved": qps, "peak": peak, "unit": "queries/s", "frac": qps / peak,
             "sectors_per_query": sectors_per_query,
@@ -438,8 +445,8 @@ def main():
         e2e = {"value": n * ke * world / e2e_s, "unit": "queries/s",
                "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h}
 
-    # The same workload and inputs in the FP32-accuracy tensor-core mode
-    # (held to the FP32 path's bars), when the headline runs in FP32.
+    # The same workload and inputs in the FP32-accuracy mode (two FP16 parts,
+    # held to the FP32 path's bars), when the headline runs in FP32.
     fp32_tc = None
     if not args.no_extras and not train_mode and w.precision == synth.FP32:
         mt = npm.NPM(npm.config_from(w, max_batch=n, precision=synth.FP32_TC))
@@ -457,17 +464,18 @@ def main():
         torch.cuda.synchronize()
         tc_ms = e0.elapsed_time(e1) / kt
         fp32_tc = {"value": n * world / (tc_ms / 1e3), "unit": "queries/s", "ms_per_step": tc_ms,
-                   "over_fp32_cuda_cores": (n / (tc_ms / 1e3)) / (n / (kern_ms / 1e3)),
-                   "sectors_per_query": gather_sector_counts(mt, w, pos[0][:, :1 << 16].contiguous()) / (1 << 16),
+                   "over_fp32": (n / (tc_ms / 1e3)) / (n / (kern_ms / 1e3)),
+                   "sectors_per_query": gather_sector_counts(mt, w, pos[0][:, :1 << 16].contiguous(),
+                                                             n >= 1 << 18) / (1 << 16),
                    "mode": "NPM_FP32_TC: FP32 grid table; activations and weights as FP16 high part plus "
                            "FP16 residual, three tcgen05 MMAs per K step, FP32 accumulation; the FP32 "
                            "path's decode and sampler. Held to the FP32 bars (density and direction "
                            "within 1e-4 of the FP64 oracle)",
-                   "kernel": "k_forward_tc<8, 1, 0, 0, 1, 3> (three tile groups per SM)"}
+                   "kernel": "k_forward_tc (two FP16 parts, four tile groups per SM)"}
         mt.close()
 
     # Reduced-precision serving path: the tiny model at 2^22 queries per
-    # call in split BF16 on tensor cores, next to the FP32 CUDA-core path on
+    # call in split BF16, next to the FP32 path (three BF16 parts) on
     # the same inputs.
     reduced = None
     if not args.no_extras:
@@ -655,9 +663,9 @@ def main():
     props = torch.cuda.get_device_properties(local)
     clocks = clk.summary()
     sm_max = clocks.get("sm_max_mhz") or pk.get("sm_max_mhz", 2070.0)
-    # FP32 CUDA-core peak: SMs x 128 FP32 lanes x 2 flop x max SM clock.
-    alu_peak = props.multi_processor_count * 128 * 2 * sm_max * 1e6 / 1e12
-    achieved = mlp_flops(w) * n / (kern_ms / 1e3) / 1e12
+    # FP32 inference: six BF16 products of every weight and activation part
+    # on the tensor cores.
+    achieved = 6 * mlp_flops(w) * n / (kern_ms / 1e3) / 1e12
     per_sorted = sorted(per)
     line = {
         "metric": ("train samples/s (forward + backward + Adam)" if train_mode
@@ -679,23 +687,24 @@ def main():
                             f"{'samples' if train_mode else 'queries'} (the serving loop's "
                             "per-bounce latencies are under serving)"},
         "e2e": e2e,
-        # Kernels per step: one fused query kernel; a training step launches
-        # the training kernel, Adam, the step counter, the FP32 weight
-        # arrangement and the loss copy, and on tensor cores also the BF16
-        # weights, the FP16 grid copy and (2-feature grids) the encode kernel.
-        "gpu_launches": K * ((7 + (1 if w.feat == 2 else 0) if w.precision != synth.FP32 else 5)
-                             if train_mode else 1),
-        "roofline": ({"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
-                      "frac": achieved / alu_peak, "traffic": FP32_FORWARD_DRAM_BYTES,
+        # Kernels per step: one fused query kernel, and the check of the corner
+        # blocks before it for large batches on 2- and 4-feature grids (not
+        # the serving networks, one level); a training step launches
+        # the weights' arrangement, the training kernel and Adam, and on
+        # tensor cores with 2-feature grids the encode kernel before them.
+        "gpu_launches": K * ((3 + (1 if w.feat == 2 and w.precision != synth.FP32 else 0))
+                             if train_mode else
+                             2 if n >= 1 << 18 and w.feat in (2, 4) and len(w.level_res) > 1 else 1),
+        "roofline": ({"bound": "tensor", "achieved": achieved, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
+                      "frac": achieved / pk["bf16_tflops"], "traffic": FP32_FORWARD_DRAM_BYTES,
                       "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum of one 2^20-query "
-                                      "launch (profiles/k_forward_fp32_ws_paper_hash_2e20.md); ncu flushes "
+                                      "launch (profiles/k_forward_tc_fp32_paper_hash_2e20.md); ncu flushes "
                                       "the caches before the capture, so it includes the 41.7 MB FP32 "
-                                      "grid table that stays in L2 between calls; algorithmic HBM "
-                                      "bytes are 40 per query (41.9 MB). The same capture "
-                                      "shows the L1TEX data pipe at 82 % of its peak wavefront "
-                                      "rate (grid gathers plus the MLP's shared-memory operands)",
-                      "kernel": "k_forward_fp32_ws<sample>",
-                      "peak_source": "152 SMs x 128 FP32 lanes x 2 x max SM clock (derived)"}
+                                      "grid table and the corner blocks that stay in L2 between calls; "
+                                      "algorithmic HBM bytes are 40 per query (41.9 MB). The gathers, not "
+                                      "the MLP, bound the kernel: gather_roofline",
+                      "kernel": "k_forward_tc (three BF16 parts)",
+                      "peak_source": pk_src + " BF16 GEMM burst; six products per weight and activation"}
                      if (w.precision == synth.FP32 and not train_mode) else None),
         "clocks": clocks,
         "train": train,
@@ -708,6 +717,7 @@ def main():
     }
     if unit_peaks:
         if fp32_tc:
+            line["gather_roofline"] = gather_roofline(value / world, fp32_tc["sectors_per_query"], unit_peaks)
             fp32_tc["roofline"] = gather_roofline(fp32_tc["value"] / world, fp32_tc["sectors_per_query"],
                                                   unit_peaks)
         if reduced:

@@ -159,9 +159,10 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __re
 constexpr int kBlkChunk = 1024;
 // Queries from which a batch uses them. Tables in the L2, without and with
 // blocks (GB300; paper-shaped hash grid in FP32 and FP16, eight dense levels
-// of four features in split BF16): 2^17 queries 85 and 83, 55 and 52, 41 and
-// 39 us, about what bringing stale blocks up to date takes (9 us); 2^18 151
-// and 143, 103 and 93, 75 and 67; 2^20 562 and 509, 371 and 326, 260 and 216.
+// of four features in split BF16): 2^16 queries 36 and 37, 29 and 27, 21 and
+// 21 us; 2^17 60 and 60, 47 and 41, 33 and 31, less than bringing stale blocks
+// up to date takes (9 us); 2^18 111 and 101, 87 and 73, 60 and 52; 2^20 398
+// and 344, 288 and 230, 204 and 158.
 constexpr int64_t kBlkMinQueries = 1 << 18;
 
 // Rewrites the chunks of corner blocks whose parameters have changed since
@@ -468,8 +469,9 @@ __global__ void __launch_bounds__(256) k_train_encode(const __grid_constant__ De
 // Measured against one tile of 256 threads a CTA (GB300): product-mode
 // network, 2^19 samples, kernel 610 -> 451 us, with vector reductions in the
 // place of atomics on vectors (which return their result; 972 us with them)
-// and the flush of the weight gradients below; small network, 2^18 samples,
-// 100 -> 82 us (165 us with one scalar atomic per weight and share).
+// and the flush of the weight gradients below (383 us with elect_one and the
+// deferred scatter's turns as well); small network, 2^18 samples, 100 -> 82 us
+// (165 us with one scalar atomic per weight and share), now 67.
 __host__ __device__ constexpr int train_ctas_per_sm(int kmax, bool f2, int g) {
     return g == 1 && kmax == 4 && !f2 ? 3 : 1;
 }

@@ -23,24 +23,26 @@
 // flight (bounded), releases its tensor memory and returns.
 //
 // What bounds it on hash grids is the gathers: the L1 takes one request per
-// lane and cycle, about 6 requests per level and query. Activations in tensor
+// lane and cycle, about 6 requests per level and query, and the L2 9.9 TB/s of
+// random 32-byte sectors (0.64 to 0.83 of that reached). Activations in tensor
 // memory leave shared memory to the weights alone, so the rest of the 256 KB
 // stays L1 and four groups (16 warps, 128 registers) fit where activation
 // tiles in shared memory left room for one to three. Measured against those
-// (GB300, one call): 64-wide product-mode network in the FP32-accuracy mode,
-// 300,007 queries, 339 -> 140 us (one group -> four); paper-shaped hash grid,
-// FP16, 2,073,600 queries, 869 -> 719 us (three -> four); eight dense levels
-// of four features, split BF16, 250,007 densities, 102 -> 72 us.
+// (GB300, one call; in brackets with what followed: corner blocks, aligned
+// pairs, elect_one): 64-wide product-mode network in the FP32-accuracy mode,
+// 300,007 queries, 339 -> 140 us (107); paper-shaped hash grid, FP16,
+// 2,073,600 queries, 869 -> 719 us (416); eight dense levels of four features,
+// split BF16, 250,007 densities, 102 -> 72 us (57).
 // Large batches read the dense levels through corner blocks (npm_tc.cuh), one
 // or two 32-byte loads a level.
 //
 // FP32 models run here too, their values as three BF16 parts: 8 + 8 + 8 bits
 // hold an FP32 value, and six products of parts leave out less than 2^-24 of
 // it. Against the CUDA-core kernel (GB300): paper-shaped hash grid, 2^20
-// queries, 722 -> 567 us, 3,001 log densities 31 -> 23 us; at 2^18 queries
-// eight dense levels of four features 175 -> 115, 96-wide layers 302 -> 133,
-// 128-wide (one group by its tensor-memory columns) 357 -> 222, sixteen lobes
-// 258 -> 176, one level into 32-wide layers 46 -> 44 us. The error against
+// queries, 717 -> 346 us, 3,001 log densities 31 -> 18 us; at 2^18 queries
+// eight dense levels of four features 175 -> 76, 96-wide layers 303 -> 107,
+// 128-wide 357 -> 124, sixteen lobes 258 -> 138, three features a level 173 ->
+// 131, one level into 32-wide layers 47 -> 32 us. The error against
 // FP64 stays where it was (density 3.6e-6 and 3.7e-6 relative, log density
 // 2.7e-7 and 2.1e-7): the hardware exponentials decide it.
 #pragma once
@@ -694,10 +696,10 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
                  long long wait_limit) {
     extern __shared__ __align__(1024) uint8_t smem[];
     // Levels of 2-feature grids gathered before the first is blended: what the
-    // registers hold without spilling (2^20 queries of the paper-shaped grid,
-    // FP16 with 2, 3, 4: 302, 290, 327 us, four spilling 116 bytes; FP32
-    // accuracy with 1, 2: 377, 407 us, two spilling 120 bytes; FP32, three
-    // groups, with 2, 3: 461, 469 us).
+    // registers hold without spilling (GB300, 2^20 queries of the paper-shaped
+    // grid: FP16 with 2, 3, 4: 241, 229, 241 us; split BF16 254, 247, 256;
+    // FP32 accuracy with 1, 2: 312, 324; FP32 in three groups with 1, 2, 3:
+    // 369, 345, 348).
     constexpr int NF = GMAX == 3 ? 2 : OpsTraits<OPS>::fp32 ? 1 : 3;
     const int G = (int)(blockDim.x >> 7);
     const int g = (int)warp_uniform(threadIdx.x >> 7);  // tile group
@@ -947,12 +949,14 @@ cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint4* blk, c
         // FP32 has instances that keep the third part in tensor memory too.
         // 4-feature grids take theirs where its columns suffice for four
         // groups (2^18 queries of a 16-wide network: 44 us, with the part in
-        // shared memory 47). 2-feature grids' has three groups with two
-        // levels' gathers in flight, against four with one, whose rounds of
-        // tiles take 1.37 times as long: whichever needs less for the rounds
-        // of this batch (paper-shaped grid, three and four groups: 3,000
-        // queries 20 and 21 us; 2^16 50 and 42; 2^17 78 and 71; 2^18 128 and
-        // 132; 2^20 449 and 461).
+        // shared memory 47, before elect_one). 2-feature grids' has three
+        // groups with two levels' gathers in flight, against four with one,
+        // whose rounds of tiles take 1.37 times as long: whichever needs less
+        // for the rounds of this batch (GB300, paper-shaped grid, three and
+        // four groups: 3,000 queries 16.9 and 18.9 us; 2^16 41.0 and 36.6;
+        // 2^17 63.6 and 59.9; 2^18 100.8 and 110.7; 2^20 345 and 373). Of the
+        // two-part formats three groups gain nothing (FP32 accuracy, 2^20:
+        // 320 against 312).
         if (c.base.feat == 4 && 4u * fwd_group_cols<OPS, false>(c) <= 512u)
             return launch_fwd<8, 4, OPS, false, 4, false>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
         if (c.base.feat == 2 && fwd_group_count<OPS, false>(c, 3) == 3) {
