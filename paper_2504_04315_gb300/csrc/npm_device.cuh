@@ -54,7 +54,13 @@ struct DevCfg {
 // serialization may start while its predecessor in the stream is still
 // running; grid_dep_wait() returns once that predecessor has completed and
 // its writes are visible (at once for a kernel launched without it).
-// grid_dep_launch() lets the stream's next such kernel be scheduled.
+// grid_dep_launch() lets the stream's next such kernel be scheduled. What the
+// predecessor writes is read after the wait through pointers without
+// __restrict__, which the compiler may take for constant memory and read
+// before it. Adam, the weights' arrangement and the forward behind the corner
+// blocks' check are launched so (GB300: small network's training step 77 -> 74
+// us, the paper's own grid in FP32 250 -> 247; 300,007 product-mode queries
+// 107.5 -> 105). The training kernel behind its encode is not (594 -> 595).
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -437,7 +443,7 @@ __device__ __forceinline__ void end_update(const UpdateEnd& e) {
 // Arrange layer l of the MLP weights (row-major [out][in] per layer, packed)
 // into the padded blob W^T [in][np_fwd] of the CUDA-core kernels; thread tid
 // of nt.
-__device__ __forceinline__ void arrange_layer(const DevCfg& cfg, int l, const float* __restrict__ mlp,
+__device__ __forceinline__ void arrange_layer(const DevCfg& cfg, int l, const float* mlp,
                                               float* __restrict__ wfwd, int tid, int nt) {
     for (int m = 0; m < l; ++m) mlp += cfg.widths[m] * cfg.widths[m + 1];
     const int K = cfg.widths[l], N = cfg.widths[l + 1], np = cfg.np_fwd[l];

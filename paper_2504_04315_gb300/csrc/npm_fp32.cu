@@ -836,6 +836,7 @@ __global__ void __launch_bounds__(kTrainGroups* kTrainT, 1)
                  const float* __restrict__ spdf, const float* __restrict__ dlogv, float inv_n,
                  float* __restrict__ grad, double* __restrict__ loss) {
     extern __shared__ float4 smem4[];
+    grid_dep_launch();
     float* sW = reinterpret_cast<float*>(smem4);
     const int L = cfg.n_layers;
     const int G = blockDim.x / kTrainT, group = threadIdx.x / kTrainT, t = threadIdx.x % kTrainT;
@@ -897,8 +898,9 @@ __global__ void __launch_bounds__(kTrainGroups* kTrainT, 1)
 // ------------------------------------------------------- utility kernels
 
 // blockIdx.y: layer.
-__global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const float* __restrict__ mlp,
-                                  float* __restrict__ wfwd, UpdateEnd end) {
+__global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const float* mlp, float* __restrict__ wfwd,
+                                  UpdateEnd end) {
+    grid_dep_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) end_update(end);
     arrange_layer(cfg, blockIdx.y, mlp, wfwd, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
@@ -913,9 +915,10 @@ __global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const floa
 // (Sec. 5.3); the FP16 copy (inference only) is then taken from e.
 __global__ void k_adam(int64_t n4, float4* __restrict__ p, float4* __restrict__ g,
                        float4* __restrict__ m, float4* __restrict__ v, float lr, float b1, float b2,
-                       float eps, const int* __restrict__ steps, const double* __restrict__ loss,
-                       int* __restrict__ status, __half2* __restrict__ half_copy, int64_t n_half,
+                       float eps, const int* steps, const double* loss, int* __restrict__ status, __half2* __restrict__ half_copy, int64_t n_half,
                        float4* __restrict__ ema, float ema_decay) {
+    grid_dep_wait();
+    grid_dep_launch();
     const bool skip = loss != nullptr && !isfinite((float)*loss);
     if (skip && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kStatusNumeric);
     const float t = (float)(*steps + 1);
@@ -1157,8 +1160,7 @@ cudaError_t launch_train_fp32(const DevCfg& cfg, const float* params, int64_t ml
 
 cudaError_t launch_arrange_weights(const DevCfg& cfg, const float* mlp, float* wfwd, const UpdateEnd& end,
                                    cudaStream_t st) {
-    k_arrange_weights<<<dim3(16, cfg.n_layers), 256, 0, st>>>(cfg, mlp, wfwd, end);
-    return cudaGetLastError();
+    return launch_maybe_pdl(k_arrange_weights, dim3(16, cfg.n_layers), dim3(256), 0, st, true, cfg, mlp, wfwd, end);
 }
 
 cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float lr, float b1,
@@ -1170,12 +1172,10 @@ cudaError_t launch_adam(int64_t n, float* p, float* g, float* m, float* v, float
     const int cap = sm_count() * 16;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    k_adam<<<grid, 256, 0, st>>>(n4, reinterpret_cast<float4*>(p), reinterpret_cast<float4*>(g),
-                                 reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v), lr, b1,
-                                 b2, eps, steps, loss, status,
-                                 reinterpret_cast<__half2*>(half_copy), n_half,
-                                 reinterpret_cast<float4*>(ema), ema_decay);
-    return cudaGetLastError();
+    return launch_maybe_pdl(k_adam, dim3(grid), dim3(256), 0, st, true, n4, reinterpret_cast<float4*>(p),
+                            reinterpret_cast<float4*>(g), reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v),
+                            lr, b1, b2, eps, steps, loss, status, reinterpret_cast<__half2*>(half_copy), n_half,
+                            reinterpret_cast<float4*>(ema), ema_decay);
 }
 
 cudaError_t launch_grid_indices(const DevCfg& cfg, int64_t n, int64_t ld, const float* pos,

@@ -120,8 +120,9 @@ __device__ __forceinline__ void tc_encode(const TcCfg& tc, const float* __restri
 // the UMMA K-major layout, zero padded to Np x Kp per layer; with wfwd also
 // the CUDA-core kernels' padded copy. blockIdx.y: layer (one pass of load latency for all layers
 // instead of one each).
-__global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* __restrict__ mlp,
-                             uint8_t* __restrict__ blob, float* __restrict__ wfwd, UpdateEnd end) {
+__global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp, uint8_t* __restrict__ blob,
+                             float* __restrict__ wfwd, UpdateEnd end) {
+    grid_dep_wait();
     const int l = blockIdx.y;
     if (l == 0 && blockIdx.x == 0 && threadIdx.x == 0) end_update(end);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(256) k_corner_blocks(const __grid_constant__ T
                                                        int force) {
     constexpr int C = blk_corners(F, sizeof(GT)), V = 8 / C;  // corners, 32-bit values a corner
     __shared__ int now, stale;
+    grid_dep_launch();
     if (threadIdx.x == 0) {
         now = *version;
         stale = force || built[blockIdx.x] != now;
@@ -528,6 +530,7 @@ __global__ void __launch_bounds__(kTrainThreads* G, train_ctas_per_sm(KMAX, F2, 
     }
     bool ok = !__syncthreads_or(threadIdx.x < 32 && !mbar_wait_bounded(bar_w, 0));
     tc_fence_after();
+    if (G == 1) grid_dep_launch();  // (two groups: 593 -> 600 us with it)
     uint32_t phase = 0;
     bool issued = false;
     const uint32_t acc = tmem + tt.acc_col + (uint32_t)g * tt.acc_cols;
@@ -1119,20 +1122,23 @@ void tc_destroy(npm_handle* h) {
 cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, const UpdateEnd& end, cudaStream_t st) {
     TcState* s = h->tc;
     // The launch that ends the update comes last.
-    const dim3 grid(16, h->dc.n_layers);
+    auto arrange = [&](const TcCfg& cfg, const float* mlp, uint8_t* blob, float* wfwd, const UpdateEnd& e) {
+        return launch_maybe_pdl(k_tc_weights, dim3(16, h->dc.n_layers), dim3(256), 0, st, true, cfg, mlp, blob, wfwd, e);
+    };
+    cudaError_t e = cudaSuccess;
     if (s->wblob_train)
-        k_tc_weights<<<grid, 256, 0, st>>>(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, UpdateEnd{});
-    if (h->ema) {
+        e = arrange(s->train_cfg, h->params + h->mlp_off, s->wblob_train, nullptr, UpdateEnd{});
+    if (e == cudaSuccess && h->ema) {
         if (!s->wblob_inf) {
             const size_t bytes = (size_t)s->cfg.wparts * s->cfg.w_bytes;
-            cudaError_t e = cudaMalloc(&s->wblob_inf, bytes);
+            e = cudaMalloc(&s->wblob_inf, bytes);
             if (e != cudaSuccess) return e;
             cudaMemsetAsync(s->wblob_inf, 0, bytes, st);
         }
-        k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, UpdateEnd{});
+        e = arrange(s->cfg, h->ema + h->mlp_off, s->wblob_inf, nullptr, UpdateEnd{});
     }
-    k_tc_weights<<<grid, 256, 0, st>>>(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr, end);
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return arrange(s->cfg, h->params + h->mlp_off, s->wblob, cuda_cores ? h->wfwd : nullptr, end);
 }
 
 template <int KMAX, bool F2, int G>

@@ -741,6 +741,9 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
     const uint32_t sW_addr = smem_u32(smem);
     const int L = tc.base.n_layers;
     const bool sample = qb.sample != 0;
+    // Launched as a programmatic dependent (of the corner blocks' check), the
+    // steps above overlap that kernel, which writes the blocks alone.
+    grid_dep_wait();
     const GridView<typename OpsTraits<OPS>::GridT> grid{table, blk, blk ? tc.blk_mask : 0u};
 
     // Tiles and queries of a segment in 32 bits: batches hold at most 2^31
@@ -932,9 +935,9 @@ cudaError_t launch_fwd(const TcCfg& cfg, const void* grid, const uint4* blk, con
     int64_t blocks = qb.n_dev ? (max_n + kTile - 1) / kTile : t0;
     if (blocks > sms) blocks = sms;
     if (blocks < 1) blocks = 1;
-    kern<<<(int)blocks, kThreads * G, smem, st>>>(
-        c, static_cast<const typename OpsTraits<OPS>::GridT*>(grid), blk, wblob, qb, status, wait_limit);
-    return cudaGetLastError();
+    return launch_maybe_pdl(kern, dim3((unsigned)blocks), dim3(kThreads * G), smem, st, blk != nullptr, c,
+                            static_cast<const typename OpsTraits<OPS>::GridT*>(grid), blk, wblob, qb, status,
+                            wait_limit);
 }
 
 // The instance of an operand format for this model: up to eight lobes with
