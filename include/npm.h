@@ -447,7 +447,11 @@ npm_status npm_set_params_device(npm_handle* h, const float* dev, int64_t count,
 npm_status npm_get_grads_device(npm_handle* h, float* dev, int64_t count, void* stream);
 
 /* Device pointers to the FP32 master parameters and gradient (owned by the
- * handle, valid until npm_destroy). */
+ * handle, valid until npm_destroy; npm_params_device returns NULL if a CUDA
+ * call fails). The grid's part of the parameters is the table that NPM_FP32
+ * and NPM_FP32_TC queries read: what the caller writes there counts for every
+ * query ordered after the write, also in graphs captured before the pointer
+ * was asked for. */
 float* npm_params_device(npm_handle* h);
 float* npm_grads_device(npm_handle* h);
 

@@ -385,7 +385,24 @@ int64_t npm_num_params(const npm_handle* h) { return h ? h->ng + h->nmlp : -1; }
 
 float* npm_params_device(npm_handle* h) {
     if (!h) return nullptr;
-    h->params_shared = true;
+    if (!h->params_shared) {
+        // On a stream of the library's own, and in relaxed mode, so that a
+        // capture in progress neither records nor refuses it.
+        int dev = h->device;
+        cudaGetDevice(&dev);
+        if (dev != h->device) cudaSetDevice(h->device);
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaError_t e = cudaMemsetAsync(shared_word(h), 1, sizeof(int), h->side[0]);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->side[0]);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (dev != h->device) cudaSetDevice(dev);
+        if (e != cudaSuccess) {
+            cuda_fail(e, "npm_params_device");
+            return nullptr;
+        }
+        h->params_shared = true;
+    }
     return h->params;
 }
 float* npm_grads_device(npm_handle* h) { return h ? h->grads : nullptr; }

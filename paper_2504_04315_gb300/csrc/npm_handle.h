@@ -27,11 +27,12 @@ struct npm_handle {
     float* wfwd = nullptr;     // padded W^T blob of the CUDA-core kernels
     __half* grid_h = nullptr;  // FP16 grid copy (BF16 precision)
     // [0] loss accumulator (64 bits; zero between training steps), [8] status
-    // word, [16] Adam steps, [24] version of
-    // the parameters (both counted on the device, so that replayed graphs
-    // count too)
+    // word, [16] Adam steps, [24] version of the parameters (both counted on
+    // the device, so that replayed graphs count too), [28] not zero once
+    // npm_params_device has handed the parameters out (on the device, so that
+    // graphs captured before that see it)
     float* scalars = nullptr;
-    bool params_shared = false;  // npm_params_device has handed them out
+    bool params_shared = false;  // [28] has been set
     float* stage = nullptr;    // device staging for the _host entry points
     cudaStream_t side[2] = {nullptr, nullptr};  // internal streams (host staging)
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -57,6 +58,8 @@ inline double* loss_acc(npm_handle* h) { return reinterpret_cast<double*>(h->sca
 inline int* status_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 8); }
 // Device-side counter of changes to the parameters.
 inline int* version_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 24); }
+// Device-side flag: the caller holds the parameters' address.
+inline int* shared_word(npm_handle* h) { return reinterpret_cast<int*>(h->scalars + 28); }
 
 namespace npm {
 // NVTX range named after an entry point for the lifetime of the object, so

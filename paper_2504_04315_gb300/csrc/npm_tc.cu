@@ -167,7 +167,8 @@ constexpr int kBlkChunk = 1024;
 constexpr int64_t kBlkMinQueries = 1 << 18;
 
 // Rewrites the chunks of corner blocks whose parameters have changed since
-// (built[chunk] != *version), or all (force). Each chunk's mark is set by the
+// (built[chunk] != *version), or all where the table may have changed unseen
+// (shared not NULL and *shared not zero). Each chunk's mark is set by the
 // thread block that wrote all of it, so that launches on several streams may
 // overlap: they write the same bytes, and a query sees its own stream's
 // launch complete. Bound by its writes: 33 MB for 1.02 M entries.
@@ -175,13 +176,13 @@ template <typename GT, int F>
 __global__ void __launch_bounds__(256) k_corner_blocks(const __grid_constant__ TcCfg tc, const GT* __restrict__ table,
                                                        uint4* __restrict__ blk, uint32_t total,
                                                        int* __restrict__ built, const int* __restrict__ version,
-                                                       int force) {
+                                                       const int* __restrict__ shared) {
     constexpr int C = blk_corners(F, sizeof(GT)), V = 8 / C;  // corners, 32-bit values a corner
     __shared__ int now, stale;
     grid_dep_launch();
     if (threadIdx.x == 0) {
         now = *version;
-        stale = force || built[blockIdx.x] != now;
+        stale = built[blockIdx.x] != now || (shared && *shared);
     }
     __syncthreads();
     if (!stale) return;
@@ -1200,15 +1201,15 @@ cudaError_t tc_train(npm_handle* h, int64_t n, int64_t ld, const float* pos, con
 
 // The corner blocks of the inference table, brought up to date on st.
 template <typename GT>
-static cudaError_t update_blocks(npm_handle* h, const GT* table, int force, cudaStream_t st) {
+static cudaError_t update_blocks(npm_handle* h, const GT* table, const int* shared, cudaStream_t st) {
     TcState* s = h->tc;
     const unsigned chunks = (s->blk_total + kBlkChunk - 1) / kBlkChunk;
     if (h->cfg.feat_per_level == 2)
         k_corner_blocks<GT, 2><<<chunks, 256, 0, st>>>(s->cfg, table, s->blk, s->blk_total, s->blk_built,
-                                                       version_word(h), force);
+                                                       version_word(h), shared);
     else
         k_corner_blocks<GT, 4><<<chunks, 256, 0, st>>>(s->cfg, table, s->blk, s->blk_total, s->blk_built,
-                                                       version_word(h), force);
+                                                       version_word(h), shared);
     return cudaGetLastError();
 }
 
@@ -1229,9 +1230,10 @@ cudaError_t tc_query_batch(npm_handle* h, QueryBatch& qb, int64_t max_n, cudaStr
     const uint4* blk = s->blk && queries >= kBlkMinQueries ? s->blk : nullptr;
     if (blk) {
         // FP32 tables are the parameters themselves: a caller that holds
-        // their address may change them unseen.
-        cudaError_t e = c.fp32 ? update_blocks(h, inf_params(h), h->params_shared ? 1 : 0, st)
-                               : update_blocks(h, h->grid_h, 0, st);
+        // their address may change them unseen. The flag is read on the
+        // device: a graph may be captured before the address is handed out.
+        cudaError_t e = c.fp32 ? update_blocks(h, inf_params(h), shared_word(h), st)
+                               : update_blocks(h, h->grid_h, nullptr, st);
         if (e != cudaSuccess) return e;
     }
     const long long limit = 1ll << 32;  // the 16-bit kernels' fixed bound

@@ -59,3 +59,53 @@ def test_blocks_equal_the_table(w, precision):
     _same(m, pos, u)
     m.check_device_status()
     m.close()
+
+
+@pytest.mark.parametrize("precision", [synth.FP32, synth.FP32_TC], ids=["fp32", "fp32tc"])
+def test_write_through_the_address_reaches_an_earlier_capture(precision):
+    # A query captured before the parameters' address was first asked for
+    # reads, at each replay, what has been written through it.
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    w = TWO
+    pos, u = cuda(synth.positions(5, N)), cuda(synth.sample_uniforms(5, N))
+    m = make_model(w, synth.random_params(w, 53), N, precision=precision)
+    out = torch.empty(3, N, device="cuda"), torch.empty(N, device="cuda")
+    m.query_sample(pos, u, out=out)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        m.query_sample(pos, u, out=out)
+    ptr = m._L.npm_params_device(m.handle)
+    ng = sum(synth.grid_sizes(w)) * w.feat
+
+    class Grid:
+        __cuda_array_interface__ = {"shape": (ng,), "typestr": "<f4", "data": (ptr, False), "version": 2}
+
+    grid = torch.as_tensor(Grid(), device="cuda")
+    for scale in (0.5, -1.0):
+        grid.mul_(scale)
+        graph.replay()
+        for a, b in ((0, N // 2), (N // 2, N)):
+            d, p, _ = m.query_sample(pos[:, a:b].contiguous(), u[:, a:b].contiguous())
+            assert torch.equal(out[0][:, a:b], d) and torch.equal(out[1][a:b], p), (scale, a)
+    m.check_device_status()
+    m.close()
+
+
+def test_address_asked_for_during_a_capture():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    w = TWO
+    pos, u = cuda(synth.positions(6, 4096)), cuda(synth.sample_uniforms(6, 4096))
+    m = make_model(w, synth.random_params(w, 54), 4096, precision=synth.FP32)
+    out = torch.empty(3, 4096, device="cuda"), torch.empty(4096, device="cuda")
+    want = m.query_sample(pos, u)[1]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        m.query_sample(pos, u, out=out)
+        assert m._L.npm_params_device(m.handle)
+    graph.replay()
+    assert torch.equal(out[1], want)
+    m.close()
