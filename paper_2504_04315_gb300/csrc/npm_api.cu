@@ -181,15 +181,15 @@ npm_status arrange_all_weights(npm_handle* h, const npm::UpdateEnd& end, cudaStr
     return NPM_OK;
 }
 
-// Every copy derived from the parameters: the arranged weights and the FP16
-// grid.
+// Every copy derived from the parameters: the FP16 grid and the arranged
+// weights. The version moves last, once the table that it stands for is
+// written: a query on another stream in between would mark corner blocks of
+// the old table with the new version, for good.
 npm_status refresh_derived(npm_handle* h, cudaStream_t st) {
+    if (h->grid_h) NPM_CUDA(npm::launch_to_half(h->ng, inf_params(h), h->grid_h, st), "grid fp16 copy");
     npm::UpdateEnd end{};
     end.version = version_word(h);
-    npm_status s = arrange_all_weights(h, end, st);
-    if (s != NPM_OK) return s;
-    if (h->grid_h) NPM_CUDA(npm::launch_to_half(h->ng, inf_params(h), h->grid_h, st), "grid fp16 copy");
-    return NPM_OK;
+    return arrange_all_weights(h, end, st);
 }
 
 }  // namespace

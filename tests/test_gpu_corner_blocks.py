@@ -109,3 +109,29 @@ def test_address_asked_for_during_a_capture():
     graph.replay()
     assert torch.equal(out[1], want)
     m.close()
+
+
+def test_query_beside_an_update_leaves_no_stale_blocks():
+    # A query on another stream while the parameters are being replaced may
+    # see either set; the next query ordered after both sees the new one. The
+    # second stream's delay walks over the update's launches.
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    w = synth.Workload(name="dense 40, then 12 levels of 2^20", mode=synth.RADIANCE, level_res=[40] + [128] * 12,
+                       feat=2, log2_table=20, widths=[28, 16, 8], K=2, n_train=4096)
+    pos, u = cuda(synth.positions(7, N)), cuda(synth.sample_uniforms(7, N))
+    sets = [cuda(synth.random_params(w, s)) for s in (55, 56)]
+    m = make_model(w, synth.random_params(w, 57), N, precision=synth.FP16)
+    _same(m, pos, u)
+    side = torch.cuda.Stream()
+    out = torch.empty(3, N, device="cuda"), torch.empty(N, device="cuda")
+    for i in range(60):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(1 + 4000 * i)  # 2 us a step
+            m.query_sample(pos, u, out=out)
+        m.set_params_device(sets[i & 1])
+        torch.cuda.synchronize()
+        _same(m, pos, u)
+    m.check_device_status()
+    m.close()
