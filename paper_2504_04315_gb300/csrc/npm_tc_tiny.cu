@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
                 tc_fence_before();
             }
         }
-        // (after a wait that gave up the loop ends at the next barrier)
+        const bool put = ok && j < n;  // (after a wait that gave up the loop ends at the next barrier)
         // ---- decode (Table 1), sample (Sec. 5.3) and density (Eq. 4).
         float r[16];
 #pragma unroll
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
         const float ssum = (e01.x + e01.y) + (e23.x + e23.y);  // in [1, 4]
         const float inv = hw_rcp(ssum);
         LobePair P0, P1;
-        float* mix = valid ? S.mix : nullptr;
+        float* mix = put ? S.mix : nullptr;
         decode_pair(mul2(e01, f2(inv)), make_float2(r[1], r[5]), make_float2(r[2], r[6]), make_float2(r[3], r[7]),
                     P0, mix, 0, ld, j);
         decode_pair(mul2(e23, f2(inv)), make_float2(r[9], r[13]), make_float2(r[10], r[14]),
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
             }
             float pv = pair_pdf(P0, w) + pair_pdf(P1, w);
             if (S.ufrac > 0.0f) pv = S.ufrac * kInv4Pi + (1.0f - S.ufrac) * pv;
-            if (valid) {
+            if (put) {
                 S.dir[j] = w[0];
                 S.dir[ld + j] = w[1];
                 S.dir[2 * ld + j] = w[2];
@@ -495,11 +495,12 @@ __global__ void __launch_bounds__(kThreads * kGroups, 1) k_forward_tiny(const __
             } else {
                 pv = pair_pdf(P0, w) + pair_pdf(P1, w);
             }
-            if (valid) S.pdf[j] = pv;
+            if (put) S.pdf[j] = pv;
         }
     }
     if (!ok) {
-        if (t == 0) atomicOr(status, kStatusTimeout);
+        // (by warp: after the last tile no barrier passes a give-up on)
+        if ((t & 31) == 0) atomicOr(status, kStatusTimeout);
         // Drain this group's own asynchronous work (bounded) before the
         // tensor memory is released: the MMA batch whose wait gave up (and,
         // for group 0, the weights' and grid's bulk copies).
