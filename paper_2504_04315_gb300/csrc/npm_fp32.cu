@@ -913,10 +913,9 @@ __global__ void k_arrange_weights(const __grid_constant__ DevCfg cfg, const floa
 // (the grid). With ema set, also the exponential moving average
 // e <- d e + (1 - d) p of the updated parameters that inference evaluates
 // (Sec. 5.3); the FP16 copy (inference only) is then taken from e.
-__global__ void k_adam(int64_t n4, float4* __restrict__ p, float4* __restrict__ g,
-                       float4* __restrict__ m, float4* __restrict__ v, float lr, float b1, float b2,
-                       float eps, const int* steps, const double* loss, int* __restrict__ status, __half2* __restrict__ half_copy, int64_t n_half,
-                       float4* __restrict__ ema, float ema_decay) {
+__global__ void k_adam(int64_t n4, float4* p, float4* g, float4* m, float4* v, float lr, float b1, float b2,
+                       float eps, const int* steps, const double* loss, int* __restrict__ status,
+                       __half2* __restrict__ half_copy, int64_t n_half, float4* ema, float ema_decay) {
     grid_dep_wait();
     grid_dep_launch();
     const bool skip = loss != nullptr && !isfinite((float)*loss);
