@@ -403,9 +403,12 @@ __host__ __device__ constexpr int blk_corners(int feat, int value_bytes) { retur
 struct Block32 {
     uint32_t r[8];
 };
-__device__ __forceinline__ Block32 load_block(const uint4* __restrict__ blk, uint32_t e) {
+// Plain loads, unlike the table's: a forward launched as a dependent of
+// k_corner_blocks runs while that still writes the blocks, and reads them
+// after its wait (their addresses depend on positions that it reads after it).
+__device__ __forceinline__ Block32 load_block(const uint4* blk, uint32_t e) {
     Block32 b;
-    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=r"(b.r[0]), "=r"(b.r[1]), "=r"(b.r[2]), "=r"(b.r[3]), "=r"(b.r[4]), "=r"(b.r[5]), "=r"(b.r[6]),
           "=r"(b.r[7])
         : "l"(blk + 2 * (size_t)e));
@@ -462,7 +465,7 @@ template <>
 struct Level2<float> {
     float r[16];
     uint32_t swap;  // bit i: pair i swapped
-    __device__ __forceinline__ void load_blocks(const uint4* __restrict__ blk, uint32_t e, uint32_t DD) {
+    __device__ __forceinline__ void load_blocks(const uint4* blk, uint32_t e, uint32_t DD) {
         const Block32 b[2] = {load_block(blk, e), load_block(blk, e + DD)};
 #pragma unroll
         for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(b[i >> 3].r[i & 7]);
@@ -504,7 +507,7 @@ template <>
 struct Level2<__half> {
     uint32_t r[8];  // corners; from the table pair i may come swapped
     uint32_t swap;
-    __device__ __forceinline__ void load_blocks(const uint4* __restrict__ blk, uint32_t e, uint32_t) {
+    __device__ __forceinline__ void load_blocks(const uint4* blk, uint32_t e, uint32_t) {
         const Block32 b = load_block(blk, e);
 #pragma unroll
         for (int i = 0; i < 8; ++i) r[i] = b.r[i];
@@ -545,13 +548,13 @@ struct Level2<__half> {
 };
 
 // Corner features of 4 features of a cell with lowest block e; DD = D^2.
-__device__ __forceinline__ void gather_blocks4(const uint4* __restrict__ blk, uint32_t e, uint32_t, uint32_t DD,
+__device__ __forceinline__ void gather_blocks4(const uint4* blk, uint32_t e, uint32_t, uint32_t DD,
                                                const __half*, uint2 (&v)[8]) {
     const Block32 b[2] = {load_block(blk, e), load_block(blk, e + DD)};
 #pragma unroll
     for (int c = 0; c < 8; ++c) v[c] = make_uint2(b[c >> 2].r[2 * (c & 3)], b[c >> 2].r[2 * (c & 3) + 1]);
 }
-__device__ __forceinline__ void gather_blocks4(const uint4* __restrict__ blk, uint32_t e, uint32_t D, uint32_t DD,
+__device__ __forceinline__ void gather_blocks4(const uint4* blk, uint32_t e, uint32_t D, uint32_t DD,
                                                const float*, float4 (&v)[8]) {
     const Block32 b[4] = {load_block(blk, e), load_block(blk, e + D), load_block(blk, e + DD),
                           load_block(blk, e + DD + D)};

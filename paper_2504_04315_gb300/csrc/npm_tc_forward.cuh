@@ -692,8 +692,8 @@ template <int KMAX, int FEAT, int OPS, bool WARPDEC = false, int GMAX = fwd_grou
           bool THIRD = (OPS == kThreeBf16)>
 __global__ void __launch_bounds__(kThreads * GMAX, 1)
     k_forward_tc(const __grid_constant__ TcCfg tc, const typename OpsTraits<OPS>::GridT* __restrict__ table,
-                 const uint4* __restrict__ blk, const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb, int* __restrict__ status,
-                 long long wait_limit) {
+                 const uint4* blk, const uint8_t* __restrict__ wblob, const __grid_constant__ QueryBatch qb,
+                 int* __restrict__ status, long long wait_limit) {
     extern __shared__ __align__(1024) uint8_t smem[];
     // Levels of 2-feature grids gathered before the first is blended: what the
     // registers hold without spilling (GB300, 2^20 queries of the paper-shaped

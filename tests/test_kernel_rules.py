@@ -26,7 +26,7 @@ def test_every_warp_reports_its_own_timeout():
 # Parameters that a kernel behind griddepcontrol.wait may hold as __restrict__:
 # those it only writes, and those that no kernel before it in its chain writes.
 _RESTRICT = {"k_adam": {"status", "half_copy"}, "k_arrange_weights": {"wfwd"}, "k_tc_weights": {"blob", "wfwd"},
-             "k_forward_tc": {"table", "blk", "wblob", "status"}, "k_forward_tiny": {"grid4", "wblob", "status"}}
+             "k_forward_tc": {"table", "wblob", "status"}, "k_forward_tiny": {"grid4", "wblob", "status"}}
 
 
 def _kernels(text):
