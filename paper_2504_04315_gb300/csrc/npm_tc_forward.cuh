@@ -373,7 +373,7 @@ struct LobePair2 {
                      rp = make_float2(raw(4 * i + 3), raw(4 * i + 7));
         if (kappa_act == NPM_EXP) {
             const float2 e = __fmul2_rn(rk, f2(kL2E));
-            kap = make_float2(hw_ex2(e.x), hw_ex2(e.y));
+            kap = make_float2(hw_ex2_tiny(e.x), hw_ex2_tiny(e.y));
         } else {
             // max(t, 0) + ln(1 + e^{-|t|})
             const float2 e = __fmul2_rn(make_float2(fabsf(rk.x), fabsf(rk.y)), f2(-kL2E));
@@ -518,7 +518,7 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
                     }
                 }
                 const float2 e = p.exponent(w);
-                const float2 v = __fmul2_rn(l, __fmul2_rn(p.norm(), make_float2(hw_ex2(e.x), hw_ex2(e.y))));
+                const float2 v = __fmul2_rn(l, __fmul2_rn(p.norm(), make_float2(hw_ex2_tiny(e.x), hw_ex2_tiny(e.y))));
                 pv += v.x;
                 if (two) pv += v.y;
             }
