@@ -92,7 +92,11 @@ enum { NPM_FP32 = 0, NPM_BF16 = 1, NPM_BF16X3 = 2, NPM_FP16 = 3, NPM_FP32_TC = 4
  *                  as three BF16 parts, which hold all 24 bits of an FP32
  *                  value (products down to 2^-24 kept, FP32 accumulation);
  *                  networks whose weights do not fit there in that form (more
- *                  than about 34,000), and training, on the CUDA cores.
+ *                  than about 34,000), and training, on the CUDA cores. On the
+ *                  tensor cores a query's density and guided direction are NaN
+ *                  where a weight, one of its inputs or one of its hidden
+ *                  values is infinite; on both, ReLU makes zero of the outputs
+ *                  of a NaN weight of a hidden layer or of a NaN input.
  *                  NPM_BF16: FP16 grid copy, BF16 tensor-core MLP (tcgen05)
  *                  with FP32 accumulation; all vMF math stays FP32. Single-
  *                  pass BF16 inference does NOT meet the reduced-precision

@@ -129,9 +129,23 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp,
     if (wfwd) arrange_layer(tc.base, l, mlp, wfwd, tid, nt);
     const TcLayer& ly = tc.layer[l];
     for (int m = 0; m < l; ++m) mlp += tc.layer[m].K * tc.layer[m].N;
-    for (int i = tid; i < ly.Np * ly.Kp; i += nt) {
-        const int nn = i / ly.Kp, k = i % ly.Kp;
-        const float v = (nn < ly.N && k < ly.K) ? mlp[nn * ly.K + k] : 0.0f;
+    // Whole rows (outputs) at a time, a thread per weight.
+    __shared__ int bad[17];
+    const int rows = (int)blockDim.x / ly.Kp, r = (int)threadIdx.x / ly.Kp, k = (int)threadIdx.x % ly.Kp;
+    for (int n0 = blockIdx.x * rows; n0 < ly.Np; n0 += gridDim.x * rows) {
+        const int nn = n0 + r;
+        const bool mine = r < rows && nn < ly.Np;
+        float v = (mine && nn < ly.N && k < ly.K) ? mlp[nn * ly.K + k] : 0.0f;
+        // FP32 arithmetic: a NaN weight makes its output NaN for every query,
+        // which a hidden layer's ReLU takes for zero (three_bf16).
+        if (tc.wparts == 3 && l + 1 < tc.base.n_layers && __syncthreads_or(isnan(v))) {
+            if (threadIdx.x < 17) bad[threadIdx.x] = 0;
+            __syncthreads();
+            if (isnan(v)) bad[r] = 1;
+            __syncthreads();
+            if (bad[r]) v = 0.0f;
+        }
+        if (!mine) continue;
         uint8_t* at = blob + ly.w_off + tile_off(nn, k, ly.Kp);
         if (tc.f16) {
             // FP16 high part and FP16 residual (the weights to ~22 bits)
@@ -141,13 +155,11 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp,
             continue;
         }
         // BF16 parts, each rounded to nearest from what the ones before
-        // leave (three hold all 24 bits). An infinite weight becomes the
-        // largest finite value in FP32 arithmetic, where its residuals
-        // would be NaN.
+        // leave (three hold all 24 bits).
         float rest = v;
         for (int p = 0; p < tc.wparts; ++p) {
             __nv_bfloat16 b = __float2bfloat16_rn(rest);
-            if (tc.wparts == 3 && __hisinf(b)) b = __float2bfloat16_rz(copysignf(3.38e38f, rest));
+            if (tc.wparts == 3 && p == 0 && __hisinf(b)) b = __float2bfloat16_rz(copysignf(3.38e38f, rest));
             *reinterpret_cast<__nv_bfloat16*>(at + p * tc.w_bytes) = b;
             rest -= __bfloat162float(b);
         }

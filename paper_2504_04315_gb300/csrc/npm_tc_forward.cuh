@@ -77,23 +77,38 @@ __host__ __device__ constexpr int fwd_groups(int kmax) { return kmax > 8 ? 2 : 4
 // ----------------------------------------------------------- operands
 
 // Three BF16 parts of a pair: each rounded to nearest from what the ones
-// before leave, so that they add up to all 24 bits of the value. Infinities
-// become the largest finite value (an infinite part would make the others
-// NaN).
-__device__ __forceinline__ uint32_t bf16x2_finite(float a, float b) {
-    uint32_t d;
-    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
-    return d;
-}
+// before leave, so that they add up to all 24 bits of the value. The first
+// stays finite where a finite value would round to infinity.
+//
+// Infinite and NaN values: an infinite one has parts (largest, inf, NaN), so
+// that every output of the row becomes NaN and, with the NaN kept by ReLU
+// (relu_nan), the query's density NaN. FP32 arithmetic ends there too but for
+// the cases in which ReLU takes infinity less infinity for zero. Where it takes
+// a NaN weight's output, or those of a NaN input, for zero, so does this: the
+// arrangement of the weights clears the rows of hidden layers that hold a NaN,
+// and a row of inputs that holds one is cleared (clear_row).
 __device__ __forceinline__ void three_bf16(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
-    p0 = bf16x2_finite(a, b);
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(b), "f"(a));
     a -= __uint_as_float(p0 << 16);
     b -= __uint_as_float(p0 & 0xffff0000u);
-    p1 = bf16x2_finite(a, b);
+    p1 = pack_bf16(a, b);
     a -= __uint_as_float(p1 << 16);
     b -= __uint_as_float(p1 & 0xffff0000u);
-    p2 = bf16x2_finite(a, b);
+    p2 = pack_bf16(a, b);
 }
+__device__ __forceinline__ float relu_nan(float a) {
+    float d;
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(d) : "f"(a));
+    return d;
+}
+// NaN once a row of inputs has held one.
+template <int OPS>
+struct NanNote {
+    float v;
+    __device__ __forceinline__ void put(float a, float b) {
+        if constexpr (OPS == kThreeBf16) asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(v) : "f"(a), "f"(b));
+    }
+};
 
 // The operand parts of a pair of values (the first in the low half).
 template <int OPS>
@@ -122,8 +137,10 @@ __device__ __forceinline__ void relu_split_pair(float a, float b, uint32_t (&p)[
         asm("cvt.rn.satfinite.relu.f16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
     } else if constexpr (OPS == kOneBf16) {
         asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
-    } else if constexpr (OPS == kTwoFp16 || OPS == kThreeBf16) {
+    } else if constexpr (OPS == kTwoFp16) {
         split_pair<OPS>(fmaxf(a, 0.0f), fmaxf(b, 0.0f), p);
+    } else if constexpr (OPS == kThreeBf16) {
+        split_pair<OPS>(relu_nan(a), relu_nan(b), p);
     } else {
         asm("cvt.rz.relu.bf16x2.f32 %0, %1, %2;" : "=r"(p[0]) : "f"(b), "f"(a));
         const float ra = a - __uint_as_float(p[0] << 16), rb = b - __uint_as_float(p[0] & 0xffff0000u);
@@ -224,11 +241,13 @@ __device__ __forceinline__ float4 blend_level4(const TcCfg& tc, const GridView<G
 template <int OPS, bool THIRD>
 struct RowPacker {
     ActRow<THIRD> act;
+    NanNote<OPS>& nan;
     int k;
     float prev;
     __device__ __forceinline__ void put(float v) {
         if (k & 1) {
             uint32_t p[1][OpsTraits<OPS>::parts];
+            nan.put(prev, v);
             split_pair<OPS>(prev, v, p[0]);
             __syncwarp();
             put_pairs<OPS, THIRD, 1>(act, (uint32_t)(k >> 1), p);
@@ -258,7 +277,7 @@ __device__ __forceinline__ void product_inputs(const QuerySeg& S, uint32_t j, bo
 template <int FEAT, int OPS, int NF, bool THIRD>
 __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typename OpsTraits<OPS>::GridT>& grid,
                                            float x, float y, float z, const QuerySeg& S, uint32_t j, bool valid,
-                                           const ActRow<THIRD>& act) {
+                                           const ActRow<THIRD>& act, NanNote<OPS>& nan) {
     const DevCfg& cfg = tc.base;
     constexpr int P = OpsTraits<OPS>::parts;
     __syncwarp();
@@ -278,6 +297,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
 #pragma unroll
             for (int i = 0; i < NF; ++i) {
                 const float2 a = v[i].blend(cl[i]);
+                nan.put(a.x, a.y);
                 split_pair<OPS>(a.x, a.y, p[i]);
             }
             put_pairs<OPS, THIRD, NF>(act, (uint32_t)l, p);
@@ -288,6 +308,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             gather_level2(tc, grid, l, cl, v);
             const float2 a = v.blend(cl);
             uint32_t p[1][P];
+            nan.put(a.x, a.y);
             split_pair<OPS>(a.x, a.y, p[0]);
             put_pairs<OPS, THIRD, 1>(act, (uint32_t)l, p);
         }
@@ -298,13 +319,15 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
             for (int h = 0; h < (F >> 2); ++h) {
                 const float4 a = blend_level4(tc, grid, l, cl, F, h);
                 uint32_t p[2][P];
+                nan.put(a.x, a.y);
+                nan.put(a.z, a.w);
                 split_pair<OPS>(a.x, a.y, p[0]);
                 split_pair<OPS>(a.z, a.w, p[1]);
                 put_pairs<OPS, THIRD, 2>(act, (uint32_t)((l * F + 4 * h) >> 1), p);
             }
         }
     } else {
-        RowPacker<OPS, THIRD> row{act, 0, 0.0f};
+        RowPacker<OPS, THIRD> row{act, nan, 0, 0.0f};
         for (int l = 0; l < L; ++l) {
             const Cell cl = make_cell_in(x, y, z, cfg.level_res[l]);
             if (F == 2) {
@@ -344,6 +367,7 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
 #pragma unroll
             for (int i = 0; i < 22; i += 2) {
                 uint32_t p[1][P];
+                nan.put(e[i], e[i + 1]);
                 split_pair<OPS>(e[i], e[i + 1], p[0]);
                 put_pairs<OPS, THIRD, 1>(act, col + (uint32_t)(i >> 1), p);
             }
@@ -354,6 +378,30 @@ __device__ __forceinline__ void encode_row(const TcCfg& tc, const GridView<typen
     for (; col < end; ++col) {
         const uint32_t p[1][P] = {};
         put_pairs<OPS, THIRD, 1>(act, col, p);
+    }
+}
+
+// This thread's row of the first layer's input set to zero where `clear`. All
+// 32 lanes take part; rare.
+template <int OPS, bool THIRD>
+__device__ __noinline__ void clear_row(const TcCfg& tc, const ActRow<THIRD> act, bool clear) {
+    const uint32_t keep = clear ? 0u : ~0u;
+    tmem_wait_st();
+    for (uint32_t col = 0; col < (uint32_t)tc.layer[0].Kp >> 1; col += 2) {
+#pragma unroll
+        for (int p = 0; p < OpsTraits<OPS>::parts; ++p) {
+            if (THIRD && p == 2) {
+                uint2* at = reinterpret_cast<uint2*>(act.third + (col >> 2) * kPlane + (col & 3u) * 4u);
+                *at = make_uint2(at->x & keep, at->y & keep);
+                continue;
+            }
+            uint32_t r[2];
+            tmem_ld2(act.tmem + p * act.part_cols + col, r);
+            tmem_wait2(r);
+            r[0] &= keep;
+            r[1] &= keep;
+            tmem_st(act.tmem + p * act.part_cols + col, r);
+        }
     }
 }
 
@@ -784,7 +832,10 @@ __global__ void __launch_bounds__(kThreads * GMAX, 1)
                 if (b2 < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(S2.pos + r * S2.ld + b2));
             }
         }
-        encode_row<FEAT, OPS, NF, THIRD>(tc, grid, x, y, z, S, j, valid, row);
+        NanNote<OPS> nan{0.0f};
+        encode_row<FEAT, OPS, NF, THIRD>(tc, grid, x, y, z, S, j, valid, row, nan);
+        if constexpr (OPS == kThreeBf16)
+            if (L > 1 && __any_sync(0xffffffffu, isnan(nan.v))) clear_row<OPS, THIRD>(tc, row, isnan(nan.v));
         // The uniforms (or the direction), loaded now so that their latency
         // passes during the layers.
         float u[4] = {0.0f, 0.0f, sample ? 0.0f : 1.0f, 0.0f};
