@@ -89,6 +89,9 @@ npm_status set_error(npm_status s, const char* msg);
 // gets NPM_ERR_UNSUPPORTED from tc_create and runs on the CUDA-core kernels.
 npm_status tc_create(npm_handle* h);
 void tc_destroy(npm_handle* h);
+// The memory that launches of up to `queries` queries use beside what the
+// handle already has (corner blocks). Allocates: not a hot call.
+void tc_reserve_blocks(npm_handle* h, int64_t queries);
 // Weights arranged for the MMAs; with cuda_cores also h->wfwd.
 cudaError_t tc_refresh_weights(npm_handle* h, bool cuda_cores, const UpdateEnd& end, cudaStream_t st);
 // pdl: the small networks' kernel may be launched as a programmatic

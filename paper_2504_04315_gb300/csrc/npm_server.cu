@@ -340,6 +340,7 @@ npm_status npm_server_create(npm_handle* h, int64_t pool_queries, npm_server** o
         delete s;
         return npm::set_error(NPM_ERR_CUDA, msg);
     }
+    npm::tc_reserve_blocks(h, pool_queries);  // (a launch serves up to the pool's queries)
     s->free_list[0] = pool_queries;
     s->worker = std::thread(worker_loop, s);
     *out = s;

@@ -927,7 +927,8 @@ struct TcState {
     TcTrain train;
     bool can_train = false;
     // Corner blocks of the inference table (npm_tc.cuh), the version of the
-    // parameters that each chunk was built from, and their number; NULL: none.
+    // parameters that each chunk was built from, and their number; NULL: none
+    // (a handle whose batches cannot be large enough to use them).
     uint4* blk = nullptr;
     int* blk_built = nullptr;
     uint32_t blk_total = 0;
@@ -1091,9 +1092,9 @@ npm_status tc_create(npm_handle* h) {
             s->enc = nullptr;
         }
     }
-    // Optional too: corner blocks, in level order while they stay a part of
-    // the L2 (64 of 129 MB).
-    if (c.feat_per_level == 2 || c.feat_per_level == 4) {
+    // Corner blocks, in level order while they stay a part of the L2 (64 of 129
+    // MB).
+    if ((c.feat_per_level == 2 || c.feat_per_level == 4) && !tiny_qualifies(t)) {  // (that keeps its table in shared memory)
         constexpr uint64_t kMost = (64ull << 20) / 32;
         uint64_t total = 0;
         for (int l = 0; l < c.n_levels; ++l) {
@@ -1103,21 +1104,30 @@ npm_status tc_create(npm_handle* h) {
             t.blk_off[l] = (uint32_t)total;
             total += entries;
         }
-        const size_t chunks = (size_t)((total + kBlkChunk - 1) / kBlkChunk);
-        if (tiny_qualifies(t)) total = 0;  // keeps its table in shared memory
-        if (total && device_alloc((void**)&s->blk, 32 * (size_t)total) == cudaSuccess) {
-            if (device_alloc((void**)&s->blk_built, chunks * sizeof(int)) != cudaSuccess) {
-                cudaFree(s->blk);
-                s->blk = nullptr;
-            } else {
-                cudaMemset(s->blk_built, 0, chunks * sizeof(int));
-                s->blk_total = (uint32_t)total;
-            }
-        }
-        cudaGetLastError();
+        s->blk_total = (uint32_t)total;
     }
     h->tc = s;
+    tc_reserve_blocks(h, c.max_batch);
     return NPM_OK;
+}
+
+void tc_reserve_blocks(npm_handle* h, int64_t queries) {
+    TcState* s = h->tc;
+    if (!s || s->blk || !s->blk_total || queries < kBlkMinQueries) return;
+    const size_t chunks = (s->blk_total + kBlkChunk - 1) / kBlkChunk;
+    uint4* blk = nullptr;
+    int* built = nullptr;
+    // Optional: without them large batches read the table too.
+    if (device_alloc((void**)&blk, 32 * (size_t)s->blk_total) == cudaSuccess &&
+        device_alloc((void**)&built, chunks * sizeof(int)) == cudaSuccess &&
+        cudaMemset(built, 0, chunks * sizeof(int)) == cudaSuccess && cudaStreamSynchronize(0) == cudaSuccess) {
+        s->blk = blk;
+        s->blk_built = built;
+        return;
+    }
+    cudaGetLastError();
+    if (blk) cudaFree(blk);
+    if (built) cudaFree(built);
 }
 
 void tc_destroy(npm_handle* h) {

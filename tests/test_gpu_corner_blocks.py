@@ -135,3 +135,50 @@ def test_query_beside_an_update_leaves_no_stale_blocks():
         _same(m, pos, u)
     m.check_device_status()
     m.close()
+
+
+def _used(make):
+    """Device memory that an object takes, in MB (rounded by the driver)."""
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    made = make()
+    torch.cuda.synchronize()
+    return (before - torch.cuda.mem_get_info()[0]) / 2 ** 20, made
+
+
+def test_memory_only_where_batches_are_large_enough():
+    # 33 MB on this grid: a handle for smaller batches has none, until a
+    # server gathers larger ones from them.
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2504_04315_gb300 as npm
+    w = synth.PAPER_HASH
+    make = {n: (lambda n=n: npm.NPM(npm.config_from(w, max_batch=n))) for n in (N - 1, N)}
+    make[N]().close()  # (the context's and the driver's own memory)
+    small, m = _used(make[N - 1])
+    large, big = _used(make[N])
+    big.close()
+    assert 24 < large - small < 48, (small, large)
+    first, server = _used(lambda: npm.Server(m, 2 * N))
+    server.close()
+    second, server = _used(lambda: npm.Server(m, 2 * N))
+    server.close()
+    assert 24 < first - second < 48, (first, second)
+    params = synth.random_params(w, 58)
+    m.set_params(params)
+    # Four requests of 2^17 queries that the server takes in one launch give
+    # what the model gives one of them.
+    n = N // 2
+    pos, u = synth.positions(8, n), synth.sample_uniforms(8, n)
+    want = m.query_sample(cuda(pos), cuda(u))[1].cpu()
+    with npm.Server(m, 2 * N) as s:
+        t = torch.from_numpy(pos).pin_memory(), torch.from_numpy(u).pin_memory()
+        out = [(torch.zeros(3, n).pin_memory(), torch.zeros(n).pin_memory()) for _ in range(4)]
+        s.hold(True)
+        tickets = [s.submit_query(t[0], t[1], d, p) for d, p in out]
+        s.hold(False)
+        for k in tickets:
+            s.wait(k)
+        for _, p in out:
+            assert torch.equal(p, want)
+    m.close()
