@@ -452,8 +452,16 @@ npm_status npm_get_grads_device(npm_handle* h, float* dev, int64_t count, void* 
 
 /* Device pointers to the FP32 master parameters and gradient (owned by the
  * handle, valid until npm_destroy; npm_params_device returns NULL if a CUDA
- * call fails). The grid's part of the parameters is the table that NPM_FP32
- * and NPM_FP32_TC queries read: what the caller writes there counts for every
+ * call fails). Layout: the grid, then from the next multiple of 64 values on
+ * the weight matrices.
+ *   Alignment: 8 bytes, and no more can be relied on. A grid of 2 features
+ * starts 0, 8, 16 or 24 bytes past a 32-byte boundary, so that its hashed
+ * levels start on one (their gathers and gradient sums take 16-byte accesses
+ * there). Code that reads or writes through these pointers 16 bytes at a time
+ * has to look at their alignment; npm_set_params_device and
+ * npm_get_grads_device copy to and from buffers of the caller's own.
+ *   The grid's part of the parameters is the table that NPM_FP32 and
+ * NPM_FP32_TC queries read: what the caller writes there counts for every
  * query ordered after the write, also in graphs captured before the pointer
  * was asked for. */
 float* npm_params_device(npm_handle* h);

@@ -282,7 +282,9 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
     // Tables of 2 features start so that the first hashed level (and with it,
     // where they follow one another, every hashed level) starts on a 32-byte
     // (FP32) or 16-byte (FP16) boundary: half of its x-neighbours then share
-    // a 16-byte FP32 load, three quarters a 16-byte FP16 one.
+    // one load of twice the width. Without it (GB300): 2^20 FP32 queries of the
+    // 16-level grid 379 us against 346, an FP16 frame 440 against 416, a
+    // product-mode training step 617 against 588.
     if (d.feat == 2)
         for (int l = 0; l < d.n_levels; ++l)
             if (!((d.dense_mask >> l) & 1u)) {

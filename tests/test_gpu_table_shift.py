@@ -57,3 +57,27 @@ def test_shifted_tables(w, precision, bar):
     assert np.abs(m.get_ema_params() - (0.25 * params + 0.75 * got)).max() <= 1e-6
     assert not m.get_grads().any()
     m.check_device_status()
+
+
+@pytest.mark.parametrize("w", NETS, ids=lambda w: w.name.replace(" ", "-"))
+def test_pointers_are_aligned_as_documented(w):
+    # 8 bytes, the first hashed level on 32, parameters and gradient alike;
+    # the grid and the weights lie where the header says.
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    params = synth.random_params(w, 62)
+    m = make_model(w, params, 256)
+    sizes = synth.grid_sizes(w)
+    dense = sum(s for s, d in zip(sizes, w.level_res) if d ** 3 <= 1 << w.log2_table)
+    at, grad = m._L.npm_params_device(m.handle), m._L.npm_grads_device(m.handle)
+    assert at % 8 == 0 and (at + 8 * dense) % 32 == 0 and at % 32 == grad % 32
+    ng = 2 * sum(sizes)
+    mlp = (ng + 63) // 64 * 64
+
+    class Own:
+        __cuda_array_interface__ = {"shape": (mlp + params.size - ng,), "typestr": "<f4", "data": (at, False),
+                                    "version": 2}
+
+    own = torch.as_tensor(Own(), device="cuda").cpu().numpy()
+    assert np.array_equal(own[:ng], params[:ng]) and np.array_equal(own[mlp:], params[ng:])
+    m.close()
