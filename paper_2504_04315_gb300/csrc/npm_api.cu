@@ -441,13 +441,38 @@ npm_status npm_get_params(npm_handle* h, float* host, int64_t count) {
     return copy_public(h, h ? h->params : nullptr, host, count, false);
 }
 
+// Whether kernels on the handle's device may access p: its own memory or managed
+// memory. (Another device's needs peer access, and host memory a mapping; a copy
+// call knows about both.)
+static bool kernel_can_access(const npm_handle* h, const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == h->device);
+}
+
+// The grid and the MLP between the public layout and the library's: in one
+// launch where the caller's buffer lies on the handle's device, else by copies.
+static npm_status copy_both(npm_handle* h, const float* src, const float* src_mlp, float* dst, float* dst_mlp,
+                            const void* callers, const char* what, cudaStream_t st) {
+    if (kernel_can_access(h, callers)) {
+        NPM_CUDA(npm::launch_copy_params(src, dst, h->ng, src_mlp, dst_mlp, h->nmlp, st), what);
+        return NPM_OK;
+    }
+    NPM_CUDA(cudaMemcpyAsync(dst, src, h->ng * sizeof(float), cudaMemcpyDeviceToDevice, st), what);
+    NPM_CUDA(cudaMemcpyAsync(dst_mlp, src_mlp, h->nmlp * sizeof(float), cudaMemcpyDeviceToDevice, st), what);
+    return NPM_OK;
+}
+
 npm_status npm_set_params_device(npm_handle* h, const float* dev, int64_t count, void* stream) {
     npm::CallRange range("npm_set_params_device");
     if (!h || !dev) return fail(NPM_ERR_INVALID_ARG, "NULL argument");
     if (count != h->ng + h->nmlp) return fail(NPM_ERR_INVALID_ARG, "count != npm_num_params");
     cudaStream_t st = (cudaStream_t)stream;
-    NPM_CUDA(npm::launch_copy_params(dev, h->params, h->ng, dev + h->ng, h->params + h->mlp_off, h->nmlp, st),
-             "copy parameters");
+    npm_status s = copy_both(h, dev, dev + h->ng, h->params, h->params + h->mlp_off, dev, "copy parameters", st);
+    if (s != NPM_OK) return s;
     if (h->ema)
         NPM_CUDA(cudaMemcpyAsync(h->ema, h->params, h->n_int * sizeof(float), cudaMemcpyDeviceToDevice, st),
                  "reset ema");
@@ -459,9 +484,7 @@ npm_status npm_get_grads_device(npm_handle* h, float* dev, int64_t count, void* 
     if (!h || !dev) return fail(NPM_ERR_INVALID_ARG, "NULL argument");
     if (count != h->ng + h->nmlp) return fail(NPM_ERR_INVALID_ARG, "count != npm_num_params");
     cudaStream_t st = (cudaStream_t)stream;
-    NPM_CUDA(npm::launch_copy_params(h->grads, dev, h->ng, h->grads + h->mlp_off, dev + h->ng, h->nmlp, st),
-             "copy gradient");
-    return NPM_OK;
+    return copy_both(h, h->grads, h->grads + h->mlp_off, dev, dev + h->ng, dev, "copy gradient", st);
 }
 
 npm_status npm_set_ema(npm_handle* h, float decay, void* stream) {

@@ -85,3 +85,23 @@ def test_log_density_gradient_matches_finite_differences():
         fd = (f(params + h * v) - f(params - h * v)) / (2 * h)
         an = float(g @ v)
         assert abs(fd - an) <= 1e-2 * max(abs(an), 1e-3), (fd, an)
+
+
+@pytest.mark.parametrize("w", [synth.TINY, PRODUCT_SMALL], ids=["tiny", "product"])
+def test_parameters_and_gradient_through_other_memory(w):
+    # Buffers that are not the device's own (pinned host memory here, another
+    # device's elsewhere) are copied, not accessed by a kernel.
+    from paper_2504_04315_gb300 import _lib
+    n = 512
+    params = synth.random_params(w, 22)
+    b, wts = _batch(w, n, 22)
+    m = make_model(w, synth.init_params(w), n)
+    st = torch.cuda.current_stream().cuda_stream
+    theta = torch.from_numpy(params.astype(np.float32)).pin_memory()
+    _lib.check(m._L.npm_set_params_device(m.handle, theta.data_ptr(), theta.numel(), st), "set")
+    assert np.array_equal(m.get_params(), params)
+    m.backward(cuda(b.pos), cuda(b.dir), cuda(wts), None if b.aux is None else cuda(b.aux))
+    grad = torch.zeros(theta.numel()).pin_memory()
+    _lib.check(m._L.npm_get_grads_device(m.handle, grad.data_ptr(), grad.numel(), st), "get")
+    torch.cuda.synchronize()
+    assert grad.abs().max() > 0 and np.array_equal(grad.numpy(), m.get_grads())
