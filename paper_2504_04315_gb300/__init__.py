@@ -70,21 +70,30 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
-_raw_stream = None  # (device index) -> cudaStream_t of its current stream
+_raw_stream = None  # () -> cudaStream_t of torch's current stream
+
+
+def _raw_stream_of(torch):
+    """A function that gives the current stream's handle: without a
+    torch.cuda.Stream object around it (4 us of a small call's 20 us on the
+    host) where this torch has the two internal functions that takes, else
+    through the public call."""
+    raw, dev = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if raw is None or dev is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(dev())
 
 
 def _stream_ptr(stream) -> Optional[int]:
     if stream is not None:
         return stream.cuda_stream
-    # The current stream's handle without a torch.cuda.Stream object around it
-    # (4 us of a small call's 20 us on the host).
     global _raw_stream
-    torch = _torch()
     if _raw_stream is None:
+        torch = _torch()
         ptr = torch.cuda.current_stream().cuda_stream  # initialises CUDA in torch
-        _raw_stream = torch._C._cuda_getCurrentRawStream
+        _raw_stream = _raw_stream_of(torch)
         return ptr
-    return _raw_stream(torch._C._cuda_getDevice())
+    return _raw_stream()
 
 
 def _soa(t, rows: int, name: str):

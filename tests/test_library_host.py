@@ -87,3 +87,25 @@ def test_normal_build_compiles_bounds_checks_out(lib):
     # The bounds-checking kernels exist only in the debug build
     # (_build.build_debug, NPM_DEBUG_BOUNDS); the normal build reports -1.
     assert lib.npm_debug_bounds_violations() == -1
+
+
+def test_current_stream_without_torchs_internal_functions():
+    # The stream's handle through the internal functions of torch where it has
+    # them, else through its public call.
+    class Stream:
+        cuda_stream = 77
+
+    class Torch:
+        class cuda:
+            @staticmethod
+            def current_stream():
+                return Stream
+
+        class _C:
+            pass
+
+    assert npm._raw_stream_of(Torch)() == 77
+    Torch._C._cuda_getDevice = staticmethod(lambda: 3)
+    assert npm._raw_stream_of(Torch)() == 77
+    Torch._C._cuda_getCurrentRawStream = staticmethod(lambda d: 100 + d)
+    assert npm._raw_stream_of(Torch)() == 103
