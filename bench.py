@@ -157,6 +157,37 @@ def tc_roofline(qps, w, pk, up, sms, sm_mhz):
                            "npm_measure_unit_peaks; FP32 lanes = SMs x 128 x max SM clock"}
 
 
+def entry_offsets(w):
+    """Place of each level's first entry, in entries past a 32-byte boundary of
+    the table: tables of 2 features start so that their first hashed level lies
+    on one (npm_create)."""
+    offs = np.cumsum([0] + synth.grid_sizes(w)[:-1])
+    hashed = [o for o, d in zip(offs, w.level_res) if d ** 3 > 1 << w.log2_table]
+    return offs + ((-hashed[0]) % 4 if w.feat == 2 and hashed else 0)
+
+
+def serving_network(w):
+    """Whether a model's queries take the serving networks' kernel
+    (tiny_qualifies)."""
+    return (w.precision in (synth.BF16, synth.BF16X3, synth.FP16) and w.mode == synth.RADIANCE and w.feat == 4
+            and len(w.level_res) == 1 and w.K == 4 and len(w.widths) == 4 and max(w.widths) <= 32
+            and 8 * w.level_res[0] ** 3 <= (90 if w.precision == synth.BF16X3 else 150) << 10
+            and w.kappa_act == synth.SOFTPLUS)
+
+
+def launches_per_step(w, n, train):
+    """Kernels that one step launches. A query: the fused kernel, and before it
+    the corner blocks' check for large batches on 2- and 4-feature grids with a
+    dense level. A training step: the weights' arrangement (twice where training
+    reads another form of them than inference), the encode kernel of 2-feature
+    grids on tensor cores, the training kernel and Adam."""
+    if train:
+        tc = w.precision in (synth.BF16, synth.BF16X3, synth.FP16)
+        return 3 + (tc and w.feat == 2) + (w.precision in (synth.BF16, synth.FP16))
+    dense = any(d ** 3 <= 1 << w.log2_table for d in w.level_res)
+    return 1 + (n >= 1 << 18 and w.feat in (2, 4) and dense and not serving_network(w))
+
+
 def scatter_atomic_counts(model, w, pos_dev):
     """(four-wide, two-wide) atomic operations the tensor-core training
     kernel's grid-gradient scatter issues for one batch. Four features per
@@ -171,8 +202,7 @@ def scatter_atomic_counts(model, w, pos_dev):
         return 8 * len(w.level_res) * n, 0
     assert w.feat == 2, "counts are defined for 2- and 4-feature grids"
     idx = model.grid_indices(pos_dev).to(torch.int64)  # [L][8][n], entry within the level
-    offs = torch.tensor(np.cumsum([0] + synth.grid_sizes(w)[:-1]), dtype=torch.int64,
-                        device=idx.device)[:, None, None]
+    offs = torch.tensor(entry_offsets(w), dtype=torch.int64, device=idx.device)[:, None, None]
     a, b = idx[:, 0::2, :], idx[:, 1::2, :]
     lo = torch.minimum(a, b)
     paired = ((a - b).abs() == 1) & (((offs + lo) & 1) == 0)
@@ -184,14 +214,13 @@ def scatter_atomic_counts(model, w, pos_dev):
 def gather_sector_counts(model, w, pos_dev, blocks=False):
     """32-byte L2 sectors that a batch's grid gathers must touch: per query
     and level, the distinct sectors holding the 8 corners' FP32 entries
-    (feat x 4 bytes each, at the level's table offset), counted from the
+    (feat x 4 bytes each, where the level lies in the table), counted from the
     corner indices the library forms (npm_grid_indices). blocks:
     dense levels of 2 and 4 features through corner blocks, as batches of
     2^18 queries and more read them: at most feat sectors."""
     import torch
     idx = model.grid_indices(pos_dev).to(torch.int64)  # [L][8][n], entry within the level
-    offs = torch.tensor(np.cumsum([0] + synth.grid_sizes(w)[:-1]), dtype=torch.int64,
-                        device=idx.device)[:, None, None]
+    offs = torch.tensor(entry_offsets(w), dtype=torch.int64, device=idx.device)[:, None, None]
     fb = 4 * w.feat
     first = ((offs + idx) * fb) // 32                   # sector of each entry's first byte
     last = ((offs + idx) * fb + fb - 1) // 32           # and of its last byte
@@ -663,9 +692,9 @@ def main():
     props = torch.cuda.get_device_properties(local)
     clocks = clk.summary()
     sm_max = clocks.get("sm_max_mhz") or pk.get("sm_max_mhz", 2070.0)
-    # FP32 inference: six BF16 products of every weight and activation part
-    # on the tensor cores.
-    achieved = 6 * mlp_flops(w) * n / (kern_ms / 1e3) / 1e12
+    # FP32 inference: the MLP's own operations; each takes six BF16 products of
+    # parts on the tensor cores, so a sixth of their rate is the peak.
+    achieved = mlp_flops(w) * n / (kern_ms / 1e3) / 1e12
     per_sorted = sorted(per)
     line = {
         "metric": ("train samples/s (forward + backward + Adam)" if train_mode
@@ -687,16 +716,9 @@ def main():
                             f"{'samples' if train_mode else 'queries'} (the serving loop's "
                             "per-bounce latencies are under serving)"},
         "e2e": e2e,
-        # Kernels per step: one fused query kernel, and the check of the corner
-        # blocks before it for large batches on 2- and 4-feature grids (not
-        # the serving networks, one level); a training step launches
-        # the weights' arrangement, the training kernel and Adam, and on
-        # tensor cores with 2-feature grids the encode kernel before them.
-        "gpu_launches": K * ((3 + (1 if w.feat == 2 and w.precision != synth.FP32 else 0))
-                             if train_mode else
-                             2 if n >= 1 << 18 and w.feat in (2, 4) and len(w.level_res) > 1 else 1),
-        "roofline": ({"bound": "tensor", "achieved": achieved, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
-                      "frac": achieved / pk["bf16_tflops"], "traffic": FP32_FORWARD_DRAM_BYTES,
+        "gpu_launches": K * int(launches_per_step(w, n, train_mode)),
+        "roofline": ({"bound": "tensor", "achieved": achieved, "peak": pk["bf16_tflops"] / 6,
+                      "unit": "TFLOP/s", "frac": 6 * achieved / pk["bf16_tflops"], "traffic": FP32_FORWARD_DRAM_BYTES,
                       "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum of one 2^20-query "
                                       "launch (profiles/k_forward_tc_fp32_paper_hash_2e20.md); ncu flushes "
                                       "the caches before the capture, so it includes the 41.7 MB FP32 "
@@ -704,7 +726,7 @@ def main():
                                       "algorithmic HBM bytes are 40 per query (41.9 MB). The gathers, not "
                                       "the MLP, bound the kernel: gather_roofline",
                       "kernel": "k_forward_tc (three BF16 parts)",
-                      "peak_source": pk_src + " BF16 GEMM burst; six products per weight and activation"}
+                      "peak_source": pk_src + " BF16 GEMM burst / 6 (six products of parts per weight and activation)"}
                      if (w.precision == synth.FP32 and not train_mode) else None),
         "clocks": clocks,
         "train": train,

@@ -76,7 +76,10 @@ def test_gather_sector_counts_by_hand():
     torch = pytest.importorskip("torch")
     w = synth.PAPER_HASH  # two FP32 features: 8-byte entries, four to a sector
     L = len(w.level_res)
-    offs = np.cumsum([0] + synth.grid_sizes(w)[:-1])
+    # The dense levels hold 1 entry more than a multiple of 4, so the table
+    # starts 3 entries past a sector's boundary.
+    assert sum(d ** 3 for d in w.level_res if d ** 3 <= 1 << w.log2_table) % 4 == 1
+    offs = np.cumsum([3] + synth.grid_sizes(w)[:-1])
     idx = np.zeros((L, 8, 2), np.int64)
     # Query 0: every level's corners are entries 0..7 (two sectors when the
     # level starts on a sector boundary). Query 1: eight corners 64 entries
@@ -95,3 +98,43 @@ def test_gather_roofline_arithmetic():
     r = bench.gather_roofline(2e9, 96.0, {"l2_sector_read_gbs": 9600.0})
     assert r["peak"] == pytest.approx(9600e9 / (32 * 96.0))
     assert r["frac"] == pytest.approx(2e9 / r["peak"])
+
+
+# A dense level of 5^3 = 125 entries before two hashed ones of 2^12: the table
+# starts 3 entries past a 32-byte boundary, the hashed levels on one.
+SHIFTED = synth.Workload(name="5^3, then hashed", mode=synth.RADIANCE, level_res=[5, 30, 45], feat=2, log2_table=12,
+                         widths=[8, 16, 8], K=2)
+
+
+def test_entry_offsets_follow_the_table_shift():
+    assert list(bench.entry_offsets(SHIFTED)) == [3, 128, 128 + 4096]
+    assert list(bench.entry_offsets(SHIFTED.with_(feat=4))) == [0, 125, 125 + 4096]
+    assert list(bench.entry_offsets(SHIFTED.with_(log2_table=17))) == [0, 125, 125 + 27000]  # no hashed level
+
+
+def test_counts_on_a_shifted_table_by_hand():
+    torch = pytest.importorskip("torch")
+    idx = np.zeros((3, 8, 1), np.int64)
+    # Level 0 at entries 3 + ...: pairs (0, 1) and (4, 5) lie at 3, 4 and 7, 8
+    # (not aligned), (1, 2) and (5, 6) at 4, 5 and 8, 9 (aligned).
+    idx[0, :, 0] = [0, 1, 4, 5, 1, 2, 5, 6]
+    # Hashed levels at multiples of 32 bytes: even entries pair with the next.
+    idx[1, :, 0] = [0, 1, 2, 3, 64, 65, 67, 68]
+    idx[2, :, 0] = [10, 11, 13, 12, 21, 22, 30, 31]
+    # Four-wide: 2 of level 0, 3 of level 1, 3 of level 2 (13, 12 comes swapped).
+    assert bench.scatter_atomic_counts(_FakeIdx(idx), SHIFTED, torch.zeros((3, 1))) == (8, 2 * 4)
+    # Sectors (four entries each): level 0's entries 3..9 in 0, 1, 2; level 1's
+    # 0..3, 64..67 and 68; level 2's 10, 11 | 12, 13 | 21, 22 | 30, 31.
+    assert bench.gather_sector_counts(_FakeIdx(idx), SHIFTED, torch.zeros((3, 1))) == 3 + 3 + 4
+
+
+def test_launches_per_step():
+    big, small = 1 << 18, (1 << 18) - 1
+    assert bench.launches_per_step(synth.PAPER_HASH, big, False) == 2
+    assert bench.launches_per_step(synth.PAPER_HASH, small, False) == 1
+    assert bench.launches_per_step(synth.TINY, big, False) == 2          # one dense level, FP32: corner blocks
+    assert bench.launches_per_step(synth.TINY_BF16, big, False) == 1     # the serving networks' kernel
+    assert bench.launches_per_step(synth.PAPER_HASH, 1 << 19, True) == 3
+    for prec, n in ((synth.BF16X3, 4), (synth.FP16, 5), (synth.BF16, 5), (synth.FP32_TC, 3)):
+        assert bench.launches_per_step(synth.PRODUCT_BF16.with_(precision=prec), 1 << 19, True) == n
+    assert bench.launches_per_step(synth.TINY_BF16, 1 << 18, True) == 3
