@@ -292,7 +292,6 @@ npm_status npm_create(const npm_config* cfg, npm_handle** out) {
                 break;
             }
     const size_t sh = 2 * (size_t)d.grid_shift;  // in values
-    h->fwd_smem = npm::fwd_smem_bytes(d);
     h->train_smem = npm::train_smem_bytes(d);
 
     size_t nb = (size_t)(cfg->max_batch > 0 ? cfg->max_batch : 1);

@@ -277,25 +277,9 @@ struct Lobe {
 };
 
 // kappa and mean direction of one lobe from its raw outputs
-// (kappa', theta', phi'); theta = pi s(theta'), phi = 2 pi s(phi').
-__device__ __forceinline__ void decode_lobe(int kappa_act, float rk, float rt, float rp, Lobe& L,
-                                            float* theta, float* phi) {
-    L.kap = kappa_act == NPM_EXP ? expf(rk) : softplus(rk);
-    float th = kPi * logistic(rt);
-    float ph = 2.0f * kPi * logistic(rp);
-    float st, ct, sp, cp;
-    sincosf(th, &st, &ct);
-    sincosf(ph, &sp, &cp);
-    L.mu[0] = st * cp;
-    L.mu[1] = st * sp;
-    L.mu[2] = ct;
-    if (theta) *theta = th;
-    if (phi) *phi = ph;
-}
-
-// Forward-path variant of decode_lobe on the hardware approximations
-// (__expf, __logf, __sincosf, __fdividef). Arguments stay where those are
-// accurate: sine/cosine arguments in [-pi, pi] (absolute error < 4e-7);
+// (kappa', theta', phi'), theta = pi s(theta'), phi = 2 pi s(phi'), on the
+// hardware approximations (__expf, __logf, __sincosf, __fdividef). Arguments
+// stay where those are accurate: sine/cosine arguments in [-pi, pi] (absolute error < 4e-7);
 // exponentials of arguments |x| <~ 100 (relative error ~|x| 2^-24).
 // phi = 2 pi s(phi') is evaluated as pi + pi (2 s - 1), so that
 // (sin, cos)(phi) = -(sin, cos)(pi (2 s - 1)).
@@ -335,11 +319,6 @@ __device__ __forceinline__ void decode_lobe_fast(int kappa_act, float rk, float 
 __device__ __forceinline__ float vmf_scaled_norm(float k) {
     if (k < 1e-6f) return (1.0f + k) * kInv4Pi;
     return k / (2.0f * kPi * (-expm1f(-2.0f * k)));
-}
-
-__device__ __forceinline__ float vmf_eval(const Lobe& L, float cn, float wx, float wy, float wz) {
-    float d = L.mu[0] * wx + L.mu[1] * wy + L.mu[2] * wz;
-    return cn * expf(L.kap * (d - 1.0f));
 }
 
 // Forward-path variants: 1 - e^{-2k} by its series below k = 0.05 (truncation

@@ -36,7 +36,7 @@ struct npm_handle {
     float* stage = nullptr;    // device staging for the _host entry points
     cudaStream_t side[2] = {nullptr, nullptr};  // internal streams (host staging)
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
-    size_t fwd_smem = 0, train_smem = 0;
+    size_t train_smem = 0;
     int step = 0;
     npm::TcState* tc = nullptr;  // tensor-core (BF16) path state
     // Exponential moving average of the parameters (Sec. 5.3), evaluated by

@@ -2,9 +2,10 @@
 // arrangement of the weights for the MMAs, the model's tensor-core state and
 // the dispatch of the forward kernels (npm_tc_forward.cuh, npm_tc_tiny.cu).
 //
-// The training kernel runs one CTA of 256 threads over 128-sample tiles, two
-// threads per sample; activations and gradients are BF16 operand tiles in
-// shared memory (UMMA K-major layout), one elected thread issues
+// The training kernel runs groups of 256 threads over 128-sample tiles, two
+// threads per sample: two groups a CTA that share the weights, or one group and
+// up to three CTAs an SM. Activations and gradients are BF16 operand tiles in
+// shared memory (planes of 8 columns), one elected thread of a group issues
 // tcgen05.mma kind::f16 with FP32 accumulation in tensor memory and commits
 // to an mbarrier, and the threads read their accumulator lanes with
 // tcgen05.ld. Weights arrive once per CTA by a bulk asynchronous copy. Every
@@ -1044,8 +1045,11 @@ npm_status tc_create(npm_handle* h) {
         tr.g_bytes = off;
         tr.acc_col = cols;
         tr.acc_cols = (uint32_t)wide;
-        // Two groups where they fit; the small four-lobe networks run three
-        // CTAs of one group instead, sixteen lobes take the registers of one.
+        // Two groups where they fit; sixteen lobes take the registers of one.
+        // Networks of up to four lobes on grids without 2 features run the
+        // instance of one group and three CTAs an SM instead, whatever their
+        // layers' widths: measured on the small network alone, for which it was
+        // made, and not on wide layers of which fewer CTAs fit.
         auto lay = [&](int G) {
             tr.groups = G;
             tr.x_off = (uint32_t)G * tr.g_bytes;

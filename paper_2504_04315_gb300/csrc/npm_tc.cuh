@@ -289,11 +289,6 @@ __device__ __forceinline__ uint32_t f16_residual(uint32_t hp, float a, float b) 
     return pack_f16_sat(a - hf.x, b - hf.y);
 }
 
-// A pair of MMA operands in the model's operand format.
-__device__ __forceinline__ uint32_t pack_op(float a, float b, bool f16) {
-    return f16 ? pack_f16_sat(a, b) : pack_bf16(a, b);
-}
-
 // Byte offset of element (row, k) in a K-major no-swizzle tile whose rows
 // hold kp elements: 8x8 core matrices (128 bytes), K-adjacent core matrices
 // 128 bytes apart, 8-row groups kp/8 * 128 bytes apart.
@@ -378,10 +373,6 @@ __device__ __forceinline__ void vmf_sample_rp(const Lobe& L, float u1, float u2,
 
 // ------------------------------------------------------------ grid gathers
 
-// Table entry loads of the FP32 table.
-__device__ __forceinline__ float2 load_feat2(const float* g, uint32_t idx) {
-    return __ldg(reinterpret_cast<const float2*>(g) + idx);
-}
 // Features 4h .. 4h+3 of entry idx of a table with F = 4 or 8 features: the
 // raw 8-byte FP16 or 16-byte FP32 vector, widened to float4 at use.
 __device__ __forceinline__ uint2 load_raw4(const __half* g, uint32_t idx, int F, int h) {
@@ -573,9 +564,7 @@ __device__ __forceinline__ void gather_blocks4(const uint4* blk, uint32_t e, uin
 }
 
 // Entry index of corner c of a cell (the corner_idx8 formula for one
-// corner). The two-level gather below issues each corner's load as soon as
-// its index is formed, which schedules better there than forming all 16
-// indices first.
+// corner; corner 0 is a cell's corner block).
 __device__ __forceinline__ uint32_t corner_idx1(const DevCfg& cfg, int l, const Cell& cl, int c) {
     const uint32_t i = cl.c[0] + (c & 1), j = cl.c[1] + ((c >> 1) & 1), k = cl.c[2] + ((c >> 2) & 1);
     if ((cfg.dense_mask >> l) & 1u) {
@@ -613,10 +602,9 @@ enum : int { kOneBf16 = 0, kOneFp16 = 1, kTwoBf16 = 2, kTwoFp16 = 3, kThreeBf16 
 
 // Fused forward of the small serving networks (npm_tc_tiny.cu): radiance
 // mode, one dense level of 4 features, three layers of at most 32 outputs
-// (padded input 16), K = 4, softplus kappa, layer 0 sharing the activation
-// buffer. launch_tiny takes the general kernel's configuration, FP16 grid
-// and weight blob. With pdl the kernel is launched as
-// a programmatic dependent of the stream's previous kernel: its prologue
+// (padded input 16), K = 4, softplus kappa. launch_tiny takes the general
+// kernel's configuration, FP16 grid and weight blob. With pdl the kernel is
+// launched as a programmatic dependent of the stream's previous kernel: its prologue
 // (tensor-memory allocation, copies of the weights and grid) overlaps that
 // kernel, which therefore must not write the weights or the grid.
 bool tiny_qualifies(const TcCfg& c);

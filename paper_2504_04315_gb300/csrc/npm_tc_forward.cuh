@@ -591,7 +591,8 @@ __device__ __forceinline__ void decode_row(const DevCfg& cfg, const uint32_t (&r
 // the lobe choice takes the running sum of the weights in lobe order (a
 // serial scan, the same rounding as the thread-per-row form) and a ballot;
 // every lane samples its own lobe and the chosen lane's direction is
-// broadcast. Measured against tc_decode (one thread per query).
+// broadcast. Slower than decode_row (one thread per query), so a tuning override
+// selects it: split BF16, paper-shaped grid, 1.60 against 1.96 G queries/s.
 template <int KMAX>
 __device__ __forceinline__ void tc_decode_warp(const TcCfg& tc, const float* __restrict__ sRaw, int warp, int lane,
                                                int64_t j0, int64_t n, int64_t ld, const float* __restrict__ uin,
@@ -1005,12 +1006,14 @@ cudaError_t launch_fwd_ops(const TcCfg& c, const void* grid, const uint4* blk, c
         // groups (2^18 queries of a 16-wide network: 44 us, with the part in
         // shared memory 47, before elect_one). 2-feature grids' has three
         // groups with two levels' gathers in flight, against four with one,
-        // whose rounds of tiles take 1.37 times as long: whichever needs less
-        // for the rounds of this batch (GB300, paper-shaped grid, three and
-        // four groups: 3,000 queries 16.9 and 18.9 us; 2^16 41.0 and 36.6;
-        // 2^17 63.6 and 59.9; 2^18 100.8 and 110.7; 2^20 345 and 373). Of the
-        // two-part formats three groups gain nothing (FP32 accuracy, 2^20:
-        // 320 against 312).
+        // whose rounds of tiles take about 1.37 times as long: whichever needs
+        // less for the rounds of this batch (GB300, 16 levels, 64-wide layers,
+        // three and four groups: 3,000 queries 16.5 and 18.5 us; 2^16 40.4 and
+        // 36.5; 2^17 63.2 and 60.3; 2^18 97.6 and 109.9; 2^20 343 and 378). The
+        // ratio is 1.36 to 1.42 on 16 levels and 1.23 to 1.25 on two to eight, where
+        // the rule errs on large batches (2^18 on eight levels: 69.7 and 70.8;
+        // 2^20: 237 and 227, two levels 173 and 169). Of the two-part formats
+        // three groups gain nothing (FP32 accuracy, 2^20: 320 against 312).
         if (c.base.feat == 4 && 4u * fwd_group_cols<OPS, false>(c) <= 512u)
             return launch_fwd<8, 4, OPS, false, 4, false>(c, grid, blk, wblob, qb, max_n, status, wait_limit, st);
         if (c.base.feat == 2 && fwd_group_count<OPS, false>(c, 3) == 3) {
