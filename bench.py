@@ -127,7 +127,7 @@ def mlp_flops(w):
 
 # DRAM bytes of one FP32 k_forward_tc launch on the paper-shaped workload
 # (2^20 queries) from the ncu capture summarised in profiles/.
-FP32_FORWARD_DRAM_BYTES = 147034880 + 17128704
+FP32_FORWARD_DRAM_BYTES = 148074240 + 17288960
 
 # Algorithmic work per query of the tensor-core forward on the tiny model
 # (K = 4): transcendentals of the vMF decode, sample and pdf (softmax 4,

@@ -171,12 +171,14 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp,
 
 // Entries of a chunk of corner blocks (kept up to date as a whole).
 constexpr int kBlkChunk = 1024;
-// Queries from which a batch uses them. Tables in the L2, without and with
-// blocks (GB300; paper-shaped hash grid in FP32 and FP16, eight dense levels
-// of four features in split BF16): 2^16 queries 36 and 37, 29 and 27, 21 and
-// 21 us; 2^17 60 and 60, 47 and 41, 33 and 31, less than bringing stale blocks
-// up to date takes (9 us); 2^18 111 and 101, 87 and 73, 60 and 52; 2^20 398
-// and 344, 288 and 230, 204 and 158.
+// Queries from which a batch uses them. Without and with blocks that are up to
+// date (GB300, us; 2^18 and 2^20 queries): paper-shaped hash grid in FP32 110
+// and 97, 398 and 343, in FP16 86 and 70, 288 and 229; eight dense levels of
+// four features in FP32 83 and 73, in FP16 55 and 43, 204 and 140. At 2^17 they
+// give 0 to 6 us. The first batch after an update also pays for bringing them
+// up to date, 11 to 13 us on the hash grid and 16 on the dense levels, as does
+// every batch of an FP32 model whose address was handed out: with an update
+// before each batch they repay that from a few hundred thousand queries on.
 constexpr int64_t kBlkMinQueries = 1 << 18;
 
 // Rewrites the chunks of corner blocks whose parameters have changed since
