@@ -131,22 +131,11 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp,
     const TcLayer& ly = tc.layer[l];
     for (int m = 0; m < l; ++m) mlp += tc.layer[m].K * tc.layer[m].N;
     // Whole rows (outputs) at a time, a thread per weight.
-    __shared__ int bad[17];
     const int rows = (int)blockDim.x / ly.Kp, r = (int)threadIdx.x / ly.Kp, k = (int)threadIdx.x % ly.Kp;
-    for (int n0 = blockIdx.x * rows; n0 < ly.Np; n0 += gridDim.x * rows) {
-        const int nn = n0 + r;
-        const bool mine = r < rows && nn < ly.Np;
-        float v = (mine && nn < ly.N && k < ly.K) ? mlp[nn * ly.K + k] : 0.0f;
-        // FP32 arithmetic: a NaN weight makes its output NaN for every query,
-        // which a hidden layer's ReLU takes for zero (three_bf16).
-        if (tc.wparts == 3 && l + 1 < tc.base.n_layers && __syncthreads_or(isnan(v))) {
-            if (threadIdx.x < 17) bad[threadIdx.x] = 0;
-            __syncthreads();
-            if (isnan(v)) bad[r] = 1;
-            __syncthreads();
-            if (bad[r]) v = 0.0f;
-        }
-        if (!mine) continue;
+    bool nan = false;
+    for (int nn = blockIdx.x * rows + r; r < rows && nn < ly.Np; nn += gridDim.x * rows) {
+        const float v = (nn < ly.N && k < ly.K) ? mlp[nn * ly.K + k] : 0.0f;
+        nan = nan || isnan(v);
         uint8_t* at = blob + ly.w_off + tile_off(nn, k, ly.Kp);
         if (tc.f16) {
             // FP16 high part and FP16 residual (the weights to ~22 bits)
@@ -165,6 +154,14 @@ __global__ void k_tc_weights(const __grid_constant__ TcCfg tc, const float* mlp,
             rest -= __bfloat162float(b);
         }
     }
+    // FP32 arithmetic: a NaN weight makes its output NaN for every query, which
+    // a hidden layer's ReLU takes for zero (three_bf16). Rare: the rows of this
+    // block that hold one are cleared once all are written.
+    if (tc.wparts == 3 && l + 1 < tc.base.n_layers && __syncthreads_or(nan))
+        for (int nn = blockIdx.x * rows + r; r < rows && nn < ly.N; nn += gridDim.x * rows)
+            if (k < ly.K && isnan(mlp[nn * ly.K + k]))
+                for (int i = 0; i < 3 * ly.Kp; ++i)
+                    *reinterpret_cast<uint16_t*>(blob + ly.w_off + tile_off(nn, i / 3, ly.Kp) + (i % 3) * tc.w_bytes) = 0;
 }
 
 // ------------------------------------------------------- corner blocks
