@@ -2,8 +2,10 @@
 more): the same bytes as the table, so a large batch gives exactly what the
 table gives its two halves, on every table format, with levels of the
 smallest resolutions and hashed levels between; and they follow the
-parameters through set_params, a training step, the weight average and a
-write through npm_params_device."""
+parameters through set_params, a training step, the weight average, a write
+through npm_params_device (in graphs captured before the address was asked for
+too) and a query on another stream beside an update; memory only for handles
+and servers whose batches are large enough."""
 import numpy as np
 import pytest
 
